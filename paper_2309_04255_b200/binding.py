@@ -130,7 +130,8 @@ def _check(code: int, where: str):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the raw handle of the current stream (building the Stream object costs more than the rest of a small call)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -200,8 +201,8 @@ class Verifier:
         return {
             "logits": torch.empty((n, self.cfg.vocab), dtype=torch.float32, device=dev) if want_logits else None,
             "argmax": torch.empty(n, dtype=torch.int32, device=dev),
-            "accepted_path": torch.full((self.max_tree,), -1, dtype=torch.int32, device=dev),
-            "scalars": torch.zeros(8, dtype=torch.int32, device=dev),
+            "accepted_path": torch.empty(self.max_tree, dtype=torch.int32, device=dev),   # -1 past the path, set by the pass
+            "scalars": torch.empty(8, dtype=torch.int32, device=dev),
         }
 
     def verify_tree(self, prefix_len: int, tokens: torch.Tensor, parent: torch.Tensor, out=None, want_logits=True):
@@ -223,7 +224,7 @@ class Verifier:
             "logits": torch.empty((n_new, self.cfg.vocab), dtype=torch.float32, device=dev) if want_logits else None,
             "topk_ids": torch.empty((n_new, max(top_k, 1)), dtype=torch.int32, device=dev),
             "topk_probs": torch.empty((n_new, max(top_k, 1)), dtype=torch.float32, device=dev),
-            "status": torch.zeros(1, dtype=torch.int32, device=dev),
+            "status": torch.empty(1, dtype=torch.int32, device=dev),
         }
         _check(lib().llmcad_extend_tree(self.ctx, _ptr(self.packed), _ptr(self.kv), prefix_len, _ptr(tokens), _ptr(parent),
                                         n_old, n_tree, top_k, _ptr(out["logits"]), _ptr(out["topk_ids"]),
@@ -250,8 +251,8 @@ class Verifier:
     # ---- single steps
     def accept_compact(self, prefix_len: int, tokens, parent, argmax, compact: bool = True):
         n = tokens.numel()
-        path = torch.full((self.max_tree,), -1, dtype=torch.int32, device=self.device)
-        scalars = torch.zeros(8, dtype=torch.int32, device=self.device)
+        path = torch.empty(self.max_tree, dtype=torch.int32, device=self.device)
+        scalars = torch.empty(8, dtype=torch.int32, device=self.device)
         _check(lib().llmcad_accept_compact(self.ctx, self.kv.data_ptr() if compact else None, prefix_len, _ptr(tokens),
                                            _ptr(parent), _ptr(argmax), n, _ptr(path), _ptr(scalars), _stream()),
                "llmcad_accept_compact")

@@ -103,6 +103,7 @@ struct llmcad_ctx {
     // (LLMCAD_COMP=0) turns the lo planes off.
     bool comp = false;
     // activations of up to 128 nodes; xn, q, att and h hold two planes of 128 rows (hi, lo)
+    void *arena = nullptr;    // the one allocation that holds every workspace below
     float *x = nullptr;       // residual stream [128][d] fp32
     void *xn = nullptr;       // normalised GEMM input [2][128][d]
     void *q = nullptr;        // rotated queries [2][128][d]
@@ -111,12 +112,11 @@ struct llmcad_ctx {
     void *kv_lo = nullptr;    // bf16 remainders of the current layer's tree keys and values [2][H][128][hd]
     float *logits = nullptr;  // [128][V], used when the caller does not want logits
     TreeBuffers tb{};
+    double *inv_freq = nullptr;   // rope_base^(-2t/head_dim), t < head_dim/2
     int32_t *ibuf = nullptr;  // tokens[128], parent[128], argmax[128], path[128], scalars[8], chain[128]
     float *partials = nullptr;            // segment workspace of the tensor-core GEMMs
     size_t partial_floats = 0;
     float *ssq[2] = {nullptr, nullptr};   // partial sums of squares for the folded attention / FFN norms
-    float *attn_ws = nullptr;
-    uint32_t *attn_counters = nullptr;
     // completion counters through which the kernels of a tensor-core pass hand over (common.cuh): one per
     // kernel, taken in launch order, all zeroed at the start of a forward. Off by default: measured on B200
     // (7B shape, 32 nodes) the hand-over through counters costs 4 % of the pass against grid dependencies
@@ -285,8 +285,7 @@ int run_attention(llmcad_ctx *ctx, const void *q, const void *k, const void *v, 
             ctx->launches += launched;
             return LLMCAD_OK;
         }
-        CUDA_TRY(launch_attention_tc(q, k, v, c.n_heads, c.head_dim, kv_stride, P, n, ctx->tb.anc, o, ctx->attn_ws,
-                                     ctx->attn_counters, ctx->n_sms, status, st, &launched, ctx->next_trace(), comp ? 1 : 0,
+        CUDA_TRY(launch_attention_tc(q, k, v, c.n_heads, c.head_dim, kv_stride, P, n, ctx->tb.anc, o, ctx->n_sms, status, st, &launched, ctx->next_trace(), comp ? 1 : 0,
                                      ctx->kv_lo, n_tree, q_first, sync));
         ctx->launches += launched;
         return LLMCAD_OK;
@@ -301,22 +300,22 @@ int run_attention(llmcad_ctx *ctx, const void *q, const void *k, const void *v, 
 // Decoder forward over the nodes n_old .. n_tree-1 of a tree of n_tree nodes (all of them when
 // n_old = 0): tree prep of the whole tree, embedding, all layers; K/V of node i go to cache slot
 // P+i, where the nodes below n_old already have theirs. When logits != nullptr the final norm and
-// lm_head run too (one row per processed node).
+// lm_head run too (one row per processed node). The status word starts from this tree's own check, or, with
+// keep_status, stays as an earlier chunk of the same call left it if that found an error.
 int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens,
-                const int32_t *parent, int n_tree, float *logits, int32_t *status, cudaStream_t st, int n_old = 0)
+                const int32_t *parent, int n_tree, float *logits, int32_t *status, cudaStream_t st, int n_old = 0,
+                bool keep_status = false)
 {
     const llmcad_config &c = ctx->cfg;
     const int d = c.d_model, f = c.d_ffn, hd = c.head_dim, H = c.n_heads, S = c.max_seq;
     const int n = n_tree - n_old;                    // nodes this call computes
     const int n_pad = (n + 15) / 16 * 16;
-    const int32_t *new_tokens = tokens + n_old;
     const char *base = static_cast<const char *>(packed);
     int rc;
     if ((rc = ensure_weight_maps(ctx, packed)) != LLMCAD_OK) return rc;
     if ((rc = ensure_act_maps(ctx, n_pad)) != LLMCAD_OK) return rc;
 
-    CUDA_TRY(launch_tree_prep(parent, tokens, n_tree, P, c.vocab, hd, c.rope_base, ctx->tb, status, st));
-    ctx->launches += 2;
+    ctx->launches++;
     const float2 *rope_new = ctx->tb.rope_cs + (size_t)n_old * (hd / 2);
     const size_t kv_layer = (size_t)2 * H * S * hd * ctx->elem;
 
@@ -326,9 +325,9 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
         // partial sums of squares; the consuming GEMM scales its accumulators by the per-node
         // rsqrt(mean(x^2) + eps). Activations travel as bf16 hi + lo planes (ctx->comp).
         const int tiles4 = 4 * ((d + 127) / 128);
-        CUDA_TRY(launch_embed_norm(base + ctx->lay.tok_embed, new_tokens, n, d,
-                                   c.n_layers > 0 ? base + ctx->lay.attn_norm : base + ctx->lay.final_norm, ctx->x, ctx->xn,
-                                   ctx->ssq[0], ctx->comp ? 1 : 0, status, st));
+        CUDA_TRY(launch_prep_embed(parent, tokens, n_tree, n_old, P, c.vocab, hd, ctx->inv_freq, ctx->tb, base + ctx->lay.tok_embed,
+                                   c.dtype, d, c.n_layers > 0 ? base + ctx->lay.attn_norm : base + ctx->lay.final_norm, ctx->x, ctx->xn,
+                                   ctx->ssq[0], ctx->comp ? 1 : 0, status, keep_status ? 1 : 0, st));
         auto qkv_ep = [&](int l, int parts) {
             char *kl = static_cast<char *>(kv_cache) + kv_layer * (size_t)l;
             EpiParams ep{};
@@ -405,7 +404,8 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
         return LLMCAD_OK;
     }
 
-    CUDA_TRY(launch_embed(base + ctx->lay.tok_embed, c.dtype, new_tokens, n, d, ctx->x, status, st));
+    CUDA_TRY(launch_prep_embed(parent, tokens, n_tree, n_old, P, c.vocab, hd, ctx->inv_freq, ctx->tb, base + ctx->lay.tok_embed, c.dtype,
+                               d, nullptr, ctx->x, nullptr, nullptr, 0, status, keep_status ? 1 : 0, st));
     for (int l = 0; l < c.n_layers; ++l) {
         const char *lb = base + ctx->lay.layer_bytes * (size_t)l;
         char *kl = static_cast<char *>(kv_cache) + kv_layer * (size_t)l;
@@ -523,23 +523,27 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
     }
 
     const size_t d = cfg->d_model, f = cfg->d_ffn, hd = cfg->head_dim;
-    auto alloc = [&](void **p, size_t bytes) {
-        if (!cuda_ok(cudaMalloc(p, bytes), "cudaMalloc")) return false;
-        return cuda_ok(cudaMemset(*p, 0, bytes), "cudaMemset");
+    // every workspace out of one allocation
+    struct Want { void **p; size_t off; };
+    std::vector<Want> wants;
+    size_t arena_bytes = 0;
+    auto want = [&](void **p, size_t bytes) {
+        wants.push_back({p, arena_bytes});
+        arena_bytes = align_up(arena_bytes + bytes, 1024);
     };
-    bool ok = true;
-    ok = ok && alloc((void **)&ctx->x, 128 * d * 4);
-    ok = ok && alloc(&ctx->xn, 2 * kLoRows * d * ctx->elem);
-    ok = ok && alloc(&ctx->q, 2 * kLoRows * d * ctx->elem);
-    ok = ok && alloc(&ctx->att, 2 * kLoRows * d * ctx->elem);
-    ok = ok && alloc(&ctx->h, 2 * kLoRows * f * ctx->elem);
-    ok = ok && alloc(&ctx->kv_lo, 2 * kLoRows * d * ctx->elem);
-    ok = ok && alloc((void **)&ctx->logits, (size_t)128 * cfg->vocab * 4);
-    ok = ok && alloc((void **)&ctx->tb.depth, 128 * 4);
-    ok = ok && alloc((void **)&ctx->tb.pos, 128 * 4);
-    ok = ok && alloc((void **)&ctx->tb.anc, 128 * 16);
-    ok = ok && alloc((void **)&ctx->tb.rope_cs, 128 * (hd / 2) * sizeof(float2));
-    ok = ok && alloc((void **)&ctx->ibuf, (520 + 128) * 4);
+    want((void **)&ctx->x, 128 * d * 4);
+    want(&ctx->xn, 2 * kLoRows * d * ctx->elem);
+    want(&ctx->q, 2 * kLoRows * d * ctx->elem);
+    want(&ctx->att, 2 * kLoRows * d * ctx->elem);
+    want(&ctx->h, 2 * kLoRows * f * ctx->elem);
+    want(&ctx->kv_lo, 2 * kLoRows * d * ctx->elem);
+    want((void **)&ctx->logits, (size_t)128 * cfg->vocab * 4);
+    want((void **)&ctx->tb.depth, 128 * 4);
+    want((void **)&ctx->tb.pos, 128 * 4);
+    want((void **)&ctx->tb.anc, 128 * 16);
+    want((void **)&ctx->tb.rope_cs, 128 * (hd / 2) * sizeof(float2));
+    want((void **)&ctx->inv_freq, (hd / 2) * sizeof(double));
+    want((void **)&ctx->ibuf, (520 + 128) * 4);
     {
         // segment workspace: the GEMM with the most tiles of this model (or 256 tiles, for the single-GEMM entry points)
         int max_tiles = 256;
@@ -547,14 +551,14 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
             if ((int)((rows + 127) / 128) > max_tiles) max_tiles = (int)((rows + 127) / 128);
         const int max_pad = (cfg->max_tree + 15) / 16 * 16;
         ctx->partial_floats = ctx->tc_gemm ? gemm_tc_partial_floats(ctx->n_sms, max_tiles, max_pad) : 64;
-        ok = ok && alloc((void **)&ctx->partials, ctx->partial_floats * 4);
+        want((void **)&ctx->partials, ctx->partial_floats * 4);
     }
     const size_t ssq_floats = (size_t)4 * ((d + 127) / 128) * LLMCAD_MAX_TREE;
-    ok = ok && alloc((void **)&ctx->ssq[0], ssq_floats * 4);
-    ok = ok && alloc((void **)&ctx->ssq[1], ssq_floats * 4);
-    ok = ok && alloc((void **)&ctx->attn_ws, attention_tc_workspace_bytes(cfg->n_heads, ctx->n_sms));
-    ok = ok && alloc((void **)&ctx->attn_counters, (size_t)cfg->n_heads * 8 * 4);
-    ok = ok && alloc((void **)&ctx->sync_ctrs, kSyncCounters * sizeof(uint32_t));
+    want((void **)&ctx->ssq[0], ssq_floats * 4);
+    want((void **)&ctx->ssq[1], ssq_floats * 4);
+    want((void **)&ctx->sync_ctrs, kSyncCounters * sizeof(uint32_t));
+    bool ok = cuda_ok(cudaMalloc(&ctx->arena, arena_bytes), "cudaMalloc") && cuda_ok(cudaMemset(ctx->arena, 0, arena_bytes), "cudaMemset");
+    for (const Want &w : wants) *w.p = static_cast<char *>(ctx->arena) + w.off;
     {
         const char *e = getenv("LLMCAD_SYNC_COUNTERS");
         ctx->use_counters = e != nullptr && atoi(e) != 0;
@@ -562,7 +566,10 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
     if (ok) {
         std::vector<int32_t> chain(128);
         for (int i = 0; i < 128; ++i) chain[i] = i - 1;
-        ok = cuda_ok(cudaMemcpy(ctx->chain_dev(), chain.data(), 128 * 4, cudaMemcpyHostToDevice), "cudaMemcpy");
+        std::vector<double> freq(hd / 2);
+        for (size_t t = 0; t < hd / 2; ++t) freq[t] = pow((double)cfg->rope_base, -2.0 * (double)t / (double)hd);
+        ok = ok && cuda_ok(cudaMemcpy(ctx->inv_freq, freq.data(), freq.size() * sizeof(double), cudaMemcpyHostToDevice), "cudaMemcpy");
+        ok = ok && cuda_ok(cudaMemcpy(ctx->chain_dev(), chain.data(), 128 * 4, cudaMemcpyHostToDevice), "cudaMemcpy");
     }
     if (!ok) {
         llmcad_destroy(ctx);
@@ -575,11 +582,7 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
 void llmcad_destroy(llmcad_ctx *ctx)
 {
     if (ctx == nullptr) return;
-    void *ptrs[] = {ctx->x, ctx->xn, ctx->q, ctx->att, ctx->h, ctx->kv_lo, ctx->logits, ctx->tb.depth, ctx->tb.pos, ctx->tb.anc,
-                    ctx->tb.rope_cs, ctx->ibuf, ctx->partials, ctx->attn_ws, ctx->attn_counters, ctx->sync_ctrs, ctx->ssq[0],
-                    ctx->ssq[1]};
-    for (void *p : ptrs)
-        if (p != nullptr) cudaFree(p);
+    if (ctx->arena != nullptr) cudaFree(ctx->arena);
     for (auto &t : ctx->timed) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
     for (auto e : ctx->event_pool) cudaEventDestroy(e);
     delete ctx;
@@ -651,9 +654,9 @@ int llmcad_pack_globals(llmcad_ctx *ctx, const llmcad_global_weights *src, void 
     return LLMCAD_OK;
 }
 
-int llmcad_verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t prefix_len,
-                       const int32_t *tree_tokens, const int32_t *parent_idx, int32_t n, const llmcad_result *out,
-                       void *stream)
+// path_fill: entries of out->accepted_path behind the path, up to this many in all, become -1
+static int verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t prefix_len, const int32_t *tree_tokens,
+                       const int32_t *parent_idx, int32_t n, const llmcad_result *out, int path_fill, void *stream)
 {
     int rc = check_pass_args(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n);
     if (rc != LLMCAD_OK) return rc;
@@ -663,15 +666,19 @@ int llmcad_verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int3
     const llmcad_config &c = ctx->cfg;
     int32_t *status = out->scalars + LLMCAD_S_STATUS;
     float *logits = out->logits != nullptr ? out->logits : ctx->logits;
-    CUDA_TRY(cudaMemsetAsync(out->scalars, 0, 8 * sizeof(int32_t), st));
     if ((rc = run_forward(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n, logits, status, st)) != LLMCAD_OK)
         return rc;
     CUDA_TRY(launch_argmax(logits, n, c.vocab, out->argmax, status, st));
-    CUDA_TRY(launch_accept(parent_idx, tree_tokens, out->argmax, n, prefix_len, out->accepted_path, out->scalars, st));
-    CUDA_TRY(launch_compact(kv_cache, c.dtype, c.n_layers, c.n_heads, c.max_seq, c.head_dim, prefix_len,
-                            out->accepted_path, out->scalars, st));
-    ctx->launches += 3;
+    CUDA_TRY(launch_search_rollback(parent_idx, tree_tokens, out->argmax, n, prefix_len, c.vocab, 0, out->accepted_path, path_fill,
+                                    out->scalars, kv_cache, c.dtype, c.n_layers, c.n_heads, c.max_seq, c.head_dim, st));
+    ctx->launches += 2;
     return LLMCAD_OK;
+}
+
+int llmcad_verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t prefix_len, const int32_t *tree_tokens,
+                                  const int32_t *parent_idx, int32_t n, const llmcad_result *out, void *stream)
+{
+    return verify_tree(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n, out, ctx ? ctx->cfg.max_tree : 0, stream);
 }
 
 int llmcad_verify_tree_host(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t prefix_len,
@@ -690,7 +697,7 @@ int llmcad_verify_tree_host(llmcad_ctx *ctx, const void *packed, void *kv_cache,
     dev.argmax = ctx->argmax_dev();
     dev.accepted_path = ctx->path_dev();
     dev.scalars = ctx->scalars_dev();
-    rc = llmcad_verify_tree(ctx, packed, kv_cache, prefix_len, ctx->tokens_dev(), ctx->parent_dev(), n, &dev, stream);
+    rc = verify_tree(ctx, packed, kv_cache, prefix_len, ctx->tokens_dev(), ctx->parent_dev(), n, &dev, 0, stream);
     if (rc != LLMCAD_OK) return rc;
     // argmax[128], path[128] and scalars[8] are contiguous in the context's integer buffer
     CUDA_TRY(cudaMemcpyAsync(out->argmax, ctx->argmax_dev(), n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -710,14 +717,13 @@ int llmcad_prefill(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t 
     if ((long long)prefix_len + n > ctx->cfg.max_seq) return LLMCAD_ERR_CAPACITY;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int32_t *status = ctx->scalars_dev() + LLMCAD_S_STATUS;
-    CUDA_TRY(cudaMemsetAsync(ctx->scalars_dev(), 0, 8 * sizeof(int32_t), st));
     const int chunk = ctx->cfg.max_tree;
     for (int done = 0; done < n; done += chunk) {
         const int m = n - done < chunk ? n - done : chunk;
         const bool last = done + m == n;
         // a chain whose "prefix" is everything before it; every node is committed, nothing to roll back
         int rc = run_forward(ctx, packed, kv_cache, prefix_len + done, tokens + done, ctx->chain_dev(), m,
-                             (last && last_logits != nullptr) ? ctx->logits : nullptr, status, st);
+                             (last && last_logits != nullptr) ? ctx->logits : nullptr, status, st, 0, done > 0);
         if (rc != LLMCAD_OK) return rc;
         if (last && last_logits != nullptr)
             CUDA_TRY(cudaMemcpyAsync(last_logits, ctx->logits + (size_t)(m - 1) * ctx->cfg.vocab,
@@ -737,7 +743,6 @@ int llmcad_extend_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int3
     if (top_k > ctx->cfg.vocab) return LLMCAD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float *lg = logits != nullptr ? logits : ctx->logits;
-    CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
     if ((rc = run_forward(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n_tree, lg, status, st, n_old)) != LLMCAD_OK)
         return rc;
     if (top_k > 0) {
@@ -754,9 +759,8 @@ int llmcad_tree_prep(const int32_t *parent_idx, int32_t n, int32_t prefix_len, i
     if (n < 1 || prefix_len < 0) return LLMCAD_ERR_INVALID_ARG;
     if (n > LLMCAD_MAX_TREE) return LLMCAD_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
     TreeBuffers tb{depth, pos, anc, nullptr};
-    CUDA_TRY(launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, 0, 0.f, tb, status, st));
+    CUDA_TRY(launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, tb, status, st));
     return LLMCAD_OK;
 }
 
@@ -770,17 +774,10 @@ int llmcad_accept_compact(llmcad_ctx *ctx, void *kv_cache, int32_t prefix_len, c
     if ((long long)prefix_len + n > ctx->cfg.max_seq) return LLMCAD_ERR_CAPACITY;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const llmcad_config &c = ctx->cfg;
-    CUDA_TRY(cudaMemsetAsync(scalars, 0, 8 * sizeof(int32_t), st));
-    // the search trusts the tree: validate it first (a malformed tree lands in scalars[status])
-    CUDA_TRY(launch_tree_prep(parent_idx, tree_tokens, n, prefix_len, c.vocab, c.head_dim, c.rope_base, ctx->tb,
-                              scalars + LLMCAD_S_STATUS, st));
-    CUDA_TRY(launch_accept(parent_idx, tree_tokens, argmax, n, prefix_len, accepted_path, scalars, st));
-    ctx->launches += 2;
-    if (kv_cache != nullptr) {
-        CUDA_TRY(launch_compact(kv_cache, c.dtype, c.n_layers, c.n_heads, c.max_seq, c.head_dim, prefix_len, accepted_path,
-                                scalars, st));
-        ctx->launches++;
-    }
+    // the search trusts the tree: the kernel validates it first (a malformed tree lands in scalars[status])
+    CUDA_TRY(launch_search_rollback(parent_idx, tree_tokens, argmax, n, prefix_len, c.vocab, 1, accepted_path, c.max_tree, scalars,
+                                    kv_cache, c.dtype, c.n_layers, c.n_heads, c.max_seq, c.head_dim, st));
+    ctx->launches++;
     return LLMCAD_OK;
 }
 
@@ -796,10 +793,7 @@ int llmcad_tree_attention(llmcad_ctx *ctx, const void *q, const void *k, const v
         return LLMCAD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int32_t *status = ctx->scalars_dev() + LLMCAD_S_STATUS;
-    CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
-    TreeBuffers tb = ctx->tb;
-    tb.rope_cs = nullptr;
-    CUDA_TRY(launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, 0, 0.f, tb, status, st));
+    CUDA_TRY(launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, ctx->tb, status, st));
     ctx->launches++;
     return run_attention(ctx, q, k, v, kv_stride, prefix_len, n, o, false, status, st);
 }

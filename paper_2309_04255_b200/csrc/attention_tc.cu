@@ -529,19 +529,12 @@ attention_tc_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__
     if (trace && threadIdx.x == 0 && cta < 256) trace[(size_t)cta * 16 + 12] = global_timer_ns();
 }
 
-size_t attention_tc_workspace_bytes(int n_heads, int n_sms)
-{
-    (void)n_heads; (void)n_sms;
-    return 256;   // the merge runs through distributed shared memory; no global workspace is needed
-}
-
 cudaError_t launch_attention_tc(const void *q, const void *k, const void *v, int n_heads, int hd, int kv_stride, int P,
-                                int n, const uint32_t *anc, void *o, float *ws, uint32_t *counters, int n_sms,
+                                int n, const uint32_t *anc, void *o, int n_sms,
                                 int32_t *status, cudaStream_t st, int *launched, unsigned long long *trace, int comp,
                                 const void *kv_lo, int n_tree, int q_first, const AttnSync *sync)
 {
     if (n_tree <= 0) n_tree = n;
-    (void)ws; (void)counters;
     if (hd != kHd) return cudaErrorInvalidValue;
     const int n_pad = (n + 15) / 16 * 16;
     const int n_tiles = (P + n_tree + kKeyTile - 1) / kKeyTile;

@@ -5,8 +5,6 @@
 
 namespace llmcad {
 
-size_t attention_tc_workspace_bytes(int n_heads, int n_sms);
-
 // Hand-over counters of an attention launch inside a pass (common.cuh, "completion counters"): the kernel waits
 // until *dep_ctr has reached dep_target instead of for its grid dependency, and every CTA adds one to *done_ctr
 // when its rows of the output are written; the launcher reports how many arrivals that makes.
@@ -25,7 +23,7 @@ struct AttnSync {
 // n_tree > 0: the queries are only the tree nodes q_first .. q_first + n - 1 (anc holds the rows of
 // all n_tree nodes), the keys the prefix and all n_tree tree nodes; 0 means n_tree = n, q_first = 0.
 cudaError_t launch_attention_tc(const void *q, const void *k, const void *v, int n_heads, int hd, int kv_stride, int P,
-                                int n, const uint32_t *anc, void *o, float *ws, uint32_t *counters, int n_sms,
+                                int n, const uint32_t *anc, void *o, int n_sms,
                                 int32_t *status, cudaStream_t st, int *launched, unsigned long long *trace = nullptr, int comp = 0,
                                 const void *kv_lo = nullptr, int n_tree = 0, int q_first = 0, const AttnSync *sync = nullptr);
 

@@ -264,19 +264,18 @@ struct TreeBuffers {
     float2 *rope_cs;    // [n][hd/2]
 };
 
-cudaError_t launch_tree_prep(const int32_t *parent, const int32_t *tokens, int n, int P, int vocab, int hd,
-                             float rope_base, TreeBuffers tb, int32_t *status, cudaStream_t st);
-cudaError_t launch_embed(const void *E, int dtype, const int32_t *tokens, int n, int d, float *x, const int32_t *status,
-                         cudaStream_t st);
-cudaError_t launch_embed_norm(const void *E, const int32_t *tokens, int n, int d, const void *gain, float *x, void *xg,
-                              float *ssq, int comp, const int32_t *status, cudaStream_t st);
+cudaError_t launch_tree_prep(const int32_t *parent, const int32_t *tokens, int n, int P, int vocab, TreeBuffers tb, int32_t *status,
+                             cudaStream_t st);
+// E == nullptr: the mask table only; gain == nullptr: the residual stream only
+cudaError_t launch_prep_embed(const int32_t *parent, const int32_t *tokens, int n_tree, int n_old, int P, int vocab, int hd,
+                              const double *inv_freq, TreeBuffers tb, const void *E, int dtype, int d, const void *gain, float *x,
+                              void *xg, float *ssq, int comp, int32_t *status, int keep, cudaStream_t st);
 cudaError_t launch_rmsnorm(const float *x, const void *g, int dtype, int n, int d, float eps, void *out,
                            const int32_t *status, cudaStream_t st);
 cudaError_t launch_argmax(const float *logits, int n, int vocab, int32_t *argmax, int32_t *status, cudaStream_t st);
-cudaError_t launch_accept(const int32_t *parent, const int32_t *tokens, const int32_t *argmax, int n, int P,
-                          int32_t *path, int32_t *scalars, cudaStream_t st);
-cudaError_t launch_compact(void *kv, int dtype, int n_layers, int n_heads, int S, int hd, int P, const int32_t *path,
-                           const int32_t *scalars, cudaStream_t st);
+cudaError_t launch_search_rollback(const int32_t *parent, const int32_t *tokens, const int32_t *argmax, int n, int P, int vocab,
+                                   int check, int32_t *path, int path_len, int32_t *scalars, void *kv, int dtype, int n_layers,
+                                   int n_heads, int S, int hd, cudaStream_t st);
 size_t tiled_weight_bytes(int n_out, int n_in);
 cudaError_t launch_tile_weight(const void *w, int n_out, int n_in, void *dst, cudaStream_t st);
 // INT4 weights (pack.cu): bytes of one (128 rows x 64 columns) tile: 4 KB of codes + 128 exponents

@@ -78,9 +78,7 @@ extern "C" int llmcad_tree_attention_noalloc(const void *q, const void *k, const
     int32_t *status = reinterpret_cast<int32_t *>(base + 1024 + 2048);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the array keeps what the previous call left: the status word must start at zero
-    cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int32_t), st);
-    if (e == cudaSuccess) e = launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, 0, 0.f, tb, status, st);
+    cudaError_t e = launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, tb, status, st);     // also sets the status word
     if (e == cudaSuccess) {
         int sms = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -89,7 +87,7 @@ extern "C" int llmcad_tree_attention_noalloc(const void *q, const void *k, const
             if (attention_prefers_t5(n))
                 e = launch_attention_t5(q, k, v, n_heads, 128, kv_stride, prefix_len, n, tb.anc, o, sms, status, st, nullptr);
             else
-                e = launch_attention_tc(q, k, v, n_heads, 128, kv_stride, prefix_len, n, tb.anc, o, nullptr, nullptr, sms, status, st, nullptr);
+                e = launch_attention_tc(q, k, v, n_heads, 128, kv_stride, prefix_len, n, tb.anc, o, sms, status, st, nullptr);
         }
     }
     if (e == cudaSuccess && status_out != nullptr)

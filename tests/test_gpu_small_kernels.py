@@ -1,0 +1,56 @@
+"""GPU parity of the short kernels around the decoder forward, at the sizes where their splits change: the
+verified-path search by pointer doubling, the rollback that rides in the same kernel, and the top-k that
+keeps a row of logits in registers as long as it fits."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2309_04255_b200 import binding as B
+from paper_2309_04255_b200 import inputs as gen
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def dev_i32(a):
+    return torch.as_tensor(np.asarray(a, np.int32), device=DEV)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 31, 32, 33, 64, 65, 127, 128])
+@pytest.mark.parametrize("broken", [False, True])
+def test_search_and_rollback_along_chains(n, broken):
+    """A chain is the deepest tree of its size: every doubling round is needed. Accepted whole, or up to a
+    wrong link in its middle; the entries behind the path are -1."""
+    cfg = gen.ModelConfig("chain", 2, 256, 2, 128, 256, 512, "bf16")
+    parent = gen.tree_chain(n)
+    tokens, amax = np.arange(n, dtype=np.int32), np.arange(1, n + 1, dtype=np.int32)
+    if broken and n > 1:
+        tokens[n // 2] = 400
+    v = B.Verifier(cfg, 7 + n + 1)
+    v.kv_view().normal_()
+    before = v.kv_view().clone()
+    path, sc = v.accept_compact(7, dev_i32(tokens), dev_i32(parent), dev_i32(amax))
+    acc = orc.accept(parent, tokens, amax)
+    assert sc.cpu().numpy()[:7].tolist() == [acc.accepted_len, acc.next_token, 7 + acc.accepted_len, acc.n_correct, acc.n_all, acc.rectified, 0]
+    assert path.cpu().numpy().tolist() == acc.path.tolist() + [-1] * (128 - acc.accepted_len)
+    assert torch.equal(v.kv_view(), before)      # a chain's path is already in place
+
+
+@pytest.mark.parametrize("vocab", [8, 31, 1023, 1024, 1025, 32767, 32768, 32769, 40000])
+def test_topk_of_short_and_long_rows(vocab):
+    """Rows that fill part of the block, all of its registers, and more than those. The oracle works on the
+    kernel's own logits, so the ids are exact (ties included: half the rows of the lm_head repeat); a
+    probability is one rounded exponential over a sum of up to 40000 of them, added in blocks: 1e-5."""
+    cfg = gen.ModelConfig("topk", 1, 64, 1, 64, 64, vocab, "f32")
+    v = B.Verifier(cfg, 16)
+    g = gen.gen_globals(cfg)
+    g["lm_head"] = g["lm_head"] * 20
+    g["lm_head"][vocab // 2: 2 * (vocab // 2)] = g["lm_head"][: vocab // 2]
+    v.pack_globals(g)
+    v.pack_layer(0, gen.gen_layer(cfg, 0))
+    out = v.extend_tree(3, dev_i32([1, 2, 5]), dev_i32([-1, 0, 0]), 0, top_k=8)
+    assert out["status"].item() == 0
+    ids, probs = orc.topk_softmax(out["logits"].cpu().numpy(), 8)
+    assert out["topk_ids"].cpu().numpy().tolist() == ids.tolist()
+    np.testing.assert_allclose(out["topk_probs"].cpu().numpy(), probs, rtol=1e-5)
