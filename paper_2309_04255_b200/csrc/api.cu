@@ -14,6 +14,7 @@
 #include "attention_tc.cuh"
 #include "common.cuh"
 #include "gemm_tc.cuh"
+#include "pass_small.cuh"
 
 using namespace llmcad;
 
@@ -112,6 +113,12 @@ struct llmcad_ctx {
     void *kv_lo = nullptr;    // bf16 remainders of the current layer's tree keys and values [2][H][128][hd]
     float *logits = nullptr;  // [128][V], used when the caller does not want logits
     TreeBuffers tb{};
+    // the one-kernel fp32 pass (pass_small.cu): allowed, and its own workspaces
+    bool small_pass = false;
+    float *sp_att = nullptr;
+    float2 *sp_ml = nullptr;
+    unsigned long long *sp_best = nullptr;
+    uint32_t *sp_bar = nullptr;
     double *inv_freq = nullptr;   // rope_base^(-2t/head_dim), t < head_dim/2
     int32_t *ibuf = nullptr;  // tokens[128], parent[128], argmax[128], path[128], scalars[8], chain[128]
     float *partials = nullptr;            // segment workspace of the tensor-core GEMMs
@@ -297,6 +304,11 @@ int run_attention(llmcad_ctx *ctx, const void *q, const void *k, const void *v, 
     return LLMCAD_OK;
 }
 
+bool use_small_pass(const llmcad_ctx *ctx, int n_keys);
+SmallPass small_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent,
+                            int n_tree, int n_old, float *logits, int32_t *status, bool keep_status);
+int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st);
+
 // Decoder forward over the nodes n_old .. n_tree-1 of a tree of n_tree nodes (all of them when
 // n_old = 0): tree prep of the whole tree, embedding, all layers; K/V of node i go to cache slot
 // P+i, where the nodes below n_old already have theirs. When logits != nullptr the final norm and
@@ -312,6 +324,8 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
     const int n_pad = (n + 15) / 16 * 16;
     const char *base = static_cast<const char *>(packed);
     int rc;
+    if (use_small_pass(ctx, P + n_tree))
+        return run_small_pass(ctx, small_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status), st);
     if ((rc = ensure_weight_maps(ctx, packed)) != LLMCAD_OK) return rc;
     if ((rc = ensure_act_maps(ctx, n_pad)) != LLMCAD_OK) return rc;
 
@@ -442,6 +456,43 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
     return LLMCAD_OK;
 }
 
+// Whether this pass goes through the one kernel of pass_small.cu (n_keys keys, prefix and tree).
+bool use_small_pass(const llmcad_ctx *ctx, int n_keys)
+{
+    const llmcad_config &c = ctx->cfg;
+    return ctx->small_pass && !ctx->timing && small_pass_serves(c.d_model, c.d_ffn, c.head_dim, c.n_heads, n_keys);
+}
+
+// What every pass through that kernel has in common; the caller adds what follows the logits.
+SmallPass small_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent,
+                            int n_tree, int n_old, float *logits, int32_t *status, bool keep_status)
+{
+    const llmcad_config &c = ctx->cfg;
+    const PackedLayout &y = ctx->lay;
+    SmallPass p{};
+    p.L = c.n_layers; p.d = c.d_model; p.H = c.n_heads; p.hd = c.head_dim; p.f = c.d_ffn; p.V = c.vocab; p.S = c.max_seq;
+    p.eps = c.rms_eps;
+    p.base = static_cast<const char *>(packed);
+    p.attn_norm = y.attn_norm; p.wqkv = y.wqkv; p.wo = y.wo; p.ffn_norm = y.ffn_norm; p.wgu = y.wgu; p.wdown = y.wdown;
+    p.layer_bytes = y.layer_bytes; p.tok_embed = y.tok_embed; p.final_norm = y.final_norm; p.lm_head = y.lm_head;
+    p.kv = static_cast<float *>(kv_cache);
+    p.inv_freq = ctx->inv_freq;
+    p.tokens = tokens; p.parent = parent; p.P = P; p.n_tree = n_tree; p.n_old = n_old;
+    p.x = ctx->x; p.q = static_cast<float *>(ctx->q); p.att = ctx->sp_att; p.h = static_cast<float *>(ctx->h);
+    p.att_ml = ctx->sp_ml; p.rope_cs = ctx->tb.rope_cs;
+    p.best = ctx->sp_best; p.bar = ctx->sp_bar;
+    p.logits = logits; p.status = status; p.keep_status = keep_status ? 1 : 0;
+    p.wait_limit_ns = ctx->wait_limit_ns;
+    return p;
+}
+
+int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st)
+{
+    ctx->launches++;
+    CUDA_TRY(launch_small_pass(p, ctx->n_sms, st));
+    return LLMCAD_OK;
+}
+
 int check_pass_args(const llmcad_ctx *ctx, const void *packed, const void *kv, int P, const void *tok, const void *par, int n)
 {
     if (ctx == nullptr || packed == nullptr || kv == nullptr || tok == nullptr || par == nullptr) return LLMCAD_ERR_INVALID_ARG;
@@ -552,6 +603,18 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
         const int max_pad = (cfg->max_tree + 15) / 16 * 16;
         ctx->partial_floats = ctx->tc_gemm ? gemm_tc_partial_floats(ctx->n_sms, max_tiles, max_pad) : 64;
         want((void **)&ctx->partials, ctx->partial_floats * 4);
+    }
+    {
+        // one kernel per pass at fp32 where the model fits it, unless the caller or the environment pins the others
+        const char *e = getenv("LLMCAD_SMALL_PASS");
+        ctx->small_pass = cfg->dtype == LLMCAD_F32 && cfg->flags == 0 && cfg->n_layers > 0 && !(e != nullptr && atoi(e) == 0) &&
+                          small_pass_serves(cfg->d_model, cfg->d_ffn, cfg->head_dim, cfg->n_heads, 1);
+        if (ctx->small_pass) {
+            want((void **)&ctx->sp_att, 128 * d * 4);
+            want((void **)&ctx->sp_ml, (size_t)128 * cfg->n_heads * sizeof(float2));
+            want((void **)&ctx->sp_best, 128 * 8);
+            want((void **)&ctx->sp_bar, 2 * 4);
+        }
     }
     const size_t ssq_floats = (size_t)4 * ((d + 127) / 128) * LLMCAD_MAX_TREE;
     want((void **)&ctx->ssq[0], ssq_floats * 4);
@@ -666,6 +729,12 @@ static int verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int3
     const llmcad_config &c = ctx->cfg;
     int32_t *status = out->scalars + LLMCAD_S_STATUS;
     float *logits = out->logits != nullptr ? out->logits : ctx->logits;
+    if (use_small_pass(ctx, prefix_len + n)) {
+        SmallPass sp = small_pass_params(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n, 0, logits, status, false);
+        sp.verify = 1;
+        sp.argmax = out->argmax; sp.path = out->accepted_path; sp.scalars = out->scalars; sp.path_fill = path_fill;
+        return run_small_pass(ctx, sp, st);
+    }
     if ((rc = run_forward(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n, logits, status, st)) != LLMCAD_OK)
         return rc;
     CUDA_TRY(launch_argmax(logits, n, c.vocab, out->argmax, status, st));
@@ -743,6 +812,12 @@ int llmcad_extend_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int3
     if (top_k > ctx->cfg.vocab) return LLMCAD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float *lg = logits != nullptr ? logits : ctx->logits;
+    if (use_small_pass(ctx, prefix_len + n_tree)) {
+        SmallPass sp = small_pass_params(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n_tree, n_old, lg, status, false);
+        sp.top_k = top_k;
+        sp.topk_ids = topk_ids; sp.topk_probs = topk_probs;
+        return run_small_pass(ctx, sp, st);
+    }
     if ((rc = run_forward(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n_tree, lg, status, st, n_old)) != LLMCAD_OK)
         return rc;
     if (top_k > 0) {

@@ -9,6 +9,8 @@ from oracle import oracle as orc
 from paper_2309_04255_b200 import binding as B
 from paper_2309_04255_b200 import inputs as gen
 
+from gpu_util import F32_TOL, Twin, argmax_agrees_where_decided, check_acceptance_against_oracle, logits_close
+
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
@@ -54,3 +56,27 @@ def test_topk_of_short_and_long_rows(vocab):
     ids, probs = orc.topk_softmax(out["logits"].cpu().numpy(), 8)
     assert out["topk_ids"].cpu().numpy().tolist() == ids.tolist()
     np.testing.assert_allclose(out["topk_probs"].cpu().numpy(), probs, rtol=1e-5)
+
+
+@pytest.mark.parametrize("P,n,H,hd,f,V", [(0, 1, 2, 64, 136, 129), (5, 8, 4, 64, 688, 1024), (63, 9, 2, 128, 264, 1001), (700, 3, 1, 128, 512, 300),
+                                          (2000, 40, 4, 64, 688, 512), (130, 65, 5, 64, 1200, 640), (31, 128, 4, 64, 688, 1024)])
+def test_one_kernel_fp32_pass(P, n, H, hd, f, V):
+    """The fp32 pass in one kernel where its cuts change: node blocks of eight and their remainders, several
+    staged chunks (128 nodes of 688 columns), one and two nodes per attention task, one and several key
+    ranges, both head widths, odd vocabularies; the verified path against the oracle's search."""
+    cfg = gen.ModelConfig("f32", 2, H * hd, H, hd, f, V, "f32")
+    tw = Twin(cfg, P + n + 8, scale=3.0)
+    tw.fill_prefix_synthetic(P)
+    parent = gen.tree_random(n, 12, "uniform4", n) if n > 1 else np.array([-1], np.int32)
+    tokens = gen.gen_tokens(cfg, n)
+    l0 = tw.v.launch_count()
+    ref = tw.oracle_pass(P, tokens, parent)
+    planted = gen.plant_tokens(parent, tokens, ref.logits.argmax(1).astype(np.int32), 1, prob=0.9)
+    for t in (tokens, planted):
+        ref = tw.oracle_pass(P, t, parent)
+        out = tw.gpu_pass(P, t, parent)
+        logits_close(out["logits"], ref.logits, F32_TOL)
+        argmax_agrees_where_decided(out["argmax"], ref.logits, F32_TOL)
+        check_acceptance_against_oracle(out, t, parent)
+        assert out["accepted_path"][out["scalars"][B.S_ACCEPTED_LEN]:].tolist() == [-1] * (128 - out["scalars"][B.S_ACCEPTED_LEN])
+    assert tw.v.launch_count() - l0 == 2
