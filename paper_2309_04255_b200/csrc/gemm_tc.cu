@@ -247,11 +247,18 @@ struct SharedCtl {
     uint64_t aempty[kMaxAStages];
 };
 
-// A ring item is (tile, k-block pair, half): up to two consecutive 64-wide k-blocks of one
-// 128-row weight tile (32 KB, contiguous in the tiled layout) and the matching activation tiles.
+// A weight tile is 128 rows of the packed matrix. An output tile has one of them, or two (SwiGLU: gate and up),
+// which are streamed one after the other like the tiles of different outputs: tile v belongs to output tile
+// v / halves. A ring item is (tile, k-block pair): up to two consecutive 64-wide k-blocks of a tile (32 KB,
+// contiguous in the tiled layout) and the matching activation tiles.
 __host__ __device__ __forceinline__ int pairs_per_tile(const GemmDesc &g) { return (g.kb_per_tile + g.pair_k - 1) / g.pair_k; }
 // the same with the k-blocks per item as a compile-time constant (the kernel is instantiated for 1 and 2)
 template <int PK> __device__ __forceinline__ int pairs_per_tile_c(const GemmDesc &g) { return (g.kb_per_tile + PK - 1) / PK; }
+// position of tile v in the packed matrix (all gate tiles, then all up tiles)
+__host__ __device__ __forceinline__ int packed_tile(const GemmDesc &g, int v)
+{
+    return g.halves == 2 ? (v >> 1) + (v & 1) * g.up_tile_offset : v;
+}
 
 // CTA cta's share of the GEMM: items [begin, end) of its item list.
 struct Range {
@@ -260,7 +267,7 @@ struct Range {
 template <int PK>
 __device__ __forceinline__ Range cta_range(const GemmDesc &g, int cta)
 {
-    const int total = g.n_tiles * pairs_per_tile_c<PK>(g) * g.halves;
+    const int total = g.n_tiles * g.halves * pairs_per_tile_c<PK>(g);
     Range r;
     r.begin = min(total, cta * g.items_per_cta);
     r.end = min(total, r.begin + g.items_per_cta);
@@ -271,21 +278,17 @@ __device__ __forceinline__ Range cta_range(const GemmDesc &g, int cta)
 // roles have well under a microsecond per item.
 template <int PK>
 struct Cursor {
-    int tile, kp, half;    // coordinates of the current item (kp: k-block pair)
+    int tile, kp;          // coordinates of the current item (kp: k-block pair)
     int left;              // items left in this CTA's range, the current one included
-    int ppt, halves, kbpt;
+    int ppt, kbpt;
     __device__ void init(const GemmDesc &d)
     {
         const Range r = cta_range<PK>(d, (int)blockIdx.x);
         left = r.end - r.begin;
         kbpt = d.kb_per_tile;
         ppt = pairs_per_tile_c<PK>(d);
-        halves = d.halves;
-        const int ipt = ppt * halves;
-        tile = r.begin / ipt;
-        const int q = r.begin - tile * ipt;
-        kp = q / halves;
-        half = q - kp * halves;
+        tile = r.begin / ppt;
+        kp = r.begin - tile * ppt;
     }
     __device__ bool done() const { return left <= 0; }
     __device__ int kb0() const { return kp * PK; }
@@ -293,19 +296,16 @@ struct Cursor {
     __device__ void advance()
     {
         --left;
-        if (++half == halves) {
-            half = 0;
-            if (++kp == ppt) { kp = 0; ++tile; }
-        }
+        if (++kp == ppt) { kp = 0; ++tile; }
     }
 };
 
-// Floats of one segment slot of the workspace: [4 row groups][halves][n_pad nodes][32 rows].
-__host__ __device__ __forceinline__ size_t slot_floats(int halves, int n_pad) { return (size_t)halves * n_pad * kTileM; }
+// Floats of one segment slot of the workspace: [4 row groups][n_pad nodes][32 rows].
+__host__ __device__ __forceinline__ size_t slot_floats(int n_pad) { return (size_t)n_pad * kTileM; }
 
 // ------------------------------------------------------------------------------------------------
 // Finishing (the work of gemm_finish_kernel). Every streaming CTA that holds items of a tile has left
-// its accumulators in the workspace as [row group][gate|up][node][32 rows] fp32 (a "segment").
+// its accumulators in the workspace as [row group][node][32 rows] fp32 (a "segment").
 __device__ __forceinline__ uint2 pack4_bf16(const __nv_bfloat16 (&h)[4])
 {
     uint2 r;
@@ -314,10 +314,22 @@ __device__ __forceinline__ uint2 pack4_bf16(const __nv_bfloat16 (&h)[4])
     return r;
 }
 
-// Where CTA cc left its segment of tile `tile`, rows of row group lane_grp: slot tile + cc.
-__device__ __forceinline__ const float *share_ptr(const GemmParams &p, const GemmDesc &d, int cc, int tile, int lane_grp)
+// Where CTA cc left its segment of tile v, rows of row group lane_grp: slot v + cc.
+__device__ __forceinline__ const float *share_ptr(const GemmParams &p, int cc, int v, int lane_grp)
 {
-    return p.partials + (size_t)(tile + cc) * slot_floats(d.halves, p.n_pad) + (size_t)lane_grp * d.halves * p.n_pad * 32;
+    return p.partials + (size_t)(v + cc) * slot_floats(p.n_pad) + (size_t)lane_grp * p.n_pad * 32;
+}
+
+// The CTAs that hold items of tile v: first .. first + n - 1.
+struct Holders {
+    int first, n;
+};
+__device__ __forceinline__ Holders holders_of(const GemmDesc &d, int ppt, int v)
+{
+    Holders h;
+    h.first = v * ppt / d.items_per_cta;
+    h.n = ((v + 1) * ppt - 1) / d.items_per_cta - h.first + 1;
+    return h;
 }
 
 // What a warp of the finishing kernel works on.
@@ -325,7 +337,8 @@ struct FinishArgs {
     const GemmParams *p;
     const GemmDesc *d;              // in shared memory
     const float *rs;                // per-node factors of the folded input norm (shared memory)
-    int tile, first_cta, last_cta, lane_grp;
+    int tile, lane_grp;             // output tile, 32-row group
+    Holders a, b;                   // who holds it (b: the up projection of a SwiGLU)
     int it_first, it_step;          // this warp finishes node groups it_first, it_first + it_step, ...
 };
 
@@ -357,8 +370,9 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
     const int row0 = tile * kTileM + lane_grp * 32 + 4 * r4;   // first of this lane's four output rows
     const int n_valid = min(4, n_out - row0);                  // how many of them exist
     const bool rows_ok = n_valid == 4;                         // all modes but EPI_PLAIN have n_out % 4 == 0
-    const int n_parts = fa.last_cta - fa.first_cta + 1;
-    if (!LLMCAD_CHECK(fa.first_cta >= 0 && fa.last_cta < d.grid && tile < d.n_tiles && row0 >= 0, p.status)) return;
+    const int n_parts = dual ? max(fa.a.n, fa.b.n) : fa.a.n;
+    const int va = dual ? 2 * tile : tile;                     // the tile (of the gate; the up projection's is the next)
+    if (!LLMCAD_CHECK(fa.a.first >= 0 && fa.a.first + fa.a.n <= d.grid && tile < d.n_tiles && row0 >= 0, p.status)) return;
     if (mode == EPI_QKV && !LLMCAD_CHECK(ep.P + n_nodes <= ep.S && row0 < 3 * ep.d, p.status)) return;
 
     // per-lane constants of the mode
@@ -395,22 +409,22 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
             float4 t[G][kB], u[G][kB];
 #pragma unroll
             for (int k = 0; k < kB; ++k) {
-                const float *sk = share_ptr(p, d, fa.first_cta + min(k0 + k, n_parts - 1), tile, lane_grp) + 4 * r4;
+                const float *sk = share_ptr(p, fa.a.first + min(k0 + k, fa.a.n - 1), va, lane_grp) + 4 * r4;
+                const float *su = dual ? share_ptr(p, fa.b.first + min(k0 + k, fa.b.n - 1), va + 1, lane_grp) + 4 * r4 : nullptr;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
                     const int node = min(itg + g * fa.it_step, iters - 1) * 4 + ns;
                     t[g][k] = __ldcg(reinterpret_cast<const float4 *>(sk + (size_t)node * 32));
-                    if (dual) u[g][k] = __ldcg(reinterpret_cast<const float4 *>(sk + (size_t)(n_pad + node) * 32));
+                    if (dual) u[g][k] = __ldcg(reinterpret_cast<const float4 *>(su + (size_t)node * 32));
                 }
             }
 #pragma unroll
             for (int k = 0; k < kB; ++k) {
-                if (k0 + k < n_parts) {          // CTA order
+                // CTA order
 #pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        as[g].x += t[g][k].x; as[g].y += t[g][k].y; as[g].z += t[g][k].z; as[g].w += t[g][k].w;
-                        if (dual) { bs[g].x += u[g][k].x; bs[g].y += u[g][k].y; bs[g].z += u[g][k].z; bs[g].w += u[g][k].w; }
-                    }
+                for (int g = 0; g < G; ++g) {
+                    if (k0 + k < fa.a.n) { as[g].x += t[g][k].x; as[g].y += t[g][k].y; as[g].z += t[g][k].z; as[g].w += t[g][k].w; }
+                    if (dual && k0 + k < fa.b.n) { bs[g].x += u[g][k].x; bs[g].y += u[g][k].y; bs[g].z += u[g][k].z; bs[g].w += u[g][k].w; }
                 }
             }
         }
@@ -515,8 +529,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
     const uint32_t astage_bytes = PK * b_tile_bytes;
     const uint32_t act_base = smem_base + (uint32_t)p.stages * wstage_bytes;
     const uint32_t packed_base = W4 ? act_base + (uint32_t)p.astages * astage_bytes : smem_base + (uint32_t)p.stages * stage_bytes;
-    const uint32_t acc_cols = 2u * nb;                    // TMEM columns of one accumulator buffer (gate | up)
-    const bool two_bufs = p.acc_bufs == 2;
+    const uint32_t acc_cols = nb;                         // TMEM columns of one of the two accumulator buffers
     const uint64_t wait_limit = p.wait_limit_ns;          // every wait below gives up after this many ns
     const DepWait dep{p.dep_ctr, p.dep_target, wait_limit};
 
@@ -536,7 +549,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             // packed tiles go to the packed ring; the dump warps turn them into MMA stages
             const uint32_t pf = smem_u32(&ctl.pfull[ps]);
             mbar_expect_tx(pf, (uint32_t)nk * kW4TileBytes);
-            const size_t t = (size_t)(pc.tile + (pc.half ? d.up_tile_offset : 0)) * d.kb_per_tile + pc.kb0();
+            const size_t t = (size_t)packed_tile(d, pc.tile) * d.kb_per_tile + pc.kb0();
             bulk_load_1d(packed_base + ps * pstage_bytes, d.w_tiled + t * kW4TileBytes, (uint32_t)nk * kW4TileBytes, pf, pol_stream);
             if (pissued == 0) LLMCAD_TRACE(2);
             ++pissued;
@@ -549,12 +562,12 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
         mbar_expect_tx(full, (uint32_t)nk * (kATileBytes + b_tile_bytes));
         if (d.w_tiled != nullptr) {
             // consecutive k-blocks of a tile are contiguous in the tiled layout: one copy
-            const size_t t = (size_t)(pc.tile + (pc.half ? d.up_tile_offset : 0)) * d.kb_per_tile + pc.kb0();
+            const size_t t = (size_t)packed_tile(d, pc.tile) * d.kb_per_tile + pc.kb0();
             bulk_load_1d(dst, d.w_tiled + t * kATileBytes, (uint32_t)nk * kATileBytes, full, pol_stream);
         } else {
             for (int k = 0; k < nk; ++k)
                 tma_load_2d(dst + k * kATileBytes, &maps.w, (pc.kb0() + k) * kBlockK,
-                            (pc.half ? d.up_row_offset : 0) + pc.tile * kTileM, full, pol_stream);
+                            pc.tile * kTileM, full, pol_stream);
         }
         __threadfence_block();
         if (pissued == 0) LLMCAD_TRACE(2);
@@ -688,9 +701,9 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             uint32_t aph = 0;
             while (!c.done() && !timed_out) {
                 // one segment: the items of one tile that belong to this CTA
-                const int tile = c.tile, halves = c.halves;
-                const int buf = two_bufs ? (seg & 1) : 0;
-                const uint32_t use = two_bufs ? (seg >> 1) : seg;     // how often this buffer has been used before
+                const int tile = c.tile;
+                const int buf = seg & 1;
+                const uint32_t use = seg >> 1;                        // how often this buffer has been used before
                 if (!mbar_wait(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
                 tc_fence_after();
                 const uint32_t d0 = tmem_base + buf * acc_cols;
@@ -700,9 +713,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                     tc_fence_after();
                     const uint32_t a_addr = W4 ? smem_base + s * wstage_bytes : smem_base + s * stage_bytes;
                     const uint32_t b_addr = W4 ? act_base + as * astage_bytes : a_addr + b_off;
-                    // segments of a two-half GEMM start on a gate item, so the first `halves` items
-                    // of a segment are the ones that must overwrite their accumulator
-                    const uint32_t dcol = d0 + c.half * nb;
                     const int nk = c.nk();
                     for (int k = 0; k < nk; ++k) {
                         const uint64_t a_desc = make_smem_desc(a_addr + k * kATileBytes);
@@ -710,7 +720,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
 #pragma unroll
                         for (int k4 = 0; k4 < kBlockK / 16; ++k4) {
                             // advancing 16 bf16 = 32 bytes inside the swizzle row: +2 in the >>4 address field
-                            tc_mma_bf16(dcol, a_desc + 2 * k4, b_desc + 2 * k4, idesc, (q >= halves || k > 0 || k4 > 0) ? 1u : 0u);
+                            tc_mma_bf16(d0, a_desc + 2 * k4, b_desc + 2 * k4, idesc, (q > 0 || k > 0 || k4 > 0) ? 1u : 0u);
                         }
                     }
                     tc_commit(smem_u32(&ctl.empty[s]));  // frees the stage when these MMAs have read it
@@ -739,8 +749,8 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             if (threadIdx.x == 64) LLMCAD_TRACE(3);
         }
         const Range r = cta_range<PK>(d, (int)blockIdx.x);
-        const int ipt = pairs_per_tile_c<PK>(d) * d.halves;
-        const size_t slot_stride = slot_floats(d.halves, p.n_pad);
+        const int ipt = pairs_per_tile_c<PK>(d);
+        const size_t slot_stride = slot_floats(p.n_pad);
         // ---- INT4 weights: these warps also turn every packed item into the bf16 tiles the MMA reads, a quarter
         // of the rows each, in the next free slot of the ring of expanded items. Element j of a word sits where
         // (word >> 4k) & 0x000f000f picks elements 2k, 2k+1; OR-ing 0x4300 into each half makes the bf16 values
@@ -804,8 +814,8 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
         for (int seg_begin = r.begin; seg_begin < r.end && !timed_out; ++seg) {
             const int tile = seg_begin / ipt;
             const int seg_end = min(r.end, (tile + 1) * ipt);
-            const int buf = two_bufs ? (seg & 1) : 0;
-            const uint32_t use = two_bufs ? (seg >> 1) : seg;
+            const int buf = seg & 1;
+            const uint32_t use = seg >> 1;
             if (W4) {
                 for (int i = seg_begin; i < seg_end && !timed_out; ++i)
                     if (!dequant_item()) timed_out = true;
@@ -823,31 +833,29 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             // this CTA's segment of the tile goes to slot tile + CTA, lane = row of the 32-row group;
             // with hi + lo activations a node's two accumulator columns are added first
             const uint32_t t_lane = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + buf * acc_cols;
-            if (!LLMCAD_CHECK(tile >= 0 && tile < d.n_tiles && tile + (int)blockIdx.x < d.n_tiles + d.grid, p.status)) { timed_out = true; break; }
-            float *dst = p.partials + (size_t)(tile + (int)blockIdx.x) * slot_stride + (size_t)lane_grp * d.halves * p.n_pad * 32 + lane;
-            for (int hf = 0; hf < d.halves; ++hf) {
-                int c0 = 0;
+            if (!LLMCAD_CHECK(tile >= 0 && tile < d.n_tiles * d.halves && tile + (int)blockIdx.x < d.n_tiles * d.halves + d.grid, p.status)) { timed_out = true; break; }
+            float *dst = p.partials + (size_t)(tile + (int)blockIdx.x) * slot_stride + (size_t)lane_grp * p.n_pad * 32 + lane;
+            int c0 = 0;
+            if (p.comp) {
+                // 32 nodes at a time, hi and lo columns in one round trip
+                for (; c0 + 32 <= p.n_pad; c0 += 32) {
+                    float v[32];
+                    tc_ld32_sum2(t_lane + c0, t_lane + p.n_pad + c0, v);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) dst[(size_t)(c0 + j) * 32] = v[j];
+                }
+            }
+            for (; c0 < p.n_pad; c0 += 16) {
+                float v[16];
+                tc_ld16(t_lane + c0, v);
                 if (p.comp) {
-                    // 32 nodes at a time, hi and lo columns in one round trip
-                    for (; c0 + 32 <= p.n_pad; c0 += 32) {
-                        float v[32];
-                        tc_ld32_sum2(t_lane + hf * nb + c0, t_lane + hf * nb + p.n_pad + c0, v);
+                    float t[16];
+                    tc_ld16(t_lane + p.n_pad + c0, t);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) dst[(size_t)(hf * p.n_pad + c0 + j) * 32] = v[j];
-                    }
+                    for (int j = 0; j < 16; ++j) v[j] += t[j];
                 }
-                for (; c0 < p.n_pad; c0 += 16) {
-                    float v[16];
-                    tc_ld16(t_lane + hf * nb + c0, v);
-                    if (p.comp) {
-                        float t[16];
-                        tc_ld16(t_lane + hf * nb + p.n_pad + c0, t);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] += t[j];
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) dst[(size_t)(hf * p.n_pad + c0 + j) * 32] = v[j];
-                }
+                for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * 32] = v[j];
             }
             // the accumulator has left TMEM: hand the buffer back to the MMA warp
             tc_fence_before();
@@ -944,7 +952,7 @@ gemm_finish_kernel(const __grid_constant__ GemmParams p)
         __syncthreads();
     }
 
-    const int ipt = pairs_per_tile(d) * d.halves;
+    const int ppt = pairs_per_tile(d);
     const int pairs = d.n_tiles * 4, iters = p.n_pad >> 2;
     const int W = (int)gridDim.x * (kFinThreads / 32);
     int k = W / pairs;
@@ -968,9 +976,8 @@ gemm_finish_kernel(const __grid_constant__ GemmParams p)
                 FinishArgs fa;
                 fa.p = &p; fa.d = &d; fa.rs = s_rs;
                 fa.tile = pair >> 2; fa.lane_grp = pair & 3;
-                const int tile_i0 = fa.tile * ipt;
-                fa.first_cta = tile_i0 / d.items_per_cta;
-                fa.last_cta = (tile_i0 + ipt - 1) / d.items_per_cta;
+                fa.a = holders_of(d, ppt, fa.tile * d.halves);
+                if (MODE == EPI_SWIGLU) fa.b = holders_of(d, ppt, fa.tile * 2 + 1);
                 fa.it_first = wg % k; fa.it_step = k;
                 finish_rows_t<G, KB, MODE>(fa, lane, dry);
                 if (dry) break;          // one pair is enough to have walked through the code
@@ -1051,7 +1058,7 @@ bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t 
     return r == CUDA_SUCCESS;
 }
 
-size_t gemm_tc_partial_floats(int n_sms, int max_tiles, int max_n_pad) { return (size_t)(max_tiles + n_sms) * slot_floats(2, max_n_pad); }
+size_t gemm_tc_partial_floats(int n_sms, int max_tiles, int max_n_pad) { return (size_t)2 * (max_tiles + n_sms) * slot_floats(max_n_pad); }
 
 GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool w4)
 {
@@ -1060,7 +1067,6 @@ GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool
     d.n_tiles = (ep.n_out + kTileM - 1) / kTileM;
     d.kb_per_tile = (n_in + kBlockK - 1) / kBlockK;
     d.pair_k = kMaxPairK;
-    d.up_row_offset = ep.n_out;
     d.items_per_cta = 0;
     d.grid = 0;
     d.w_tiled = static_cast<const uint8_t *>(w_tiled);
@@ -1102,11 +1108,10 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
     GemmDesc &d = p.g;
     d.pair_k = pair_k;
     // the items are split evenly over one CTA per SM (fewer CTAs when there are fewer items)
-    const long long total = (long long)d.n_tiles * pairs_per_tile(d) * d.halves;
+    const long long total = (long long)d.n_tiles * d.halves * pairs_per_tile(d);
     if (total < 1) return cudaErrorInvalidValue;
     int grid = total < n_sms ? (int)total : n_sms;
-    long long ipc = (total + grid - 1) / grid;
-    if (d.halves == 2) ipc += ipc & 1;   // ranges of a two-half GEMM start on a gate item
+    const long long ipc = (total + grid - 1) / grid;
     d.items_per_cta = (int)ipc;
     grid = (int)((total + ipc - 1) / ipc);
     d.grid = grid;
@@ -1125,12 +1130,11 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     const int nb = p.n_pad * (p.comp ? 2 : 1);
     const int pair_k = d.pair_k, grid = d.grid;
     const long long ipc = d.items_per_cta;
-    if ((size_t)(d.n_tiles + grid) * slot_floats(d.halves, p.n_pad) > partial_floats) return cudaErrorInvalidValue;
+    if ((size_t)(d.n_tiles * d.halves + grid) * slot_floats(p.n_pad) > partial_floats) return cudaErrorInvalidValue;
     const size_t stage_bytes = (size_t)pair_k * ((size_t)kATileBytes + (size_t)nb * kBlockK * 2);
     // One CTA per SM with the whole shared memory as the ring.
-    // accumulators: (gate | up) x MMA N columns each, double-buffered when two of them fit
-    p.acc_bufs = 4 * nb <= 512 ? 2 : 1;
-    int cols = p.acc_bufs * 2 * nb, pow2 = 32;
+    // two accumulator buffers of MMA N columns each
+    int cols = 2 * nb, pow2 = 32;
     while (pow2 < cols) pow2 <<= 1;
     p.tmem_cols = pow2;
     // the ring takes what the SM has, less the room that the finishing CTA of the previous GEMM needs beside it
@@ -1195,7 +1199,7 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     int fgrid = (int)((units + warps_per_cta - 1) / warps_per_cta);
     if (fgrid > n_sms) fgrid = n_sms;
     const long long per_warp = (units + (long long)fgrid * warps_per_cta - 1) / ((long long)fgrid * warps_per_cta);
-    const int max_parts = (int)(((long long)pairs_per_tile(d) * d.halves + ipc - 1) / ipc) + 1;
+    const int max_parts = (int)((pairs_per_tile(d) + ipc - 1) / ipc) + 1;
     const bool wide = max_parts > 4;           // many segments per tile (tiles split over many CTAs)
     const bool two = per_warp >= 2;            // several node groups per warp
     typedef void (*FinKernel)(GemmParams);

@@ -14,9 +14,8 @@ struct GemmDesc {
     int n_tiles;        // tiles of 128 output features
     int kb_per_tile;    // 64-wide k-blocks per tile
     int pair_k;         // k-blocks per ring item (1 or 2), set by the launcher
-    int halves;         // 2: every tile carries a gate and an up accumulator (SwiGLU), else 1
-    int up_row_offset;  // row of the first up-projection row in the packed [2f][d] matrix
-    int items_per_cta;  // ring items ((tile, k-block, half) triples) per CTA of the streaming grid
+    int halves;         // weight tiles per output tile: 2 (gate and up, SwiGLU), else 1
+    int items_per_cta;  // ring items ((weight tile, k-blocks) pairs) per CTA of the streaming grid
     int grid;           // CTAs of the streaming grid
     const uint8_t *w_tiled;  // weights as a sequence of pre-swizzled 16 KB tiles [tile][k-block] (see pack.cu),
                              // or nullptr: row-major weights through the tensor map
@@ -34,13 +33,12 @@ struct GemmMaps {
 struct GemmParams {
     int n_pad;          // tree nodes padded to a multiple of 16
     int comp;           // 1: activations come as hi + lo planes; the MMA N is 2 * n_pad and the two columns of a node are added
-    int acc_bufs;       // accumulator buffers in TMEM: 2, or 1 when 2 x (gate | up) x MMA N exceeds the 512 columns
     int stages;         // depth of the shared-memory ring (INT4 weights: of the ring of expanded weight items)
     int pstages;        // INT4 weights: depth of the ring of packed tiles that feeds it
     int astages;        // INT4 weights: depth of the ring of activation items (with bf16 weights they share the weights' stages)
     int tmem_cols;      // allocated TMEM columns (power of two)
-    float *partials;    // segment slots [n_tiles + grid][4 row groups][halves][n_pad][32 rows] fp32: the segment of
-                        // tile t held by CTA c sits in slot t + c
+    float *partials;    // segment slots [weight tiles + grid][4 row groups][n_pad][32 rows] fp32: the segment of
+                        // weight tile v held by CTA c sits in slot v + c
     int32_t *status;
     unsigned long long *trace;  // optional [256][16] timeline in ns of this GEMM (nullptr: off)
     int withhold_act;   // self-test of the wait limit: the activation copies are never issued
@@ -69,7 +67,7 @@ bool make_act_map_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64
 bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t dims[3], const uint64_t strides_bytes[2],
                              const uint32_t box[3]);
 
-// Floats of segment workspace that GEMMs of up to max_tiles tiles on up to max_n_pad nodes need.
+// Floats of segment workspace that GEMMs of up to max_tiles output tiles (of one or two weight tiles) on up to max_n_pad nodes need.
 size_t gemm_tc_partial_floats(int n_sms, int max_tiles, int max_n_pad);
 
 // Describes one GEMM (fills everything but items_per_cta and grid, which the launcher sets).
