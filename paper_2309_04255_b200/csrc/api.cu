@@ -143,7 +143,10 @@ struct llmcad_ctx {
         return trace + (size_t)(trace_launch++) * 256 * 16;
     }
     const void *maps_for = nullptr;    // packed weight buffer of the current call
+    std::vector<CUtensorMap> weight_maps;   // its matrices, for the GEMMs on CTA pairs: four per layer, then the lm_head
+    const void *weight_maps_for = nullptr;
     CUtensorMap act_maps[9][3];        // [n_pad/16][xn, att, h]
+    CUtensorMap pair_maps[9][3];       // the same for the GEMMs on CTA pairs
     bool act_ready[9] = {false, false, false, false, false, false, false, false, false};
     // optional per-launch timing (events around every GEMM / attention launch)
     bool timing = false;
@@ -193,11 +196,28 @@ struct TimedLaunch {
     }
 };
 
-int ensure_weight_maps(llmcad_ctx *ctx, const void *packed)
+// Remembers which packed buffer the pass addresses; GEMMs on CTA pairs (see gemm_takes_pairs) also want a tensor
+// map per matrix, encoded when the buffer is first seen.
+int ensure_weight_maps(llmcad_ctx *ctx, const void *packed, int n_pad)
 {
-    // the pass reads its weights as pre-swizzled tiles through plain bulk copies, so there is no
-    // tensor map to encode for them: remember which packed buffer the chains address
     ctx->maps_for = packed;
+    if (!ctx->tc_gemm || ctx->weight_maps_for == packed || !gemm_takes_pairs(n_pad, ctx->comp)) return LLMCAD_OK;
+    const llmcad_config &c = ctx->cfg;
+    const int d = c.d_model, f = c.d_ffn;
+    const char *base = static_cast<const char *>(packed);
+    ctx->weight_maps.resize(4 * (size_t)c.n_layers + 1);
+    bool ok = make_packed_map(&ctx->weight_maps.back(), base + ctx->lay.lm_head, tiled_weight_bytes(c.vocab, d));
+    for (int l = 0; l < c.n_layers && ok && !ctx->w4; ++l) {
+        const char *lb = base + ctx->lay.layer_bytes * (size_t)l;
+        CUtensorMap *m = &ctx->weight_maps[4 * (size_t)l];
+        ok = make_packed_map(m, lb + ctx->lay.wqkv, 3 * tiled_weight_bytes(d, d)) && make_packed_map(m + 1, lb + ctx->lay.wo, tiled_weight_bytes(d, d)) &&
+             make_packed_map(m + 2, lb + ctx->lay.wgu, 2 * tiled_weight_bytes(f, d)) && make_packed_map(m + 3, lb + ctx->lay.wdown, tiled_weight_bytes(d, f));
+    }
+    if (!ok) {
+        snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for a weight matrix");
+        return LLMCAD_ERR_CUDA;
+    }
+    ctx->weight_maps_for = packed;
     return LLMCAD_OK;
 }
 
@@ -208,9 +228,14 @@ int ensure_act_maps(llmcad_ctx *ctx, int n_pad)
     const llmcad_config &c = ctx->cfg;
     bool ok = true;
     const uint32_t planes = ctx->comp ? 2 : 1;
-    ok &= make_act_map_bf16(&ctx->act_maps[slot][0], ctx->xn, 128, c.d_model, n_pad, planes, kLoRows);
-    ok &= make_act_map_bf16(&ctx->act_maps[slot][1], ctx->att, 128, c.d_model, n_pad, planes, kLoRows);
-    ok &= make_act_map_bf16(&ctx->act_maps[slot][2], ctx->h, 128, c.d_ffn, n_pad, planes, kLoRows);
+    const void *bufs[3] = {ctx->xn, ctx->att, ctx->h};
+    for (int i = 0; i < 3; ++i) {
+        const int cols = i == 2 ? c.d_ffn : c.d_model;
+        ok &= make_act_map_bf16(&ctx->act_maps[slot][i], bufs[i], 128, cols, n_pad, planes, kLoRows, planes);
+        // a CTA pair: one plane, or half of the rows of the only plane
+        if (gemm_takes_pairs(n_pad, ctx->comp))
+            ok &= make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], 128, cols, ctx->comp ? n_pad : n_pad / 2, planes, kLoRows, 1);
+    }
     if (!ok) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for an activation buffer");
         return LLMCAD_ERR_CUDA;
@@ -235,8 +260,11 @@ struct TcGemm {
     }
     void set(llmcad_ctx *ctx, int l, int which, int act, int n_in, const EpiParams &ep, int n_pad)
     {
-        maps.x = ctx->act_maps[n_pad / 16][act];
-        p.g = make_gemm_desc(n_in, ep, weight_ptr(ctx, l, which), ctx->w4 && l >= 0);
+        const bool w4 = ctx->w4 && l >= 0;
+        p.pairs = !w4 && gemm_takes_pairs(n_pad, ctx->comp);
+        maps.x = p.pairs ? ctx->pair_maps[n_pad / 16][act] : ctx->act_maps[n_pad / 16][act];
+        if (p.pairs) maps.w = l < 0 ? ctx->weight_maps.back() : ctx->weight_maps[4 * (size_t)l + which];
+        p.g = make_gemm_desc(n_in, ep, weight_ptr(ctx, l, which), w4);
         p.n_pad = n_pad;
         p.comp = ctx->comp ? 1 : 0;
     }
@@ -326,7 +354,7 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
     int rc;
     if (use_small_pass(ctx, P + n_tree))
         return run_small_pass(ctx, small_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status), st);
-    if ((rc = ensure_weight_maps(ctx, packed)) != LLMCAD_OK) return rc;
+    if ((rc = ensure_weight_maps(ctx, packed, n_pad)) != LLMCAD_OK) return rc;
     if ((rc = ensure_act_maps(ctx, n_pad)) != LLMCAD_OK) return rc;
 
     ctx->launches++;
@@ -888,7 +916,7 @@ int llmcad_skinny_gemm(llmcad_ctx *ctx, const void *w, const void *x, float *y, 
         const int n_pad = (n + 15) / 16 * 16;
         TcGemm g;
         // rows of x beyond n are outside the tensor: the copy engine fills them with zeros
-        if (!make_tensor_map_bf16(&g.maps.w, w, n_out, n_in, 128) || !make_act_map_bf16(&g.maps.x, x, n, n_in, n_pad, 1, n)) {
+        if (!make_tensor_map_bf16(&g.maps.w, w, n_out, n_in, 128) || !make_act_map_bf16(&g.maps.x, x, n, n_in, n_pad, 1, n, 1)) {
             snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
             return LLMCAD_ERR_CUDA;
         }
@@ -930,7 +958,9 @@ int llmcad_skinny_gemm_tiled(llmcad_ctx *ctx, const void *w_tiled, const void *x
     ep.mode = EPI_PLAIN; ep.n = n; ep.n_out = n_out; ep.y = y; ep.ldy = n_out;
     const int n_pad = (n + 15) / 16 * 16;
     TcGemm g;
-    if (!make_act_map_bf16(&g.maps.x, x, n, n_in, n_pad, 1, n)) {
+    g.p.pairs = gemm_takes_pairs(n_pad, false);
+    if (!make_act_map_bf16(&g.maps.x, x, n, n_in, g.p.pairs ? n_pad / 2 : n_pad, 1, n, 1) ||
+        (g.p.pairs && !make_packed_map(&g.maps.w, w_tiled, tiled_weight_bytes(n_out, n_in)))) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
         return LLMCAD_ERR_CUDA;
     }
@@ -976,7 +1006,7 @@ int llmcad_skinny_gemm_tiled_int4(llmcad_ctx *ctx, const void *w_tiled, const vo
     ep.mode = EPI_PLAIN; ep.n = n; ep.n_out = n_out; ep.y = y; ep.ldy = n_out;
     const int n_pad = (n + 15) / 16 * 16;
     TcGemm g;
-    if (!make_act_map_bf16(&g.maps.x, x, n, n_in, n_pad, 1, n)) {
+    if (!make_act_map_bf16(&g.maps.x, x, n, n_in, n_pad, 1, n, 1)) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
         return LLMCAD_ERR_CUDA;
     }

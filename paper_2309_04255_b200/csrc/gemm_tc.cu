@@ -193,6 +193,20 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float *v)
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// 32 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float *v)
+{
+    uint32_t a[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]), "=r"(a[16]), "=r"(a[17]), "=r"(a[18]), "=r"(a[19]), "=r"(a[20]), "=r"(a[21]), "=r"(a[22]), "=r"(a[23]), "=r"(a[24]), "=r"(a[25]), "=r"(a[26]), "=r"(a[27]), "=r"(a[28]), "=r"(a[29]), "=r"(a[30]), "=r"(a[31])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(a[j]);
+}
+
 // 32 consecutive fp32 columns of this thread's TMEM lane at each of two addresses, summed. A load plus
 // its wait costs ~0.15 us whatever the width, so the two loads share one wait; everything sits in one
 // statement so that no register of the result can be touched before the wait.
@@ -314,21 +328,22 @@ __device__ __forceinline__ uint2 pack4_bf16(const __nv_bfloat16 (&h)[4])
     return r;
 }
 
-// Where CTA cc left its segment of tile v, rows of row group lane_grp: slot v + cc.
-__device__ __forceinline__ const float *share_ptr(const GemmParams &p, int cc, int v, int lane_grp)
+// Where CTA (or CTA pair) cc left its segment of tile v, rows of row group lane_grp: slot v + cc (v + 2 cc).
+__device__ __forceinline__ const float *share_ptr(const GemmParams &p, const GemmDesc &d, int cc, int v, int lane_grp)
 {
-    return p.partials + (size_t)(v + cc) * slot_floats(p.n_pad) + (size_t)lane_grp * p.n_pad * 32;
+    return p.partials + (size_t)(v + d.group * cc) * slot_floats(p.n_pad) + (size_t)lane_grp * p.n_pad * 32;
 }
 
-// The CTAs that hold items of tile v: first .. first + n - 1.
+// The CTAs (pairs) that hold items of tile v: first .. first + n - 1.
 struct Holders {
     int first, n;
 };
 __device__ __forceinline__ Holders holders_of(const GemmDesc &d, int ppt, int v)
 {
     Holders h;
-    h.first = v * ppt / d.items_per_cta;
-    h.n = ((v + 1) * ppt - 1) / d.items_per_cta - h.first + 1;
+    const int t = d.group == 2 ? v >> 1 : v;
+    h.first = t * ppt / d.items_per_cta;
+    h.n = ((t + 1) * ppt - 1) / d.items_per_cta - h.first + 1;
     return h;
 }
 
@@ -372,7 +387,7 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
     const bool rows_ok = n_valid == 4;                         // all modes but EPI_PLAIN have n_out % 4 == 0
     const int n_parts = dual ? max(fa.a.n, fa.b.n) : fa.a.n;
     const int va = dual ? 2 * tile : tile;                     // the tile (of the gate; the up projection's is the next)
-    if (!LLMCAD_CHECK(fa.a.first >= 0 && fa.a.first + fa.a.n <= d.grid && tile < d.n_tiles && row0 >= 0, p.status)) return;
+    if (!LLMCAD_CHECK(fa.a.first >= 0 && d.group * (fa.a.first + fa.a.n) <= d.grid && tile < d.n_tiles && row0 >= 0, p.status)) return;
     if (mode == EPI_QKV && !LLMCAD_CHECK(ep.P + n_nodes <= ep.S && row0 < 3 * ep.d, p.status)) return;
 
     // per-lane constants of the mode
@@ -409,13 +424,15 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
             float4 t[G][kB], u[G][kB];
 #pragma unroll
             for (int k = 0; k < kB; ++k) {
-                const float *sk = share_ptr(p, fa.a.first + min(k0 + k, fa.a.n - 1), va, lane_grp) + 4 * r4;
-                const float *su = dual ? share_ptr(p, fa.b.first + min(k0 + k, fa.b.n - 1), va + 1, lane_grp) + 4 * r4 : nullptr;
+                // (no load for a holder that does not exist: at many nodes the segments' bytes are what this costs)
+                const bool has = k0 + k < fa.a.n, has_u = dual && k0 + k < fa.b.n;
+                const float *sk = share_ptr(p, d, fa.a.first + k0 + k, va, lane_grp) + 4 * r4;
+                const float *su = dual ? share_ptr(p, d, fa.b.first + k0 + k, va + 1, lane_grp) + 4 * r4 : nullptr;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
                     const int node = min(itg + g * fa.it_step, iters - 1) * 4 + ns;
-                    t[g][k] = __ldcg(reinterpret_cast<const float4 *>(sk + (size_t)node * 32));
-                    if (dual) u[g][k] = __ldcg(reinterpret_cast<const float4 *>(su + (size_t)node * 32));
+                    t[g][k] = has ? __ldcg(reinterpret_cast<const float4 *>(sk + (size_t)node * 32)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (dual) u[g][k] = has_u ? __ldcg(reinterpret_cast<const float4 *>(su + (size_t)node * 32)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
 #pragma unroll
@@ -423,8 +440,8 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
                 // CTA order
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    if (k0 + k < fa.a.n) { as[g].x += t[g][k].x; as[g].y += t[g][k].y; as[g].z += t[g][k].z; as[g].w += t[g][k].w; }
-                    if (dual && k0 + k < fa.b.n) { bs[g].x += u[g][k].x; bs[g].y += u[g][k].y; bs[g].z += u[g][k].z; bs[g].w += u[g][k].w; }
+                    as[g].x += t[g][k].x; as[g].y += t[g][k].y; as[g].z += t[g][k].z; as[g].w += t[g][k].w;
+                    if (dual) { bs[g].x += u[g][k].x; bs[g].y += u[g][k].y; bs[g].z += u[g][k].z; bs[g].w += u[g][k].w; }
                 }
             }
         }
@@ -885,6 +902,287 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
     }
 }
 
+// ------------------------------------------------------------------------------------------------
+// The streaming kernel for wide inputs, on CTA pairs (cta_group::2).
+//
+// With many nodes the bound moves from HBM to what an SM can take in from L2, of which gemm_stream_kernel spends
+// n_pad * 256 bytes per 16 KB of weights on activation tiles (128 nodes: two thirds of the traffic), and to power
+// (30B shape, 128 nodes: 1000 W, the clock drops to 1.65 GHz). Here the two CTAs of a cluster work on two weight tiles at once: one
+// tcgen05.mma of 256 rows reads each CTA's own weight tile and half of the activation rows from each
+// CTA's shared memory, so that every activation tile enters an SM pair once: half the traffic, and room for
+// more weights in the ring (30B shape, 128 nodes, 12 layers: 4.70 -> 4.45 ms a pass; its stream alone, unthrottled,
+// 53 -> 46 us for the QKV GEMM). Each CTA keeps the accumulator of its own tile and dumps it as before.
+//
+// Roles as in gemm_stream_kernel; the MMA warp of the first CTA of the pair issues for both. Copies of both
+// CTAs complete on the first CTA's "full" barrier (its producer announces the bytes of both), the MMAs' commits
+// release the stage and announce the accumulator in both CTAs, and the dump warps of both hand an
+// accumulator buffer back on the first CTA's barrier. Weights travel as tensor-map boxes of 512-byte rows over
+// the packed tiles: a plain bulk copy can only complete on a barrier of its own CTA.
+//
+// kWide (128 < nodes <= 256, prefill): hi and lo activation planes are multiplied one after the other into the
+// same 256 columns; the MMA is at full rate at N = 256 either way and twice the nodes fit tensor memory.
+__device__ __forceinline__ uint32_t map_to_cta0(uint32_t addr)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ void tma_pair_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar0, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3}], [%4], %5;"
+        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar0), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tma_pair_3d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, uint32_t bar0, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;"
+        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar0), "l"(policy)
+        : "memory");
+}
+// both CTAs' barriers at this offset
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(bar), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int PK, bool kWide>
+__global__ void __launch_bounds__(kThreads, 1)
+gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ SharedCtl ctl;
+    const GemmDesc &d = p.g;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)blockIdx.x & 1, group = (int)blockIdx.x >> 1;
+    const int n_vtiles = d.n_tiles * d.halves;
+    const uint32_t nb = (uint32_t)p.n_pad * (p.comp && !kWide ? 2u : 1u);      // MMA N
+    const uint32_t b_half = nb / 2 * kBlockK * 2;                              // this CTA's activation rows of a k-block, one pass
+    const uint32_t b_tile_bytes = b_half * (kWide ? 2u : 1u);
+    const uint32_t stage_bytes = PK * (kATileBytes + b_tile_bytes);
+    const uint32_t b_off = PK * kATileBytes;
+    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint64_t wait_limit = p.wait_limit_ns;
+    const DepWait dep{p.dep_ctr, p.dep_target, wait_limit};
+    if (threadIdx.x == 0) LLMCAD_TRACE(0);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            mbar_init(smem_u32(&ctl.full[s]), 1);
+            mbar_init(smem_u32(&ctl.empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&ctl.tmem_full[b]), 1);
+            mbar_init(smem_u32(&ctl.tmem_empty[b]), 8);
+        }
+        ctl.abort_flag = 0;
+        ctl.a_issued = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    // Allocating and freeing tensor memory for a pair are acts of both CTAs: neither may start before the other CTA
+    // is running, nor leave before the other has done its part. (The first barrier also says that the mbarriers of
+    // both exist before a copy or a commit signals them.)
+    __syncwarp();
+    cluster_sync_all();
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)),
+                     "r"((uint32_t)p.tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl.tmem_base;
+    volatile int *abort_flag = &ctl.abort_flag;
+    bool timed_out = false;
+    if (threadIdx.x == 0) LLMCAD_TRACE(1);
+
+    // the pair's items: (pair of weight tiles, PK k-blocks), the same list in both CTAs
+    const int ppt = pairs_per_tile_c<PK>(d), total = (n_vtiles + 1) / 2 * ppt;
+    const int begin = min(total, group * d.items_per_cta), end = min(total, begin + d.items_per_cta);
+
+    if (warp == 0) {
+        // ================================================= weight producer
+        if (lane == 0) {
+            uint64_t pol_stream;
+            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
+            int s = 0, pt = begin / ppt, kp = begin - pt * ppt;
+            uint32_t par = 1;
+            uint64_t t_idle = 0;
+            for (int i = begin; i < end;) {
+                if (!mbar_try(smem_u32(&ctl.empty[s]), par)) {
+                    if (t_idle == 0) t_idle = global_timer_ns();
+                    else if (*abort_flag || global_timer_ns() - t_idle > wait_limit) { timed_out = true; break; }
+                    continue;
+                }
+                t_idle = 0;
+                const uint32_t full = smem_u32(&ctl.full[s]);
+                if (rank == 0) mbar_expect_tx(full, 2u * stage_bytes);
+                // (an odd last tile is loaded twice; an item past the end of a tile's k-blocks brings bytes nobody multiplies)
+                const int v = min(2 * pt + rank, n_vtiles - 1);
+                for (int k = 0; k < PK; ++k)
+                    tma_pair_2d(smem_base + s * stage_bytes + k * kATileBytes, &maps.w, 0, (packed_tile(d, v) * d.kb_per_tile + kp * PK + k) * 32, map_to_cta0(full), pol_stream);
+                __threadfence_block();
+                if (i == begin) LLMCAD_TRACE(2);
+                ctl.a_issued = (uint32_t)(++i - begin);
+                if (++kp == ppt) { kp = 0; ++pt; }
+                if (++s == p.stages) { s = 0; par ^= 1u; }
+            }
+            LLMCAD_TRACE(6);
+        }
+    } else if (warp == 6) {
+        // ================================================= activation loader: this CTA's half of the rows
+        if (lane == 0) {
+            uint64_t pol_keep;
+            asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
+            int s = 0, kp = begin % ppt;
+            if (!dep_wait_thread(dep)) timed_out = true;
+            fence_proxy_async();
+            pdl_launch_dependents();
+            for (int i = begin; i < end && !timed_out; ++i) {
+                uint64_t t0 = 0;
+                for (uint32_t spin = 0; (int32_t)(ctl.a_issued - (uint32_t)(i + 1 - begin)) < 0; ++spin) {
+                    __nanosleep(32);
+                    if ((spin & 255u) == 255u) {
+                        if (t0 == 0) t0 = global_timer_ns();
+                        if (*abort_flag || global_timer_ns() - t0 > wait_limit) { timed_out = true; break; }
+                    }
+                }
+                if (timed_out) break;
+                const uint32_t full = map_to_cta0(smem_u32(&ctl.full[s]));
+                const uint32_t dst = smem_base + s * stage_bytes + b_off;
+                // hi | lo planes: the first CTA has the hi rows, the second the lo rows; one plane, or wide: half of the rows each
+                const bool by_plane = p.comp && !kWide;
+                for (int k = 0; k < PK; ++k)
+                    tma_pair_3d(dst + k * b_tile_bytes, &maps.x, (kp * PK + k) * kBlockK, by_plane ? 0 : rank * (int)(nb / 2), by_plane ? rank : 0, full, pol_keep);
+                if (++kp == ppt) kp = 0;
+                if (++s == p.stages) s = 0;
+            }
+        }
+    } else if (warp == 1) {
+        // ================================================= MMA issuer (first CTA of the pair)
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = make_idesc(2 * kTileM, (int)nb);
+            uint32_t seg = 0, ph = 0;
+            int s = 0;
+            for (int i = begin; i < end && !timed_out; ++seg) {
+                const int pt = i / ppt, seg_end = min(end, (pt + 1) * ppt), first = i;
+                int kb = (i - pt * ppt) * PK;
+                const int buf = seg & 1;
+                if (!mbar_wait(smem_u32(&ctl.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+                tc_fence_after();
+                const uint32_t d0 = tmem_base + buf * nb;
+                for (; i < seg_end; ++i, kb += PK) {
+                    if (!mbar_wait(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
+                    tc_fence_after();
+                    const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off;
+                    const int nk = min(PK, d.kb_per_tile - kb);
+                    for (int k = 0; k < nk; ++k) {
+                        const uint64_t a_desc = make_smem_desc(a_addr + k * kATileBytes);
+#pragma unroll
+                        for (int pl = 0; pl < (kWide ? 2 : 1); ++pl) {
+                            const uint64_t b_desc = make_smem_desc(b_addr + k * b_tile_bytes + pl * b_half);
+#pragma unroll
+                            for (int k4 = 0; k4 < kBlockK / 16; ++k4)
+                                tc_mma_pair(d0, a_desc + 2 * k4, b_desc + 2 * k4, idesc, (i > first || k > 0 || pl > 0 || k4 > 0) ? 1u : 0u);
+                        }
+                    }
+                    tc_commit_pair(smem_u32(&ctl.empty[s]));
+                    if (++s == p.stages) { s = 0; ph ^= 1u; }
+                }
+                if (timed_out) break;
+                tc_commit_pair(smem_u32(&ctl.tmem_full[buf]));
+            }
+            LLMCAD_TRACE(7);
+        }
+    } else {
+        // ================================================= accumulator dump (warps 2..5): this CTA's weight tile
+        const int lane_grp = warp & 3;
+        if (!dep_wait_warp(dep, lane)) timed_out = true;
+        pdl_launch_dependents();
+        if (threadIdx.x == 64) LLMCAD_TRACE(3);
+        const size_t slot_stride = slot_floats(p.n_pad);
+        uint32_t seg = 0;
+        for (int i = begin; i < end && !timed_out; ++seg) {
+            const int pt = i / ppt, v = 2 * pt + rank, buf = seg & 1;
+            i = min(end, (pt + 1) * ppt);
+            if (!mbar_wait_warp(smem_u32(&ctl.tmem_full[buf]), (seg >> 1) & 1u, abort_flag, lane, wait_limit)) { timed_out = true; break; }
+            tc_fence_after();
+            if (threadIdx.x == 64 && seg == 0) LLMCAD_TRACE(4);
+            const uint32_t t_lane = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + buf * nb;
+            if (v < n_vtiles) {
+                if (!LLMCAD_CHECK(v >= 0 && v + 2 * group < n_vtiles + d.grid, p.status)) { timed_out = true; break; }
+                float *dst = p.partials + (size_t)(v + 2 * group) * slot_stride + (size_t)lane_grp * p.n_pad * 32 + lane;
+                int c0 = 0;
+                for (; c0 + 32 <= p.n_pad; c0 += 32) {
+                    float t[32];
+                    if (p.comp && !kWide) tc_ld32_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
+                    else tc_ld32(t_lane + c0, t);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) dst[(size_t)(c0 + j) * 32] = t[j];
+                }
+                for (; c0 < p.n_pad; c0 += 16) {
+                    float t[16];
+                    tc_ld16(t_lane + c0, t);
+                    if (p.comp && !kWide) {
+                        float u[16];
+                        tc_ld16(t_lane + p.n_pad + c0, u);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) t[j] += u[j];
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * 32] = t[j];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_to_cta0(smem_u32(&ctl.tmem_empty[buf])));
+        }
+        if (threadIdx.x == 64) LLMCAD_TRACE(8);
+    }
+    __syncwarp();
+    timed_out = __any_sync(0xffffffffu, timed_out);
+    if (warp >= 2 && warp <= 5 && lane == 0) dep_arrive(p.s_done);
+    if (timed_out) {
+        *abort_flag = 1;
+        atomicCAS(p.status, 0, LLMCAD_ERR_TIMEOUT);
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncwarp();
+    cluster_sync_all();            // the other CTA has stopped signalling this one's barriers and using its shared memory
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
+    __syncwarp();
+    cluster_sync_all();            // and both have given their tensor memory back
+    if (threadIdx.x == 32) LLMCAD_TRACE(13);
+}
+
 // Adds the segments of every tile and applies the fused epilogue; see the head of the file. The
 // work is cut into (tile, 32-row group) pairs; k warps share a pair's node groups, k chosen so that
 // all warps of the grid have work. G node groups and KB segments of each are loaded in one go
@@ -1029,18 +1327,30 @@ bool make_tensor_map_bf16(CUtensorMap *map, const void *base, uint64_t rows, uin
 }
 
 bool make_act_map_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t planes,
-                       uint64_t plane_rows)
+                       uint64_t plane_rows, uint32_t box_planes)
 {
     auto fn = get_encode_fn();
     if (fn == nullptr) return false;
     cuuint64_t dims[3] = {cols, rows, planes};
     cuuint64_t strides[2] = {cols * 2, plane_rows * cols * 2};
-    cuuint32_t box[3] = {(cuuint32_t)kBlockK, box_rows, planes};
+    cuuint32_t box[3] = {(cuuint32_t)kBlockK, box_rows, box_planes};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
+}
+
+bool make_packed_map(CUtensorMap *map, const void *tiled, uint64_t bytes)
+{
+    auto fn = get_encode_fn();
+    if (fn == nullptr) return false;
+    cuuint64_t dims[2] = {256, bytes / 512};
+    cuuint64_t strides[1] = {512};
+    cuuint32_t box[2] = {256, kATileBytes / 512};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(tiled), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t dims[3], const uint64_t strides_bytes[2],
@@ -1079,11 +1389,12 @@ GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool
 namespace {
 // tuning aids from the environment, read once per process
 struct Tuning {
-    int pair_k = 0, stages_cap = 0, w4_wstages = 3, w4_pstages = 4;
+    int pair_k = 0, stages_cap = 0, w4_wstages = 3, w4_pstages = 4, cta_pair_min = 80;
     Tuning()
     {
         if (const char *e = getenv("LLMCAD_GEMM_PAIR_K")) { const int v = atoi(e); if (v == 1 || v == 2) pair_k = v; }
         if (const char *e = getenv("LLMCAD_GEMM_STAGES")) { const int v = atoi(e); if (v >= 2) stages_cap = v; }
+        if (const char *e = getenv("LLMCAD_CTA_PAIR_MIN")) cta_pair_min = atoi(e);
         if (const char *e = getenv("LLMCAD_W4_WSTAGES")) { const int v = atoi(e); if (v >= 2 && v <= kMaxStages) w4_wstages = v; }
         if (const char *e = getenv("LLMCAD_W4_PSTAGES")) { const int v = atoi(e); if (v >= 2 && v <= kMaxPStages) w4_pstages = v; }
     }
@@ -1095,26 +1406,39 @@ const Tuning &tuning()
 }
 }  // namespace
 
+// Pairs from 80 nodes on (measured in whole passes, one kernel per CTA against pairs: 48 nodes 2 % slower, 64 nodes
+// level, 128 nodes 4-5 % faster; 16 and 32 nodes 3-6 % slower, the two cluster barriers at either end of the kernel
+// sit in every hand-over). The MMA's N has to be a multiple of 32.
+bool gemm_takes_pairs(int n_pad, bool comp)
+{
+    if (n_pad > 128) return true;
+    const int nb = n_pad * (comp ? 2 : 1);
+    return tuning().cta_pair_min > 0 && n_pad >= tuning().cta_pair_min && nb % 32 == 0;
+}
+
 cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
 {
     const Tuning &tune = tuning();
     // Ring items of two k-blocks (one 32 KB weight copy each) unless the activation tiles are so wide
     // (hi | lo planes of more than 64 nodes) that only two stages would fit; measured on B200:
     // single k-blocks cost 10-17 % up to 64 nodes and gain 6 % at 128.
-    const int nb = p.n_pad * (p.comp ? 2 : 1);       // MMA N
-    if (nb > 256 || p.n_pad < 16 || p.n_pad % 16) return cudaErrorInvalidValue;
+    const bool wide = p.n_pad > 128;
+    const int nb = p.n_pad * (p.comp && !wide ? 2 : 1);       // MMA N
+    if (nb > 256 || p.n_pad < 16 || p.n_pad % 16 || (wide && (!p.pairs || !p.comp || p.n_pad != 256))) return cudaErrorInvalidValue;
     int pair_k = nb > 128 ? 1 : kMaxPairK;
     if (tune.pair_k) pair_k = tune.pair_k;
     GemmDesc &d = p.g;
     d.pair_k = pair_k;
-    // the items are split evenly over one CTA per SM (fewer CTAs when there are fewer items)
-    const long long total = (long long)d.n_tiles * d.halves * pairs_per_tile(d);
+    // the items are split evenly over one CTA (CTA pair) per SM (two SMs), fewer when there are fewer items
+    d.group = p.pairs ? 2 : 1;
+    const int vtiles = d.n_tiles * d.halves;
+    const long long total = (long long)(p.pairs ? (vtiles + 1) / 2 : vtiles) * pairs_per_tile(d);
     if (total < 1) return cudaErrorInvalidValue;
-    int grid = total < n_sms ? (int)total : n_sms;
-    const long long ipc = (total + grid - 1) / grid;
+    long long groups = n_sms / d.group;
+    if (groups > total) groups = total;
+    const long long ipc = (total + groups - 1) / groups;
     d.items_per_cta = (int)ipc;
-    grid = (int)((total + ipc - 1) / ipc);
-    d.grid = grid;
+    d.grid = (int)((total + ipc - 1) / ipc) * d.group;
     return cudaSuccess;
 }
 
@@ -1127,11 +1451,14 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
         if (e != cudaSuccess) return e;
     }
     GemmDesc &d = p.g;
-    const int nb = p.n_pad * (p.comp ? 2 : 1);
+    const bool wide_in = p.n_pad > 128;
+    const int nb = p.n_pad * (p.comp && !wide_in ? 2 : 1);
     const int pair_k = d.pair_k, grid = d.grid;
     const long long ipc = d.items_per_cta;
     if ((size_t)(d.n_tiles * d.halves + grid) * slot_floats(p.n_pad) > partial_floats) return cudaErrorInvalidValue;
-    const size_t stage_bytes = (size_t)pair_k * ((size_t)kATileBytes + (size_t)nb * kBlockK * 2);
+    // activation bytes of a k-block per CTA: all rows, or half of them in a pair (both planes when wide)
+    const size_t act_bytes = (size_t)nb * kBlockK * 2 / (p.pairs && !wide_in ? 2 : 1);
+    const size_t stage_bytes = (size_t)pair_k * ((size_t)kATileBytes + act_bytes);
     // One CTA per SM with the whole shared memory as the ring.
     // two accumulator buffers of MMA N columns each
     int cols = 2 * nb, pow2 = 32;
@@ -1170,11 +1497,12 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     if (attr_set.needed()) {
         cudaError_t e = cudaSuccess;
         typedef void (*SKernel)(GemmMaps, GemmParams);
-        const SKernel all[4] = {gemm_stream_kernel<1, false>, gemm_stream_kernel<2, false>, gemm_stream_kernel<1, true>, gemm_stream_kernel<2, true>};
+        const SKernel all[8] = {gemm_stream_kernel<1, false>, gemm_stream_kernel<2, false>, gemm_stream_kernel<1, true>, gemm_stream_kernel<2, true>,
+                                gemm_pair_kernel<1, false>, gemm_pair_kernel<2, false>, gemm_pair_kernel<1, true>, gemm_pair_kernel<2, true>};
         // An SM splits its on-chip memory between shared memory and L1 when it is empty, to fit the kernel that
         // arrives; a streaming CTA of 195 KB would get a 196 KB split, and the finishing CTA of the same GEMM
         // could not settle beside it. Every kernel of the GEMM asks for the largest shared-memory split.
-        for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+        for (int i = 0; i < 8 && e == cudaSuccess; ++i) {
             e = cudaFuncSetAttribute(all[i], cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(all[i], cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         }
@@ -1183,9 +1511,13 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     }
     if (p.wait_limit_ns == 0) p.wait_limit_ns = kDefaultWaitLimitNs;
     {
-        LaunchCfg lc(grid, kThreads, smem, st);
+        LaunchCfg lc(grid, kThreads, smem, st, p.pairs ? 2 : 0);
         cudaError_t e;
-        if (d.w4) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<1, true>, maps, p)
+        if (p.pairs && wide_in) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<1, true>, maps, p)
+                                                : cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<2, true>, maps, p);
+        else if (p.pairs) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<1, false>, maps, p)
+                                          : cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<2, false>, maps, p);
+        else if (d.w4) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<1, true>, maps, p)
                                   : cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<2, true>, maps, p);
         else e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<1, false>, maps, p)
                              : cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<2, false>, maps, p);
@@ -1202,11 +1534,13 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     const int max_parts = (int)((pairs_per_tile(d) + ipc - 1) / ipc) + 1;
     const bool wide = max_parts > 4;           // many segments per tile (tiles split over many CTAs)
     const bool two = per_warp >= 2;            // several node groups per warp
+    const bool four = per_warp >= 4 && max_parts <= 2;   // many of them, and one or two segments each
     typedef void (*FinKernel)(GemmParams);
     FinKernel fk = nullptr;
 #define LLMCAD_PICK(MODE)                                                                                            \
     fk = wide ? (FinKernel)gemm_finish_kernel<MODE, 1, 8>                                                            \
-              : (two ? (FinKernel)gemm_finish_kernel<MODE, 2, 4> : (FinKernel)gemm_finish_kernel<MODE, 1, 4>)
+              : (four ? (FinKernel)gemm_finish_kernel<MODE, 4, 2>                                                            \
+                      : (two ? (FinKernel)gemm_finish_kernel<MODE, 2, 4> : (FinKernel)gemm_finish_kernel<MODE, 1, 4>))
     switch (d.ep.mode) {
     case EPI_QKV: LLMCAD_PICK(EPI_QKV); break;
     case EPI_RESID: LLMCAD_PICK(EPI_RESID); break;
@@ -1218,8 +1552,8 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
 #undef LLMCAD_PICK
     {
         // once per finishing kernel and device (see above)
-        static PerDeviceOnce fin_set[4][3];
-        PerDeviceOnce &once = fin_set[d.ep.mode & 3][wide ? 0 : (two ? 1 : 2)];
+        static PerDeviceOnce fin_set[4][4];
+        PerDeviceOnce &once = fin_set[d.ep.mode & 3][wide ? 0 : (four ? 3 : (two ? 1 : 2))];
         if (once.needed()) {
             const cudaError_t e = cudaFuncSetAttribute(fk, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
             if (e != cudaSuccess) return e;

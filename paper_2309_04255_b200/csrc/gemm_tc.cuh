@@ -17,6 +17,7 @@ struct GemmDesc {
     int halves;         // weight tiles per output tile: 2 (gate and up, SwiGLU), else 1
     int items_per_cta;  // ring items ((weight tile, k-blocks) pairs) per CTA of the streaming grid
     int grid;           // CTAs of the streaming grid
+    int group;          // 1, or 2: CTA pairs share items (items_per_cta counts a pair's)
     const uint8_t *w_tiled;  // weights as a sequence of pre-swizzled 16 KB tiles [tile][k-block] (see pack.cu),
                              // or nullptr: row-major weights through the tensor map
     int up_tile_offset;      // first tile of the up projection in the tiled sequence
@@ -33,6 +34,8 @@ struct GemmMaps {
 struct GemmParams {
     int n_pad;          // tree nodes padded to a multiple of 16
     int comp;           // 1: activations come as hi + lo planes; the MMA N is 2 * n_pad and the two columns of a node are added
+    int pairs;          // 1: CTA pairs (gemm_pair_kernel): maps.w is the packed matrix (make_packed_map), maps.x has boxes of half
+                        // of the MMA's rows (gemm_takes_pairs)
     int stages;         // depth of the shared-memory ring (INT4 weights: of the ring of expanded weight items)
     int pstages;        // INT4 weights: depth of the ring of packed tiles that feeds it
     int astages;        // INT4 weights: depth of the ring of activation items (with bf16 weights they share the weights' stages)
@@ -59,9 +62,15 @@ bool make_tensor_map_bf16(CUtensorMap *map, const void *base, uint64_t rows, uin
 
 // Tensor map over `planes` (1 or 2) row-major bf16 matrices [rows][cols] that lie plane_rows rows
 // apart, with a box of 64 columns x box_rows rows x planes: one copy brings the hi and the lo tile
-// of an activation k-block, one after the other, into shared memory. Rows beyond `rows` read as zero.
+// of an activation k-block, one after the other, into shared memory (box_planes of the planes). Rows beyond `rows`
+// read as zero.
 bool make_act_map_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t planes,
-                       uint64_t plane_rows);
+                       uint64_t plane_rows, uint32_t box_planes);
+// Tensor map over a packed weight matrix of `bytes` bytes (a sequence of 16 KB tiles): one box = one tile.
+bool make_packed_map(CUtensorMap *map, const void *tiled, uint64_t bytes);
+
+// Whether a GEMM with bf16 weights on this many (padded) nodes runs on CTA pairs. comp: hi and lo planes.
+bool gemm_takes_pairs(int n_pad, bool comp);
 // Any three-dimensional bf16 tensor with 128-byte swizzle and zero fill outside its bounds: dims and box
 // innermost first, strides (bytes) of dimensions 1 and 2.
 bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t dims[3], const uint64_t strides_bytes[2],

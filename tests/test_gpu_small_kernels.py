@@ -80,3 +80,20 @@ def test_one_kernel_fp32_pass(P, n, H, hd, f, V):
         check_acceptance_against_oracle(out, t, parent)
         assert out["accepted_path"][out["scalars"][B.S_ACCEPTED_LEN]:].tolist() == [-1] * (128 - out["scalars"][B.S_ACCEPTED_LEN])
     assert tw.v.launch_count() - l0 == 2
+
+
+@pytest.mark.parametrize("n_out,n_in,n", [(128, 64, 64), (300, 520, 64), (640, 128, 96), (257, 72, 128), (4096, 1000, 120), (9600, 4096, 128)])
+def test_gemm_on_cta_pairs(n_out, n_in, n):
+    """Weight tiles paired over two CTAs: one tile only (its pair is empty), an odd number of them, a ragged last
+    k-block, an odd number of k-blocks, half of the activation rows per CTA. bf16 inputs, fp32 sums: the error of
+    a sum of n_in products is at most n_in * 2^-24 of the sum of their magnitudes; 2e-6 * sqrt(n_in) of the largest
+    result is far inside what the random signs leave of that and far below a single wrong element."""
+    cfg = gen.ModelConfig("g", 0, 256, 2, 128, 256, 512, "bf16")
+    v = B.Verifier(cfg, 16)
+    g = torch.Generator(device=DEV).manual_seed(n_out + n_in + n)
+    w = torch.randn(n_out, n_in, generator=g, device=DEV).to(torch.bfloat16)
+    x = torch.randn(n, n_in, generator=g, device=DEV).to(torch.bfloat16)
+    y = v.skinny_gemm_tiled(v.tile_weight(w), n_out, x)
+    assert v.last_status() == 0
+    ref = x.double() @ w.double().t()
+    assert (y.double() - ref).abs().max() <= 2e-6 * n_in ** 0.5 * ref.abs().max()
