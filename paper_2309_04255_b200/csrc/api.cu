@@ -261,9 +261,9 @@ struct TcGemm {
     void set(llmcad_ctx *ctx, int l, int which, int act, int n_in, const EpiParams &ep, int n_pad)
     {
         const bool w4 = ctx->w4 && l >= 0;
-        p.pairs = !w4 && gemm_takes_pairs(n_pad, ctx->comp);
-        maps.x = p.pairs ? ctx->pair_maps[n_pad / 16][act] : ctx->act_maps[n_pad / 16][act];
-        if (p.pairs) maps.w = l < 0 ? ctx->weight_maps.back() : ctx->weight_maps[4 * (size_t)l + which];
+        p.pairs = gemm_takes_pairs(n_pad, ctx->comp);
+        maps.x = p.pairs && !w4 ? ctx->pair_maps[n_pad / 16][act] : ctx->act_maps[n_pad / 16][act];
+        if (p.pairs && !w4) maps.w = l < 0 ? ctx->weight_maps.back() : ctx->weight_maps[4 * (size_t)l + which];
         p.g = make_gemm_desc(n_in, ep, weight_ptr(ctx, l, which), w4);
         p.n_pad = n_pad;
         p.comp = ctx->comp ? 1 : 0;
@@ -1010,6 +1010,7 @@ int llmcad_skinny_gemm_tiled_int4(llmcad_ctx *ctx, const void *w_tiled, const vo
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
         return LLMCAD_ERR_CUDA;
     }
+    g.p.pairs = gemm_takes_pairs(n_pad, false);
     g.p.g = make_gemm_desc(n_in, ep, w_tiled, true);
     g.p.n_pad = n_pad;
     return g.launch(ctx, status, st);

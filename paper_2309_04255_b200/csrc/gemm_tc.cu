@@ -62,8 +62,6 @@ constexpr size_t kFinSmem = 24 * 1024;   // dynamic shared memory the finishing 
                                          // there for the next GEMM's streaming CTA
 constexpr int kATileBytes = kTileM * kBlockK * 2;  // 16 KB
 constexpr int kMaxStages = 16;
-constexpr int kMaxPStages = 24;   // INT4 weights: ring of packed tiles
-constexpr int kMaxAStages = 8;    // INT4 weights: ring of activation k-block sets, apart from the expanded weight tiles
 constexpr int kMaxPairK = 2;     // k-blocks per ring item (GemmDesc::pair_k): 2 = one 32 KB weight copy feeds 8 MMAs;
                                  // 1 for wide activation tiles, which would leave too few ring stages otherwise
 
@@ -255,10 +253,6 @@ struct SharedCtl {
     uint32_t tmem_base;
     volatile int abort_flag;
     volatile uint32_t a_issued;     // ring items whose weight copy (and expect_tx) has been issued
-    uint64_t pfull[kMaxPStages];    // INT4 weights: packed tile landed / packed stage free again
-    uint64_t pempty[kMaxPStages];
-    uint64_t afull[kMaxAStages];    // INT4 weights: activation tiles of an item landed / their slot free again
-    uint64_t aempty[kMaxAStages];
 };
 
 // A weight tile is 128 rows of the packed matrix. An output tile has one of them, or two (SwiGLU: gate and up),
@@ -521,7 +515,7 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
 
 #define LLMCAD_TRACE(slot) do { if (p.trace && blockIdx.x < 256) p.trace[(size_t)blockIdx.x * 16 + (slot)] = global_timer_ns(); } while (0)
 
-template <int PK, bool W4>
+template <int PK>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmParams p)
 {
@@ -536,16 +530,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
     const uint32_t stage_bytes = PK * (kATileBytes + b_tile_bytes);
     const uint32_t b_off = PK * kATileBytes;
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    // INT4 weights: three rings of their own. [p.stages expanded weight items of PK bf16 tiles, written by the dump
-    // warps and read by the MMA][p.astages activation items, PK k-blocks each, filled by the activation loader as far
-    // ahead as slots are free][p.pstages packed items of PK tiles of 4224 bytes each, filled by the weight producer].
-    // Every item needs its activation tiles from L2 (~1.5 us under load) and they are larger than its packed weights:
-    // kept in the stage of the expanded weights, as in the bf16 path, too few of them would be in flight.
-    constexpr uint32_t pstage_bytes = PK * kW4TileBytes;
-    constexpr uint32_t wstage_bytes = PK * kATileBytes;
-    const uint32_t astage_bytes = PK * b_tile_bytes;
-    const uint32_t act_base = smem_base + (uint32_t)p.stages * wstage_bytes;
-    const uint32_t packed_base = W4 ? act_base + (uint32_t)p.astages * astage_bytes : smem_base + (uint32_t)p.stages * stage_bytes;
     const uint32_t acc_cols = nb;                         // TMEM columns of one of the two accumulator buffers
     const uint64_t wait_limit = p.wait_limit_ns;          // every wait below gives up after this many ns
     const DepWait dep{p.dep_ctr, p.dep_target, wait_limit};
@@ -562,18 +546,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
     uint64_t pol_stream = 0;
     auto issue_item = [&]() {          // the next item of the stream into ring stage ps (which must be free)
         const int nk = pc.nk();
-        if (W4) {
-            // packed tiles go to the packed ring; the dump warps turn them into MMA stages
-            const uint32_t pf = smem_u32(&ctl.pfull[ps]);
-            mbar_expect_tx(pf, (uint32_t)nk * kW4TileBytes);
-            const size_t t = (size_t)packed_tile(d, pc.tile) * d.kb_per_tile + pc.kb0();
-            bulk_load_1d(packed_base + ps * pstage_bytes, d.w_tiled + t * kW4TileBytes, (uint32_t)nk * kW4TileBytes, pf, pol_stream);
-            if (pissued == 0) LLMCAD_TRACE(2);
-            ++pissued;
-            pc.advance();
-            if (++ps == p.pstages) { ps = 0; ppar ^= 1u; }
-            return;
-        }
         const uint32_t full = smem_u32(&ctl.full[ps]);
         const uint32_t dst = smem_base + ps * stage_bytes;
         mbar_expect_tx(full, (uint32_t)nk * (kATileBytes + b_tile_bytes));
@@ -594,19 +566,8 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
     };
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
-            // INT4: an expanded weight item is full when the four dump warps have written their quarters of it
-            mbar_init(smem_u32(&ctl.full[s]), W4 ? 4 : 1);
+            mbar_init(smem_u32(&ctl.full[s]), 1);
             mbar_init(smem_u32(&ctl.empty[s]), 1);
-        }
-        if (W4) {
-            for (int s = 0; s < p.pstages; ++s) {
-                mbar_init(smem_u32(&ctl.pfull[s]), 1);
-                mbar_init(smem_u32(&ctl.pempty[s]), 4);
-            }
-            for (int s = 0; s < p.astages; ++s) {
-                mbar_init(smem_u32(&ctl.afull[s]), 1);
-                mbar_init(smem_u32(&ctl.aempty[s]), 1);
-            }
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&ctl.tmem_full[b]), 1);
@@ -618,7 +579,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
         pc.init(d);
-        while (!pc.done() && pissued < (uint32_t)(W4 ? p.pstages : p.stages)) issue_item();
+        while (!pc.done() && pissued < (uint32_t)p.stages) issue_item();
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)),
@@ -645,7 +606,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             // into the ring.)
             uint64_t t_idle = 0;
             while (!pc.done()) {
-                if (mbar_try(smem_u32(W4 ? &ctl.pempty[ps] : &ctl.empty[ps]), ppar)) {
+                if (mbar_try(smem_u32(&ctl.empty[ps]), ppar)) {
                     issue_item();
                     t_idle = 0;
                     continue;
@@ -670,22 +631,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             if (!dep_wait_thread(dep)) timed_out = true;
             fence_proxy_async();          // the activations were written by ordinary stores; the copies below read them
             pdl_launch_dependents();
-            if (W4) {
-                // a ring of its own: item i goes to slot i % astages as soon as the MMAs of item i - astages have read it
-                uint32_t apar = 1;         // a fresh barrier passes a wait on parity 1
-                while (!c.done() && !timed_out && !p.withhold_act) {
-                    if (!mbar_wait(smem_u32(&ctl.aempty[s]), apar, abort_flag, wait_limit)) { timed_out = true; break; }
-                    const uint32_t full = smem_u32(&ctl.afull[s]);
-                    const uint32_t dst = act_base + s * astage_bytes;
-                    const int nk = c.nk();
-                    mbar_expect_tx(full, (uint32_t)nk * b_tile_bytes);
-                    for (int k = 0; k < nk; ++k)
-                        tma_load_3d(dst + k * b_tile_bytes, &maps.x, (c.kb0() + k) * kBlockK, full, pol_keep);
-                    c.advance();
-                    if (++s == p.astages) { s = 0; apar ^= 1u; }
-                }
-            }
-            while (!W4 && !c.done() && !timed_out && !p.withhold_act) {
+            while (!c.done() && !timed_out && !p.withhold_act) {
                 uint64_t t0 = 0;
                 // the stage is ours: the producer has passed its "empty" wait and armed the barrier
                 for (uint32_t spin = 0; (int32_t)(ctl.a_issued - (i + 1)) < 0; ++spin) {
@@ -714,8 +660,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             c.init(d);
             uint32_t seg = 0, ph = 0;   // ph: parity the MMA warp waits for on its stage's "full" barrier
             int s = 0;
-            int as = 0;                 // INT4: slot of the activation ring, and the parity waited for on its "full" barrier
-            uint32_t aph = 0;
             while (!c.done() && !timed_out) {
                 // one segment: the items of one tile that belong to this CTA
                 const int tile = c.tile;
@@ -726,10 +670,8 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                 const uint32_t d0 = tmem_base + buf * acc_cols;
                 for (int q = 0; !c.done() && c.tile == tile; ++q) {
                     if (!mbar_wait(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
-                    if (W4 && !mbar_wait(smem_u32(&ctl.afull[as]), aph, abort_flag, wait_limit)) { timed_out = true; break; }
                     tc_fence_after();
-                    const uint32_t a_addr = W4 ? smem_base + s * wstage_bytes : smem_base + s * stage_bytes;
-                    const uint32_t b_addr = W4 ? act_base + as * astage_bytes : a_addr + b_off;
+                    const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off;
                     const int nk = c.nk();
                     for (int k = 0; k < nk; ++k) {
                         const uint64_t a_desc = make_smem_desc(a_addr + k * kATileBytes);
@@ -741,10 +683,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                         }
                     }
                     tc_commit(smem_u32(&ctl.empty[s]));  // frees the stage when these MMAs have read it
-                    if (W4) {
-                        tc_commit(smem_u32(&ctl.aempty[as]));
-                        if (++as == p.astages) { as = 0; aph ^= 1u; }
-                    }
                     c.advance();
                     if (++s == p.stages) { s = 0; ph ^= 1u; }
                 }
@@ -758,92 +696,18 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
         // ================================================= accumulator dump (warps 2..5)
         const int lane_grp = warp & 3;                 // TMEM lanes 32*lane_grp .. +31 belong to this warp
         // the workspace may still be read by the finishing kernel of the previous GEMM
-        bool dep_ok = false;
-        if (!W4) {
-            if (!dep_wait_warp(dep, lane)) timed_out = true;
-            pdl_launch_dependents();
-            dep_ok = true;
-            if (threadIdx.x == 64) LLMCAD_TRACE(3);
-        }
+        if (!dep_wait_warp(dep, lane)) timed_out = true;
+        pdl_launch_dependents();
+        if (threadIdx.x == 64) LLMCAD_TRACE(3);
         const Range r = cta_range<PK>(d, (int)blockIdx.x);
         const int ipt = pairs_per_tile_c<PK>(d);
         const size_t slot_stride = slot_floats(p.n_pad);
-        // ---- INT4 weights: these warps also turn every packed item into the bf16 tiles the MMA reads, a quarter
-        // of the rows each, in the next free slot of the ring of expanded items. Element j of a word sits where
-        // (word >> 4k) & 0x000f000f picks elements 2k, 2k+1; OR-ing 0x4300 into each half makes the bf16 values
-        // 128 + u (u = q + 8), and one fused multiply-add per pair, (128 + u) * 2^e - 136 * 2^e, gives q * 2^e exactly.
-        Cursor<PK> dc;
-        dc.init(d);
-        int ds = 0, dps = 0;
-        uint32_t dpar = 1, dppar = 0;                  // a fresh "empty" barrier passes a wait on parity 1
-        uint8_t *const smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-        auto dequant_item = [&]() -> bool {
-            const int nk = dc.nk();
-            if (!mbar_wait_warp(smem_u32(&ctl.empty[ds]), dpar, abort_flag, lane, wait_limit)) return false;
-            if (!mbar_wait_warp(smem_u32(&ctl.pfull[dps]), dppar, abort_flag, lane, wait_limit)) return false;
-            const uint8_t *pk = smem_gen + (packed_base - smem_base) + (size_t)dps * pstage_bytes;
-            uint8_t *wt = smem_gen + (size_t)ds * wstage_bytes;
-            // lane = (row within a group of four, chunk): iteration `it` handles row 32 * lane_grp + 4 * it + lane / 8,
-            // words and stores of a warp instruction are contiguous (no bank conflicts). All loads of a k-block go
-            // out before the first conversion: a warp is alone on its scheduler here, so latency is what counts.
-            const int r_in = lane >> 3, c = lane & 7;
-            for (int k = 0; k < nk; ++k) {
-                const uint32_t *words = reinterpret_cast<const uint32_t *>(pk + (size_t)k * kW4TileBytes) + (lane_grp * 32 + r_in) * 8 + c;
-                const int8_t *exps = reinterpret_cast<const int8_t *>(pk + (size_t)k * kW4TileBytes + 4096) + lane_grp * 32 + r_in;
-                uint8_t *dst = wt + (size_t)k * kATileBytes + (size_t)(lane_grp * 32 + r_in) * 128;
-                uint32_t x[8];
-                int e[8];
-#pragma unroll
-                for (int it = 0; it < 8; ++it) {
-                    x[it] = words[it * 32];
-                    e[it] = exps[it * 4];
-                }
-#pragma unroll
-                for (int it = 0; it < 8; ++it) {
-                    const uint32_t s16 = (uint32_t)(e[it] + 127) << 7;                       // bf16 bits of 2^e
-                    const uint32_t b16 = 0x8000u | ((uint32_t)(e[it] + 134) << 7) | 8u;      // bf16 bits of -136 * 2^e
-                    const uint32_t s2 = s16 | (s16 << 16), b2 = b16 | (b16 << 16);
-                    uint32_t o[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint32_t t2 = ((x[it] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
-                        const __nv_bfloat162 rr = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2),
-                                                          *reinterpret_cast<const __nv_bfloat162 *>(&s2),
-                                                          *reinterpret_cast<const __nv_bfloat162 *>(&b2));
-                        o[j] = *reinterpret_cast<const uint32_t *>(&rr);
-                    }
-                    // row & 7 = (4 * it + r_in) & 7: the 128-byte swizzle of the MMA tile
-                    *reinterpret_cast<uint4 *>(dst + (size_t)it * 512 + ((c ^ ((4 * it + r_in) & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
-                }
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the tensor core reads what these threads wrote
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(smem_u32(&ctl.full[ds]));
-                mbar_arrive(smem_u32(&ctl.pempty[dps]));
-            }
-            dc.advance();
-            if (++ds == p.stages) { ds = 0; dpar ^= 1u; }
-            if (++dps == p.pstages) { dps = 0; dppar ^= 1u; }
-            return true;
-        };
         uint32_t seg = 0;
         for (int seg_begin = r.begin; seg_begin < r.end && !timed_out; ++seg) {
             const int tile = seg_begin / ipt;
             const int seg_end = min(r.end, (tile + 1) * ipt);
             const int buf = seg & 1;
             const uint32_t use = seg >> 1;
-            if (W4) {
-                for (int i = seg_begin; i < seg_end && !timed_out; ++i)
-                    if (!dequant_item()) timed_out = true;
-                if (timed_out) break;
-                if (!dep_ok) {          // the workspace may still be read by the previous GEMM's finishing kernel
-                    if (!dep_wait_warp(dep, lane)) { timed_out = true; break; }
-                    pdl_launch_dependents();
-                    dep_ok = true;
-                    if (threadIdx.x == 64) LLMCAD_TRACE(3);
-                }
-            }
             if (!mbar_wait_warp(smem_u32(&ctl.tmem_full[buf]), use & 1u, abort_flag, lane, wait_limit)) { timed_out = true; break; }
             tc_fence_after();
             if (threadIdx.x == 64 && seg == 0) LLMCAD_TRACE(4);
@@ -1183,6 +1047,336 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
     if (threadIdx.x == 32) LLMCAD_TRACE(13);
 }
 
+// ------------------------------------------------------------------------------------------------
+// The streaming kernel for INT4 weights.
+//
+// A quarter of the bytes, so HBM no longer sets the pace: expanding the weights and the MMAs do (a
+// tcgen05.mma of K = 16 takes ~48 cycles for up to 64 columns, 17 us per layer of the 7B shape, about what its
+// packed weights take from HBM). The weights are therefore expanded straight into tensor memory and multiplied
+// from there: thread = weight row = TMEM lane, eight codes of a word become four packed bf16 pairs (three
+// instructions a pair), 32 of which are the row's share of a k-block. The previous form wrote the expanded tiles
+// to shared memory, with four warps that also dumped the accumulators, and slots were handed around at 0.5 us an
+// item (7B shape, 32 nodes: 3.53 ms a pass).
+//
+// Warps: 0 producer of packed items (bulk copies), 1 TMEM allocator and MMA issuer, 2 activation loader (TMA),
+// 4..11 expansion and dump: warp w works on rows 32 * (w % 4) .., the two sets of four take alternate items and
+// alternate 16-node chunks of a dump. Three rings of items (PK k-blocks): packed (shared memory), expanded
+// (tensor memory, what the accumulators leave of the 512 columns), activations (shared memory). Until the grid
+// dependency the packed ring fills and the expanded ring as far as it reaches. 72 registers a thread: three warps
+// per scheduler beside the finishing CTA's three.
+//
+// The items are cut and ordered exactly as the kernels for bf16 weights cut theirs on the same number of nodes
+// (CTA pairs included, which here only means how tiles and ranges are dealt out), so that the sums are the same
+// to the bit.
+constexpr int kW4Threads = 384;
+constexpr int kMaxPStages = 16, kMaxXStages = 12, kMaxAStages = 12;
+
+struct W4Ctl {
+    uint64_t pfull[kMaxPStages], pempty[kMaxPStages];     // packed items
+    uint64_t xfull[kMaxXStages], xempty[kMaxXStages];     // expanded items
+    uint64_t afull[kMaxAStages], aempty[kMaxAStages];     // activation items
+    uint64_t tmem_full[2], tmem_empty[2];
+    uint32_t tmem_base;
+    volatile int abort_flag;
+};
+
+// D[tmem] (+)= A[tmem] * B[smem]^T; A: lanes = rows, one 32-bit column = two bf16 along K
+__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// 16 consecutive 32-bit columns of this thread's TMEM lane
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+          "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+// 16 columns at each of two addresses, summed (one wait for both loads)
+__device__ __forceinline__ void tc_ld16_sum2(uint32_t taddr_a, uint32_t taddr_b, float *v)
+{
+    uint32_t a[16], b[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%33];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]),
+          "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15])
+        : "r"(taddr_a), "r"(taddr_b)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(a[j]) + __uint_as_float(b[j]);
+}
+
+// slot and parity of a ring, stepped through n slots at a time
+struct RingPos {
+    int slot;
+    uint32_t par;
+    __device__ void step(int by, int n)
+    {
+        slot += by;
+        if (slot >= n) { slot -= n; par ^= 1u; }
+    }
+};
+
+template <int PK>
+__global__ void __maxnreg__(72)
+gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ W4Ctl ctl;
+    const GemmDesc &d = p.g;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t nb = (uint32_t)p.n_pad * (p.comp ? 2u : 1u);
+    const uint32_t b_tile_bytes = nb * kBlockK * 2, astage_bytes = PK * b_tile_bytes;
+    constexpr uint32_t pstage_bytes = PK * kW4TileBytes;
+    const uint32_t act_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t packed_base = act_base + (uint32_t)p.astages * astage_bytes;
+    const int acc_bufs = p.acc_bufs;
+    const uint64_t wait_limit = p.wait_limit_ns;
+    const DepWait dep{p.dep_ctr, p.dep_target, wait_limit};
+    if (threadIdx.x == 0) LLMCAD_TRACE(0);
+
+    // this CTA's items: with group == 2 two CTAs walk the same list of (pair of tiles, k-blocks), each for its tile
+    const int rank = d.group == 2 ? (int)blockIdx.x & 1 : 0, group = (int)blockIdx.x / d.group;
+    const int n_vtiles = d.n_tiles * d.halves, ppt = pairs_per_tile_c<PK>(d);
+    const int total = (n_vtiles + d.group - 1) / d.group * ppt;
+    const int begin = min(total, group * d.items_per_cta), end = min(total, begin + d.items_per_cta);
+    auto tile_of = [&](int unit) { return d.group == 2 ? 2 * unit + rank : unit; };
+
+    // ---- weight producer, across the start-up barrier: the first ring-full goes out at once
+    int pi = begin, put = begin / ppt, pkp = begin - put * ppt;
+    RingPos pp{0, 1};                              // a fresh barrier passes a wait on parity 1
+    uint64_t pol_stream = 0;
+    auto issue_item = [&]() {
+        const int nk = min(PK, d.kb_per_tile - pkp * PK), v = min(tile_of(put), n_vtiles - 1);
+        const uint32_t full = smem_u32(&ctl.pfull[pp.slot]);
+        mbar_expect_tx(full, (uint32_t)nk * kW4TileBytes);
+        bulk_load_1d(packed_base + pp.slot * pstage_bytes, d.w_tiled + ((size_t)packed_tile(d, v) * d.kb_per_tile + pkp * PK) * kW4TileBytes,
+                     (uint32_t)nk * kW4TileBytes, full, pol_stream);
+        ++pi;
+        if (++pkp == ppt) { pkp = 0; ++put; }
+        pp.step(1, p.pstages);
+    };
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.pstages; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), 4); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.xfull[s]), 4); mbar_init(smem_u32(&ctl.xempty[s]), 1); }
+        for (int s = 0; s < p.astages; ++s) { mbar_init(smem_u32(&ctl.afull[s]), 1); mbar_init(smem_u32(&ctl.aempty[s]), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&ctl.tmem_full[b]), 1); mbar_init(smem_u32(&ctl.tmem_empty[b]), 8); }
+        ctl.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
+        while (pi < end && pi - begin < p.pstages) issue_item();
+        LLMCAD_TRACE(2);
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl.tmem_base)),
+                     "r"((uint32_t)p.tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl.tmem_base, x_base = tmem_base + (uint32_t)acc_bufs * nb;
+    volatile int *abort_flag = &ctl.abort_flag;
+    bool timed_out = false;
+    if (threadIdx.x == 0) LLMCAD_TRACE(1);
+
+    if (warp == 0) {
+        if (lane == 0) {
+            uint64_t t_idle = 0;
+            while (pi < end) {
+                if (mbar_try(smem_u32(&ctl.pempty[pp.slot]), pp.par)) {
+                    issue_item();
+                    t_idle = 0;
+                    continue;
+                }
+                __nanosleep(32);
+                if (t_idle == 0) t_idle = global_timer_ns();
+                else if (*abort_flag || global_timer_ns() - t_idle > wait_limit) { timed_out = true; break; }
+            }
+            LLMCAD_TRACE(6);
+        }
+    } else if (warp == 2) {
+        // ================================================= activation loader
+        if (lane == 0) {
+            uint64_t pol_keep;
+            asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
+            RingPos a{0, 1};
+            int kp = begin % ppt;
+            if (!dep_wait_thread(dep)) timed_out = true;
+            fence_proxy_async();          // the activations were written by ordinary stores; the copies below read them
+            pdl_launch_dependents();
+            for (int i = begin; i < end && !timed_out; ++i) {
+                if (!mbar_wait(smem_u32(&ctl.aempty[a.slot]), a.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                const uint32_t full = smem_u32(&ctl.afull[a.slot]), dst = act_base + a.slot * astage_bytes;
+                const int nk = min(PK, d.kb_per_tile - kp * PK);
+                mbar_expect_tx(full, (uint32_t)nk * b_tile_bytes);
+                for (int k = 0; k < nk; ++k) tma_load_3d(dst + k * b_tile_bytes, &maps.x, (kp * PK + k) * kBlockK, full, pol_keep);
+                if (++kp == ppt) kp = 0;
+                a.step(1, p.astages);
+            }
+        }
+    } else if (warp == 1) {
+        // ================================================= MMA issuer
+        if (lane == 0) {
+            const uint32_t idesc = make_idesc(kTileM, (int)nb);
+            RingPos x{0, 0}, a{0, 0};
+            uint32_t seg = 0;
+            for (int i = begin; i < end && !timed_out; ++seg) {
+                const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt), first = i;
+                int kp = i - unit * ppt;
+                const int buf = acc_bufs == 2 ? (int)(seg & 1) : 0;
+                const uint32_t use = acc_bufs == 2 ? seg >> 1 : seg;
+                if (!mbar_wait(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+                const uint32_t d0 = tmem_base + buf * nb;
+                for (; i < seg_end; ++i, ++kp) {
+                    if (!mbar_wait(smem_u32(&ctl.xfull[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                    if (!mbar_wait(smem_u32(&ctl.afull[a.slot]), a.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                    tc_fence_after();
+                    const uint32_t at = x_base + x.slot * (PK * 32);
+                    const uint32_t b_addr = act_base + a.slot * astage_bytes;
+                    const int nk = min(PK, d.kb_per_tile - kp * PK);
+                    for (int k = 0; k < nk; ++k) {
+                        const uint64_t b_desc = make_smem_desc(b_addr + k * b_tile_bytes);
+#pragma unroll
+                        for (int k4 = 0; k4 < kBlockK / 16; ++k4)
+                            tc_mma_ts(d0, at + k * 32 + k4 * 8, b_desc + 2 * k4, idesc, (i > first || k > 0 || k4 > 0) ? 1u : 0u);
+                    }
+                    tc_commit(smem_u32(&ctl.xempty[x.slot]));
+                    tc_commit(smem_u32(&ctl.aempty[a.slot]));
+                    x.step(1, p.stages);
+                    a.step(1, p.astages);
+                }
+                if (timed_out) break;
+                tc_commit(smem_u32(&ctl.tmem_full[buf]));
+            }
+            LLMCAD_TRACE(7);
+        }
+    } else if (warp >= 4) {
+        // ================================================= expansion and dump
+        const int quad = warp & 3, set = (warp - 4) >> 2, row = quad * 32 + lane;
+        const uint32_t t_quad = (uint32_t)(quad * 32) << 16;
+        RingPos pk{0, 0}, x{0, 1};
+        pk.step(set, p.pstages);
+        x.step(set, p.stages);
+        int next = begin + set;                    // this set's next item
+        int kp = (begin + set) % ppt;
+        bool dep_ok = false;
+        uint32_t seg = 0;
+        for (int i = begin; i < end && !timed_out; ++seg) {
+            const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt);
+            // Items of the next segments are expanded ahead of this one's dump, as far as their slots are freed by MMAs
+            // that do not wait for it: the tensor cores have work while the accumulators leave.
+            const int limit = min(end, seg_end + p.stages);
+            while (next < limit && !timed_out) {
+                const int nk = min(PK, d.kb_per_tile - kp * PK);
+                if (!mbar_wait_warp(smem_u32(&ctl.pfull[pk.slot]), pk.par, abort_flag, lane, wait_limit)) { timed_out = true; break; }
+                // a row's 64 codes of a k-block: two 16-byte words, [half][row], and its exponent
+                const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes;
+                uint4 w[PK][2];
+                int e[PK];
+#pragma unroll
+                for (int k = 0; k < PK; ++k) {
+                    w[k][0] = *reinterpret_cast<const uint4 *>(src + k * kW4TileBytes + row * 16);
+                    w[k][1] = *reinterpret_cast<const uint4 *>(src + k * kW4TileBytes + 2048 + row * 16);
+                    e[k] = reinterpret_cast<const int8_t *>(src + k * kW4TileBytes + 4096)[row];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.pempty[pk.slot]));
+                if (!mbar_wait_warp(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, lane, wait_limit)) { timed_out = true; break; }
+                tc_fence_after();
+                const uint32_t dst = x_base + t_quad + x.slot * (PK * 32);
+#pragma unroll
+                for (int k = 0; k < PK; ++k) {
+                    if (k >= nk) break;
+                    // OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact
+                    const uint32_t s16 = (uint32_t)(e[k] + 127) << 7, b16 = 0x8000u | ((uint32_t)(e[k] + 134) << 7) | 8u;
+                    const uint32_t s2 = s16 | (s16 << 16), b2 = b16 | (b16 << 16);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t ww[4] = {w[k][h].x, w[k][h].y, w[k][h].z, w[k][h].w};
+                        uint32_t o[16];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint32_t t2 = ((ww[q] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
+                                const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2), *reinterpret_cast<const __nv_bfloat162 *>(&s2),
+                                                                 *reinterpret_cast<const __nv_bfloat162 *>(&b2));
+                                o[q * 4 + j] = *reinterpret_cast<const uint32_t *>(&r);
+                            }
+                        tc_st16(dst + k * 32 + h * 16, o);
+                    }
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.xfull[x.slot]));
+                next += 2;
+                kp += 2;
+                while (kp >= ppt) kp -= ppt;
+                pk.step(2, p.pstages);
+                x.step(2, p.stages);
+            }
+            if (timed_out) break;
+            // ---- dump
+            if (!dep_ok) {                          // the workspace may still be read by the previous GEMM's finishing kernel
+                if (!dep_wait_warp(dep, lane)) { timed_out = true; break; }
+                pdl_launch_dependents();
+                dep_ok = true;
+                if (threadIdx.x == 128) LLMCAD_TRACE(3);
+            }
+            const int v = tile_of(unit), buf = acc_bufs == 2 ? (int)(seg & 1) : 0;
+            const uint32_t use = acc_bufs == 2 ? seg >> 1 : seg;
+            if (!mbar_wait_warp(smem_u32(&ctl.tmem_full[buf]), use & 1u, abort_flag, lane, wait_limit)) { timed_out = true; break; }
+            tc_fence_after();
+            if (v < n_vtiles) {
+                if (!LLMCAD_CHECK(v >= 0 && v + d.group * group < n_vtiles + d.grid, p.status)) { timed_out = true; break; }
+                float *dst = p.partials + (size_t)(v + d.group * group) * slot_floats(p.n_pad) + (size_t)quad * p.n_pad * 32 + lane;
+                const uint32_t t_lane = tmem_base + t_quad + buf * nb;
+                for (int c0 = 16 * set; c0 < p.n_pad; c0 += 32) {
+                    float t[16];
+                    if (p.comp) tc_ld16_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
+                    else tc_ld16(t_lane + c0, t);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * 32] = t[j];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&ctl.tmem_empty[buf]));
+            i = seg_end;
+        }
+        if (threadIdx.x == 128) LLMCAD_TRACE(8);
+    }
+    __syncwarp();
+    timed_out = __any_sync(0xffffffffu, timed_out);
+    if (timed_out) {
+        *abort_flag = 1;
+        atomicCAS(p.status, 0, LLMCAD_ERR_TIMEOUT);
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp >= 4 && warp <= 7 && lane == 0) dep_arrive(p.s_done);      // four arrivals per CTA, behind the barrier: both sets have dumped
+    if (warp == 1) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
+        if (lane == 0) LLMCAD_TRACE(13);
+    }
+}
+
 // Adds the segments of every tile and applies the fused epilogue; see the head of the file. The
 // work is cut into (tile, 32-row group) pairs; k warps share a pair's node groups, k chosen so that
 // all warps of the grid have work. G node groups and KB segments of each are loaded in one go
@@ -1389,13 +1583,13 @@ GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool
 namespace {
 // tuning aids from the environment, read once per process
 struct Tuning {
-    int pair_k = 0, stages_cap = 0, w4_wstages = 3, w4_pstages = 4, cta_pair_min = 80;
+    int pair_k = 0, stages_cap = 0, w4_xstages = kMaxXStages, w4_pstages = kMaxPStages, cta_pair_min = 80;
     Tuning()
     {
         if (const char *e = getenv("LLMCAD_GEMM_PAIR_K")) { const int v = atoi(e); if (v == 1 || v == 2) pair_k = v; }
         if (const char *e = getenv("LLMCAD_GEMM_STAGES")) { const int v = atoi(e); if (v >= 2) stages_cap = v; }
         if (const char *e = getenv("LLMCAD_CTA_PAIR_MIN")) cta_pair_min = atoi(e);
-        if (const char *e = getenv("LLMCAD_W4_WSTAGES")) { const int v = atoi(e); if (v >= 2 && v <= kMaxStages) w4_wstages = v; }
+        if (const char *e = getenv("LLMCAD_W4_XSTAGES")) { const int v = atoi(e); if (v >= 2 && v <= kMaxXStages) w4_xstages = v; }
         if (const char *e = getenv("LLMCAD_W4_PSTAGES")) { const int v = atoi(e); if (v >= 2 && v <= kMaxPStages) w4_pstages = v; }
     }
 };
@@ -1457,7 +1651,7 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     const long long ipc = d.items_per_cta;
     if ((size_t)(d.n_tiles * d.halves + grid) * slot_floats(p.n_pad) > partial_floats) return cudaErrorInvalidValue;
     // activation bytes of a k-block per CTA: all rows, or half of them in a pair (both planes when wide)
-    const size_t act_bytes = (size_t)nb * kBlockK * 2 / (p.pairs && !wide_in ? 2 : 1);
+    const size_t act_bytes = (size_t)nb * kBlockK * 2 / (p.pairs && !d.w4 && !wide_in ? 2 : 1);
     const size_t stage_bytes = (size_t)pair_k * ((size_t)kATileBytes + act_bytes);
     // One CTA per SM with the whole shared memory as the ring.
     // two accumulator buffers of MMA N columns each
@@ -1471,33 +1665,38 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     if (tune.stages_cap && tune.stages_cap < stages) stages = tune.stages_cap;   // tuning aid: cap the ring depth
     if (stages < 2) return cudaErrorInvalidConfiguration;
     size_t smem = (size_t)stages * stage_bytes + 1024;
-    p.pstages = 0;
-    p.astages = 0;
+    p.pstages = p.astages = p.acc_bufs = 0;
     if (d.w4) {
-        // INT4 weights: three rings (see the kernel). Three expanded items (8-layer pass of the 7B shape at 32 nodes:
-        // 1.08 ms with two, 0.97 ms with three or four), a few packed items (they are small, 8.4 KB per 32 KB of
-        // bf16; 3 to 12 of them measure the same), and the rest of the shared memory for activation items.
+        // Three rings (see the kernel). Tensor memory, all 512 columns: two accumulators if at least four k-blocks of
+        // expanded weights (32 columns each) fit beside them, else one. Shared memory: six activation items if they fit
+        // beside four packed ones, the rest packed items.
         if (d.w_tiled == nullptr) return cudaErrorInvalidValue;
-        const size_t pstage = (size_t)pair_k * kW4TileBytes, wstage = (size_t)pair_k * kATileBytes;
-        const size_t astage = (size_t)pair_k * nb * kBlockK * 2;
-        stages = tune.w4_wstages;
-        int pst = tune.w4_pstages;
-        if ((size_t)stages * wstage + (size_t)pst * pstage + 2 * astage > full_limit) return cudaErrorInvalidConfiguration;
-        int ast = (int)((full_limit - (size_t)stages * wstage - (size_t)pst * pstage) / astage);
-        if (ast > kMaxAStages) ast = kMaxAStages;
-        // what the activation ring does not use goes to the packed ring
-        pst = (int)((full_limit - (size_t)stages * wstage - (size_t)ast * astage) / pstage);
-        if (pst > kMaxPStages) pst = kMaxPStages;
+        p.acc_bufs = 512 - 2 * nb >= 4 * 32 ? 2 : 1;
+        stages = (512 - p.acc_bufs * nb) / (32 * pair_k);
+        if (stages > tune.w4_xstages) stages = tune.w4_xstages;
+        // The two sets of expanding warps take alternate items. The rings they wait on have an even number of slots, so
+        // that a set comes back to a slot every lap: every second lap the parity would be the one it has already seen.
+        stages &= ~1;
+        const size_t pstage = (size_t)pair_k * kW4TileBytes, astage = (size_t)pair_k * nb * kBlockK * 2;
+        int ast = (int)((full_limit - 4 * pstage) / astage);
+        if (ast > 6) ast = 6;
+        int pst = (int)((full_limit - (size_t)ast * astage) / pstage);
+        if (pst > tune.w4_pstages) pst = tune.w4_pstages;
+        pst &= ~1;
+        if (ast < 2 || pst < 2 || stages < 2) return cudaErrorInvalidConfiguration;
         p.pstages = pst;
         p.astages = ast;
-        smem = (size_t)stages * wstage + (size_t)ast * astage + (size_t)pst * pstage + 1024;
+        p.tmem_cols = 512;
+        smem = (size_t)ast * astage + (size_t)pst * pstage + 1024;
+        // as much as the bf16 kernels ask for, so that no second streaming CTA (and its tensor memory) settles beside it
+        if (smem < full_limit) smem = full_limit;
     }
     p.stages = stages;
     static PerDeviceOnce attr_set;
     if (attr_set.needed()) {
         cudaError_t e = cudaSuccess;
         typedef void (*SKernel)(GemmMaps, GemmParams);
-        const SKernel all[8] = {gemm_stream_kernel<1, false>, gemm_stream_kernel<2, false>, gemm_stream_kernel<1, true>, gemm_stream_kernel<2, true>,
+        const SKernel all[8] = {gemm_stream_kernel<1>, gemm_stream_kernel<2>, gemm_w4_kernel<1>, gemm_w4_kernel<2>,
                                 gemm_pair_kernel<1, false>, gemm_pair_kernel<2, false>, gemm_pair_kernel<1, true>, gemm_pair_kernel<2, true>};
         // An SM splits its on-chip memory between shared memory and L1 when it is empty, to fit the kernel that
         // arrives; a streaming CTA of 195 KB would get a 196 KB split, and the finishing CTA of the same GEMM
@@ -1511,16 +1710,15 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     }
     if (p.wait_limit_ns == 0) p.wait_limit_ns = kDefaultWaitLimitNs;
     {
-        LaunchCfg lc(grid, kThreads, smem, st, p.pairs ? 2 : 0);
+        LaunchCfg lc(grid, d.w4 ? kW4Threads : kThreads, smem, st, p.pairs && !d.w4 ? 2 : 0);
         cudaError_t e;
-        if (p.pairs && wide_in) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<1, true>, maps, p)
-                                                : cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<2, true>, maps, p);
-        else if (p.pairs) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<1, false>, maps, p)
-                                          : cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<2, false>, maps, p);
-        else if (d.w4) e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<1, true>, maps, p)
-                                  : cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<2, true>, maps, p);
-        else e = pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<1, false>, maps, p)
-                             : cudaLaunchKernelEx(&lc.cfg, gemm_stream_kernel<2, false>, maps, p);
+#define LLMCAD_BY_K(KERNEL1, KERNEL2) \
+    (pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, KERNEL1, maps, p) : cudaLaunchKernelEx(&lc.cfg, KERNEL2, maps, p))
+        if (d.w4) e = LLMCAD_BY_K(gemm_w4_kernel<1>, gemm_w4_kernel<2>);
+        else if (p.pairs && wide_in) e = LLMCAD_BY_K((gemm_pair_kernel<1, true>), (gemm_pair_kernel<2, true>));
+        else if (p.pairs) e = LLMCAD_BY_K((gemm_pair_kernel<1, false>), (gemm_pair_kernel<2, false>));
+        else e = LLMCAD_BY_K(gemm_stream_kernel<1>, gemm_stream_kernel<2>);
+#undef LLMCAD_BY_K
         if (e != cudaSuccess) return e;
         if (launched) ++*launched;
     }

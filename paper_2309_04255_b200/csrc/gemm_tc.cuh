@@ -34,11 +34,12 @@ struct GemmMaps {
 struct GemmParams {
     int n_pad;          // tree nodes padded to a multiple of 16
     int comp;           // 1: activations come as hi + lo planes; the MMA N is 2 * n_pad and the two columns of a node are added
-    int pairs;          // 1: CTA pairs (gemm_pair_kernel): maps.w is the packed matrix (make_packed_map), maps.x has boxes of half
+    int pairs;          // 1: items are dealt out to CTA pairs; with bf16 weights (gemm_pair_kernel) maps.w is the packed matrix (make_packed_map), maps.x has boxes of half
                         // of the MMA's rows (gemm_takes_pairs)
-    int stages;         // depth of the shared-memory ring (INT4 weights: of the ring of expanded weight items)
-    int pstages;        // INT4 weights: depth of the ring of packed tiles that feeds it
+    int stages;         // depth of the shared-memory ring (INT4 weights: of the ring of expanded items in tensor memory)
+    int pstages;        // INT4 weights: depth of the ring of packed items that feeds it
     int astages;        // INT4 weights: depth of the ring of activation items (with bf16 weights they share the weights' stages)
+    int acc_bufs;       // INT4 weights: accumulator buffers (always two with bf16 weights)
     int tmem_cols;      // allocated TMEM columns (power of two)
     float *partials;    // segment slots [weight tiles + grid][4 row groups][n_pad][32 rows] fp32: the segment of
                         // weight tile v held by CTA c sits in slot v + c

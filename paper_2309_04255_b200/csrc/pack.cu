@@ -98,11 +98,12 @@ __global__ void quantize_int4_plain_kernel(const uint4 *__restrict__ w, int n_ou
     for (int i = 0; i < 64; ++i) q[(size_t)row * n_in + (size_t)g * 64 + i] = (int8_t)((int)u[i] - 8);
 }
 
-// The layout the GEMM streams: per (tile of 128 rows, k-block of 64 columns) 4224 bytes: 128 rows x 8
-// words of eight codes each (word c of row r = columns 8c .. 8c+7, element j of the word in the nibble
-// at bit 4 * (j / 2) + 16 * (j % 2), so that (word >> 4k) & 0x000f000f holds elements 2k and 2k + 1 in
-// its two halves), then the 128 exponents of the rows. Tiles in the order [tile][k-block]. Rows past
-// the matrix are zero (code 8 = 0, exponent -126).
+// The layout the GEMM streams: per (tile of 128 rows, k-block of 64 columns) 4224 bytes: 2 x 128 rows x 4
+// words of eight codes each (word c of row r = columns 8c .. 8c+7; words 0-3 of all rows, then words 4-7, so that
+// 32 threads reading 16 bytes of a row each touch 512 consecutive bytes; element j of a word in the nibble at bit
+// 4 * (j / 2) + 16 * (j % 2), so that (word >> 4k) & 0x000f000f holds elements 2k and 2k + 1 in its two halves),
+// then the 128 exponents of the rows. Tiles in the order [tile][k-block]. Rows past the matrix are zero (code 8
+// = 0, exponent -126).
 __global__ void tile_weight_int4_kernel(const uint4 *__restrict__ w, int n_out, int n_in, int kb_per_tile, long long n_rows,
                                         uint8_t *__restrict__ dst)
 {
@@ -132,9 +133,9 @@ __global__ void tile_weight_int4_kernel(const uint4 *__restrict__ w, int n_out, 
 #pragma unroll
         for (int c = 0; c < 8; ++c) words[c] = 0x88888888u;
     }
-    uint4 *tw = reinterpret_cast<uint4 *>(t) + (size_t)r * 2;
+    uint4 *tw = reinterpret_cast<uint4 *>(t) + r;
     tw[0] = make_uint4(words[0], words[1], words[2], words[3]);
-    tw[1] = make_uint4(words[4], words[5], words[6], words[7]);
+    tw[128] = make_uint4(words[4], words[5], words[6], words[7]);
     reinterpret_cast<int8_t *>(t + 4096)[r] = (int8_t)ex;
 }
 
