@@ -125,6 +125,49 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
+// Wait of a warp whose lanes stay together (the MMA warps): every lane tries, so that no broadcast follows.
+__device__ __forceinline__ bool mbar_wait_all(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint64_t wait_limit)
+{
+    uint64_t t0 = 0;
+    for (uint32_t it = 1; !__all_sync(0xffffffffu, mbar_try(bar, parity)); ++it) {
+        if ((it & 255u) == 0) {
+            bool out = *abort_flag != 0;
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else out |= now - t0 > wait_limit;
+            if (__any_sync(0xffffffffu, out)) return false;
+        }
+    }
+    return true;
+}
+// Whether the phase is complete, without waiting.
+__device__ __forceinline__ bool mbar_test_all(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
+}
+// Threads that issue MMAs: the code between two of them is what limits the rate (one lane under `if (lane == 0)` got
+// through 8 MMAs, their commit and two barrier waits in 1250 cycles, four times what the tensor pipe needs for 64
+// columns: every operand went through a per-thread register). The MMA warps therefore stay converged, so that
+// addresses and descriptors live in uniform registers, and one elected lane issues.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)::"memory");
+    return ok != 0;
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar,
                                             uint64_t policy)
@@ -523,7 +566,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
     __shared__ SharedCtl ctl;
     const GemmDesc &d = p.g;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const uint32_t nb = (uint32_t)p.n_pad * (p.comp ? 2u : 1u);   // activation rows per k-block = the MMA N: nodes (hi | lo)
     const uint32_t b_tile_bytes = nb * kBlockK * 2;
     // stage: [weights k-block 0 | weights k-block 1 | activations k-block 0 | activations k-block 1]
@@ -654,44 +697,48 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
         }
     } else if (warp == 1) {
         // ================================================= MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc(kTileM, (int)nb);
-            Cursor<PK> c;
-            c.init(d);
-            uint32_t seg = 0, ph = 0;   // ph: parity the MMA warp waits for on its stage's "full" barrier
-            int s = 0;
-            while (!c.done() && !timed_out) {
-                // one segment: the items of one tile that belong to this CTA
-                const int tile = c.tile;
-                const int buf = seg & 1;
-                const uint32_t use = seg >> 1;                        // how often this buffer has been used before
-                if (!mbar_wait(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+        const uint32_t idesc = make_idesc(kTileM, (int)nb);
+        const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
+        const bool leader = elect_one();
+        const Range r = cta_range<PK>(d, (int)blockIdx.x);
+        const int ppt = pairs_per_tile_c<PK>(d), kbpt = d.kb_per_tile;
+        uint32_t seg = 0, ph = 0;       // ph: parity to wait for on the stage's "full" barrier
+        int s = 0;
+        bool ready = false;             // the next item's barrier has been seen complete
+        for (int i = r.begin; i < r.end && !timed_out; ++seg) {
+            // one segment: the items of one tile that belong to this CTA
+            const int tile = i / ppt, seg_end = min(r.end, (tile + 1) * ppt);
+            int kb = (i - tile * ppt) * PK;
+            const int buf = seg & 1;
+            // (seg >> 1: how often this buffer has been used before)
+            if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+            const uint32_t d0 = tmem + buf * acc_cols;
+            uint32_t acc = 0;
+            for (; i < seg_end; ++i, kb += PK) {
+                if (!ready && !mbar_wait_all(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
                 tc_fence_after();
-                const uint32_t d0 = tmem_base + buf * acc_cols;
-                for (int q = 0; !c.done() && c.tile == tile; ++q) {
-                    if (!mbar_wait(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
-                    tc_fence_after();
-                    const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off;
-                    const int nk = c.nk();
-                    for (int k = 0; k < nk; ++k) {
-                        const uint64_t a_desc = make_smem_desc(a_addr + k * kATileBytes);
-                        const uint64_t b_desc = make_smem_desc(b_addr + k * b_tile_bytes);
+                const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off, empty = smem_u32(&ctl.empty[s]);
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
+                ready = i + 1 < r.end && mbar_test_all(smem_u32(&ctl.full[s]), ph);
+                const int nk = min(PK, kbpt - kb);
+                const uint64_t a_desc = make_smem_desc(a_addr), b_desc = make_smem_desc(b_addr);
+                if (leader) {
 #pragma unroll
-                        for (int k4 = 0; k4 < kBlockK / 16; ++k4) {
+                    for (int k = 0; k < PK; ++k) {
+                        if (k >= nk) break;
+#pragma unroll
+                        for (int k4 = 0; k4 < kBlockK / 16; ++k4)
                             // advancing 16 bf16 = 32 bytes inside the swizzle row: +2 in the >>4 address field
-                            tc_mma_bf16(d0, a_desc + 2 * k4, b_desc + 2 * k4, idesc, (q > 0 || k > 0 || k4 > 0) ? 1u : 0u);
-                        }
+                            tc_mma_bf16(d0, a_desc + k * (kATileBytes >> 4) + 2 * k4, b_desc + k * (b_tile_bytes >> 4) + 2 * k4, idesc,
+                                        k > 0 || k4 > 0 ? 1u : acc);
                     }
-                    tc_commit(smem_u32(&ctl.empty[s]));  // frees the stage when these MMAs have read it
-                    c.advance();
-                    if (++s == p.stages) { s = 0; ph ^= 1u; }
+                    tc_commit(empty);                        // frees the stage when these MMAs have read it
+                    if (i + 1 == seg_end) tc_commit(smem_u32(&ctl.tmem_full[buf]));
                 }
-                if (timed_out) break;
-                tc_commit(smem_u32(&ctl.tmem_full[buf]));
-                ++seg;
+                acc = 1;
             }
-            LLMCAD_TRACE(7);
         }
+        if (lane == 0) LLMCAD_TRACE(7);
     } else {
         // ================================================= accumulator dump (warps 2..5)
         const int lane_grp = warp & 3;                 // TMEM lanes 32*lane_grp .. +31 belong to this warp
@@ -839,7 +886,7 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
     __shared__ SharedCtl ctl;
     const GemmDesc &d = p.g;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const int rank = (int)blockIdx.x & 1, group = (int)blockIdx.x >> 1;
     const int n_vtiles = d.n_tiles * d.halves;
     const uint32_t nb = (uint32_t)p.n_pad * (p.comp && !kWide ? 2u : 1u);      // MMA N
@@ -949,39 +996,46 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
         }
     } else if (warp == 1) {
         // ================================================= MMA issuer (first CTA of the pair)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc = make_idesc(2 * kTileM, (int)nb);
+            const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
+            const bool leader = elect_one();
             uint32_t seg = 0, ph = 0;
             int s = 0;
+            bool ready = false;
             for (int i = begin; i < end && !timed_out; ++seg) {
-                const int pt = i / ppt, seg_end = min(end, (pt + 1) * ppt), first = i;
+                const int pt = i / ppt, seg_end = min(end, (pt + 1) * ppt);
                 int kb = (i - pt * ppt) * PK;
                 const int buf = seg & 1;
-                if (!mbar_wait(smem_u32(&ctl.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
-                tc_fence_after();
-                const uint32_t d0 = tmem_base + buf * nb;
+                if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+                const uint32_t d0 = tmem + buf * nb;
+                uint32_t acc = 0;
                 for (; i < seg_end; ++i, kb += PK) {
-                    if (!mbar_wait(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
+                    if (!ready && !mbar_wait_all(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
                     tc_fence_after();
-                    const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off;
-                    const int nk = min(PK, d.kb_per_tile - kb);
-                    for (int k = 0; k < nk; ++k) {
-                        const uint64_t a_desc = make_smem_desc(a_addr + k * kATileBytes);
-#pragma unroll
-                        for (int pl = 0; pl < (kWide ? 2 : 1); ++pl) {
-                            const uint64_t b_desc = make_smem_desc(b_addr + k * b_tile_bytes + pl * b_half);
-#pragma unroll
-                            for (int k4 = 0; k4 < kBlockK / 16; ++k4)
-                                tc_mma_pair(d0, a_desc + 2 * k4, b_desc + 2 * k4, idesc, (i > first || k > 0 || pl > 0 || k4 > 0) ? 1u : 0u);
-                        }
-                    }
-                    tc_commit_pair(smem_u32(&ctl.empty[s]));
+                    const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off, empty = smem_u32(&ctl.empty[s]);
                     if (++s == p.stages) { s = 0; ph ^= 1u; }
+                    ready = i + 1 < end && mbar_test_all(smem_u32(&ctl.full[s]), ph);
+                    const int nk = min(PK, d.kb_per_tile - kb);
+                    const uint64_t a_desc = make_smem_desc(a_addr), b_desc = make_smem_desc(b_addr);
+                    if (leader) {
+#pragma unroll
+                        for (int k = 0; k < PK; ++k) {
+                            if (k >= nk) break;
+#pragma unroll
+                            for (int pl = 0; pl < (kWide ? 2 : 1); ++pl)
+#pragma unroll
+                                for (int k4 = 0; k4 < kBlockK / 16; ++k4)
+                                    tc_mma_pair(d0, a_desc + k * (kATileBytes >> 4) + 2 * k4, b_desc + ((k * b_tile_bytes + pl * b_half) >> 4) + 2 * k4, idesc,
+                                                k > 0 || pl > 0 || k4 > 0 ? 1u : acc);
+                        }
+                        tc_commit_pair(empty);
+                        if (i + 1 == seg_end) tc_commit_pair(smem_u32(&ctl.tmem_full[buf]));
+                    }
+                    acc = 1;
                 }
-                if (timed_out) break;
-                tc_commit_pair(smem_u32(&ctl.tmem_full[buf]));
             }
-            LLMCAD_TRACE(7);
+            if (lane == 0) LLMCAD_TRACE(7);
         }
     } else {
         // ================================================= accumulator dump (warps 2..5): this CTA's weight tile
@@ -1074,7 +1128,7 @@ constexpr int kMaxPStages = 16, kMaxXStages = 12, kMaxAStages = 12;
 struct W4Ctl {
     uint64_t pfull[kMaxPStages], pempty[kMaxPStages];     // packed items
     uint64_t xfull[kMaxXStages], xempty[kMaxXStages];     // expanded items
-    uint64_t afull[kMaxAStages], aempty[kMaxAStages];     // activation items
+    uint64_t afull[kMaxAStages];                          // activation items
     uint64_t tmem_full[2], tmem_empty[2];
     uint32_t tmem_base;
     volatile int abort_flag;
@@ -1134,7 +1188,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     __shared__ W4Ctl ctl;
     const GemmDesc &d = p.g;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const uint32_t nb = (uint32_t)p.n_pad * (p.comp ? 2u : 1u);
     const uint32_t b_tile_bytes = nb * kBlockK * 2, astage_bytes = PK * b_tile_bytes;
     constexpr uint32_t pstage_bytes = PK * kW4TileBytes;
@@ -1169,7 +1223,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.pstages; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), 4); }
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.xfull[s]), 4); mbar_init(smem_u32(&ctl.xempty[s]), 1); }
-        for (int s = 0; s < p.astages; ++s) { mbar_init(smem_u32(&ctl.afull[s]), 1); mbar_init(smem_u32(&ctl.aempty[s]), 1); }
+        for (int s = 0; s < p.astages; ++s) mbar_init(smem_u32(&ctl.afull[s]), 1);
         for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&ctl.tmem_full[b]), 1); mbar_init(smem_u32(&ctl.tmem_empty[b]), 8); }
         ctl.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1212,13 +1266,19 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         if (lane == 0) {
             uint64_t pol_keep;
             asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
-            RingPos a{0, 1};
+            // Item i goes where item i - astages was, once the MMAs have read that: the barrier of its expanded slot says
+            // so. (There are at least as many expanded slots as activation slots: the barrier cannot be a lap further,
+            // because the item that would take it there has no activations yet.)
+            RingPos a{0, 0}, x{0, 0};
             int kp = begin % ppt;
             if (!dep_wait_thread(dep)) timed_out = true;
             fence_proxy_async();          // the activations were written by ordinary stores; the copies below read them
             pdl_launch_dependents();
             for (int i = begin; i < end && !timed_out; ++i) {
-                if (!mbar_wait(smem_u32(&ctl.aempty[a.slot]), a.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                if (i - begin >= p.astages) {
+                    if (!mbar_wait(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                    x.step(1, p.stages);
+                }
                 const uint32_t full = smem_u32(&ctl.afull[a.slot]), dst = act_base + a.slot * astage_bytes;
                 const int nk = min(PK, d.kb_per_tile - kp * PK);
                 mbar_expect_tx(full, (uint32_t)nk * b_tile_bytes);
@@ -1229,40 +1289,46 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         }
     } else if (warp == 1) {
         // ================================================= MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc(kTileM, (int)nb);
-            RingPos x{0, 0}, a{0, 0};
-            uint32_t seg = 0;
-            for (int i = begin; i < end && !timed_out; ++seg) {
-                const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt), first = i;
-                int kp = i - unit * ppt;
-                const int buf = acc_bufs == 2 ? (int)(seg & 1) : 0;
-                const uint32_t use = acc_bufs == 2 ? seg >> 1 : seg;
-                if (!mbar_wait(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
-                const uint32_t d0 = tmem_base + buf * nb;
-                for (; i < seg_end; ++i, ++kp) {
-                    if (!mbar_wait(smem_u32(&ctl.xfull[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
-                    if (!mbar_wait(smem_u32(&ctl.afull[a.slot]), a.par, abort_flag, wait_limit)) { timed_out = true; break; }
-                    tc_fence_after();
-                    const uint32_t at = x_base + x.slot * (PK * 32);
-                    const uint32_t b_addr = act_base + a.slot * astage_bytes;
-                    const int nk = min(PK, d.kb_per_tile - kp * PK);
-                    for (int k = 0; k < nk; ++k) {
-                        const uint64_t b_desc = make_smem_desc(b_addr + k * b_tile_bytes);
+        const uint32_t idesc = make_idesc(kTileM, (int)nb);
+        const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0), xb = tmem + (uint32_t)acc_bufs * nb;
+        const bool leader = elect_one();
+        RingPos x{0, 0}, a{0, 0};
+        uint32_t seg = 0;
+        bool ready_x = false, ready_a = false;
+        for (int i = begin; i < end && !timed_out; ++seg) {
+            const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt);
+            int kb = (i - unit * ppt) * PK;
+            const int buf = acc_bufs == 2 ? (int)(seg & 1) : 0;
+            const uint32_t use = acc_bufs == 2 ? seg >> 1 : seg;
+            if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+            const uint32_t d0 = tmem + buf * nb;
+            uint32_t acc = 0;
+            for (; i < seg_end; ++i, kb += PK) {
+                if (!ready_x && !mbar_wait_all(smem_u32(&ctl.xfull[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                if (!ready_a && !mbar_wait_all(smem_u32(&ctl.afull[a.slot]), a.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                tc_fence_after();
+                const uint32_t at = xb + x.slot * (PK * 32), empty = smem_u32(&ctl.xempty[x.slot]);
+                const uint64_t b_desc = make_smem_desc(act_base + a.slot * astage_bytes);
+                x.step(1, p.stages);
+                a.step(1, p.astages);
+                ready_x = i + 1 < end && mbar_test_all(smem_u32(&ctl.xfull[x.slot]), x.par);
+                ready_a = i + 1 < end && mbar_test_all(smem_u32(&ctl.afull[a.slot]), a.par);
+                const int nk = min(PK, d.kb_per_tile - kb);
+                if (leader) {
+#pragma unroll
+                    for (int k = 0; k < PK; ++k) {
+                        if (k >= nk) break;
 #pragma unroll
                         for (int k4 = 0; k4 < kBlockK / 16; ++k4)
-                            tc_mma_ts(d0, at + k * 32 + k4 * 8, b_desc + 2 * k4, idesc, (i > first || k > 0 || k4 > 0) ? 1u : 0u);
+                            tc_mma_ts(d0, at + k * 32 + k4 * 8, b_desc + k * (b_tile_bytes >> 4) + 2 * k4, idesc, k > 0 || k4 > 0 ? 1u : acc);
                     }
-                    tc_commit(smem_u32(&ctl.xempty[x.slot]));
-                    tc_commit(smem_u32(&ctl.aempty[a.slot]));
-                    x.step(1, p.stages);
-                    a.step(1, p.astages);
+                    tc_commit(empty);                        // the expanded item's slot, and with it the activation item's (see the loader)
+                    if (i + 1 == seg_end) tc_commit(smem_u32(&ctl.tmem_full[buf]));
                 }
-                if (timed_out) break;
-                tc_commit(smem_u32(&ctl.tmem_full[buf]));
+                acc = 1;
             }
-            LLMCAD_TRACE(7);
         }
+        if (lane == 0) LLMCAD_TRACE(7);
     } else if (warp >= 4) {
         // ================================================= expansion and dump
         const int quad = warp & 3, set = (warp - 4) >> 2, row = quad * 32 + lane;
@@ -1292,8 +1358,6 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                     w[k][1] = *reinterpret_cast<const uint4 *>(src + k * kW4TileBytes + 2048 + row * 16);
                     e[k] = reinterpret_cast<const int8_t *>(src + k * kW4TileBytes + 4096)[row];
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ctl.pempty[pk.slot]));
                 if (!mbar_wait_warp(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, lane, wait_limit)) { timed_out = true; break; }
                 tc_fence_after();
                 const uint32_t dst = x_base + t_quad + x.slot * (PK * 32);
@@ -1319,6 +1383,11 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                         tc_st16(dst + k * 32 + h * 16, o);
                     }
                 }
+                // The packed slot is given back only here, where every word has gone through the arithmetic above: given back
+                // right after the loads it was refilled before cold code (an instruction fetch of half a microsecond at the
+                // start of the kernel) had got to them.
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.pempty[pk.slot]));
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
                 __syncwarp();
@@ -1680,6 +1749,7 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
         const size_t pstage = (size_t)pair_k * kW4TileBytes, astage = (size_t)pair_k * nb * kBlockK * 2;
         int ast = (int)((full_limit - 4 * pstage) / astage);
         if (ast > 6) ast = 6;
+        if (ast > stages) ast = stages;      // (the loader relies on it)
         int pst = (int)((full_limit - (size_t)ast * astage) / pstage);
         if (pst > tune.w4_pstages) pst = tune.w4_pstages;
         pst &= ~1;
