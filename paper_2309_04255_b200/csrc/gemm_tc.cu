@@ -153,6 +153,21 @@ __device__ __forceinline__ bool mbar_test_all(uint32_t bar, uint32_t parity)
         : "memory");
     return __all_sync(0xffffffffu, ok != 0);
 }
+// The same for two barriers at once.
+__device__ __forceinline__ bool mbar_test2_all(uint32_t bar_a, uint32_t parity_a, uint32_t bar_b, uint32_t parity_b)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 q, [%3], %4;\n\t"
+        "and.pred p, p, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar_a), "r"(parity_a), "r"(bar_b), "r"(parity_b)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
+}
 // Threads that issue MMAs: the code between two of them is what limits the rate (one lane under `if (lane == 0)` got
 // through 8 MMAs, their commit and two barrier waits in 1250 cycles, four times what the tensor pipe needs for 64
 // columns: every operand went through a per-thread register). The MMA warps therefore stay converged, so that
@@ -718,8 +733,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                 if (!ready && !mbar_wait_all(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
                 tc_fence_after();
                 const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off, empty = smem_u32(&ctl.empty[s]);
-                if (++s == p.stages) { s = 0; ph ^= 1u; }
-                ready = i + 1 < r.end && mbar_test_all(smem_u32(&ctl.full[s]), ph);
                 const int nk = min(PK, kbpt - kb);
                 const uint64_t a_desc = make_smem_desc(a_addr), b_desc = make_smem_desc(b_addr);
                 if (leader) {
@@ -736,6 +749,8 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                     if (i + 1 == seg_end) tc_commit(smem_u32(&ctl.tmem_full[buf]));
                 }
                 acc = 1;
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
+                ready = i + 1 < r.end && mbar_test_all(smem_u32(&ctl.full[s]), ph);    // while the tensor pipe works on this item
             }
         }
         if (lane == 0) LLMCAD_TRACE(7);
@@ -1014,8 +1029,6 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
                     if (!ready && !mbar_wait_all(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) { timed_out = true; break; }
                     tc_fence_after();
                     const uint32_t a_addr = smem_base + s * stage_bytes, b_addr = a_addr + b_off, empty = smem_u32(&ctl.empty[s]);
-                    if (++s == p.stages) { s = 0; ph ^= 1u; }
-                    ready = i + 1 < end && mbar_test_all(smem_u32(&ctl.full[s]), ph);
                     const int nk = min(PK, d.kb_per_tile - kb);
                     const uint64_t a_desc = make_smem_desc(a_addr), b_desc = make_smem_desc(b_addr);
                     if (leader) {
@@ -1033,6 +1046,8 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
                         if (i + 1 == seg_end) tc_commit_pair(smem_u32(&ctl.tmem_full[buf]));
                     }
                     acc = 1;
+                    if (++s == p.stages) { s = 0; ph ^= 1u; }
+                    ready = i + 1 < end && mbar_test_all(smem_u32(&ctl.full[s]), ph);
                 }
             }
             if (lane == 0) LLMCAD_TRACE(7);
@@ -1112,16 +1127,19 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
 // to shared memory, with four warps that also dumped the accumulators, and slots were handed around at 0.5 us an
 // item (7B shape, 32 nodes: 3.53 ms a pass).
 //
+// What paces it is the MMA warp: ~520 cycles per ring item for its barriers, fences and addresses beside the MMAs
+// themselves. An item here is therefore two of the items that the kernels for bf16 weights move, 2 PK k-blocks, as
+// far as the segment reaches.
+//
 // Warps: 0 producer of packed items (bulk copies), 1 TMEM allocator and MMA issuer, 2 activation loader (TMA),
-// 4..11 expansion and dump: warp w works on rows 32 * (w % 4) .., the two sets of four take alternate items and
-// alternate 16-node chunks of a dump. Three rings of items (PK k-blocks): packed (shared memory), expanded
+// 4..11 expansion and dump: warp w works on rows 32 * (w % 4) .., the two sets of four on one half of an item's
+// k-blocks each, and on alternate 16-node chunks of a dump. Three rings of items: packed (shared memory), expanded
 // (tensor memory, what the accumulators leave of the 512 columns), activations (shared memory). Until the grid
 // dependency the packed ring fills and the expanded ring as far as it reaches. 72 registers a thread: three warps
 // per scheduler beside the finishing CTA's three.
 //
-// The items are cut and ordered exactly as the kernels for bf16 weights cut theirs on the same number of nodes
-// (CTA pairs included, which here only means how tiles and ranges are dealt out), so that the sums are the same
-// to the bit.
+// Work is cut and ordered exactly as the kernels for bf16 weights cut theirs on the same number of nodes (CTA pairs
+// included, which here only means how tiles and ranges are dealt out), so that the sums are the same to the bit.
 constexpr int kW4Threads = 384;
 constexpr int kMaxPStages = 16, kMaxXStages = 12, kMaxAStages = 12;
 
@@ -1169,14 +1187,43 @@ __device__ __forceinline__ void tc_ld16_sum2(uint32_t taddr_a, uint32_t taddr_b,
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(a[j]) + __uint_as_float(b[j]);
 }
 
-// slot and parity of a ring, stepped through n slots at a time
+// slot and parity of a ring of n slots
 struct RingPos {
     int slot;
     uint32_t par;
-    __device__ void step(int by, int n)
+    __device__ void step(int n)
     {
-        slot += by;
-        if (slot >= n) { slot -= n; par ^= 1u; }
+        if (++slot == n) { slot = 0; par ^= 1u; }
+    }
+};
+
+// Walks a CTA's share [i, end) of the (tile, PK k-blocks) list in steps of up to two entries of one tile.
+template <int PK>
+struct W4Walk {
+    int i, end, ppt, kbpt;
+    int unit, kb, nk;       // tile (or pair of tiles), first k-block and number of k-blocks of the current step
+    bool last;              // it ends a segment: the entries of one tile that belong to this CTA
+    int n_items;
+    __device__ void init(int begin, int e, int p, int k)
+    {
+        i = begin; end = e; ppt = p; kbpt = k;
+        unit = begin / p;
+        load();
+    }
+    __device__ void load()
+    {
+        const int at = i - unit * ppt, left = min(end - i, ppt - at);
+        n_items = min(2, left);
+        last = n_items == left;
+        kb = at * PK;
+        nk = min(n_items * PK, kbpt - kb);
+    }
+    __device__ bool done() const { return i >= end; }
+    __device__ void next()
+    {
+        i += n_items;
+        if (i == (unit + 1) * ppt) ++unit;
+        load();
     }
 };
 
@@ -1190,8 +1237,9 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const uint32_t nb = (uint32_t)p.n_pad * (p.comp ? 2u : 1u);
-    const uint32_t b_tile_bytes = nb * kBlockK * 2, astage_bytes = PK * b_tile_bytes;
-    constexpr uint32_t pstage_bytes = PK * kW4TileBytes;
+    constexpr int SK = 2 * PK;                     // k-blocks per item
+    const uint32_t b_tile_bytes = nb * kBlockK * 2, astage_bytes = SK * b_tile_bytes;
+    constexpr uint32_t pstage_bytes = SK * kW4TileBytes;
     const uint32_t act_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t packed_base = act_base + (uint32_t)p.astages * astage_bytes;
     const int acc_bufs = p.acc_bufs;
@@ -1207,29 +1255,29 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     auto tile_of = [&](int unit) { return d.group == 2 ? 2 * unit + rank : unit; };
 
     // ---- weight producer, across the start-up barrier: the first ring-full goes out at once
-    int pi = begin, put = begin / ppt, pkp = begin - put * ppt;
+    W4Walk<PK> pw;
     RingPos pp{0, 1};                              // a fresh barrier passes a wait on parity 1
     uint64_t pol_stream = 0;
     auto issue_item = [&]() {
-        const int nk = min(PK, d.kb_per_tile - pkp * PK), v = min(tile_of(put), n_vtiles - 1);
-        const uint32_t full = smem_u32(&ctl.pfull[pp.slot]);
-        mbar_expect_tx(full, (uint32_t)nk * kW4TileBytes);
-        bulk_load_1d(packed_base + pp.slot * pstage_bytes, d.w_tiled + ((size_t)packed_tile(d, v) * d.kb_per_tile + pkp * PK) * kW4TileBytes,
-                     (uint32_t)nk * kW4TileBytes, full, pol_stream);
-        ++pi;
-        if (++pkp == ppt) { pkp = 0; ++put; }
-        pp.step(1, p.pstages);
+        const int v = min(tile_of(pw.unit), n_vtiles - 1);
+        const uint32_t full = smem_u32(&ctl.pfull[pp.slot]), bytes = (uint32_t)pw.nk * kW4TileBytes;
+        mbar_expect_tx(full, bytes);
+        bulk_load_1d(packed_base + pp.slot * pstage_bytes, d.w_tiled + ((size_t)packed_tile(d, v) * d.kb_per_tile + pw.kb) * kW4TileBytes,
+                     bytes, full, pol_stream);
+        pw.next();
+        pp.step(p.pstages);
     };
     if (threadIdx.x == 0) {
-        for (int s = 0; s < p.pstages; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), 4); }
-        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.xfull[s]), 4); mbar_init(smem_u32(&ctl.xempty[s]), 1); }
+        for (int s = 0; s < p.pstages; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), 8); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.xfull[s]), 8); mbar_init(smem_u32(&ctl.xempty[s]), 1); }
         for (int s = 0; s < p.astages; ++s) mbar_init(smem_u32(&ctl.afull[s]), 1);
         for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&ctl.tmem_full[b]), 1); mbar_init(smem_u32(&ctl.tmem_empty[b]), 8); }
         ctl.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
-        while (pi < end && pi - begin < p.pstages) issue_item();
+        pw.init(begin, end, ppt, d.kb_per_tile);
+        for (int q = 0; q < p.pstages && !pw.done(); ++q) issue_item();
         LLMCAD_TRACE(2);
     }
     if (warp == 1) {
@@ -1249,7 +1297,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     if (warp == 0) {
         if (lane == 0) {
             uint64_t t_idle = 0;
-            while (pi < end) {
+            while (!pw.done()) {
                 if (mbar_try(smem_u32(&ctl.pempty[pp.slot]), pp.par)) {
                     issue_item();
                     t_idle = 0;
@@ -1270,21 +1318,21 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
             // so. (There are at least as many expanded slots as activation slots: the barrier cannot be a lap further,
             // because the item that would take it there has no activations yet.)
             RingPos a{0, 0}, x{0, 0};
-            int kp = begin % ppt;
+            W4Walk<PK> w;
+            w.init(begin, end, ppt, d.kb_per_tile);
             if (!dep_wait_thread(dep)) timed_out = true;
             fence_proxy_async();          // the activations were written by ordinary stores; the copies below read them
             pdl_launch_dependents();
-            for (int i = begin; i < end && !timed_out; ++i) {
-                if (i - begin >= p.astages) {
+            for (int q = 0; !w.done() && !timed_out; ++q) {
+                if (q >= p.astages) {
                     if (!mbar_wait(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
-                    x.step(1, p.stages);
+                    x.step(p.stages);
                 }
                 const uint32_t full = smem_u32(&ctl.afull[a.slot]), dst = act_base + a.slot * astage_bytes;
-                const int nk = min(PK, d.kb_per_tile - kp * PK);
-                mbar_expect_tx(full, (uint32_t)nk * b_tile_bytes);
-                for (int k = 0; k < nk; ++k) tma_load_3d(dst + k * b_tile_bytes, &maps.x, (kp * PK + k) * kBlockK, full, pol_keep);
-                if (++kp == ppt) kp = 0;
-                a.step(1, p.astages);
+                mbar_expect_tx(full, (uint32_t)w.nk * b_tile_bytes);
+                for (int k = 0; k < w.nk; ++k) tma_load_3d(dst + k * b_tile_bytes, &maps.x, (w.kb + k) * kBlockK, full, pol_keep);
+                w.next();
+                a.step(p.astages);
             }
         }
     } else if (warp == 1) {
@@ -1293,40 +1341,39 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0), xb = tmem + (uint32_t)acc_bufs * nb;
         const bool leader = elect_one();
         RingPos x{0, 0}, a{0, 0};
-        uint32_t seg = 0;
-        bool ready_x = false, ready_a = false;
-        for (int i = begin; i < end && !timed_out; ++seg) {
-            const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt);
-            int kb = (i - unit * ppt) * PK;
-            const int buf = acc_bufs == 2 ? (int)(seg & 1) : 0;
-            const uint32_t use = acc_bufs == 2 ? seg >> 1 : seg;
-            if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
-            const uint32_t d0 = tmem + buf * nb;
-            uint32_t acc = 0;
-            for (; i < seg_end; ++i, kb += PK) {
-                if (!ready_x && !mbar_wait_all(smem_u32(&ctl.xfull[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
-                if (!ready_a && !mbar_wait_all(smem_u32(&ctl.afull[a.slot]), a.par, abort_flag, wait_limit)) { timed_out = true; break; }
-                tc_fence_after();
-                const uint32_t at = xb + x.slot * (PK * 32), empty = smem_u32(&ctl.xempty[x.slot]);
-                const uint64_t b_desc = make_smem_desc(act_base + a.slot * astage_bytes);
-                x.step(1, p.stages);
-                a.step(1, p.astages);
-                ready_x = i + 1 < end && mbar_test_all(smem_u32(&ctl.xfull[x.slot]), x.par);
-                ready_a = i + 1 < end && mbar_test_all(smem_u32(&ctl.afull[a.slot]), a.par);
-                const int nk = min(PK, d.kb_per_tile - kb);
-                if (leader) {
-#pragma unroll
-                    for (int k = 0; k < PK; ++k) {
-                        if (k >= nk) break;
-#pragma unroll
-                        for (int k4 = 0; k4 < kBlockK / 16; ++k4)
-                            tc_mma_ts(d0, at + k * 32 + k4 * 8, b_desc + k * (b_tile_bytes >> 4) + 2 * k4, idesc, k > 0 || k4 > 0 ? 1u : acc);
-                    }
-                    tc_commit(empty);                        // the expanded item's slot, and with it the activation item's (see the loader)
-                    if (i + 1 == seg_end) tc_commit(smem_u32(&ctl.tmem_full[buf]));
-                }
-                acc = 1;
+        W4Walk<PK> w;
+        w.init(begin, end, ppt, d.kb_per_tile);
+        uint32_t seg = 0, acc = 0;
+        int buf = 0;
+        bool ready = false;
+        while (!w.done()) {
+            if (acc == 0) {                                  // a segment begins
+                buf = acc_bufs == 2 ? (int)(seg & 1) : 0;
+                const uint32_t use = acc_bufs == 2 ? seg >> 1 : seg;
+                if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+                ++seg;
             }
+            if (!ready && !(mbar_wait_all(smem_u32(&ctl.xfull[x.slot]), x.par, abort_flag, wait_limit) &&
+                            mbar_wait_all(smem_u32(&ctl.afull[a.slot]), a.par, abort_flag, wait_limit))) { timed_out = true; break; }
+            tc_fence_after();
+            const uint32_t d0 = tmem + buf * nb, at = xb + x.slot * (SK * 32), empty = smem_u32(&ctl.xempty[x.slot]);
+            const uint64_t b_desc = make_smem_desc(act_base + a.slot * astage_bytes);
+            if (leader) {
+#pragma unroll
+                for (int k = 0; k < SK; ++k) {
+                    if (k >= w.nk) break;
+#pragma unroll
+                    for (int k4 = 0; k4 < kBlockK / 16; ++k4)
+                        tc_mma_ts(d0, at + k * 32 + k4 * 8, b_desc + k * (b_tile_bytes >> 4) + 2 * k4, idesc, k > 0 || k4 > 0 ? 1u : acc);
+                }
+                tc_commit(empty);                            // the expanded item's slot, and with it the activation item's (see the loader)
+                if (w.last) tc_commit(smem_u32(&ctl.tmem_full[buf]));
+            }
+            acc = w.last ? 0 : 1;
+            w.next();
+            x.step(p.stages);
+            a.step(p.astages);
+            ready = !w.done() && mbar_test2_all(smem_u32(&ctl.xfull[x.slot]), x.par, smem_u32(&ctl.afull[a.slot]), a.par);
         }
         if (lane == 0) LLMCAD_TRACE(7);
     } else if (warp >= 4) {
@@ -1334,54 +1381,49 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         const int quad = warp & 3, set = (warp - 4) >> 2, row = quad * 32 + lane;
         const uint32_t t_quad = (uint32_t)(quad * 32) << 16;
         RingPos pk{0, 0}, x{0, 1};
-        pk.step(set, p.pstages);
-        x.step(set, p.stages);
-        int next = begin + set;                    // this set's next item
-        int kp = (begin + set) % ppt;
+        W4Walk<PK> w;                              // the items to expand
+        w.init(begin, end, ppt, d.kb_per_tile);
+        int expanded = 0, dumpable = 0;            // items expanded; items up to and including the ones of the segment to be dumped next
         bool dep_ok = false;
         uint32_t seg = 0;
         for (int i = begin; i < end && !timed_out; ++seg) {
             const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt);
             // Items of the next segments are expanded ahead of this one's dump, as far as their slots are freed by MMAs
             // that do not wait for it: the tensor cores have work while the accumulators leave.
-            const int limit = min(end, seg_end + p.stages);
-            while (next < limit && !timed_out) {
-                const int nk = min(PK, d.kb_per_tile - kp * PK);
-                if (!mbar_wait_warp(smem_u32(&ctl.pfull[pk.slot]), pk.par, abort_flag, lane, wait_limit)) { timed_out = true; break; }
-                // a row's 64 codes of a k-block: two 16-byte words, [half][row], and its exponent
-                const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes;
-                uint4 w[PK][2];
-                int e[PK];
-#pragma unroll
-                for (int k = 0; k < PK; ++k) {
-                    w[k][0] = *reinterpret_cast<const uint4 *>(src + k * kW4TileBytes + row * 16);
-                    w[k][1] = *reinterpret_cast<const uint4 *>(src + k * kW4TileBytes + 2048 + row * 16);
-                    e[k] = reinterpret_cast<const int8_t *>(src + k * kW4TileBytes + 4096)[row];
-                }
-                if (!mbar_wait_warp(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, lane, wait_limit)) { timed_out = true; break; }
+            dumpable += (seg_end - i + 1) / 2;
+            while (!w.done() && expanded < dumpable + p.stages && !timed_out) {
+                if (!mbar_wait_all(smem_u32(&ctl.pfull[pk.slot]), pk.par, abort_flag, wait_limit) ||
+                    !mbar_wait_all(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
                 tc_fence_after();
-                const uint32_t dst = x_base + t_quad + x.slot * (PK * 32);
-#pragma unroll
-                for (int k = 0; k < PK; ++k) {
-                    if (k >= nk) break;
+                // A row's 64 codes of a k-block are two 16-byte words, [half][row], its exponent follows them. The loop over
+                // the halves is not unrolled: the expanding warps share their scheduler's instruction cache with the MMA
+                // warp, and with 400 instructions here that warp's 60 were fetched anew for every item.
+                const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes;
+                const uint32_t dst = x_base + t_quad + x.slot * (SK * 32);
+                const int h0 = 2 * PK * set, h1 = min(h0 + 2 * PK, 2 * w.nk);
+                uint4 codes = *reinterpret_cast<const uint4 *>(src + (h0 >> 1) * kW4TileBytes + row * 16);
+#pragma unroll 1
+                for (int h = h0; h < h1; ++h) {
+                    const uint8_t *blk = src + (h >> 1) * kW4TileBytes;
+                    const int e = reinterpret_cast<const int8_t *>(blk + 4096)[row];
+                    const uint4 cur = codes;
+                    const int hn = h + 1 < h1 ? h + 1 : h;
+                    codes = *reinterpret_cast<const uint4 *>(src + (hn >> 1) * kW4TileBytes + (hn & 1) * 2048 + row * 16);
                     // OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact
-                    const uint32_t s16 = (uint32_t)(e[k] + 127) << 7, b16 = 0x8000u | ((uint32_t)(e[k] + 134) << 7) | 8u;
+                    const uint32_t s16 = (uint32_t)(e + 127) << 7, b16 = 0x8000u | ((uint32_t)(e + 134) << 7) | 8u;
                     const uint32_t s2 = s16 | (s16 << 16), b2 = b16 | (b16 << 16);
+                    const uint32_t ww[4] = {cur.x, cur.y, cur.z, cur.w};
+                    uint32_t o[16];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t ww[4] = {w[k][h].x, w[k][h].y, w[k][h].z, w[k][h].w};
-                        uint32_t o[16];
+                    for (int q = 0; q < 4; ++q)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const uint32_t t2 = ((ww[q] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
-                                const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2), *reinterpret_cast<const __nv_bfloat162 *>(&s2),
-                                                                 *reinterpret_cast<const __nv_bfloat162 *>(&b2));
-                                o[q * 4 + j] = *reinterpret_cast<const uint32_t *>(&r);
-                            }
-                        tc_st16(dst + k * 32 + h * 16, o);
-                    }
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t t2 = ((ww[q] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
+                            const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2), *reinterpret_cast<const __nv_bfloat162 *>(&s2),
+                                                             *reinterpret_cast<const __nv_bfloat162 *>(&b2));
+                            o[q * 4 + j] = *reinterpret_cast<const uint32_t *>(&r);
+                        }
+                    tc_st16(dst + h * 16, o);
                 }
                 // The packed slot is given back only here, where every word has gone through the arithmetic above: given back
                 // right after the loads it was refilled before cold code (an instruction fetch of half a microsecond at the
@@ -1392,11 +1434,10 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.xfull[x.slot]));
-                next += 2;
-                kp += 2;
-                while (kp >= ppt) kp -= ppt;
-                pk.step(2, p.pstages);
-                x.step(2, p.stages);
+                ++expanded;
+                w.next();
+                pk.step(p.pstages);
+                x.step(p.stages);
             }
             if (timed_out) break;
             // ---- dump
@@ -1736,23 +1777,19 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     size_t smem = (size_t)stages * stage_bytes + 1024;
     p.pstages = p.astages = p.acc_bufs = 0;
     if (d.w4) {
-        // Three rings (see the kernel). Tensor memory, all 512 columns: two accumulators if at least four k-blocks of
-        // expanded weights (32 columns each) fit beside them, else one. Shared memory: six activation items if they fit
-        // beside four packed ones, the rest packed items.
+        // Three rings of items of 2 pair_k k-blocks (see the kernel). Tensor memory, all 512 columns: two accumulators if
+        // two items of expanded weights (32 columns per k-block) fit beside them, else one. Shared memory: as many
+        // activation items as there are expanded ones if they fit beside two packed ones, the rest packed items.
         if (d.w_tiled == nullptr) return cudaErrorInvalidValue;
-        p.acc_bufs = 512 - 2 * nb >= 4 * 32 ? 2 : 1;
-        stages = (512 - p.acc_bufs * nb) / (32 * pair_k);
+        const int sk = 2 * pair_k;
+        p.acc_bufs = 512 - 2 * nb >= 2 * sk * 32 ? 2 : 1;
+        stages = (512 - p.acc_bufs * nb) / (32 * sk);
         if (stages > tune.w4_xstages) stages = tune.w4_xstages;
-        // The two sets of expanding warps take alternate items. The rings they wait on have an even number of slots, so
-        // that a set comes back to a slot every lap: every second lap the parity would be the one it has already seen.
-        stages &= ~1;
-        const size_t pstage = (size_t)pair_k * kW4TileBytes, astage = (size_t)pair_k * nb * kBlockK * 2;
-        int ast = (int)((full_limit - 4 * pstage) / astage);
-        if (ast > 6) ast = 6;
+        const size_t pstage = (size_t)sk * kW4TileBytes, astage = (size_t)sk * nb * kBlockK * 2;
+        int ast = (int)((full_limit - 2 * pstage) / astage);
         if (ast > stages) ast = stages;      // (the loader relies on it)
         int pst = (int)((full_limit - (size_t)ast * astage) / pstage);
         if (pst > tune.w4_pstages) pst = tune.w4_pstages;
-        pst &= ~1;
         if (ast < 2 || pst < 2 || stages < 2) return cudaErrorInvalidConfiguration;
         p.pstages = pst;
         p.astages = ast;
