@@ -1132,15 +1132,16 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
 // far as the segment reaches.
 //
 // Warps: 0 producer of packed items (bulk copies), 1 TMEM allocator and MMA issuer, 2 activation loader (TMA),
-// 4..11 expansion and dump: warp w works on rows 32 * (w % 4) .., the two sets of four on one half of an item's
-// k-blocks each, and on alternate 16-node chunks of a dump. Three rings of items: packed (shared memory), expanded
-// (tensor memory, what the accumulators leave of the 512 columns), activations (shared memory). Until the grid
-// dependency the packed ring fills and the expanded ring as far as it reaches. 72 registers a thread: three warps
-// per scheduler beside the finishing CTA's three.
+// 4..15 expansion and dump: warp w works on rows 32 * (w % 4) .., the three sets of four take every third half of an
+// item's k-blocks, and every third 16-node chunk of a dump (with two sets the expansion, 150 cycles a half and warp
+// most of which is latency, set the pace: 1750 cycles an item against ~770 of MMAs at 64 columns). Three rings of
+// items: packed (shared memory), expanded (tensor memory, what the accumulators leave of the 512 columns), activations
+// (shared memory). Until the grid dependency the packed ring fills and the expanded ring as far as it reaches. 56
+// registers a thread: four warps per scheduler beside the finishing CTA's three of 96.
 //
 // Work is cut and ordered exactly as the kernels for bf16 weights cut theirs on the same number of nodes (CTA pairs
 // included, which here only means how tiles and ranges are dealt out), so that the sums are the same to the bit.
-constexpr int kW4Threads = 384;
+constexpr int kW4Sets = 2, kW4Threads = 128 + 128 * kW4Sets;
 constexpr int kMaxPStages = 16, kMaxXStages = 12, kMaxAStages = 12;
 
 struct W4Ctl {
@@ -1268,10 +1269,10 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         pp.step(p.pstages);
     };
     if (threadIdx.x == 0) {
-        for (int s = 0; s < p.pstages; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), 8); }
-        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.xfull[s]), 8); mbar_init(smem_u32(&ctl.xempty[s]), 1); }
+        for (int s = 0; s < p.pstages; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), 4 * kW4Sets); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.xfull[s]), 4 * kW4Sets); mbar_init(smem_u32(&ctl.xempty[s]), 1); }
         for (int s = 0; s < p.astages; ++s) mbar_init(smem_u32(&ctl.afull[s]), 1);
-        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&ctl.tmem_full[b]), 1); mbar_init(smem_u32(&ctl.tmem_empty[b]), 8); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&ctl.tmem_full[b]), 1); mbar_init(smem_u32(&ctl.tmem_empty[b]), 4 * kW4Sets); }
         ctl.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1384,7 +1385,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         W4Walk<PK> w;                              // the items to expand
         w.init(begin, end, ppt, d.kb_per_tile);
         int expanded = 0, dumpable = 0;            // items expanded; items up to and including the ones of the segment to be dumped next
-        bool dep_ok = false;
+        bool dep_ok = false, ready = false;
         uint32_t seg = 0;
         for (int i = begin; i < end && !timed_out; ++seg) {
             const int unit = i / ppt, seg_end = min(end, (unit + 1) * ppt);
@@ -1392,26 +1393,25 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
             // that do not wait for it: the tensor cores have work while the accumulators leave.
             dumpable += (seg_end - i + 1) / 2;
             while (!w.done() && expanded < dumpable + p.stages && !timed_out) {
-                if (!mbar_wait_all(smem_u32(&ctl.pfull[pk.slot]), pk.par, abort_flag, wait_limit) ||
-                    !mbar_wait_all(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, wait_limit)) { timed_out = true; break; }
+                if (!ready && !(mbar_wait_all(smem_u32(&ctl.pfull[pk.slot]), pk.par, abort_flag, wait_limit) &&
+                                mbar_wait_all(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, wait_limit))) { timed_out = true; break; }
                 tc_fence_after();
                 // A row's 64 codes of a k-block are two 16-byte words, [half][row], its exponent follows them. The loop over
                 // the halves is not unrolled: the expanding warps share their scheduler's instruction cache with the MMA
                 // warp, and with 400 instructions here that warp's 60 were fetched anew for every item.
                 const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes;
                 const uint32_t dst = x_base + t_quad + x.slot * (SK * 32);
-                const int h0 = 2 * PK * set, h1 = min(h0 + 2 * PK, 2 * w.nk);
-                uint4 codes = *reinterpret_cast<const uint4 *>(src + (h0 >> 1) * kW4TileBytes + row * 16);
+                auto codes_of = [&](int h) { return *reinterpret_cast<const uint4 *>(src + (h >> 1) * kW4TileBytes + (h & 1) * 2048 + row * 16); };
+                const int halves = 2 * w.nk;
+                uint4 codes = codes_of(min(set, halves - 1));
 #pragma unroll 1
-                for (int h = h0; h < h1; ++h) {
-                    const uint8_t *blk = src + (h >> 1) * kW4TileBytes;
-                    const int e = reinterpret_cast<const int8_t *>(blk + 4096)[row];
+                for (int h = set; h < halves; h += kW4Sets) {
+                    const int e = reinterpret_cast<const int8_t *>(src + (h >> 1) * kW4TileBytes + 4096)[row];
                     const uint4 cur = codes;
-                    const int hn = h + 1 < h1 ? h + 1 : h;
-                    codes = *reinterpret_cast<const uint4 *>(src + (hn >> 1) * kW4TileBytes + (hn & 1) * 2048 + row * 16);
-                    // OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact
-                    const uint32_t s16 = (uint32_t)(e + 127) << 7, b16 = 0x8000u | ((uint32_t)(e + 134) << 7) | 8u;
-                    const uint32_t s2 = s16 | (s16 << 16), b2 = b16 | (b16 << 16);
+                    codes = codes_of(min(h + kW4Sets, halves - 1));
+                    // OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact. The bf16 bits
+                    // of 2^e are (e + 127) << 7, those of -136 * 2^e are that + 0x8388.
+                    const uint32_t s2 = (uint32_t)(e + 127) * 0x00800080u, b2 = s2 + 0x83888388u;
                     const uint32_t ww[4] = {cur.x, cur.y, cur.z, cur.w};
                     uint32_t o[16];
 #pragma unroll
@@ -1430,14 +1430,16 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                 // start of the kernel) had got to them.
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.pempty[pk.slot]));
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ctl.xfull[x.slot]));
+                const uint32_t xfull = smem_u32(&ctl.xfull[x.slot]);
                 ++expanded;
                 w.next();
                 pk.step(p.pstages);
                 x.step(p.stages);
+                ready = !w.done() && mbar_test2_all(smem_u32(&ctl.pfull[pk.slot]), pk.par, smem_u32(&ctl.xempty[x.slot]), x.par);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(xfull);
             }
             if (timed_out) break;
             // ---- dump
@@ -1455,7 +1457,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                 if (!LLMCAD_CHECK(v >= 0 && v + d.group * group < n_vtiles + d.grid, p.status)) { timed_out = true; break; }
                 float *dst = p.partials + (size_t)(v + d.group * group) * slot_floats(p.n_pad) + (size_t)quad * p.n_pad * 32 + lane;
                 const uint32_t t_lane = tmem_base + t_quad + buf * nb;
-                for (int c0 = 16 * set; c0 < p.n_pad; c0 += 32) {
+                for (int c0 = 16 * set; c0 < p.n_pad; c0 += 16 * kW4Sets) {
                     float t[16];
                     if (p.comp) tc_ld16_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
                     else tc_ld16(t_lane + c0, t);
@@ -1480,7 +1482,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     }
     tc_fence_before();
     __syncthreads();
-    if (warp >= 4 && warp <= 7 && lane == 0) dep_arrive(p.s_done);      // four arrivals per CTA, behind the barrier: both sets have dumped
+    if (warp >= 4 && warp <= 7 && lane == 0) dep_arrive(p.s_done);      // four arrivals per CTA, behind the barrier: all sets have dumped
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
         if (lane == 0) LLMCAD_TRACE(13);
