@@ -163,6 +163,9 @@ class Verifier:
         self.packed = torch.empty(lib().llmcad_packed_weight_bytes(C.byref(self.c)), dtype=torch.uint8, device=self.device)
         self.kv = torch.zeros(lib().llmcad_kv_cache_bytes(C.byref(self.c)), dtype=torch.uint8, device=self.device)
         self.tdtype = torch.float32 if cfg.dtype == "f32" else torch.bfloat16
+        self._i32 = torch.empty(1, dtype=torch.int32, device=self.device)      # new_empty of these is the cheapest allocation
+        self._f32 = torch.empty(1, dtype=torch.float32, device=self.device)
+        self._kv_view = None
 
     def close(self):
         if getattr(self, "ctx", None):
@@ -192,17 +195,18 @@ class Verifier:
     # ---- cache views
     def kv_view(self) -> torch.Tensor:
         """[L][2][H][max_seq][hd] view of the cache in the model dtype."""
-        c = self.cfg
-        return self.kv.view(self.tdtype).view(c.n_layers, 2, c.n_heads, self.max_seq, c.head_dim)
+        if self._kv_view is None or self._kv_view[0] is not self.kv:
+            c = self.cfg
+            self._kv_view = (self.kv, self.kv.view(self.tdtype).view(c.n_layers, 2, c.n_heads, self.max_seq, c.head_dim))
+        return self._kv_view[1]
 
     # ---- the pass
     def new_outputs(self, n: int, want_logits: bool = True):
-        dev = self.device
         return {
-            "logits": torch.empty((n, self.cfg.vocab), dtype=torch.float32, device=dev) if want_logits else None,
-            "argmax": torch.empty(n, dtype=torch.int32, device=dev),
-            "accepted_path": torch.empty(self.max_tree, dtype=torch.int32, device=dev),   # -1 past the path, set by the pass
-            "scalars": torch.empty(8, dtype=torch.int32, device=dev),
+            "logits": self._f32.new_empty((n, self.cfg.vocab)) if want_logits else None,
+            "argmax": self._i32.new_empty(n),
+            "accepted_path": self._i32.new_empty(self.max_tree),   # -1 past the path, set by the pass
+            "scalars": self._i32.new_empty(8),
         }
 
     def verify_tree(self, prefix_len: int, tokens: torch.Tensor, parent: torch.Tensor, out=None, want_logits=True):
@@ -219,12 +223,11 @@ class Verifier:
         returns logits [n_new][vocab] (or None), top-k ids and probabilities [n_new][top_k], status."""
         n_tree = tokens.numel()
         n_new = n_tree - n_old
-        dev = self.device
         out = {
-            "logits": torch.empty((n_new, self.cfg.vocab), dtype=torch.float32, device=dev) if want_logits else None,
-            "topk_ids": torch.empty((n_new, max(top_k, 1)), dtype=torch.int32, device=dev),
-            "topk_probs": torch.empty((n_new, max(top_k, 1)), dtype=torch.float32, device=dev),
-            "status": torch.empty(1, dtype=torch.int32, device=dev),
+            "logits": self._f32.new_empty((n_new, self.cfg.vocab)) if want_logits else None,
+            "topk_ids": self._i32.new_empty((n_new, max(top_k, 1))),
+            "topk_probs": self._f32.new_empty((n_new, max(top_k, 1))),
+            "status": self._i32.new_empty(1),
         }
         _check(lib().llmcad_extend_tree(self.ctx, _ptr(self.packed), _ptr(self.kv), prefix_len, _ptr(tokens), _ptr(parent),
                                         n_old, n_tree, top_k, _ptr(out["logits"]), _ptr(out["topk_ids"]),
@@ -251,8 +254,8 @@ class Verifier:
     # ---- single steps
     def accept_compact(self, prefix_len: int, tokens, parent, argmax, compact: bool = True):
         n = tokens.numel()
-        path = torch.empty(self.max_tree, dtype=torch.int32, device=self.device)
-        scalars = torch.empty(8, dtype=torch.int32, device=self.device)
+        path = self._i32.new_empty(self.max_tree)
+        scalars = self._i32.new_empty(8)
         _check(lib().llmcad_accept_compact(self.ctx, self.kv.data_ptr() if compact else None, prefix_len, _ptr(tokens),
                                            _ptr(parent), _ptr(argmax), n, _ptr(path), _ptr(scalars), _stream()),
                "llmcad_accept_compact")

@@ -304,9 +304,10 @@ int run_gemm(llmcad_ctx *ctx, const void *packed, int l, int which, int act, int
 }
 
 // comp: q carries a lo plane kLoRows rows after the hi plane, and o gets one too (the pass);
-// the single-step entry points work on plain bf16 buffers.
+// the single-step entry points work on plain bf16 buffers, and pass the tree for the kernel to make its own mask table.
 int run_attention(llmcad_ctx *ctx, const void *q, const void *k, const void *v, int kv_stride, int P, int n, void *o,
-                  bool comp, int32_t *status, cudaStream_t st, int n_tree = 0, int q_first = 0, const AttnSync *sync = nullptr)
+                  bool comp, int32_t *status, cudaStream_t st, int n_tree = 0, int q_first = 0, const AttnSync *sync = nullptr,
+                  const int32_t *parent = nullptr)
 {
     const llmcad_config &c = ctx->cfg;
     TimedLaunch tl(ctx, 1, st);
@@ -316,12 +317,12 @@ int run_attention(llmcad_ctx *ctx, const void *q, const void *k, const void *v, 
                         : (c.flags & LLMCAD_FLAG_MMA_ATTN) ? false : attention_prefers_t5(n);
         if (t5) {
             CUDA_TRY(launch_attention_t5(q, k, v, c.n_heads, c.head_dim, kv_stride, P, n, ctx->tb.anc, o, ctx->n_sms, status, st,
-                                         &launched, ctx->next_trace(), comp ? 1 : 0, ctx->kv_lo, n_tree, q_first, ctx->wait_limit_ns, sync));
+                                         &launched, ctx->next_trace(), comp ? 1 : 0, ctx->kv_lo, n_tree, q_first, ctx->wait_limit_ns, sync, parent));
             ctx->launches += launched;
             return LLMCAD_OK;
         }
         CUDA_TRY(launch_attention_tc(q, k, v, c.n_heads, c.head_dim, kv_stride, P, n, ctx->tb.anc, o, ctx->n_sms, status, st, &launched, ctx->next_trace(), comp ? 1 : 0,
-                                     ctx->kv_lo, n_tree, q_first, sync));
+                                     ctx->kv_lo, n_tree, q_first, sync, parent));
         ctx->launches += launched;
         return LLMCAD_OK;
     }
@@ -896,6 +897,8 @@ int llmcad_tree_attention(llmcad_ctx *ctx, const void *q, const void *k, const v
         return LLMCAD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int32_t *status = ctx->scalars_dev() + LLMCAD_S_STATUS;
+    if (ctx->tc_attn)      // the tensor-core kernels make the mask table themselves
+        return run_attention(ctx, q, k, v, kv_stride, prefix_len, n, o, false, status, st, 0, 0, nullptr, parent_idx);
     CUDA_TRY(launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, ctx->tb, status, st));
     ctx->launches++;
     return run_attention(ctx, q, k, v, kv_stride, prefix_len, n, o, false, status, st);

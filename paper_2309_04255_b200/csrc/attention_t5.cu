@@ -27,6 +27,7 @@
 
 #include "attention_tc.cuh"
 #include "gemm_tc.cuh"
+#include "tree_dev.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -299,8 +300,10 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
                     const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_lo, int n_heads, int P,
                     int n, const uint32_t *__restrict__ anc, __nv_bfloat16 *o, int splits, int tiles_per_split,
                     int32_t *status, unsigned long long *trace, int comp, int n_tree, int q_first, uint64_t wait_limit,
-                    DepWait dep, uint32_t *done_ctr)
+                    DepWait dep, uint32_t *done_ctr, const int32_t *__restrict__ parent)
 {
+    // parent != null: a call of its own, see attention_tc.cu
+    const bool own = parent != nullptr;
     const int cta = blockIdx.y * gridDim.x + blockIdx.x;
     if (trace && threadIdx.x == 0 && cta < 256) trace[(size_t)cta * 16 + 0] = global_timer_ns();
     pdl_launch_dependents();
@@ -352,6 +355,41 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
     const uint32_t tmem_base = ctl.tmem_base;
     volatile int *abort_flag = &ctl.abort_flag;
     bool failed = false;
+
+    // State of the producer (thread 0), which starts before the roles do: the prefix tiles that fit in the ring.
+    int s = 0, t = t_begin, issued = 0;
+    uint32_t par = 1;              // a fresh barrier passes a wait on parity 1
+    auto issue_kv = [&](int tile) {
+        const uint32_t full = smem_u32(&ctl.full[s]);
+        const uint32_t dst = s_ring + s * kStageBytes;
+        mbar_expect_tx(full, kStageBytes);
+        for (int j = 0; j < 2; ++j) {
+            tma_load_3d(dst + j * kSubTile, &map_k, j * 64, tile * kKeyTile, head, full);
+            tma_load_3d(dst + (2 + j) * kSubTile, &map_v, j * 64, tile * kKeyTile, head, full);
+        }
+        if (++s == kStages) { s = 0; par ^= 1u; }
+    };
+    if (own) pdl_wait();
+    if (tid == 0) {
+        if (own) fence_proxy_async();
+        // in a pass they go out before the grid dependency: earlier passes wrote them
+        while (t < t_end && (own || !reaches_tree(t)) && issued < kStages) {
+            issue_kv(t++);
+            ++issued;
+        }
+    }
+    int own_err = 0;
+    uint32_t own_anc[4] = {0, 0, 0, 0};
+    if (own) {
+        MaskTable &table = *reinterpret_cast<MaskTable *>(q_stage);
+        own_err = mask_table(table, parent, nullptr, n_tree, 0);
+        if (cta == 0 && tid == 0) *status = own_err;
+        const int r = (warp & 3) * 32 + lane;
+        if (r < n)
+            for (int w = 0; w < 4; ++w) own_anc[w] = table.anc[q_first + r][w];
+        __syncthreads();           // the space is the query staging buffer from here on
+    }
+    auto status_says_no = [&]() { return own ? own_err != 0 : *reinterpret_cast<const volatile int32_t *>(status) != 0; };
     // A pass whose tree or tokens an earlier phase refused (status word set) does no work here: every
     // role looks at the word once the grid dependency has resolved, and all see the same value.
     // (the dependency is the grid dependency or the producer's completion counter; the one thread that feeds the
@@ -359,28 +397,12 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
     auto refused = [&]() {
         dep_wait_thread(dep);
         fence_proxy_async();
-        return *reinterpret_cast<const volatile int32_t *>(status) != 0;
-    };
-    auto refused_warp = [&]() {
-        dep_wait_warp(dep, lane);
-        return *reinterpret_cast<const volatile int32_t *>(status) != 0;
+        return status_says_no();
     };
 
     if (warp == 0) {
         // ================================================= producer
         if (lane == 0) {
-            int s = 0;
-            uint32_t par = 1;          // a fresh barrier passes a wait on parity 1
-            auto issue_kv = [&](int t) {
-                const uint32_t full = smem_u32(&ctl.full[s]);
-                const uint32_t dst = s_ring + s * kStageBytes;
-                mbar_expect_tx(full, kStageBytes);
-                for (int j = 0; j < 2; ++j) {
-                    tma_load_3d(dst + j * kSubTile, &map_k, j * 64, t * kKeyTile, head, full);
-                    tma_load_3d(dst + (2 + j) * kSubTile, &map_v, j * 64, t * kKeyTile, head, full);
-                }
-                if (++s == kStages) { s = 0; par ^= 1u; }
-            };
             auto issue_lo = [&](int t) {
                 const uint32_t full = smem_u32(&ctl.full[s]);
                 const uint32_t dst = s_ring + s * kStageBytes;
@@ -392,12 +414,6 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
                 }
                 if (++s == kStages) { s = 0; par ^= 1u; }
             };
-            // prefix tiles that fit in the ring go out before the grid dependency: earlier passes wrote them
-            int t = t_begin, issued = 0;
-            while (t < t_end && !reaches_tree(t) && issued < kStages) {
-                issue_kv(t++);
-                ++issued;
-            }
             if (refused()) {
                 // nothing will consume the tiles already requested: let them land before the ring goes away
                 for (int i = 0; i < issued; ++i) mbar_wait(smem_u32(&ctl.full[i]), 0, abort_flag, wait_limit);
@@ -525,7 +541,7 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
         uint32_t a4[4] = {0, 0, 0, 0};
         if (row < n) {
 #pragma unroll
-            for (int w = 0; w < 4; ++w) a4[w] = __ldcg(anc + (q_first + row) * 4 + w);   // L2: written earlier in this pass
+            for (int w = 0; w < 4; ++w) a4[w] = own ? own_anc[w] : __ldcg(anc + (q_first + row) * 4 + w);   // L2: written earlier in this pass
         }
         uint4 g[2][16];
         if (warp_active) {
@@ -541,7 +557,7 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
                 }
             }
         }
-        const bool skip = *reinterpret_cast<const volatile int32_t *>(status) != 0;
+        const bool skip = status_says_no();
         if (!skip) {
         // The queries become the A operand of Q K^T in tensor memory: 64 packed columns per plane, thread =
         // row. A warp fetches its 32 rows with coalesced loads (two rows of 256 bytes per instruction, both
@@ -700,7 +716,7 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
     }
     // (the softmax warps have passed the grid dependency, so the status word is final for every thread)
-    const bool bad = ctl.abort_flag != 0 || *reinterpret_cast<const volatile int32_t *>(status) != 0;
+    const bool bad = ctl.abort_flag != 0 || status_says_no();
 
     // four outputs of one row, normalised, as bf16 hi (and lo) to global memory
     auto store4 = [&](int row, int dim, float4 a, float inv) {
@@ -754,7 +770,7 @@ bool attention_prefers_t5(int n)
 cudaError_t launch_attention_t5(const void *q, const void *k, const void *v, int n_heads, int hd, int kv_stride, int P,
                                 int n, const uint32_t *anc, void *o, int n_sms, int32_t *status, cudaStream_t st,
                                 int *launched, unsigned long long *trace, int comp, const void *kv_lo, int n_tree, int q_first, uint64_t wait_limit_ns,
-                                const AttnSync *sync)
+                                const AttnSync *sync, const int32_t *parent)
 {
     if (n_tree <= 0) n_tree = n;
     if (hd != kHd || n < 1 || n > 128 || P + n_tree > kv_stride) return cudaErrorInvalidValue;
@@ -801,7 +817,7 @@ cudaError_t launch_attention_t5(const void *q, const void *k, const void *v, int
         sync->arrivals = (uint32_t)(splits * n_heads);
     }
     return cudaLaunchKernelEx(&lc.cfg, attention_t5_kernel, (const __nv_bfloat16 *)q, mk, mv, ml, n_heads, P, n, anc, (__nv_bfloat16 *)o, splits,
-                              tiles_per_split, status, trace, comp, n_tree, q_first, wait_limit_ns, dep, done);
+                              tiles_per_split, status, trace, comp, n_tree, q_first, wait_limit_ns, dep, done, parent);
 }
 
 }  // namespace llmcad

@@ -20,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include "attention_tc.cuh"
+#include "tree_dev.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -84,6 +85,10 @@ __device__ __forceinline__ void pack_split(float a, float b, uint32_t &hi, uint3
     lo = *reinterpret_cast<uint32_t *>(&l);
 }
 
+// shared memory of a kernel that makes the mask table itself (the calls on plain operands)
+template <bool COMP> struct OwnTable { typedef MaskTable type; };
+template <> struct OwnTable<true> { typedef int type; };
+
 }  // namespace
 
 // GROUPS key groups per CTA: warp w works on query tile w % q_tiles and on the keys
@@ -104,9 +109,15 @@ __global__ void __launch_bounds__(kAtThreads)
 attention_tc_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k,
                     const __nv_bfloat16 *__restrict__ v, int n_heads, int kv_stride, int P, int n, int n_pad,
                     const uint32_t *__restrict__ anc, __nv_bfloat16 *o, int splits, int tiles_base, int tiles_rem,
-                    const int32_t *status, unsigned long long *trace, const __nv_bfloat16 *__restrict__ kv_lo,
-                    int n_tree, int q_first, DepWait dep, uint32_t *done_ctr, int recv_off)
+                    int32_t *status, unsigned long long *trace, const __nv_bfloat16 *__restrict__ kv_lo,
+                    int n_tree, int q_first, DepWait dep, uint32_t *done_ctr, int recv_off, const int32_t *__restrict__ parent)
 {
+    // A call of its own (parent != null; plain operands): every CTA makes the mask table itself while its first key
+    // tiles travel, and the call is this one kernel (a second one in front of it was a third of a short call's time:
+    // prefix 256, 8 nodes, bound by launches on the host). Nothing is read before earlier kernels are done, whatever
+    // they wrote.
+    __shared__ typename OwnTable<COMP>::type s_table;
+    const bool own = !COMP && parent != nullptr;
     // PUSH: partial rows travel to their owners (see the head of the file); recv_off = where the receive
     // buffer starts in this CTA's shared memory, [splits][rows per CTA][kWsRow] floats behind everything else
     constexpr bool PUSH = GROUPS == 4;
@@ -161,7 +172,7 @@ attention_tc_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__
     bool early[kStages - 1];
 #pragma unroll
     for (int st = 0; st < kStages - 1; ++st) {
-        early[st] = t_begin + st < t_end && (t_begin + st + 1) * kKeyTile <= P;
+        early[st] = !own && t_begin + st < t_end && (t_begin + st + 1) * kKeyTile <= P;
         if (early[st]) load_tile(t_begin + st, st);
     }
     // the queries and the tree nodes' K/V are final: grid dependency, or the producer's completion counter
@@ -197,7 +208,15 @@ attention_tc_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__
     }
     // The status word is looked at only now, with the copies above already on their way (they read buffers that
     // exist whatever an earlier phase found): a refused pass waits for them and leaves.
-    if (*reinterpret_cast<const volatile int32_t *>(status)) {   // uniform over the grid: set only by kernels that ran before this one
+    int refused = 0;
+    if constexpr (!COMP) {
+        if (own) {
+            refused = mask_table(s_table, parent, nullptr, n_tree, 0);
+            if (cta == 0 && tid == 0) *status = refused;
+        }
+    }
+    if (!own) refused = *reinterpret_cast<const volatile int32_t *>(status);
+    if (refused) {   // uniform over the grid: set only by kernels that ran before this one
         cp_wait<0>();          // nothing may still be writing this CTA's shared memory when it exits
         if (threadIdx.x == 0) dep_arrive(done_ctr);
         return;
@@ -210,6 +229,13 @@ attention_tc_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__
     uint32_t anc0[4] = {0, 0, 0, 0}, anc1[4] = {0, 0, 0, 0};
     if (active) {
         for (int w = 0; w < 4; ++w) {
+            if constexpr (!COMP) {
+                if (own) {
+                    if (row0 < n) anc0[w] = s_table.anc[q_first + row0][w];
+                    if (row1 < n) anc1[w] = s_table.anc[q_first + row1][w];
+                    continue;
+                }
+            }
             if (row0 < n) anc0[w] = __ldcg(anc + (q_first + row0) * 4 + w);     // L2: written earlier in this pass
             if (row1 < n) anc1[w] = __ldcg(anc + (q_first + row1) * 4 + w);
         }
@@ -532,7 +558,7 @@ attention_tc_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__
 cudaError_t launch_attention_tc(const void *q, const void *k, const void *v, int n_heads, int hd, int kv_stride, int P,
                                 int n, const uint32_t *anc, void *o, int n_sms,
                                 int32_t *status, cudaStream_t st, int *launched, unsigned long long *trace, int comp,
-                                const void *kv_lo, int n_tree, int q_first, const AttnSync *sync)
+                                const void *kv_lo, int n_tree, int q_first, const AttnSync *sync, const int32_t *parent)
 {
     if (n_tree <= 0) n_tree = n;
     if (hd != kHd) return cudaErrorInvalidValue;
@@ -556,17 +582,17 @@ cudaError_t launch_attention_tc(const void *q, const void *k, const void *v, int
     const size_t recv = groups == 4 ? (size_t)splits * ((n_pad + splits - 1) / splits) * kWsRow * sizeof(float) : 0;
     const size_t smem = recv_off + recv;
     typedef void (*Kern)(const __nv_bfloat16 *, const __nv_bfloat16 *, const __nv_bfloat16 *, int, int, int, int, int,
-                         const uint32_t *, __nv_bfloat16 *, int, int, int, const int32_t *, unsigned long long *,
-                         const __nv_bfloat16 *, int, int, DepWait, uint32_t *, int);
+                         const uint32_t *, __nv_bfloat16 *, int, int, int, int32_t *, unsigned long long *,
+                         const __nv_bfloat16 *, int, int, DepWait, uint32_t *, int, const int32_t *);
     static const Kern kerns[2][3] = {{attention_tc_kernel<1, false>, attention_tc_kernel<2, false>, attention_tc_kernel<4, false>},
                                      {attention_tc_kernel<1, true>, attention_tc_kernel<2, true>, attention_tc_kernel<4, true>}};
     static PerDeviceOnce attr_set;
     if (attr_set.needed()) {
-        // 128 nodes, hi + lo; with <= 32 nodes: a deeper ring, and the receive buffer behind it
+        // 128 nodes, hi + lo (one plane of operands: 180 KB at most); with <= 32 nodes: a deeper ring, and the receive buffer behind it
         const int max_smem = 2 * 128 * kRowBytes + 2 * 3 * kKeyTile * kRowBytes + 2 * 129 * kRowBytes + 128;
         for (int c = 0; c < 2; ++c)
             for (int g = 0; g < 3; ++g) {
-                cudaError_t e = cudaFuncSetAttribute(kerns[c][g], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+                cudaError_t e = cudaFuncSetAttribute(kerns[c][g], cudaFuncAttributeMaxDynamicSharedMemorySize, c == 0 ? 200 * 1024 : max_smem);
                 // the largest shared-memory split of the SM, so that the next GEMM's streaming CTA can settle beside this kernel's
                 if (e == cudaSuccess) e = cudaFuncSetAttribute(kerns[c][g], cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
                 if (e != cudaSuccess) return e;
@@ -585,8 +611,8 @@ cudaError_t launch_attention_tc(const void *q, const void *k, const void *v, int
     }
     return cudaLaunchKernelEx(&lc.cfg, kern, (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k,
                               (const __nv_bfloat16 *)v, n_heads, kv_stride, P, n, n_pad, anc, (__nv_bfloat16 *)o, splits,
-                              tiles_base, tiles_rem, (const int32_t *)status, trace, (const __nv_bfloat16 *)kv_lo, n_tree, q_first, dep, done,
-                              (int)recv_off);
+                              tiles_base, tiles_rem, status, trace, (const __nv_bfloat16 *)kv_lo, n_tree, q_first, dep, done,
+                              (int)recv_off, parent);
 }
 
 }  // namespace llmcad

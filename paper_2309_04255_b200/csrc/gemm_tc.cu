@@ -1256,7 +1256,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     auto tile_of = [&](int unit) { return d.group == 2 ? 2 * unit + rank : unit; };
 
     // ---- weight producer, across the start-up barrier: the first ring-full goes out at once
-    W4Walk<PK> pw;
+    W4Walk<PK> pw{};
     RingPos pp{0, 1};                              // a fresh barrier passes a wait on parity 1
     uint64_t pol_stream = 0;
     auto issue_item = [&]() {

@@ -4,9 +4,9 @@
 // that has handed every byte of the device to its own pool at start-up, a plug-in loaded after
 // that point, or a latency-critical loop in which cudaMalloc (a device-wide synchronising call)
 // is forbidden. llmcad_tree_attention() needs a context, and creating one allocates its work
-// buffers. The variant below needs no context: the few kilobytes of scratch it uses (per-node
-// depth, position, ancestor bit rows and a status word) live in a static device array that comes
-// with the library image, so nothing is allocated at any time.
+// buffers. The variant below needs no context: the kernels make the mask table in shared memory, and the
+// status word, when the caller does not want it, lives in a static device array that comes with the
+// library image, so nothing is allocated at any time.
 #include <cstdio>
 
 #include "attention_tc.cuh"
@@ -15,8 +15,7 @@
 namespace {
 
 constexpr int kMaxNodes = LLMCAD_MAX_TREE;      // 128 tree nodes
-// depth[128] | pos[128] | anc[128][4] | status: 128*4 + 128*4 + 128*16 + 4 bytes, rounded up
-constexpr size_t kScratchBytes = 4096;
+constexpr size_t kScratchBytes = 256;           // a status word
 
 // One copy per GPU that loads the library, held until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -41,7 +40,7 @@ extern "C" int llmcad_tree_attention_noalloc(const void *q, const void *k, const
         return LLMCAD_ERR_INVALID_ARG;
     }
     if (n > kMaxNodes) {
-        snprintf(g_err, sizeof(g_err), "n=%d exceeds the %d nodes the static scratch holds", n, kMaxNodes);
+        snprintf(g_err, sizeof(g_err), "n=%d exceeds the %d nodes a mask table holds", n, kMaxNodes);
         return LLMCAD_ERR_UNSUPPORTED;
     }
     if (n_heads > 65535) { snprintf(g_err, sizeof(g_err), "n_heads=%d exceeds 65535", n_heads); return LLMCAD_ERR_UNSUPPORTED; }
@@ -69,29 +68,20 @@ extern "C" int llmcad_tree_attention_noalloc(const void *q, const void *k, const
         }
         __atomic_store_n(&g_scratch_ptr[dev], ptr, __ATOMIC_RELEASE);
     }
-    unsigned char *base = static_cast<unsigned char *>(__atomic_load_n(&g_scratch_ptr[dev], __ATOMIC_ACQUIRE));
-    TreeBuffers tb;
-    tb.depth = reinterpret_cast<int32_t *>(base);
-    tb.pos = reinterpret_cast<int32_t *>(base + 512);
-    tb.anc = reinterpret_cast<uint32_t *>(base + 1024);
-    tb.rope_cs = nullptr;
-    int32_t *status = reinterpret_cast<int32_t *>(base + 1024 + 2048);
-
+    int32_t *status = status_out != nullptr ? status_out : static_cast<int32_t *>(__atomic_load_n(&g_scratch_ptr[dev], __ATOMIC_ACQUIRE));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = launch_tree_prep(parent_idx, nullptr, n, prefix_len, 0, tb, status, st);     // also sets the status word
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) {
-        int sms = 0;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) {
-            // neither kernel needs global scratch; same choice as the regular entry point
-            if (attention_prefers_t5(n))
-                e = launch_attention_t5(q, k, v, n_heads, 128, kv_stride, prefix_len, n, tb.anc, o, sms, status, st, nullptr);
-            else
-                e = launch_attention_tc(q, k, v, n_heads, 128, kv_stride, prefix_len, n, tb.anc, o, sms, status, st, nullptr);
-        }
+        // neither kernel needs global scratch, and both make the mask table and set the status word themselves; same
+        // choice as the regular entry point
+        if (attention_prefers_t5(n))
+            e = launch_attention_t5(q, k, v, n_heads, 128, kv_stride, prefix_len, n, nullptr, o, sms, status, st, nullptr, nullptr, 0, nullptr, 0, 0,
+                                    kDefaultWaitLimitNs, nullptr, parent_idx);
+        else
+            e = launch_attention_tc(q, k, v, n_heads, 128, kv_stride, prefix_len, n, nullptr, o, sms, status, st, nullptr, nullptr, 0, nullptr, 0, 0,
+                                    nullptr, parent_idx);
     }
-    if (e == cudaSuccess && status_out != nullptr)
-        e = cudaMemcpyAsync(status_out, status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) {
         snprintf(g_err, sizeof(g_err), "CUDA: %s", cudaGetErrorString(e));
         return LLMCAD_ERR_CUDA;
