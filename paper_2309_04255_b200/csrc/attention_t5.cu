@@ -7,10 +7,10 @@
 //   warp 0    producer: TMA boxes of K and V (and, for the tiles that hold tree nodes, of the bf16
 //             remainders of their K and V) into a ring of shared-memory stages;
 //   warp 1    MMA issuer of S = Q K^T into one of two TMEM score buffers (queries on the 128 TMEM
-//             lanes, 64 keys on the columns), two tiles ahead of the softmax;
+//             lanes, 64 keys on the columns), as soon as the softmax has read that buffer;
 //   warp 6    MMA issuer of O += P V into another TMEM region; the A operands (Q, P) are read from
 //             tensor memory, only K and V come from shared memory;
-//   warps 2-5 softmax: thread = query row. Puts its row of Q into TMEM once; per tile reads its row of
+//   warps 2-5 and 7-10 softmax, two groups that take alternate tiles: thread = query row. Puts its row of Q into TMEM once; per tile reads its row of
 //             S from TMEM, masks, keeps a running reference and sum, and writes P (hi + lo bf16
 //             pairs) back to TMEM for the second MMA, which accumulates the outputs in TMEM over all
 //             tiles; the rare move of a row's reference value rescales that row in TMEM.
@@ -27,6 +27,7 @@
 
 #include "attention_tc.cuh"
 #include "gemm_tc.cuh"
+#include "mbar.cuh"
 #include "tree_dev.cuh"
 
 namespace cg = cooperative_groups;
@@ -37,7 +38,7 @@ namespace {
 
 constexpr int kHd = 128;
 constexpr int kKeyTile = 64;
-constexpr int kT5Threads = 224;                   // producer, score MMAs, four softmax warps, P V MMAs
+constexpr int kT5Threads = 352;                   // producer, score MMAs, four softmax warps, P V MMAs, four more softmax warps
 constexpr int kStages = 6;                       // three tiles in flight, each possibly with a remainder stage
 constexpr int kSubTile = 64 * 64 * 2;            // [64 rows][64 columns] bf16, 128-byte rows
 constexpr int kStageBytes = 4 * kSubTile;        // K dims 0-63, K dims 64-127, V dims 0-63, V dims 64-127
@@ -57,42 +58,18 @@ struct Ctl {
     uint64_t full[kStages];
     uint64_t empty[kStages];
     uint64_t q_full;
-    uint64_t s_full[2];
+    uint64_t s_full[2], s_empty[2];
     uint64_t p_full[2];
     uint64_t o_full[2];
     uint32_t tmem_base;
     volatile int abort_flag;
+    volatile int seq[4];                         // per 32 rows: tiles whose reference has been decided
+    float ref[128];                              // the rows' references
 };
 
 constexpr int kQStage = 32 * 256;                   // per softmax warp: 32 query rows of one plane on their way to TMEM
 constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + 4 * kQStage + sizeof(Ctl);
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
 // Bounded wait of one thread: gives up after wait_limit ns or when another role has raised `abort`.
 __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint64_t wait_limit)
 {
@@ -108,14 +85,6 @@ __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile i
         }
     }
 }
-// The same for a whole warp: lane 0 polls, the warp follows.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, int lane, uint64_t wait_limit)
-{
-    int ok = 1;
-    if (lane == 0) ok = mbar_wait(bar, parity, abort_flag, wait_limit) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
-
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, uint32_t bar)
 {
     asm volatile(
@@ -151,6 +120,29 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t *r)
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// 16 consecutive 32-bit columns of this thread's TMEM lane
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+          "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+// 32 consecutive fp32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float *v)
+{
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
 // 64 consecutive fp32 columns of this thread's TMEM lane in one instruction (a load and its wait cost
 // ~0.2 us however many columns they move, so the score row is fetched whole).
 __device__ __forceinline__ void tc_ld64(uint32_t taddr, float *v)
@@ -165,18 +157,6 @@ __device__ __forceinline__ void tc_ld64(uint32_t taddr, float *v)
 #pragma unroll
     for (int j = 0; j < 64; ++j) v[j] = __uint_as_float(r[j]);
 }
-__device__ __forceinline__ void tc_st64(uint32_t taddr, const float *v)
-{
-    uint32_t r[64];
-#pragma unroll
-    for (int j = 0; j < 64; ++j) r[j] = __float_as_uint(v[j]);
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x64.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63, %64};"
-        :: "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(r[32]), "r"(r[33]), "r"(r[34]), "r"(r[35]), "r"(r[36]), "r"(r[37]), "r"(r[38]), "r"(r[39]), "r"(r[40]), "r"(r[41]), "r"(r[42]), "r"(r[43]), "r"(r[44]), "r"(r[45]), "r"(r[46]), "r"(r[47]), "r"(r[48]), "r"(r[49]), "r"(r[50]), "r"(r[51]), "r"(r[52]), "r"(r[53]), "r"(r[54]), "r"(r[55]), "r"(r[56]), "r"(r[57]), "r"(r[58]), "r"(r[59]), "r"(r[60]), "r"(r[61]), "r"(r[62]), "r"(r[63])
-        : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
 // Shared-memory matrix descriptors, 128-byte swizzle (layout type 2 at bits 61-63, version 1 at bit
 // 46), start address >> 4 at bits 0-13.
 // K-major operand (rows of 64 bf16 = 128 bytes, as a TMA box of 64 columns leaves them): groups of
@@ -220,6 +200,12 @@ __device__ __forceinline__ void pack_split(float a, float b, uint32_t &hi, uint3
     __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
     hi = *reinterpret_cast<uint32_t *>(&h);
     lo = *reinterpret_cast<uint32_t *>(&l);
+}
+
+__device__ __forceinline__ uint32_t pack2(float a, float b)
+{
+    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t *>(&h);
 }
 
 // 2^x, one instruction; 2^(-inf) = +0
@@ -317,7 +303,7 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
     float *part = reinterpret_cast<float *>(smp);   // the ring's space, once the loop is over
 
     const int split = blockIdx.x, head = blockIdx.y;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: known to be uniform
     const int n_keys = P + n_tree;
     const int n_tiles = (n_keys + kKeyTile - 1) / kKeyTile;
     const int t_begin = min(n_tiles, split * tiles_per_split);
@@ -333,9 +319,11 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
             mbar_init(smem_u32(&ctl.full[s]), 1);
             mbar_init(smem_u32(&ctl.empty[s]), 1);
         }
-        mbar_init(smem_u32(&ctl.q_full), 4);
+        mbar_init(smem_u32(&ctl.q_full), comp ? 8 : 4);
+        for (int w = 0; w < 4; ++w) ctl.seq[w] = 0;
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&ctl.s_full[b]), 1);
+            mbar_init(smem_u32(&ctl.s_empty[b]), 4);
             mbar_init(smem_u32(&ctl.p_full[b]), 4);
             mbar_init(smem_u32(&ctl.o_full[b]), 1);
         }
@@ -399,6 +387,10 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
         fence_proxy_async();
         return status_says_no();
     };
+    auto refused_warp = [&]() {
+        dep_wait_warp(dep, lane);
+        return status_says_no();
+    };
 
     if (warp == 0) {
         // ================================================= producer
@@ -432,104 +424,97 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
         }
     } else if (warp == 1) {
         // ================================================= MMA issuer of S = Q K^T
-        if (lane == 0 && T > 0 && !refused()) {
+        // (the issuing warps stay converged, so that addresses and descriptors live in uniform registers, and one elected
+        // lane issues: see gemm_tc.cu)
+        if (T > 0 && !refused_warp()) {
             constexpr uint32_t idesc_s = make_idesc(128, kKeyTile, false);
-            int s = 0;
+            const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
+            const bool leader = elect_one();
+            int rs = 0;
             uint32_t ph = 0;
-            int st_kv[4] = {0, 0, 0, 0}, st_lo[4] = {-1, -1, -1, -1};   // ring stages of the (up to three) tiles in flight, by tile & 3
-            auto issue_s = [&](int i) -> bool {             // S of tile t_begin + i into score buffer i & 1
-                const int t = t_begin + i, b = i & 1;
-                const bool lo = comp && reaches_tree(t);
-                st_kv[i & 3] = s;
-                if (!mbar_wait(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) return false;
-                if (++s == kStages) { s = 0; ph ^= 1u; }
-                st_lo[i & 3] = -1;
-                if (lo) {
-                    st_lo[i & 3] = s;
-                    if (!mbar_wait(smem_u32(&ctl.full[s]), ph, abort_flag, wait_limit)) return false;
-                    if (++s == kStages) { s = 0; ph ^= 1u; }
-                }
-                // (the softmax warps have read tile i - 2 out of this score buffer: their P of that tile, which
-                // the caller has waited for, came after it)
-                tc_fence_after();
-                // One thread issues every MMA, so the code between two of them is what limits the rate:
-                // descriptors are a base plus compile-time offsets (address field in units of 16 bytes).
-                const uint32_t d = tmem_base + (uint32_t)b * kKeyTile;
-                const uint64_t dk = desc_k_major(s_ring + st_kv[i & 3] * kStageBytes);
-                // k-step ks = 16 head dims: 8 columns of the queries in tensor memory, 32 bytes in a row of
-                // the K sub-tile that holds dims 64 * (ks / 4) ..
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    tc_mma_ts(d, tmem_base + kColQ + 8 * ks, dk + (uint64_t)(((ks >> 2) * kSubTile >> 4) + 2 * (ks & 3)), idesc_s, ks != 0 ? 1u : 0u);
-                if (comp) {
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        tc_mma_ts(d, tmem_base + kColQ + 64 + 8 * ks, dk + (uint64_t)(((ks >> 2) * kSubTile >> 4) + 2 * (ks & 3)), idesc_s, 1u);
-                }
-                if (lo) {
-                    const uint64_t dl = desc_k_major(s_ring + st_lo[i & 3] * kStageBytes);
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        tc_mma_ts(d, tmem_base + kColQ + 8 * ks, dl + (uint64_t)(((ks >> 2) * kSubTile >> 4) + 2 * (ks & 3)), idesc_s, 1u);
-                }
-                tc_commit(smem_u32(&ctl.s_full[b]));
-                return true;
-            };
-            if (!mbar_wait(smem_u32(&ctl.q_full), 0, abort_flag, wait_limit)) failed = true;
-            // Scores run two tiles ahead of the softmax: tile i goes into the buffer that the weights of
-            // tile i - 2 have been computed from.
+            if (!mbar_wait_all(smem_u32(&ctl.q_full), 0, abort_flag, wait_limit)) failed = true;
+            // S of tile i goes into score buffer i & 1 as soon as the softmax warps have read tile i - 2 out of it
             for (int i = 0; i < T && !failed; ++i) {
-                if (i >= 2 && !mbar_wait(smem_u32(&ctl.p_full[i & 1]), (uint32_t)((i - 2) >> 1) & 1u, abort_flag, wait_limit)) { failed = true; break; }
-                if (!issue_s(i)) failed = true;
+                const int b = i & 1;
+                const bool lo = comp && reaches_tree(t_begin + i);
+                if (i >= 2 && !mbar_wait_all(smem_u32(&ctl.s_empty[b]), (uint32_t)((i - 2) >> 1) & 1u, abort_flag, wait_limit)) { failed = true; break; }
+                if (!mbar_wait_all(smem_u32(&ctl.full[rs]), ph, abort_flag, wait_limit)) { failed = true; break; }
+                const uint64_t dk = desc_k_major(s_ring + rs * kStageBytes);
+                uint64_t dl = 0;
+                if (++rs == kStages) { rs = 0; ph ^= 1u; }
+                if (lo) {
+                    if (!mbar_wait_all(smem_u32(&ctl.full[rs]), ph, abort_flag, wait_limit)) { failed = true; break; }
+                    dl = desc_k_major(s_ring + rs * kStageBytes);
+                    if (++rs == kStages) { rs = 0; ph ^= 1u; }
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)b * kKeyTile;
+                if (leader) {
+                    // k-step ks = 16 head dims: 8 columns of the queries in tensor memory, 32 bytes in a row of
+                    // the K sub-tile that holds dims 64 * (ks / 4) ..
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        tc_mma_ts(d, tmem + kColQ + 8 * ks, dk + (uint64_t)(((ks >> 2) * kSubTile >> 4) + 2 * (ks & 3)), idesc_s, ks != 0 ? 1u : 0u);
+                    if (comp) {
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)
+                            tc_mma_ts(d, tmem + kColQ + 64 + 8 * ks, dk + (uint64_t)(((ks >> 2) * kSubTile >> 4) + 2 * (ks & 3)), idesc_s, 1u);
+                    }
+                    if (lo) {
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)
+                            tc_mma_ts(d, tmem + kColQ + 8 * ks, dl + (uint64_t)(((ks >> 2) * kSubTile >> 4) + 2 * (ks & 3)), idesc_s, 1u);
+                    }
+                    tc_commit(smem_u32(&ctl.s_full[b]));
+                }
             }
         }
     } else if (warp == 6) {
         // ================================================= MMA issuer of O += P V
-        // A second issuing thread: a run of MMAs into one accumulator holds its thread for the ~420 cycles
+        // A second issuing warp: a run of MMAs into one accumulator holds its thread for the ~420 cycles
         // of pipeline latency on top of the MMAs themselves, and two threads keep two runs (scores of a
         // later tile, P V of this one) in flight at once (measured: 1460 cycles for both against 1870 in turn).
-        if (lane == 0 && T > 0 && !refused()) {
+        if (T > 0 && !refused_warp()) {
             constexpr uint32_t idesc_o = make_idesc(128, kHd, true);
-            int s = 0;                                    // walks the ring like the score issuer (it has waited for the copies)
+            const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0), d = tmem + kColO;
+            const bool leader = elect_one();
+            int rs = 0;                                   // walks the ring like the score issuer (it has waited for the copies)
             for (int i = 0; i < T && !failed; ++i) {
                 const bool lo = comp && reaches_tree(t_begin + i);
-                const int s_kv = s;
-                if (++s == kStages) s = 0;
-                int s_lo = -1;
-                if (lo) {
-                    s_lo = s;
-                    if (++s == kStages) s = 0;
-                }
-                if (!mbar_wait(smem_u32(&ctl.p_full[i & 1]), (uint32_t)(i >> 1) & 1u, abort_flag, wait_limit)) { failed = true; break; }
-                tc_fence_after();
+                const int s_kv = rs;
+                if (++rs == kStages) rs = 0;
+                const int s_lo = rs;
+                if (lo && ++rs == kStages) rs = 0;
                 const int b = i & 1;
-                const uint32_t d = tmem_base + kColO;
+                if (!mbar_wait_all(smem_u32(&ctl.p_full[b]), (uint32_t)(i >> 1) & 1u, abort_flag, wait_limit)) { failed = true; break; }
+                tc_fence_after();
                 // 16 keys further: 8 columns of P in tensor memory, 16 rows (2048 bytes) in V
-                const uint32_t tp = tmem_base + kColP + 64 * (uint32_t)b;
+                const uint32_t tp = tmem + kColP + 64 * (uint32_t)b;
                 const uint64_t dv = desc_mn_major(s_ring + s_kv * kStageBytes + 2 * kSubTile, kSubTile);
-                if (i > 0) {                              // the outputs accumulate in TMEM over the tiles
+                const uint64_t dvl = desc_mn_major(s_ring + s_lo * kStageBytes + 2 * kSubTile, kSubTile);
+                const uint32_t acc = i > 0 ? 1u : 0u;     // the outputs accumulate in TMEM over the tiles
+                if (leader) {
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 8 * ks, dv + (uint64_t)(ks * 2048 >> 4), idesc_o, 1u);
-                } else {
+                    for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 8 * ks, dv + (uint64_t)(ks * 2048 >> 4), idesc_o, ks != 0 ? 1u : acc);
+                    if (comp) {
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 8 * ks, dv + (uint64_t)(ks * 2048 >> 4), idesc_o, ks != 0 ? 1u : 0u);
+                        for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 32 + 8 * ks, dv + (uint64_t)(ks * 2048 >> 4), idesc_o, 1u);
+                    }
+                    if (lo) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 8 * ks, dvl + (uint64_t)(ks * 2048 >> 4), idesc_o, 1u);
+                    }
+                    tc_commit(smem_u32(&ctl.o_full[b]));
+                    tc_commit(smem_u32(&ctl.empty[s_kv]));
+                    if (lo) tc_commit(smem_u32(&ctl.empty[s_lo]));
                 }
-                if (comp) {
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 32 + 8 * ks, dv + (uint64_t)(ks * 2048 >> 4), idesc_o, 1u);
-                }
-                if (s_lo >= 0) {
-                    const uint64_t dvl = desc_mn_major(s_ring + s_lo * kStageBytes + 2 * kSubTile, kSubTile);
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) tc_mma_ts(d, tp + 8 * ks, dvl + (uint64_t)(ks * 2048 >> 4), idesc_o, 1u);
-                }
-                tc_commit(smem_u32(&ctl.o_full[b]));
-                tc_commit(smem_u32(&ctl.empty[s_kv]));
-                if (s_lo >= 0) tc_commit(smem_u32(&ctl.empty[s_lo]));
             }
         }
-    } else if (warp < 6) {
-        // ================================================= softmax (warps 2..5): thread = query row
+    } else {
+        // ================================================= softmax: thread = query row, two groups of four warps
+        // (2..5 and 7..10) that take alternate tiles: group g owns score buffer g and weight buffer g. With one group a
+        // tile took 2670 cycles, of which 1600 were its own work and the rest waits that nobody filled.
+        const int grp = warp > 6 ? 1 : 0;
         const int lg = warp & 3;                          // TMEM lanes 32*lg .. 32*lg + 31 belong to this warp
         const int row = lg * 32 + lane;
         const bool warp_active = lg * 32 < n;             // a warp whose rows are all padding only keeps the barriers going
@@ -543,73 +528,91 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
 #pragma unroll
             for (int w = 0; w < 4; ++w) a4[w] = own ? own_anc[w] : __ldcg(anc + (q_first + row) * 4 + w);   // L2: written earlier in this pass
         }
-        uint4 g[2][16];
-        if (warp_active) {
+        const bool stages_q = warp_active && (comp || grp == 0);   // group 0 fetches the hi plane of the queries, group 1 the lo plane
+        uint4 g[16];
+        if (stages_q) {
 #pragma unroll
-            for (int pl = 0; pl < 2; ++pl) {
-                if (pl < (comp ? 2 : 1)) {
-#pragma unroll
-                    for (int it = 0; it < 16; ++it) {
-                        const int rr = it * 2 + (lane >> 4);
-                        const int qrow = min(lg * 32 + rr, n - 1);
-                        g[pl][it] = __ldcg(reinterpret_cast<const uint4 *>(q + (size_t)pl * lo_off + ((size_t)qrow * n_heads + head) * kHd) + (lane & 15));
-                    }
-                }
+            for (int it = 0; it < 16; ++it) {
+                const int qrow = min(lg * 32 + it * 2 + (lane >> 4), n - 1);
+                g[it] = __ldcg(reinterpret_cast<const uint4 *>(q + (size_t)grp * lo_off + ((size_t)qrow * n_heads + head) * kHd) + (lane & 15));
             }
         }
         const bool skip = status_says_no();
         if (!skip) {
         // The queries become the A operand of Q K^T in tensor memory: 64 packed columns per plane, thread =
-        // row. A warp fetches its 32 rows with coalesced loads (two rows of 256 bytes per instruction, both
-        // planes in flight together), turns them through a small shared-memory buffer (16-byte chunks
-        // XOR-swizzled by row) and every thread stores its own row. Rows beyond n repeat row n - 1: a row
-        // of A only ever influences the same row of the product, and nobody reads those rows of the result.
-        if (warp_active) {
-            const int planes = comp ? 2 : 1;
-            const uint32_t stg = smem_u32(q_stage + (size_t)lg * kQStage);
+        // row. A warp fetches its 32 rows with coalesced loads (two rows of 256 bytes per instruction), turns them
+        // through a small shared-memory buffer, 16 rows at a time (16-byte chunks XOR-swizzled by row), and every
+        // thread stores its own row. Rows beyond n repeat row n - 1: a row of A only ever influences the same row of
+        // the product, and nobody reads those rows of the result.
+        if (stages_q) {
+            const uint32_t stg = smem_u32(q_stage + (size_t)(grp * 4 + lg) * (kQStage / 2));
+            uint32_t qr[64];
 #pragma unroll
-            for (int pl = 0; pl < 2; ++pl) {
-                if (pl < planes) {
+            for (int half = 0; half < 2; ++half) {
 #pragma unroll
-                    for (int it = 0; it < 16; ++it) {
-                        const int rr = it * 2 + (lane >> 4);
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + rr * 256 + (((lane & 15) ^ (rr & 15)) << 4)),
-                                     "r"(g[pl][it].x), "r"(g[pl][it].y), "r"(g[pl][it].z), "r"(g[pl][it].w) : "memory");
-                    }
-                    __syncwarp();
-                    uint32_t qr[64];
+                for (int it = 0; it < 8; ++it) {
+                    const int rr = it * 2 + (lane >> 4);
+                    const uint4 v = g[half * 8 + it];
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + rr * 256 + (((lane & 15) ^ rr) << 4)),
+                                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+                }
+                __syncwarp();
+                if ((lane >> 4) == half) {
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                                      : "=r"(qr[4 * c]), "=r"(qr[4 * c + 1]), "=r"(qr[4 * c + 2]), "=r"(qr[4 * c + 3])
-                                     : "r"(stg + lane * 256 + ((c ^ (lane & 15)) << 4)) : "memory");
+                                     : "r"(stg + (lane & 15) * 256 + ((c ^ (lane & 15)) << 4)) : "memory");
                     }
-                    __syncwarp();                         // the buffer is reused for the lo plane
-                    tc_st32(tlane + kColQ + 64 * pl, qr);
-                    tc_st32(tlane + kColQ + 64 * pl + 32, qr + 32);
                 }
+                __syncwarp();
             }
+            tc_st32(tlane + kColQ + 64 * grp, qr);
+            tc_st32(tlane + kColQ + 64 * grp + 32, qr + 32);
             tc_wait_st();
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&ctl.q_full));
+        if (lane == 0 && (comp || grp == 0)) mbar_arrive(smem_u32(&ctl.q_full));
         const float scale_log2 = 1.4426950408889634f * rsqrtf((float)kHd);
         // Online softmax with a lazy reference: the weights of a row are 2^(s - ref), and ref only moves
         // (with a rescale of the row's running sum and of its outputs in TMEM) when a tile's maximum
         // exceeds it by more than kSlack, so that the outputs can stay and accumulate in TMEM across the
-        // tiles; weights then reach at most 2^kSlack, harmless in fp32 and in hi + lo bf16.
+        // tiles; weights then reach at most 2^kSlack, harmless in fp32 and in hi + lo bf16. The two groups share
+        // a row's reference: it is decided tile by tile, in tile order (ctl.seq counts the decided tiles of a warp's
+        // rows), so that results do not depend on timing; each keeps the sum of its own tiles' weights.
         constexpr float kSlack = 8.f;
         float ref = -INFINITY, l = 0.f;
+        volatile float *s_ref = ctl.ref;
+        auto decided = [&](int tiles) -> bool {           // waits until the reference after the first `tiles` tiles stands
+            uint64_t t0 = 0;
+            for (uint32_t it = 1; ctl.seq[lg] < tiles; ++it) {
+                if ((it & 255u) == 0) {
+                    const uint64_t now = global_timer_ns();
+                    if (t0 == 0) t0 = now;
+                    if (*abort_flag || now - t0 > wait_limit) return false;
+                }
+            }
+            return true;
+        };
+        auto follow = [&](float r) {                      // this thread's sum onto reference r
+            if (r != ref) {
+                l = ref == -INFINITY ? 0.f : l * ex2(ref - r);
+                ref = r;
+            }
+        };
 
-        for (int i = 0; i < T; ++i) {
-            const int t = t_begin + i, b = i & 1;
-            const int key0 = t * kKeyTile;
-            if (!mbar_wait_warp(smem_u32(&ctl.s_full[b]), (uint32_t)(i >> 1) & 1u, abort_flag, lane, wait_limit)) { failed = true; break; }
+        for (int i = grp; i < T; i += 2) {
+            const int key0 = (t_begin + i) * kKeyTile;
+            const uint32_t par_i = (uint32_t)(i >> 1) & 1u;
+            if (!mbar_wait_all(smem_u32(&ctl.s_full[grp]), par_i, abort_flag, wait_limit)) { failed = true; break; }
             tc_fence_after();
             if (trace && tid == 64 && cta < 256 && i == 0) trace[(size_t)cta * 16 + 2] = global_timer_ns();
             float sc[kKeyTile];
-            if (warp_active) tc_ld64(tlane + (uint32_t)b * kKeyTile, sc);
+            if (warp_active) tc_ld64(tlane + (uint32_t)grp * kKeyTile, sc);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&ctl.s_empty[grp]));      // the scores of tile i + 2 may come
             // Visibility of the tile's 64 keys for this row, one bit each: prefix keys always, tree keys by
             // the row's ancestor-or-self bits (bits of nodes that do not exist are never set).
             float tmax = -INFINITY;
@@ -633,74 +636,86 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
                 for (int j = 0; j < kKeyTile; ++j) tmax = fmaxf(tmax, sc[j]);
                 tmax *= scale_log2;                       // scores stay raw; the scale goes into the exponent below
             }
-            // P buffer b was last read by the P V of tile i - 2
-            if (i > 1) {
-                if (!mbar_wait_warp(smem_u32(&ctl.o_full[b]), (uint32_t)((i - 2) >> 1) & 1u, abort_flag, lane, wait_limit)) { failed = true; break; }
-            }
+            // P buffer grp was last read by the P V of tile i - 2
+            if (i > 1 && !mbar_wait_all(smem_u32(&ctl.o_full[grp]), (uint32_t)((i - 2) >> 1) & 1u, abort_flag, wait_limit)) { failed = true; break; }
             if (warp_active) {
+                if (__any_sync(0xffffffffu, !decided(i))) { failed = true; break; }
+                if (i > 0) follow(s_ref[row]);
                 const bool move = tmax > ref + kSlack || (ref == -INFINITY && tmax > -INFINITY);
                 if (__any_sync(0xffffffffu, move)) {
                     // the outputs in TMEM are about to be rescaled: the P V of tile i - 1 must have retired
-                    if (i > 0 && !mbar_wait_warp(smem_u32(&ctl.o_full[b ^ 1]), (uint32_t)((i - 1) >> 1) & 1u, abort_flag, lane, wait_limit)) { failed = true; break; }
+                    if (i > 0 && !mbar_wait_all(smem_u32(&ctl.o_full[grp ^ 1]), (uint32_t)((i - 1) >> 1) & 1u, abort_flag, wait_limit)) { failed = true; break; }
                     tc_fence_after();
                     const float factor = !move ? 1.f : (ref == -INFINITY ? 0.f : ex2(ref - tmax));
-                    if (move) ref = tmax;
-                    l *= factor;
+                    if (move) follow(tmax);
                     if (i > 0) {
+#pragma unroll 1
+                        for (int hcol = 0; hcol < 4; ++hcol) {
+                            float ov[32];
+                            tc_ld32(tlane + kColO + hcol * 32, ov);
 #pragma unroll
-                        for (int hcol = 0; hcol < 2; ++hcol) {
-                            float ov[64];
-                            tc_ld64(tlane + kColO + hcol * 64, ov);
-#pragma unroll
-                            for (int j = 0; j < 64; ++j) ov[j] *= factor;
-                            tc_st64(tlane + kColO + hcol * 64, ov);
+                            for (int j = 0; j < 32; ++j) ov[j] *= factor;
+                            tc_st32(tlane + kColO + hcol * 32, reinterpret_cast<const uint32_t *>(ov));
                         }
+                        tc_wait_st();
                     }
                 }
+                s_ref[row] = ref;
+                __threadfence_block();
+                __syncwarp();
+                if (lane == 0) ctl.seq[lg] = i + 1;
                 const float nr0 = (ref == -INFINITY) ? 0.f : -ref;   // no visible key so far: every weight is 0 anyway
-                float rs = 0.f;
-                uint32_t hi[32], lo[32];                  // packed pairs of consecutive keys: the A operand of P V
+                float rsum = 0.f;
+                const uint32_t tp = tlane + kColP + 64 * (uint32_t)grp;
 #pragma unroll
-                for (int e = 0; e < kKeyTile / 2; ++e) {
-                    const float p0 = ex2(fmaf(sc[2 * e], scale_log2, nr0));
-                    const float p1 = ex2(fmaf(sc[2 * e + 1], scale_log2, nr0));
-                    rs += p0 + p1;
-                    pack_split(p0, p1, hi[e], lo[e]);
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t hi[16], lo[16];              // packed pairs of consecutive keys: the A operand of P V
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const float p0 = ex2(fmaf(sc[32 * half + 2 * e], scale_log2, nr0));
+                        const float p1 = ex2(fmaf(sc[32 * half + 2 * e + 1], scale_log2, nr0));
+                        rsum += p0 + p1;
+                        if (comp) pack_split(p0, p1, hi[e], lo[e]);
+                        else hi[e] = pack2(p0, p1);
+                    }
+                    tc_st16(tp + 16 * half, hi);
+                    if (comp) tc_st16(tp + 32 + 16 * half, lo);
                 }
-                tc_st32(tlane + kColP + 64 * (uint32_t)b, hi);
-                if (comp) tc_st32(tlane + kColP + 64 * (uint32_t)b + 32, lo);
                 tc_wait_st();
-                l += rs;
+                l += rsum;
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl.p_full[b]));
+            if (lane == 0) mbar_arrive(smem_u32(&ctl.p_full[grp]));
         }
-        // the last two tiles' P V
+        // All P V have retired when the last tile's has; this group has followed its own buffer's barrier up to its
+        // last tile but one.
         for (int i = max(0, T - 2); i < T && !failed; ++i)
-            if (!mbar_wait_warp(smem_u32(&ctl.o_full[i & 1]), (uint32_t)(i >> 1) & 1u, abort_flag, lane, wait_limit)) failed = true;
+            if (((i & 1) == grp || i == T - 1) && !mbar_wait_all(smem_u32(&ctl.o_full[i & 1]), (uint32_t)(i >> 1) & 1u, abort_flag, wait_limit)) failed = true;
+        if (warp_active && !failed && T > 0) {
+            if (__any_sync(0xffffffffu, !decided(T))) failed = true;
+            else follow(s_ref[row]);
+        }
         tc_fence_after();
         if (trace && tid == 64 && cta < 256) trace[(size_t)cta * 16 + 3] = global_timer_ns();
         // every copy has landed and every MMA has retired (the last o_full): the ring is free for the
-        // partial of this CTA: per row 128 outputs, reference, sum
+        // partial of this CTA: per row 128 outputs (64 by each group), reference, the two groups' sums
         if (!failed && warp_active) {
             float *pr = part + (size_t)row * kWsRow;
+            float ov[64];
+            if (T > 0) {
+                tc_ld64(tlane + kColO + grp * 64, ov);
+            } else {
 #pragma unroll
-            for (int hcol = 0; hcol < 2; ++hcol) {
-                float ov[64];
-                if (T > 0) {
-                    tc_ld64(tlane + kColO + hcol * 64, ov);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 64; ++j) ov[j] = 0.f;
-                }
-                if (row < n) {
-#pragma unroll
-                    for (int j = 0; j < 64; j += 4)
-                        *reinterpret_cast<float4 *>(pr + hcol * 64 + j) = make_float4(ov[j], ov[j + 1], ov[j + 2], ov[j + 3]);
-                }
+                for (int j = 0; j < 64; ++j) ov[j] = 0.f;
             }
-            if (row < n) *reinterpret_cast<float2 *>(pr + kHd) = make_float2(ref, l);
+            if (row < n) {
+#pragma unroll
+                for (int j = 0; j < 64; j += 4)
+                    *reinterpret_cast<float4 *>(pr + grp * 64 + j) = make_float4(ov[j], ov[j + 1], ov[j + 2], ov[j + 3]);
+                if (grp == 0) *reinterpret_cast<float2 *>(pr + kHd) = make_float2(ref, l);
+                else pr[kHd + 2] = l;
+            }
         }
         }
         tc_fence_before();
@@ -717,6 +732,9 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
     }
     // (the softmax warps have passed the grid dependency, so the status word is final for every thread)
     const bool bad = ctl.abort_flag != 0 || status_says_no();
+
+    if (!bad && tid < n) part[(size_t)tid * kWsRow + kHd + 1] += part[(size_t)tid * kWsRow + kHd + 2];    // the two groups' sums
+    __syncthreads();
 
     // four outputs of one row, normalised, as bf16 hi (and lo) to global memory
     auto store4 = [&](int row, int dim, float4 a, float inv) {
