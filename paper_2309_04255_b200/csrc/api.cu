@@ -115,6 +115,7 @@ struct llmcad_ctx {
     TreeBuffers tb{};
     // the one-kernel fp32 pass (pass_small.cu): allowed, and its own workspaces
     bool small_pass = false;
+    bool wide_chunks = false;      // prefill: chunks of kLoRows tokens
     float *sp_att = nullptr;
     float2 *sp_ml = nullptr;
     unsigned long long *sp_best = nullptr;
@@ -145,9 +146,9 @@ struct llmcad_ctx {
     const void *maps_for = nullptr;    // packed weight buffer of the current call
     std::vector<CUtensorMap> weight_maps;   // its matrices, for the GEMMs on CTA pairs: four per layer, then the lm_head
     const void *weight_maps_for = nullptr;
-    CUtensorMap act_maps[9][3];        // [n_pad/16][xn, att, h]
-    CUtensorMap pair_maps[9][3];       // the same for the GEMMs on CTA pairs
-    bool act_ready[9] = {false, false, false, false, false, false, false, false, false};
+    CUtensorMap act_maps[17][3];        // [n_pad/16][xn, att, h]
+    CUtensorMap pair_maps[17][3];       // the same for the GEMMs on CTA pairs
+    bool act_ready[17] = {};
     // optional per-launch timing (events around every GEMM / attention launch)
     bool timing = false;
     struct Timed { int kind; cudaEvent_t a, b; };
@@ -231,10 +232,12 @@ int ensure_act_maps(llmcad_ctx *ctx, int n_pad)
     const void *bufs[3] = {ctx->xn, ctx->att, ctx->h};
     for (int i = 0; i < 3; ++i) {
         const int cols = i == 2 ? c.d_ffn : c.d_model;
-        ok &= make_act_map_bf16(&ctx->act_maps[slot][i], bufs[i], 128, cols, n_pad, planes, kLoRows, planes);
+        if (n_pad <= LLMCAD_MAX_TREE) ok &= make_act_map_bf16(&ctx->act_maps[slot][i], bufs[i], kLoRows, cols, n_pad, planes, kLoRows, planes);
         // a CTA pair: one plane, or half of the rows of the only plane
         if (gemm_takes_pairs(n_pad, ctx->comp))
-            ok &= make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], 128, cols, ctx->comp ? n_pad : n_pad / 2, planes, kLoRows, 1);
+            ok &= n_pad > LLMCAD_MAX_TREE
+                      ? make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], kLoRows, cols, n_pad / 2, planes, kLoRows, planes)    // half of the rows, both planes
+                      : make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], kLoRows, cols, ctx->comp ? n_pad : n_pad / 2, planes, kLoRows, 1);
     }
     if (!ok) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for an activation buffer");
@@ -342,15 +345,17 @@ int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st);
 // n_old = 0): tree prep of the whole tree, embedding, all layers; K/V of node i go to cache slot
 // P+i, where the nodes below n_old already have theirs. When logits != nullptr the final norm and
 // lm_head run too (one row per processed node). The status word starts from this tree's own check, or, with
-// keep_status, stays as an earlier chunk of the same call left it if that found an error.
+// keep_status, stays as an earlier chunk of the same call left it if that found an error. last_row (tensor-core path
+// only): logits has one row, the last node's.
 int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens,
                 const int32_t *parent, int n_tree, float *logits, int32_t *status, cudaStream_t st, int n_old = 0,
-                bool keep_status = false)
+                bool keep_status = false, bool last_row = false)
 {
     const llmcad_config &c = ctx->cfg;
     const int d = c.d_model, f = c.d_ffn, hd = c.head_dim, H = c.n_heads, S = c.max_seq;
     const int n = n_tree - n_old;                    // nodes this call computes
-    const int n_pad = (n + 15) / 16 * 16;
+    const bool wide = n > LLMCAD_MAX_TREE;           // a chunk of a prompt (a chain; parent is not read)
+    const int n_pad = wide ? kLoRows : (n + 15) / 16 * 16;
     const char *base = static_cast<const char *>(packed);
     int rc;
     if (use_small_pass(ctx, P + n_tree))
@@ -368,7 +373,11 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
         // partial sums of squares; the consuming GEMM scales its accumulators by the per-node
         // rsqrt(mean(x^2) + eps). Activations travel as bf16 hi + lo planes (ctx->comp).
         const int tiles4 = 4 * ((d + 127) / 128);
-        CUDA_TRY(launch_prep_embed(parent, tokens, n_tree, n_old, P, c.vocab, hd, ctx->inv_freq, ctx->tb, base + ctx->lay.tok_embed,
+        if (wide)
+            CUDA_TRY(launch_chain_embed(tokens, n, P, c.vocab, hd, ctx->inv_freq, ctx->tb, base + ctx->lay.tok_embed, d,
+                                        c.n_layers > 0 ? base + ctx->lay.attn_norm : base + ctx->lay.final_norm, ctx->x, ctx->xn, ctx->ssq[0],
+                                        status, keep_status ? 1 : 0, st));
+        else CUDA_TRY(launch_prep_embed(parent, tokens, n_tree, n_old, P, c.vocab, hd, ctx->inv_freq, ctx->tb, base + ctx->lay.tok_embed,
                                    c.dtype, d, c.n_layers > 0 ? base + ctx->lay.attn_norm : base + ctx->lay.final_norm, ctx->x, ctx->xn,
                                    ctx->ssq[0], ctx->comp ? 1 : 0, status, keep_status ? 1 : 0, st));
         auto qkv_ep = [&](int l, int parts) {
@@ -382,8 +391,8 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
         };
         auto head_ep = [&](int parts) {
             EpiParams ep{};
-            ep.n = n; ep.mode = EPI_PLAIN; ep.n_out = c.vocab; ep.y = logits; ep.ldy = c.vocab;
-            ep.ssq_in = ctx->ssq[0]; ep.ssq_in_parts = parts; ep.norm_d = d; ep.eps = c.rms_eps;
+            ep.n = last_row ? 1 : n; ep.mode = EPI_PLAIN; ep.n_out = c.vocab; ep.y = logits; ep.ldy = c.vocab;
+            ep.ssq_in = ctx->ssq[0] + (last_row ? n - 1 : 0); ep.ssq_in_parts = parts; ep.norm_d = d; ep.eps = c.rms_eps;
             return ep;
         };
         // the GEMMs of the pass in order; attention runs before the O GEMM of every layer
@@ -415,8 +424,18 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
             else if (logits != nullptr) specs.push_back({-1, 0, 0, d, head_ep(tiles4), false});
         }
         std::vector<TcGemm> gemms(specs.size());
-        for (size_t i = 0; i < specs.size(); ++i)
-            gemms[i].set(ctx, specs[i].l, specs[i].which, specs[i].act, specs[i].n_in, specs[i].ep, n_pad);
+        for (size_t i = 0; i < specs.size(); ++i) {
+            if (specs[i].l < 0 && last_row) {
+                // the lm_head on the last row alone
+                if ((rc = ensure_act_maps(ctx, 16)) != LLMCAD_OK) return rc;
+                gemms[i].set(ctx, -1, 0, 0, d, specs[i].ep, 16);
+                if (!make_act_map_bf16(&gemms[i].maps.x, static_cast<char *>(ctx->xn) + (size_t)(n - 1) * d * ctx->elem, 1, d, 16, ctx->comp ? 2 : 1, kLoRows,
+                                       ctx->comp ? 2 : 1)) {
+                    snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for an activation row");
+                    return LLMCAD_ERR_CUDA;
+                }
+            } else gemms[i].set(ctx, specs[i].l, specs[i].which, specs[i].act, specs[i].n_in, specs[i].ep, n_pad);
+        }
         // Hand-over between the kernels: completion counters (one per kernel, zeroed here) where both sides are
         // tensor-core kernels of this library, the grid dependency otherwise. `dep` is what the next kernel
         // waits for: null after the embedding kernel and after a plain-ALU attention kernel.
@@ -611,7 +630,7 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
         wants.push_back({p, arena_bytes});
         arena_bytes = align_up(arena_bytes + bytes, 1024);
     };
-    want((void **)&ctx->x, 128 * d * 4);
+    want((void **)&ctx->x, kLoRows * d * 4);
     want(&ctx->xn, 2 * kLoRows * d * ctx->elem);
     want(&ctx->q, 2 * kLoRows * d * ctx->elem);
     want(&ctx->att, 2 * kLoRows * d * ctx->elem);
@@ -621,7 +640,7 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
     want((void **)&ctx->tb.depth, 128 * 4);
     want((void **)&ctx->tb.pos, 128 * 4);
     want((void **)&ctx->tb.anc, 128 * 16);
-    want((void **)&ctx->tb.rope_cs, 128 * (hd / 2) * sizeof(float2));
+    want((void **)&ctx->tb.rope_cs, kLoRows * (hd / 2) * sizeof(float2));
     want((void **)&ctx->inv_freq, (hd / 2) * sizeof(double));
     want((void **)&ctx->ibuf, (520 + 128) * 4);
     {
@@ -631,6 +650,14 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
             if ((int)((rows + 127) / 128) > max_tiles) max_tiles = (int)((rows + 127) / 128);
         const int max_pad = (cfg->max_tree + 15) / 16 * 16;
         ctx->partial_floats = ctx->tc_gemm ? gemm_tc_partial_floats(ctx->n_sms, max_tiles, max_pad) : 64;
+        // Prompts go in chunks of kLoRows tokens where the GEMMs on CTA pairs and the tcgen05 attention kernel serve the
+        // layers: the weights are then read half as often, and at 256 columns the MMAs of hi and lo planes set the pace.
+        ctx->wide_chunks = ctx->tc_gemm && ctx->comp && !ctx->w4 && ctx->tc_attn && !(cfg->flags & LLMCAD_FLAG_MMA_ATTN) &&
+                           attention_prefers_t5(LLMCAD_MAX_TREE) && cfg->max_tree == LLMCAD_MAX_TREE;
+        if (ctx->wide_chunks) {
+            const size_t wide = gemm_tc_wide_partial_floats(ctx->n_sms, (int)(d > f ? d : f), (int)d);
+            if (wide > ctx->partial_floats) ctx->partial_floats = wide;
+        }
         want((void **)&ctx->partials, ctx->partial_floats * 4);
     }
     {
@@ -645,7 +672,7 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
             want((void **)&ctx->sp_bar, 2 * 4);
         }
     }
-    const size_t ssq_floats = (size_t)4 * ((d + 127) / 128) * LLMCAD_MAX_TREE;
+    const size_t ssq_floats = (size_t)4 * ((d + 127) / 128) * kLoRows;
     want((void **)&ctx->ssq[0], ssq_floats * 4);
     want((void **)&ctx->ssq[1], ssq_floats * 4);
     want((void **)&ctx->sync_ctrs, kSyncCounters * sizeof(uint32_t));
@@ -816,16 +843,20 @@ int llmcad_prefill(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int32_t *status = ctx->scalars_dev() + LLMCAD_S_STATUS;
     const int chunk = ctx->cfg.max_tree;
-    for (int done = 0; done < n; done += chunk) {
-        const int m = n - done < chunk ? n - done : chunk;
-        const bool last = done + m == n;
+    const bool wide = ctx->wide_chunks && !ctx->use_counters;
+    for (int done = 0, m; done < n; done += m) {
+        m = n - done;
+        if (wide && m > chunk) m = m < kLoRows ? m : kLoRows;
+        else if (m > chunk) m = chunk;
+        float *lg = done + m == n ? last_logits : nullptr;
+        const bool direct = ctx->tc_gemm;             // one row of logits, straight to where it is wanted
         // a chain whose "prefix" is everything before it; every node is committed, nothing to roll back
         int rc = run_forward(ctx, packed, kv_cache, prefix_len + done, tokens + done, ctx->chain_dev(), m,
-                             (last && last_logits != nullptr) ? ctx->logits : nullptr, status, st, 0, done > 0);
+                             lg == nullptr ? nullptr : (direct ? lg : ctx->logits), status, st, 0, done > 0, direct);
         if (rc != LLMCAD_OK) return rc;
-        if (last && last_logits != nullptr)
-            CUDA_TRY(cudaMemcpyAsync(last_logits, ctx->logits + (size_t)(m - 1) * ctx->cfg.vocab,
-                                     (size_t)ctx->cfg.vocab * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        if (lg != nullptr && !direct)
+            CUDA_TRY(cudaMemcpyAsync(lg, ctx->logits + (size_t)(m - 1) * ctx->cfg.vocab, (size_t)ctx->cfg.vocab * sizeof(float),
+                                     cudaMemcpyDeviceToDevice, st));
     }
     return LLMCAD_OK;
 }

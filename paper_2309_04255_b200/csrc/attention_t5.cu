@@ -288,6 +288,16 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
                     int32_t *status, unsigned long long *trace, int comp, int n_tree, int q_first, uint64_t wait_limit,
                     DepWait dep, uint32_t *done_ctr, const int32_t *__restrict__ parent)
 {
+    // Chunks of a prompt of more than 128 rows: blockIdx.y walks the heads once per block of 128 rows. A block sees the
+    // rows before it as prefix and its own as a chain (anc holds the rows of one block, all are alike).
+    const int row_block = (int)blockIdx.y / n_heads, rows_before = row_block * 128;
+    if (n > 128) {
+        q += (size_t)rows_before * n_heads * kHd;
+        o += (size_t)rows_before * n_heads * kHd;
+        P += rows_before;
+        n = min(128, n - rows_before);
+        n_tree = n;
+    }
     // parent != null: a call of its own, see attention_tc.cu
     const bool own = parent != nullptr;
     const int cta = blockIdx.y * gridDim.x + blockIdx.x;
@@ -302,7 +312,7 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
     Ctl &ctl = *reinterpret_cast<Ctl *>(q_stage + 4 * kQStage);
     float *part = reinterpret_cast<float *>(smp);   // the ring's space, once the loop is over
 
-    const int split = blockIdx.x, head = blockIdx.y;
+    const int split = blockIdx.x, head = (int)blockIdx.y - row_block * n_heads;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: known to be uniform
     const int n_keys = P + n_tree;
     const int n_tiles = (n_keys + kKeyTile - 1) / kKeyTile;
@@ -360,8 +370,9 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
     if (own) pdl_wait();
     if (tid == 0) {
         if (own) fence_proxy_async();
-        // in a pass they go out before the grid dependency: earlier passes wrote them
-        while (t < t_end && (own || !reaches_tree(t)) && issued < kStages) {
+        // in a pass they go out before the grid dependency: earlier passes wrote them (the rows before a later row block
+        // are of this pass)
+        while (t < t_end && (own || (t + 1) * kKeyTile <= P - rows_before) && issued < kStages) {
             issue_kv(t++);
             ++issued;
         }
@@ -398,7 +409,7 @@ attention_t5_kernel(const __nv_bfloat16 *__restrict__ q, const __grid_constant__
             auto issue_lo = [&](int t) {
                 const uint32_t full = smem_u32(&ctl.full[s]);
                 const uint32_t dst = s_ring + s * kStageBytes;
-                const int row0 = t * kKeyTile - P - q_first;      // query index of the tile's first key
+                const int row0 = t * kKeyTile - P - q_first + rows_before;      // query index of the tile's first key
                 mbar_expect_tx(full, kStageBytes);
                 for (int j = 0; j < 2; ++j) {
                     tma_load_3d(dst + j * kSubTile, &map_lo, j * 64, row0, head, full);
@@ -791,11 +802,13 @@ cudaError_t launch_attention_t5(const void *q, const void *k, const void *v, int
                                 const AttnSync *sync, const int32_t *parent)
 {
     if (n_tree <= 0) n_tree = n;
-    if (hd != kHd || n < 1 || n > 128 || P + n_tree > kv_stride) return cudaErrorInvalidValue;
+    if (hd != kHd || n < 1 || n > kLoRows || P + n_tree > kv_stride) return cudaErrorInvalidValue;
+    const int row_blocks = (n + 127) / 128;
+    if (row_blocks > 1 && (!comp || n_tree != n || q_first != 0)) return cudaErrorInvalidValue;
     if (comp && kv_lo == nullptr) return cudaErrorInvalidValue;
     const int n_keys = P + n_tree;
     const int n_tiles = (n_keys + kKeyTile - 1) / kKeyTile;
-    int splits = n_sms / n_heads;
+    int splits = n_sms / (n_heads * row_blocks);
     if (splits > kMaxSplits) splits = kMaxSplits;
     if (splits > n_tiles) splits = n_tiles;
     if (splits < 1) splits = 1;
@@ -825,14 +838,14 @@ cudaError_t launch_attention_t5(const void *q, const void *k, const void *v, int
         if (e != cudaSuccess) return e;
         attr_set.mark();
     }
-    LaunchCfg lc(dim3(splits, n_heads), dim3(kT5Threads), kSmemBytes, st, splits);
+    LaunchCfg lc(dim3(splits, n_heads * row_blocks), dim3(kT5Threads), kSmemBytes, st, splits);
     if (launched) *launched = 1;
     DepWait dep{nullptr, 0, wait_limit_ns};
     uint32_t *done = nullptr;
     if (sync != nullptr) {
         dep = DepWait{sync->dep_ctr, sync->dep_target, wait_limit_ns};
         done = sync->done_ctr;
-        sync->arrivals = (uint32_t)(splits * n_heads);
+        sync->arrivals = (uint32_t)(splits * n_heads * row_blocks);
     }
     return cudaLaunchKernelEx(&lc.cfg, attention_t5_kernel, (const __nv_bfloat16 *)q, mk, mv, ml, n_heads, P, n, anc, (__nv_bfloat16 *)o, splits,
                               tiles_per_split, status, trace, comp, n_tree, q_first, wait_limit_ns, dep, done, parent);

@@ -30,7 +30,8 @@ cudaError_t launch_attention_tc(const void *q, const void *k, const void *v, int
                                 const void *kv_lo = nullptr, int n_tree = 0, int q_first = 0, const AttnSync *sync = nullptr,
                                 const int32_t *parent = nullptr);
 
-// The same operation on the tcgen05 tensor cores (attention_t5.cu), for larger trees; arguments as above.
+// The same operation on the tcgen05 tensor cores (attention_t5.cu), for larger trees; arguments as above. With comp, n up
+// to kLoRows rows of a chain (n_tree == n): anc then holds the mask rows of a chain of 128 nodes.
 cudaError_t launch_attention_t5(const void *q, const void *k, const void *v, int n_heads, int hd, int kv_stride, int P,
                                 int n, const uint32_t *anc, void *o, int n_sms, int32_t *status, cudaStream_t st,
                                 int *launched, unsigned long long *trace = nullptr, int comp = 0, const void *kv_lo = nullptr,

@@ -26,7 +26,8 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
 // (16 significant bits together), in two planes of the same buffer: the lo plane of a [128][len]
 // activation buffer starts kLoRows rows after the hi plane. The weights stream once either way;
 // the MMAs see the nodes twice (N = 2 * n_pad) and the epilogue adds the two accumulator columns.
-constexpr int kLoRows = LLMCAD_MAX_TREE;
+// A buffer has twice as many rows as a tree has nodes: chunks of a prompt are up to that long.
+constexpr int kLoRows = 2 * LLMCAD_MAX_TREE;
 
 __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bfloat16 &lo)
 {
@@ -79,14 +80,14 @@ struct EpiParams {
     int d, hd, S, P;
     // RMSNorm folded into the tensor-core GEMM. Input side (any mode): the accumulator of node i
     // is multiplied by rsqrt(sum_t ssq_in[t][i] / norm_d + eps); the GEMM input then is gain * x.
-    const float *ssq_in;    // [ssq_in_parts][128] partial sums of squares per node, or nullptr
+    const float *ssq_in;    // [ssq_in_parts][kLoRows] partial sums of squares per node, or nullptr
     int ssq_in_parts, norm_d;
     float eps;
     // Output side (EPI_RESID): besides x += acc, emit gain_next * x in the activation dtype and
     // this tile's partial sums of squares (4 per tile, one per 32 rows) for the next norm.
     void *xg_out;           // [n][n_out] or nullptr
     const void *gain_next;  // [n_out]
-    float *ssq_out;         // [4 * n_tiles][128]
+    float *ssq_out;         // [4 * n_tiles][kLoRows]
     // Tensor-core path: q_out, h and xg_out also get their lo plane (see kLoRows), and the bf16
     // remainders of the keys and values go to kv_lo, [2][H][kLoRows][hd] (K then V, row = node).
     int comp;
@@ -266,6 +267,10 @@ struct TreeBuffers {
 
 cudaError_t launch_tree_prep(const int32_t *parent, const int32_t *tokens, int n, int P, int vocab, TreeBuffers tb, int32_t *status,
                              cudaStream_t st);
+// A chunk of a prompt (bf16, up to kLoRows tokens): embedding, rotary rows, and the mask rows of a chain of 128 nodes,
+// which its blocks of 128 rows share.
+cudaError_t launch_chain_embed(const int32_t *tokens, int n, int P, int vocab, int hd, const double *inv_freq, TreeBuffers tb, const void *E,
+                               int d, const void *gain, float *x, void *xg, float *ssq, int32_t *status, int keep, cudaStream_t st);
 // E == nullptr: the mask table only; gain == nullptr: the residual stream only
 cudaError_t launch_prep_embed(const int32_t *parent, const int32_t *tokens, int n_tree, int n_old, int P, int vocab, int hd,
                               const double *inv_freq, TreeBuffers tb, const void *E, int dtype, int d, const void *gain, float *x,

@@ -444,7 +444,7 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
                 ss += __shfl_xor_sync(0xffffffffu, ss, 1);
                 ss += __shfl_xor_sync(0xffffffffu, ss, 2);
                 ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-                if (r4 == 0 && !dry) ep.ssq_out[(size_t)(tile * 4 + lane_grp) * LLMCAD_MAX_TREE + node] = ss;
+                if (r4 == 0 && !dry) ep.ssq_out[(size_t)(tile * 4 + lane_grp) * kLoRows + node] = ss;
             }
         } else if (mode == EPI_SWIGLU) {
 #pragma unroll
@@ -1425,7 +1425,7 @@ gemm_finish_kernel(const __grid_constant__ GemmParams p)
     // nothing to read.
     __shared__ __align__(16) GemmDesc s_desc;
     __shared__ float s_part[kFinThreads / LLMCAD_MAX_TREE][LLMCAD_MAX_TREE];
-    __shared__ float s_rs[LLMCAD_MAX_TREE];
+    __shared__ float s_rs[kLoRows];
     {
         static_assert(sizeof(GemmDesc) % 4 == 0, "GemmDesc is copied word by word");
         const uint32_t *src = reinterpret_cast<const uint32_t *>(&p.g);
@@ -1444,33 +1444,36 @@ gemm_finish_kernel(const __grid_constant__ GemmParams p)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // ---- RMSNorm of the GEMM input folded into the epilogue: the producer of the residual stream
-    // left partial sums of squares per node ([parts][128]); the accumulators of node i are multiplied
+    // left partial sums of squares per node ([parts][kLoRows]); the accumulators of node i are multiplied
     // by rsqrt(mean(x^2) + eps). Three threads per node add every third partial row, in a fixed order.
     if (ep.ssq_in != nullptr) {
         constexpr int kSlices = kFinThreads / LLMCAD_MAX_TREE;
-        const int node = threadIdx.x & (LLMCAD_MAX_TREE - 1), slice = threadIdx.x / LLMCAD_MAX_TREE;
-        float acc = 0.f;
-        if (node < p.n_pad) {
-            const float *col = ep.ssq_in + node;
-            int t = slice;
-            for (; t + 7 * kSlices < ep.ssq_in_parts; t += 8 * kSlices) {
-                float v[8];
+        const int col128 = threadIdx.x & (LLMCAD_MAX_TREE - 1), slice = threadIdx.x / LLMCAD_MAX_TREE;
+        for (int n0 = 0; n0 < p.n_pad; n0 += LLMCAD_MAX_TREE) {
+            const int node = n0 + col128;
+            float acc = 0.f;
+            if (node < p.n_pad) {
+                const float *col = ep.ssq_in + node;
+                int t = slice;
+                for (; t + 7 * kSlices < ep.ssq_in_parts; t += 8 * kSlices) {
+                    float v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = __ldcg(col + (size_t)(t + kSlices * u) * LLMCAD_MAX_TREE);
+                    for (int u = 0; u < 8; ++u) v[u] = __ldcg(col + (size_t)(t + kSlices * u) * kLoRows);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) acc += v[u];
+                    for (int u = 0; u < 8; ++u) acc += v[u];
+                }
+                for (; t < ep.ssq_in_parts; t += kSlices) acc += __ldcg(col + (size_t)t * kLoRows);
             }
-            for (; t < ep.ssq_in_parts; t += kSlices) acc += __ldcg(col + (size_t)t * LLMCAD_MAX_TREE);
-        }
-        s_part[slice][node] = acc;
-        __syncthreads();
-        if (threadIdx.x < LLMCAD_MAX_TREE) {
-            float sum = 0.f;
+            s_part[slice][col128] = acc;
+            __syncthreads();
+            if (threadIdx.x < LLMCAD_MAX_TREE) {
+                float sum = 0.f;
 #pragma unroll
-            for (int q = 0; q < kSlices; ++q) sum += s_part[q][threadIdx.x];
-            s_rs[threadIdx.x] = rsqrtf(sum / (float)ep.norm_d + ep.eps);
+                for (int q = 0; q < kSlices; ++q) sum += s_part[q][threadIdx.x];
+                s_rs[n0 + threadIdx.x] = rsqrtf(sum / (float)ep.norm_d + ep.eps);
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
 
     const int ppt = pairs_per_tile(d);
@@ -1592,6 +1595,13 @@ bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t 
 }
 
 size_t gemm_tc_partial_floats(int n_sms, int max_tiles, int max_n_pad) { return (size_t)2 * (max_tiles + n_sms) * slot_floats(max_n_pad); }
+
+size_t gemm_tc_wide_partial_floats(int n_sms, int max_rows, int d)
+{
+    // the layer's GEMMs only: 3d and d rows, and two weight tiles per output tile of the FFN's
+    const int tiles = 2 * ((max_rows + kTileM - 1) / kTileM), qkv = (3 * d + kTileM - 1) / kTileM;
+    return (size_t)((tiles > qkv ? tiles : qkv) + n_sms) * slot_floats(kLoRows);
+}
 
 GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool w4)
 {

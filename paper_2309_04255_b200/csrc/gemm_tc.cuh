@@ -80,6 +80,9 @@ bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t 
 // Floats of segment workspace that GEMMs of up to max_tiles output tiles (of one or two weight tiles) on up to max_n_pad nodes need.
 size_t gemm_tc_partial_floats(int n_sms, int max_tiles, int max_n_pad);
 
+// The same for the layer GEMMs of prompt chunks of kLoRows tokens.
+size_t gemm_tc_wide_partial_floats(int n_sms, int max_rows, int d);
+
 // Describes one GEMM (fills everything but items_per_cta and grid, which the launcher sets).
 GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled = nullptr, bool w4 = false);
 

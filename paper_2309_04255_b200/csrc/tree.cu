@@ -89,6 +89,59 @@ cudaError_t launch_prep_embed(const int32_t *parent, const int32_t *tokens, int 
                               (const __nv_bfloat16 *)E, d, (const __nv_bfloat16 *)gain, x, (__nv_bfloat16 *)xg, ssq, comp, status, keep);
 }
 
+// Start of a prompt chunk of more than 128 tokens, block i = token i; as above with the tree known to be a chain.
+__global__ void __launch_bounds__(256)
+chain_embed_kernel(const int32_t *__restrict__ tokens, int n, int P, int vocab, int hd, const double *__restrict__ inv_freq, TreeBuffers tb,
+                   const __nv_bfloat16 *__restrict__ E, int d, const __nv_bfloat16 *__restrict__ gain, float *x, __nv_bfloat16 *xg, float *ssq,
+                   int32_t *status, int keep)
+{
+    __shared__ float red[8];
+    const int i = blockIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    int bad = 0;
+    for (int c = threadIdx.x; c < n; c += 256) { const int tk = __ldg(tokens + c); bad |= tk < 0 || tk >= vocab; }
+    const int err = __syncthreads_or(bad) ? LLMCAD_ERR_BAD_TOKEN : 0;
+    if (i == 0 && threadIdx.x == 0) {
+        if (!keep) *status = err;
+        else if (err) atomicCAS(status, 0, err);
+    }
+    if (i < LLMCAD_MAX_TREE && threadIdx.x < 4) {
+        const int left = i + 1 - 32 * (int)threadIdx.x;      // bits 0 .. i of the row
+        tb.anc[i * 4 + threadIdx.x] = left >= 32 ? 0xffffffffu : (left <= 0 ? 0u : (1u << left) - 1u);
+    }
+    if (err || (keep && *reinterpret_cast<volatile int32_t *>(status))) return;
+    for (int k = threadIdx.x; k < hd / 2; k += 256) {
+        double sn, cs;
+        sincos((double)(P + i) * inv_freq[k], &sn, &cs);
+        tb.rope_cs[(size_t)i * (hd / 2) + k] = make_float2((float)cs, (float)sn);
+    }
+    const __nv_bfloat16 *row = E + (size_t)__ldg(tokens + i) * d;
+    float ss = 0.f;
+    for (int k = threadIdx.x; k < d; k += 256) {
+        const float v = __bfloat162float(row[k]);
+        x[(size_t)i * d + k] = v;
+        store_split<__nv_bfloat16>(xg + (size_t)i * d + k, (size_t)kLoRows * d, v * __bfloat162float(gain[k]), true);
+        ss += v * v;
+    }
+    for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float tot = 0.f;
+        for (int w = 0; w < 8; ++w) tot += red[w];
+        ssq[i] = tot;
+    }
+}
+
+cudaError_t launch_chain_embed(const int32_t *tokens, int n, int P, int vocab, int hd, const double *inv_freq, TreeBuffers tb, const void *E,
+                               int d, const void *gain, float *x, void *xg, float *ssq, int32_t *status, int keep, cudaStream_t st)
+{
+    LaunchCfg lc(n, 256, 0, st);
+    return cudaLaunchKernelEx(&lc.cfg, chain_embed_kernel, tokens, n, P, vocab, hd, inv_freq, tb, (const __nv_bfloat16 *)E, d,
+                              (const __nv_bfloat16 *)gain, x, (__nv_bfloat16 *)xg, ssq, status, keep);
+}
+
 // ------------------------------------------------------------------------------------------
 // RMSNorm of the fp32 residual stream into the GEMM input dtype. One block per node; the row is
 // read once with 16-byte loads and kept in registers between the reduction and the scaling

@@ -9,7 +9,7 @@ from oracle import oracle as orc
 from paper_2309_04255_b200 import binding as B
 from paper_2309_04255_b200 import inputs as gen
 
-from gpu_util import F32_TOL, Twin, argmax_agrees_where_decided, check_acceptance_against_oracle, logits_close
+from gpu_util import BF16_TOL, F32_TOL, Twin, argmax_agrees_where_decided, check_acceptance_against_oracle, logits_close
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -97,3 +97,43 @@ def test_gemm_on_cta_pairs(n_out, n_in, n):
     assert v.last_status() == 0
     ref = x.double() @ w.double().t()
     assert (y.double() - ref).abs().max() <= 2e-6 * n_in ** 0.5 * ref.abs().max()
+
+
+PROMPT_CFG = gen.ModelConfig("prompt", 2, 512, 4, 128, 1408, 1000, "bf16")
+
+
+@pytest.mark.parametrize("cuts", [[129], [200], [255], [256], [257], [300, 140], [64, 191], [400]])
+def test_prompt_chunks_of_up_to_256_tokens(cuts):
+    """Prompts whose chunks are wider than a tree (129..256 tokens on CTA pairs, two row blocks in the attention kernel),
+    in one or two calls that start at odd cache positions, against sequential decoding: the logits of the last token
+    within the bf16 bound of the repository (2e-2 of the largest; rows of earlier chunks are read back rounded), cache
+    rows within a bf16 rounding step plus that bound, a second run bit for bit."""
+    total = sum(cuts)
+    twin = Twin(PROMPT_CFG, total + 8, scale=3.0)
+    tokens = gen.gen_prefix_tokens(PROMPT_CFG, total, seed=total)
+    dec = orc.SequentialDecoder(PROMPT_CFG, twin.glob, [twin.layer(l) for l in range(2)], total + 1)
+    for t in tokens:
+        ref = dec.step(int(t))
+    runs = []
+    for _ in range(2):
+        twin.v.kv_view().zero_()
+        done = 0
+        for m in cuts:
+            lg = twin.v.prefill(done, dev_i32(tokens[done:done + m]), want_logits=True)
+            assert twin.v.last_status() == 0
+            done += m
+        runs.append((lg.clone(), twin.v.kv_view().clone()))
+    assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])
+    logits_close(runs[0][0].cpu().numpy(), ref, BF16_TOL)
+    rows = runs[0][1][:, :, :, :total].double().cpu().numpy()
+    for l in range(2):
+        for got, want in zip(rows[l], dec.cache_heads(l, total)):
+            assert np.abs(got - want).max() <= (2.0 ** -8 + BF16_TOL) * np.abs(want).max()
+
+
+def test_prompt_with_a_bad_token_in_a_wide_chunk():
+    twin = Twin(PROMPT_CFG, 300)
+    tokens = gen.gen_prefix_tokens(PROMPT_CFG, 250, seed=1)
+    tokens[200] = PROMPT_CFG.vocab
+    twin.v.prefill(0, dev_i32(tokens))
+    assert twin.v.last_status() == B.ERR_BAD_TOKEN
