@@ -283,12 +283,36 @@ struct Cursor {
     }
 };
 
-// Floats of one segment slot of the workspace: [4 row groups][n_pad nodes][32 rows].
+// Floats of one segment slot of the workspace: [4 row groups][n_pad / 4 node groups][32 rows][4 nodes], so that the
+// dumping warps (thread = row) store four nodes at once: with one node per store the last segment of a CTA took 4-5 us
+// to leave at 128-256 nodes, four times as many instructions.
 __host__ __device__ __forceinline__ size_t slot_floats(int n_pad) { return (size_t)n_pad * kTileM; }
 
 // ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void dump4(float *dst, const float *v) { *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]); }
+
 // Finishing (the work of gemm_finish_kernel). Every streaming CTA that holds items of a tile has left
-// its accumulators in the workspace as [row group][node][32 rows] fp32 (a "segment").
+// its accumulators in the workspace as [row group][node group][32 rows][4 nodes] fp32 (a "segment").
+// A warp reads a node group with lane = row; turned so that a lane has four rows of one node (below):
+// four rounds of shuffles, in which lane L = 4r + k sends the value of node k - s in round s.
+__device__ __forceinline__ float4 rotate4(float4 v, int by)       // component j of the result = component (j - by) mod 4
+{
+    if (by & 1) v = make_float4(v.w, v.x, v.y, v.z);
+    if (by & 2) v = make_float4(v.z, v.w, v.x, v.y);
+    return v;
+}
+__device__ __forceinline__ float4 rows_of_node(float4 v, int lane)
+{
+    const int ns = lane >> 3, from = 4 * (lane & 7);
+    const float4 r = rotate4(make_float4(v.x, v.w, v.z, v.y), lane & 3);
+    float4 g;
+    g.x = __shfl_sync(0xffffffffu, r.x, from + (ns & 3));
+    g.y = __shfl_sync(0xffffffffu, r.y, from + ((ns + 1) & 3));
+    g.z = __shfl_sync(0xffffffffu, r.z, from + ((ns + 2) & 3));
+    g.w = __shfl_sync(0xffffffffu, r.w, from + ((ns + 3) & 3));
+    return rotate4(g, ns);
+}
+
 __device__ __forceinline__ uint2 pack4_bf16(const __nv_bfloat16 (&h)[4])
 {
     uint2 r;
@@ -330,7 +354,7 @@ struct FinishArgs {
 // tile, in CTA order (so the result does not depend on timing), and apply the fused epilogue. What
 // this costs is the length of its dependent chain, round trips to L2 and plain instruction latency,
 // not bytes. Hence: lane = (node sub-index ns = lane / 8, row quad r4 = lane % 8), iteration `it`
-// handles the four output rows 4 * r4 .. + 3 of node 4 * it + ns, everything moves as 16- or 8-byte
+// handles the four output rows 4 * r4 .. + 3 of node 4 * it + ns (after rows_of_node), everything moves as 16- or 8-byte
 // vectors, a rotary pair sits in one thread; the iterations of a group are dealt out to several
 // warps of the grid (it_first, it_step); G node groups travel together and kB segments of each are
 // loaded at a time, all loads issued before the first use. With `dry` nothing is stored: the
@@ -373,10 +397,25 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
     // what a node's epilogue reads besides the shares: the residual (EPI_RESID) or the rotary
     // (cos, sin) of the lane's two pairs (EPI_QKV, q and k sections)
     const float *aux = nullptr;
-    size_t aux_stride = 0;
-    if (rows_ok && resid) { aux = ep.x + row0; aux_stride = (size_t)n_out; }
-    if (rows_ok && mode == EPI_QKV && sec < 2) { aux = reinterpret_cast<const float *>(ep.rope_cs) + 2 * (e >> 1); aux_stride = (size_t)ep.hd; }
+    int aux_stride = 0;
+    if (rows_ok && resid) { aux = ep.x + row0; aux_stride = n_out; }
+    if (rows_ok && mode == EPI_QKV && sec < 2) { aux = reinterpret_cast<const float *>(ep.rope_cs) + 2 * (e >> 1); aux_stride = ep.hd; }
     const float4 aux_none = resid ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(1.f, 0.f, 1.f, 0.f);
+    // where a node's outputs go in the activation format: hi and lo plane, the same stride per node. Queries get a lo
+    // plane; keys and values go to the cache rounded, their remainders to kv_lo.
+    T *hi_at = nullptr, *lo_at = nullptr;
+    int out_stride = n_out;
+    if (resid && has_xg) hi_at = reinterpret_cast<T *>(ep.xg_out) + row0;
+    else if (mode == EPI_SWIGLU) hi_at = reinterpret_cast<T *>(ep.h) + row0;
+    else if (mode == EPI_QKV && sec == 0) { hi_at = reinterpret_cast<T *>(ep.q_out) + cidx; out_stride = ep.d; }
+    if (hi_at != nullptr) lo_at = hi_at + (size_t)kLoRows * out_stride;
+    if (mode == EPI_QKV && sec > 0) {
+        out_stride = ep.hd;
+        hi_at = reinterpret_cast<T *>(sec == 1 ? ep.k_cache : ep.v_cache) + ((size_t)head * ep.S + ep.P) * ep.hd + e;
+        lo_at = reinterpret_cast<T *>(ep.kv_lo) + (size_t)((sec - 1) * (ep.d / ep.hd) + head) * kLoRows * ep.hd + e;
+    }
+    if (!comp) lo_at = nullptr;
+    const bool y_vec = mode == EPI_PLAIN && rows_ok && (ep.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(ep.y) & 15) == 0;
 
     const int iters = n_pad >> 2;
     for (int itg = fa.it_first; itg < iters; itg += G * fa.it_step) {
@@ -395,13 +434,13 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
             for (int k = 0; k < kB; ++k) {
                 // (no load for a holder that does not exist: at many nodes the segments' bytes are what this costs)
                 const bool has = k0 + k < fa.a.n, has_u = dual && k0 + k < fa.b.n;
-                const float *sk = share_ptr(p, d, fa.a.first + k0 + k, va, lane_grp) + 4 * r4;
-                const float *su = dual ? share_ptr(p, d, fa.b.first + k0 + k, va + 1, lane_grp) + 4 * r4 : nullptr;
+                const float *sk = share_ptr(p, d, fa.a.first + k0 + k, va, lane_grp) + 4 * lane;
+                const float *su = dual ? share_ptr(p, d, fa.b.first + k0 + k, va + 1, lane_grp) + 4 * lane : nullptr;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    const int node = min(itg + g * fa.it_step, iters - 1) * 4 + ns;
-                    t[g][k] = has ? __ldcg(reinterpret_cast<const float4 *>(sk + (size_t)node * 32)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (dual) u[g][k] = has_u ? __ldcg(reinterpret_cast<const float4 *>(su + (size_t)node * 32)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const int it = min(itg + g * fa.it_step, iters - 1);
+                    t[g][k] = has ? __ldcg(reinterpret_cast<const float4 *>(sk + (size_t)it * 128)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (dual) u[g][k] = has_u ? __ldcg(reinterpret_cast<const float4 *>(su + (size_t)it * 128)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
 #pragma unroll
@@ -414,74 +453,56 @@ __device__ __forceinline__ void finish_rows_t(const FinishArgs &fa, int lane, co
                 }
             }
         }
-        // two at a time, unrolled, so that the two dependent chains overlap
-        for (int g2 = 0; g2 < G; g2 += 2) {
 #pragma unroll
-        for (int gq = 0; gq < (G < 2 ? G : 2); ++gq) {
-        const int g = g2 + gq;
-        const int it = itg + g * fa.it_step;
-        if (it >= iters) continue;
-        const int node = it * 4 + ns;
-        const bool ok = rows_ok && node < n_nodes;
-        float4 ax = axs[0], a = as[0], b = bs[0];
+        for (int g = 0; g < G; ++g) {
+            const int it = itg + g * fa.it_step;
+            if (it >= iters) break;
+            const int node = it * 4 + ns;
+            const bool ok = rows_ok && node < n_nodes;
+            const float4 ax = axs[g], a = rows_of_node(as[g], lane);
+            float4 b;
+            if (dual) b = rows_of_node(bs[g], lane);
+            const float r = has_rs ? fa.rs[node] : 1.f;
+            const float v[4] = {a.x * r, a.y * r, a.z * r, a.w * r};
+            float out[4];                 // what goes out in the activation format (hi and lo plane)
+            if (resid) {
+                const float xo[4] = {ok ? ax.x + v[0] : 0.f, ok ? ax.y + v[1] : 0.f, ok ? ax.z + v[2] : 0.f, ok ? ax.w + v[3] : 0.f};
+                if (ok && !dry) *reinterpret_cast<float4 *>(ep.x + (size_t)node * n_out + row0) = make_float4(xo[0], xo[1], xo[2], xo[3]);
 #pragma unroll
-        for (int q = 1; q < G; ++q) if (q == g) { ax = axs[q]; a = as[q]; b = bs[q]; }
-        const float r = has_rs ? fa.rs[node] : 1.f;
-        float v[4] = {a.x * r, a.y * r, a.z * r, a.w * r};
-        float out[4];                 // what goes out in the activation format (hi and lo plane)
-        T *dst = nullptr, *dst_lo = nullptr;
-        if (resid) {
-            const float xo[4] = {ok ? ax.x + v[0] : 0.f, ok ? ax.y + v[1] : 0.f, ok ? ax.z + v[2] : 0.f, ok ? ax.w + v[3] : 0.f};
-            if (ok && !dry) *reinterpret_cast<float4 *>(ep.x + (size_t)node * n_out + row0) = make_float4(xo[0], xo[1], xo[2], xo[3]);
+                for (int k = 0; k < 4; ++k) out[k] = xo[k] * gain[k];
+                if (has_xg) {
+                    // what the next RMSNorm needs: gain * x in the GEMM input format, and this row
+                    // group's share of every node's sum of squares
+                    float ss = xo[0] * xo[0] + xo[1] * xo[1] + xo[2] * xo[2] + xo[3] * xo[3];
+                    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+                    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+                    ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+                    if (r4 == 0 && !dry) ep.ssq_out[(size_t)(tile * 4 + lane_grp) * kLoRows + node] = ss;
+                }
+            } else if (mode == EPI_SWIGLU) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) out[k] = xo[k] * gain[k];
-            if (has_xg) {
-                // what the next RMSNorm needs: gain * x in the GEMM input format, and this row
-                // group's share of every node's sum of squares
-                dst = reinterpret_cast<T *>(ep.xg_out) + (size_t)node * n_out + row0;
-                dst_lo = dst + (size_t)kLoRows * n_out;
-                float ss = xo[0] * xo[0] + xo[1] * xo[1] + xo[2] * xo[2] + xo[3] * xo[3];
-                ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-                ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-                ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-                if (r4 == 0 && !dry) ep.ssq_out[(size_t)(tile * 4 + lane_grp) * kLoRows + node] = ss;
+                for (int k = 0; k < 4; ++k) out[k] = v[k] / (1.0f + __expf(-v[k]));
+                out[0] *= b.x * r; out[1] *= b.y * r; out[2] *= b.z * r; out[3] *= b.w * r;
+            } else if (mode == EPI_QKV) {
+                // rotary pairs (2t, 2t+1) = (v0, v1), (v2, v3); values pass through with (cos, sin) = (1, 0)
+                out[0] = v[0] * ax.x - v[1] * ax.y; out[1] = v[0] * ax.y + v[1] * ax.x;
+                out[2] = v[2] * ax.z - v[3] * ax.w; out[3] = v[2] * ax.w + v[3] * ax.z;
+            } else if (node < n_nodes && !dry) {
+                float *yr = ep.y + (size_t)node * ep.ldy + row0;
+                if (y_vec) *reinterpret_cast<float4 *>(yr) = make_float4(v[0], v[1], v[2], v[3]);
+                else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k < n_valid) yr[k] = v[k];
+                }
             }
-        } else if (mode == EPI_SWIGLU) {
+            if (mode != EPI_PLAIN && hi_at != nullptr && ok && !dry) {
+                T hi[4], lo[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) out[k] = v[k] / (1.0f + __expf(-v[k]));
-            out[0] *= b.x * r; out[1] *= b.y * r; out[2] *= b.z * r; out[3] *= b.w * r;
-            dst = reinterpret_cast<T *>(ep.h) + (size_t)node * n_out + row0;
-            dst_lo = dst + (size_t)kLoRows * n_out;
-        } else if (mode == EPI_QKV) {
-            // rotary pairs (2t, 2t+1) = (v0, v1), (v2, v3); values pass through with (cos, sin) = (1, 0)
-            out[0] = v[0] * ax.x - v[1] * ax.y; out[1] = v[0] * ax.y + v[1] * ax.x;
-            out[2] = v[2] * ax.z - v[3] * ax.w; out[3] = v[2] * ax.w + v[3] * ax.z;
-            // queries get a lo plane; keys and values go to the cache rounded, their remainders to kv_lo
-            if (sec == 0) {
-                dst = reinterpret_cast<T *>(ep.q_out) + (size_t)node * ep.d + cidx;
-                dst_lo = dst + (size_t)kLoRows * ep.d;
-            } else {
-                dst = reinterpret_cast<T *>(sec == 1 ? ep.k_cache : ep.v_cache) + ((size_t)head * ep.S + ep.P + node) * ep.hd + e;
-                dst_lo = reinterpret_cast<T *>(ep.kv_lo) + ((size_t)((sec - 1) * (ep.d / ep.hd) + head) * kLoRows + node) * ep.hd + e;
+                for (int k = 0; k < 4; ++k) split_bf16(out[k], hi[k], lo[k]);
+                *reinterpret_cast<uint2 *>(hi_at + (size_t)node * out_stride) = pack4_bf16(hi);
+                if (lo_at != nullptr) *reinterpret_cast<uint2 *>(lo_at + (size_t)node * out_stride) = pack4_bf16(lo);
             }
-        } else if (node < n_nodes && !dry) {
-            float *yr = ep.y + (size_t)node * ep.ldy + row0;
-            if (rows_ok && (ep.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(ep.y) & 15) == 0)
-                *reinterpret_cast<float4 *>(yr) = make_float4(v[0], v[1], v[2], v[3]);
-            else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (k < n_valid) yr[k] = v[k];
-            }
-        }
-        if (dst != nullptr && ok && !dry) {
-            T hi[4], lo[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) split_bf16(out[k], hi[k], lo[k]);
-            *reinterpret_cast<uint2 *>(dst) = pack4_bf16(hi);
-            if (comp) *reinterpret_cast<uint2 *>(dst_lo) = pack4_bf16(lo);
-        }
-        }
         }
     }
 }
@@ -694,7 +715,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
             // with hi + lo activations a node's two accumulator columns are added first
             const uint32_t t_lane = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + buf * acc_cols;
             if (!LLMCAD_CHECK(tile >= 0 && tile < d.n_tiles * d.halves && tile + (int)blockIdx.x < d.n_tiles * d.halves + d.grid, p.status)) { timed_out = true; break; }
-            float *dst = p.partials + (size_t)(tile + (int)blockIdx.x) * slot_stride + (size_t)lane_grp * p.n_pad * 32 + lane;
+            float *dst = p.partials + (size_t)(tile + (int)blockIdx.x) * slot_stride + (size_t)lane_grp * p.n_pad * 32 + 4 * lane;
             int c0 = 0;
             if (p.comp) {
                 // 32 nodes at a time, hi and lo columns in one round trip
@@ -702,7 +723,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                     float v[32];
                     tc_ld32_sum2(t_lane + c0, t_lane + p.n_pad + c0, v);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) dst[(size_t)(c0 + j) * 32] = v[j];
+                    for (int j = 0; j < 32; j += 4) dump4(dst + (size_t)(c0 + j) * 32, v + j);
                 }
             }
             for (; c0 < p.n_pad; c0 += 16) {
@@ -715,7 +736,7 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                     for (int j = 0; j < 16; ++j) v[j] += t[j];
                 }
 #pragma unroll
-                for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * 32] = v[j];
+                for (int j = 0; j < 16; j += 4) dump4(dst + (size_t)(c0 + j) * 32, v + j);
             }
             // the accumulator has left TMEM: hand the buffer back to the MMA warp
             tc_fence_before();
@@ -986,14 +1007,14 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
             const uint32_t t_lane = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + buf * nb;
             if (v < n_vtiles) {
                 if (!LLMCAD_CHECK(v >= 0 && v + 2 * group < n_vtiles + d.grid, p.status)) { timed_out = true; break; }
-                float *dst = p.partials + (size_t)(v + 2 * group) * slot_stride + (size_t)lane_grp * p.n_pad * 32 + lane;
+                float *dst = p.partials + (size_t)(v + 2 * group) * slot_stride + (size_t)lane_grp * p.n_pad * 32 + 4 * lane;
                 int c0 = 0;
                 for (; c0 + 32 <= p.n_pad; c0 += 32) {
                     float t[32];
                     if (p.comp && !kWide) tc_ld32_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
                     else tc_ld32(t_lane + c0, t);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) dst[(size_t)(c0 + j) * 32] = t[j];
+                    for (int j = 0; j < 32; j += 4) dump4(dst + (size_t)(c0 + j) * 32, t + j);
                 }
                 for (; c0 < p.n_pad; c0 += 16) {
                     float t[16];
@@ -1005,7 +1026,7 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
                         for (int j = 0; j < 16; ++j) t[j] += u[j];
                     }
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * 32] = t[j];
+                    for (int j = 0; j < 16; j += 4) dump4(dst + (size_t)(c0 + j) * 32, t + j);
                 }
             }
             tc_fence_before();
@@ -1372,14 +1393,14 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
             tc_fence_after();
             if (v < n_vtiles) {
                 if (!LLMCAD_CHECK(v >= 0 && v + d.group * group < n_vtiles + d.grid, p.status)) { timed_out = true; break; }
-                float *dst = p.partials + (size_t)(v + d.group * group) * slot_floats(p.n_pad) + (size_t)quad * p.n_pad * 32 + lane;
+                float *dst = p.partials + (size_t)(v + d.group * group) * slot_floats(p.n_pad) + (size_t)quad * p.n_pad * 32 + 4 * lane;
                 const uint32_t t_lane = tmem_base + t_quad + buf * nb;
                 for (int c0 = 16 * set; c0 < p.n_pad; c0 += 16 * kW4Sets) {
                     float t[16];
                     if (p.comp) tc_ld16_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
                     else tc_ld16(t_lane + c0, t);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * 32] = t[j];
+                    for (int j = 0; j < 16; j += 4) dump4(dst + (size_t)(c0 + j) * 32, t + j);
                 }
             }
             tc_fence_before();

@@ -41,7 +41,7 @@ struct GemmParams {
     int astages;        // INT4 weights: depth of the ring of activation items (with bf16 weights they share the weights' stages)
     int acc_bufs;       // INT4 weights: accumulator buffers (always two with bf16 weights)
     int tmem_cols;      // allocated TMEM columns (power of two)
-    float *partials;    // segment slots [weight tiles + grid][4 row groups][n_pad][32 rows] fp32: the segment of
+    float *partials;    // segment slots [weight tiles + grid][4 row groups][n_pad / 4][32 rows][4 nodes] fp32: the segment of
                         // weight tile v held by CTA c sits in slot v + c
     int32_t *status;
     unsigned long long *trace;  // optional [256][16] timeline in ns of this GEMM (nullptr: off)
