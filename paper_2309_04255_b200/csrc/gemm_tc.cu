@@ -1110,6 +1110,22 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
           "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
+// 32 codes of a row, two to a bf16 pair, into 16 columns of this thread's TMEM lane
+__device__ __forceinline__ void expand_store(const uint4 &c, uint32_t s2, uint32_t b2, uint32_t taddr)
+{
+    const uint32_t ww[4] = {c.x, c.y, c.z, c.w};
+    uint32_t o[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t t2 = ((ww[q] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
+            const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2), *reinterpret_cast<const __nv_bfloat162 *>(&s2),
+                                             *reinterpret_cast<const __nv_bfloat162 *>(&b2));
+            o[q * 4 + j] = *reinterpret_cast<const uint32_t *>(&r);
+        }
+    tc_st16(taddr, o);
+}
 // 16 columns at each of two addresses, summed (one wait for both loads)
 __device__ __forceinline__ void tc_ld16_sum2(uint32_t taddr_a, uint32_t taddr_b, float *v)
 {
@@ -1334,34 +1350,26 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                 if (!ready && !(mbar_wait_all(smem_u32(&ctl.pfull[pk.slot]), pk.par, abort_flag, wait_limit) &&
                                 mbar_wait_all(smem_u32(&ctl.xempty[x.slot]), x.par, abort_flag, wait_limit))) { timed_out = true; break; }
                 tc_fence_after();
-                // A row's 64 codes of a k-block are two 16-byte words, [half][row], its exponent follows them. The loop over
-                // the halves is not unrolled: the expanding warps share their scheduler's instruction cache with the MMA
-                // warp, and with 400 instructions here that warp's 60 were fetched anew for every item.
-                const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes;
+                // A row's 64 codes of a k-block are two 16-byte words, [half][row], its exponent follows them. A set takes every
+                // other k-block; the words of its next one are loaded while it works on this one. The loop is not unrolled:
+                // the expanding warps share their scheduler's instruction cache with the MMA warp, and with 400 instructions
+                // here that warp's 60 were fetched anew for every item.
+                const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes + set * kW4TileBytes;
                 const uint32_t dst = x_base + t_quad + x.slot * (SK * 32);
-                auto codes_of = [&](int h) { return *reinterpret_cast<const uint4 *>(src + (h >> 1) * kW4TileBytes + (h & 1) * 2048 + row * 16); };
-                const int halves = 2 * w.nk;
-                uint4 codes = codes_of(min(set, halves - 1));
+                uint4 c0 = *reinterpret_cast<const uint4 *>(src + row * 16), c1 = *reinterpret_cast<const uint4 *>(src + 2048 + row * 16);
+                int e = reinterpret_cast<const int8_t *>(src + 4096)[row];
 #pragma unroll 1
-                for (int h = set; h < halves; h += kW4Sets) {
-                    const int e = reinterpret_cast<const int8_t *>(src + (h >> 1) * kW4TileBytes + 4096)[row];
-                    const uint4 cur = codes;
-                    codes = codes_of(min(h + kW4Sets, halves - 1));
+                for (int k = set; k < w.nk; k += kW4Sets) {
                     // OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact. The bf16 bits
                     // of 2^e are (e + 127) << 7, those of -136 * 2^e are that + 0x8388.
                     const uint32_t s2 = (uint32_t)(e + 127) * 0x00800080u, b2 = s2 + 0x83888388u;
-                    const uint32_t ww[4] = {cur.x, cur.y, cur.z, cur.w};
-                    uint32_t o[16];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint32_t t2 = ((ww[q] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
-                            const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2), *reinterpret_cast<const __nv_bfloat162 *>(&s2),
-                                                             *reinterpret_cast<const __nv_bfloat162 *>(&b2));
-                            o[q * 4 + j] = *reinterpret_cast<const uint32_t *>(&r);
-                        }
-                    tc_st16(dst + h * 16, o);
+                    const uint4 h0 = c0, h1 = c1;
+                    if (k + kW4Sets < w.nk) src += kW4Sets * kW4TileBytes;
+                    c0 = *reinterpret_cast<const uint4 *>(src + row * 16);
+                    c1 = *reinterpret_cast<const uint4 *>(src + 2048 + row * 16);
+                    e = reinterpret_cast<const int8_t *>(src + 4096)[row];
+                    expand_store(h0, s2, b2, dst + k * 32);
+                    expand_store(h1, s2, b2, dst + k * 32 + 16);
                 }
                 // The packed slot is given back only here, where every word has gone through the arithmetic above: given back
                 // right after the loads it was refilled before cold code (an instruction fetch of half a microsecond at the
