@@ -1110,8 +1110,11 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
           "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
-// 32 codes of a row, two to a bf16 pair, into 16 columns of this thread's TMEM lane
-__device__ __forceinline__ void expand_store(const uint4 &c, uint32_t s2, uint32_t b2, uint32_t taddr)
+// 32 codes of a row, two to a bf16 pair, into 16 columns of this thread's TMEM lane: nibble j of each half of a word by a
+// shift, one (a & b) | c and one fused multiply-add. Shifts and logic run at half the issue rate and pace the kernel, so
+// there must be no more of them: from the plain expression the compiler made an AND and an OR, and with `nibbles` and
+// `magic` as constants it knows it is slower than with values in registers (cycles for two k-blocks: 1028 plain, 885, 839).
+__device__ __forceinline__ void expand_store(const uint4 &c, uint32_t nibbles, uint32_t magic, uint32_t s2, uint32_t b2, uint32_t taddr)
 {
     const uint32_t ww[4] = {c.x, c.y, c.z, c.w};
     uint32_t o[16];
@@ -1119,10 +1122,9 @@ __device__ __forceinline__ void expand_store(const uint4 &c, uint32_t s2, uint32
     for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint32_t t2 = ((ww[q] >> (4 * j)) & 0x000f000fu) | 0x43004300u;
-            const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&t2), *reinterpret_cast<const __nv_bfloat162 *>(&s2),
-                                             *reinterpret_cast<const __nv_bfloat162 *>(&b2));
-            o[q * 4 + j] = *reinterpret_cast<const uint32_t *>(&r);
+            uint32_t t2;
+            asm("lop3.b32 %0, %1, %2, %3, 0xea;" : "=r"(t2) : "r"(ww[q] >> (4 * j)), "r"(nibbles), "r"(magic));
+            asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(o[q * 4 + j]) : "r"(t2), "r"(s2), "r"(b2));
         }
     tc_st16(taddr, o);
 }
@@ -1334,6 +1336,8 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
     } else if (warp >= 4) {
         // ================================================= expansion and dump
         const int quad = warp & 3, set = (warp - 4) >> 2, row = quad * 32 + lane;
+        const uint32_t zero = (uint32_t)p.n_pad >> 24;        // (as the compiler cannot know)
+        const uint32_t nibbles = 0x000f000fu | zero, magic = 0x43004300u | zero;
         const uint32_t t_quad = (uint32_t)(quad * 32) << 16;
         RingPos pk{0, 0}, x{0, 1};
         W4Walk<PK> w;                              // the items to expand
@@ -1368,8 +1372,8 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                     c0 = *reinterpret_cast<const uint4 *>(src + row * 16);
                     c1 = *reinterpret_cast<const uint4 *>(src + 2048 + row * 16);
                     e = reinterpret_cast<const int8_t *>(src + 4096)[row];
-                    expand_store(h0, s2, b2, dst + k * 32);
-                    expand_store(h1, s2, b2, dst + k * 32 + 16);
+                    expand_store(h0, nibbles, magic, s2, b2, dst + k * 32);
+                    expand_store(h1, nibbles, magic, s2, b2, dst + k * 32 + 16);
                 }
                 // The packed slot is given back only here, where every word has gone through the arithmetic above: given back
                 // right after the loads it was refilled before cold code (an instruction fetch of half a microsecond at the
