@@ -1128,6 +1128,18 @@ __device__ __forceinline__ void expand_store(const uint4 &c, uint32_t nibbles, u
         }
     tc_st16(taddr, o);
 }
+__device__ __forceinline__ uint4 lds128(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ int lds_s8(uint32_t addr)
+{
+    int v;
+    asm volatile("ld.shared.s8 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
 // 16 columns at each of two addresses, summed (one wait for both loads)
 __device__ __forceinline__ void tc_ld16_sum2(uint32_t taddr_a, uint32_t taddr_b, float *v)
 {
@@ -1181,6 +1193,35 @@ struct W4Walk {
         i += n_items;
         if (i == (unit + 1) * ppt) ++unit;
         load();
+    }
+};
+
+// The same steps for the warps that only need to know how many k-blocks a step has: one subtraction per step.
+template <int PK>
+struct W4Count {
+    int i, end, ppt, kbpt, unit;
+    int left;               // k-blocks from the current step to the end of its segment; 0: no step left
+    __device__ void init(int begin, int e, int p, int k)
+    {
+        i = begin; end = e; ppt = p; kbpt = k;
+        unit = begin / p;
+        left = 0;
+        segment();
+    }
+    __device__ void segment()
+    {
+        if (i >= end) return;
+        const int at = i - unit * ppt, n = min(end - i, ppt - at);
+        left = min(n * PK, kbpt - at * PK);
+        i += n;
+        ++unit;
+    }
+    __device__ bool done() const { return left == 0; }
+    __device__ int nk() const { return min(2 * PK, left); }
+    __device__ void next(int nk)
+    {
+        left -= nk;
+        if (left == 0) segment();
     }
 };
 
@@ -1298,7 +1339,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0), xb = tmem + (uint32_t)acc_bufs * nb;
         const bool leader = elect_one();
         RingPos x{0, 0}, a{0, 0};
-        W4Walk<PK> w;
+        W4Count<PK> w;
         w.init(begin, end, ppt, d.kb_per_tile);
         uint32_t seg = 0, acc = 0;
         int buf = 0;
@@ -1315,19 +1356,21 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
             tc_fence_after();
             const uint32_t d0 = tmem + buf * nb, at = xb + x.slot * (SK * 32), empty = smem_u32(&ctl.xempty[x.slot]);
             const uint64_t b_desc = make_smem_desc(act_base + a.slot * astage_bytes);
+            const int nk = w.nk();
+            const bool last = nk == w.left;                  // the item ends its segment
             if (leader) {
 #pragma unroll
                 for (int k = 0; k < SK; ++k) {
-                    if (k >= w.nk) break;
+                    if (k >= nk) break;
 #pragma unroll
                     for (int k4 = 0; k4 < kBlockK / 16; ++k4)
                         tc_mma_ts(d0, at + k * 32 + k4 * 8, b_desc + k * (b_tile_bytes >> 4) + 2 * k4, idesc, k > 0 || k4 > 0 ? 1u : acc);
                 }
                 tc_commit(empty);                            // the expanded item's slot, and with it the activation item's (see the loader)
-                if (w.last) tc_commit(smem_u32(&ctl.tmem_full[buf]));
+                if (last) tc_commit(smem_u32(&ctl.tmem_full[buf]));
             }
-            acc = w.last ? 0 : 1;
-            w.next();
+            acc = last ? 0 : 1;
+            w.next(nk);
             x.step(p.stages);
             a.step(p.astages);
             ready = !w.done() && mbar_test2_all(smem_u32(&ctl.xfull[x.slot]), x.par, smem_u32(&ctl.afull[a.slot]), a.par);
@@ -1340,9 +1383,12 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         const uint32_t nibbles = 0x000f000fu | zero, magic = 0x43004300u | zero;
         const uint32_t t_quad = (uint32_t)(quad * 32) << 16;
         RingPos pk{0, 0}, x{0, 1};
-        W4Walk<PK> w;                              // the items to expand
+        W4Count<PK> w;                             // the items to expand
         w.init(begin, end, ppt, d.kb_per_tile);
         int expanded = 0, dumpable = 0;            // items expanded; items up to and including the ones of the segment to be dumped next
+        // this thread's codes and exponents in packed slot 0, and its set's columns in expanded slot 0
+        const uint32_t row_codes = packed_base + set * kW4TileBytes + row * 16, row_exp = packed_base + set * kW4TileBytes + 4096 + row;
+        const uint32_t x_set = x_base + t_quad + set * 32;
         bool dep_ok = false, ready = false;
         uint32_t seg = 0;
         for (int i = begin; i < end && !timed_out; ++seg) {
@@ -1358,38 +1404,37 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                 // other k-block; the words of its next one are loaded while it works on this one. The loop is not unrolled:
                 // the expanding warps share their scheduler's instruction cache with the MMA warp, and with 400 instructions
                 // here that warp's 60 were fetched anew for every item.
-                const uint8_t *src = smem_raw + (packed_base - smem_u32(smem_raw)) + (size_t)pk.slot * pstage_bytes + set * kW4TileBytes;
-                const uint32_t dst = x_base + t_quad + x.slot * (SK * 32);
-                uint4 c0 = *reinterpret_cast<const uint4 *>(src + row * 16), c1 = *reinterpret_cast<const uint4 *>(src + 2048 + row * 16);
-                int e = reinterpret_cast<const int8_t *>(src + 4096)[row];
+                uint32_t src = row_codes + pk.slot * pstage_bytes, src_e = row_exp + pk.slot * pstage_bytes, dst = x_set + x.slot * (SK * 32);
+                const int nk = w.nk();
+                uint4 c0 = lds128(src), c1 = lds128(src + 2048);
+                int e = lds_s8(src_e);
 #pragma unroll 1
-                for (int k = set; k < w.nk; k += kW4Sets) {
+                for (int k = set; k < nk; k += kW4Sets) {
                     // OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact. The bf16 bits
                     // of 2^e are (e + 127) << 7, those of -136 * 2^e are that + 0x8388.
                     const uint32_t s2 = (uint32_t)(e + 127) * 0x00800080u, b2 = s2 + 0x83888388u;
                     const uint4 h0 = c0, h1 = c1;
-                    if (k + kW4Sets < w.nk) src += kW4Sets * kW4TileBytes;
-                    c0 = *reinterpret_cast<const uint4 *>(src + row * 16);
-                    c1 = *reinterpret_cast<const uint4 *>(src + 2048 + row * 16);
-                    e = reinterpret_cast<const int8_t *>(src + 4096)[row];
-                    expand_store(h0, nibbles, magic, s2, b2, dst + k * 32);
-                    expand_store(h1, nibbles, magic, s2, b2, dst + k * 32 + 16);
+                    if (k + kW4Sets < nk) { src += kW4Sets * kW4TileBytes; src_e += kW4Sets * kW4TileBytes; }
+                    c0 = lds128(src);
+                    c1 = lds128(src + 2048);
+                    e = lds_s8(src_e);
+                    expand_store(h0, nibbles, magic, s2, b2, dst);
+                    expand_store(h1, nibbles, magic, s2, b2, dst + 16);
+                    dst += kW4Sets * 32;
                 }
-                // The packed slot is given back only here, where every word has gone through the arithmetic above: given back
-                // right after the loads it was refilled before cold code (an instruction fetch of half a microsecond at the
-                // start of the kernel) had got to them.
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ctl.pempty[pk.slot]));
-                const uint32_t xfull = smem_u32(&ctl.xfull[x.slot]);
+                const uint32_t xfull = smem_u32(&ctl.xfull[x.slot]), pempty = smem_u32(&ctl.pempty[pk.slot]);
                 ++expanded;
-                w.next();
+                w.next(nk);
                 pk.step(p.pstages);
                 x.step(p.stages);
                 ready = !w.done() && mbar_test2_all(smem_u32(&ctl.pfull[pk.slot]), pk.par, smem_u32(&ctl.xempty[x.slot]), x.par);
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(xfull);
+                // The packed slot, too, is given back only here, where every word has gone through the arithmetic above: given
+                // back right after the loads it was refilled before cold code (an instruction fetch of half a microsecond at
+                // the start of the kernel) had got to them.
+                if (lane == 0) { mbar_arrive(xfull); mbar_arrive(pempty); }
             }
             if (timed_out) break;
             // ---- dump
