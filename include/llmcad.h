@@ -249,11 +249,12 @@ int llmcad_skinny_gemm_tiled(llmcad_ctx *ctx, const void *w_tiled, const void *x
  * weights is the bf16 pass over the dequantised weights, bit for bit, at a quarter of the weight bytes.
  * A context created with LLMCAD_FLAG_INT4_WEIGHTS (bf16, d_model and d_ffn multiples of 64) quantises
  * the layer matrices inside llmcad_pack_layer and streams them as INT4 tiles, which the GEMM kernel
- * expands to bf16 tiles in shared memory; embedding and lm_head stay bf16.
+ * expands to bf16 in tensor memory; embedding and lm_head stay bf16.
  * llmcad_quantize_int4: codes and exponents of a row-major bf16 matrix [n_out][n_in] (DEVICE), n_in a
  * multiple of 64, as plain arrays q [n_out][n_in] and e [n_out][n_in / 64] (DEVICE int8).
  * llmcad_tile_weight_int4 / llmcad_tiled_weight_int4_bytes: the same quantisation in the layout the GEMM
- * streams (4224 bytes per tile of 128 rows and 64 columns: 128 x 8 words of eight codes, 128 exponents).
+ * streams (4224 bytes per tile of 128 rows and 64 columns: two halves of 32 columns, each 128 rows of 16 bytes of
+ * codes, then 128 exponents).
  * llmcad_skinny_gemm_tiled_int4: llmcad_skinny_gemm on a matrix in that layout (bf16 contexts only). */
 int llmcad_quantize_int4(const void *w, int32_t n_out, int32_t n_in, int8_t *q, int8_t *e, void *stream);
 size_t llmcad_tiled_weight_int4_bytes(int32_t n_out, int32_t n_in);

@@ -1057,25 +1057,23 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
 // ------------------------------------------------------------------------------------------------
 // The streaming kernel for INT4 weights.
 //
-// A quarter of the bytes, so HBM no longer sets the pace: expanding the weights and the MMAs do (a
-// tcgen05.mma of K = 16 takes ~48 cycles for up to 64 columns, 17 us per layer of the 7B shape, about what its
-// packed weights take from HBM). The weights are therefore expanded straight into tensor memory and multiplied
-// from there: thread = weight row = TMEM lane, eight codes of a word become four packed bf16 pairs (three
-// instructions a pair), 32 of which are the row's share of a k-block. The previous form wrote the expanded tiles
-// to shared memory, with four warps that also dumped the accumulators, and slots were handed around at 0.5 us an
-// item (7B shape, 32 nodes: 3.53 ms a pass).
+// A quarter of the bytes, so HBM no longer sets the pace: expanding the weights does (~1100 cycles per item of four
+// k-blocks, against ~770 for its MMAs at 64 columns, ~48 cycles each for K = 16, and ~650 for its bytes). The weights
+// are expanded straight into tensor memory and multiplied from there: thread = weight row = TMEM lane, eight codes of a
+// word become four packed bf16 pairs, 32 of which are the row's share of a k-block. (Expanded into shared memory, by
+// the warps that also dumped the accumulators, a pass of the 7B shape with 32 nodes took 3.53 ms; now 2.33 ms.)
 //
-// What paces it is the MMA warp: ~520 cycles per ring item for its barriers, fences and addresses beside the MMAs
-// themselves. An item here is therefore two of the items that the kernels for bf16 weights move, 2 PK k-blocks, as
-// far as the segment reaches.
+// What an item costs beside its arithmetic, its barriers, fences and addresses, is worth as much attention: ~520
+// cycles in the MMA warp, ~290 in each expanding warp. An item here is therefore two of the items that the kernels for
+// bf16 weights move, 2 PK k-blocks, as far as the segment reaches.
 //
 // Warps: 0 producer of packed items (bulk copies), 1 TMEM allocator and MMA issuer, 2 activation loader (TMA),
-// 4..15 expansion and dump: warp w works on rows 32 * (w % 4) .., the three sets of four take every third half of an
-// item's k-blocks, and every third 16-node chunk of a dump (with two sets the expansion, 150 cycles a half and warp
-// most of which is latency, set the pace: 1750 cycles an item against ~770 of MMAs at 64 columns). Three rings of
-// items: packed (shared memory), expanded (tensor memory, what the accumulators leave of the 512 columns), activations
-// (shared memory). Until the grid dependency the packed ring fills and the expanded ring as far as it reaches. 56
-// registers a thread: four warps per scheduler beside the finishing CTA's three of 96.
+// 4..11 expansion and dump: warp w works on rows 32 * (w % 4) .., the two sets of four take alternate k-blocks of an
+// item and alternate 16-node chunks of a dump. More sets do not help (three: 2.58 against 2.48 ms a pass; four, with 40
+// registers a thread: a third slower): the ALU and FMA pipes of the four schedulers are the bound, not latency. Three
+// rings of items: packed (shared memory), expanded (tensor memory, what the accumulators leave of the 512 columns),
+// activations (shared memory). Until the grid dependency the packed ring fills and the expanded ring as far as it
+// reaches. At most 72 registers a thread: three warps per scheduler beside the finishing CTA's three of 96.
 //
 // Work is cut and ordered exactly as the kernels for bf16 weights cut theirs on the same number of nodes (CTA pairs
 // included, which here only means how tiles and ranges are dealt out), so that the sums are the same to the bit.
