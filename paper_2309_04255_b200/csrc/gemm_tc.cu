@@ -607,7 +607,8 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                     t_idle = 0;
                     continue;
                 }
-                __nanosleep(32);
+                // (no sleep between the tries, here and in the activation loader: with 32 ns of it decode passes of the 7B
+                // shape took 2823 instead of 2814 us, 20 layers of the 13B shape with 64 nodes 3437 instead of 3410)
                 if (t_idle == 0) t_idle = global_timer_ns();
                 else if (*abort_flag || global_timer_ns() - t_idle > wait_limit) { timed_out = true; break; }
             }
@@ -631,7 +632,6 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
                 uint64_t t0 = 0;
                 // the stage is ours: the producer has passed its "empty" wait and armed the barrier
                 for (uint32_t spin = 0; (int32_t)(ctl.a_issued - (i + 1)) < 0; ++spin) {
-                    __nanosleep(32);
                     if ((spin & 255u) == 255u) {
                         if (t0 == 0) t0 = global_timer_ns();
                         if (*abort_flag || global_timer_ns() - t0 > wait_limit) { timed_out = true; break; }
