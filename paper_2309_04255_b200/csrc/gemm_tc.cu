@@ -930,7 +930,7 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
             for (int i = begin; i < end && !timed_out; ++i) {
                 uint64_t t0 = 0;
                 for (uint32_t spin = 0; (int32_t)(ctl.a_issued - (uint32_t)(i + 1 - begin)) < 0; ++spin) {
-                    __nanosleep(32);
+                    // (no sleep between the looks: 0.5 % of a pass at 30B widths with 128 nodes)
                     if ((spin & 255u) == 255u) {
                         if (t0 == 0) t0 = global_timer_ns();
                         if (*abort_flag || global_timer_ns() - t0 > wait_limit) { timed_out = true; break; }
