@@ -773,7 +773,7 @@ int llmcad_pack_globals(llmcad_ctx *ctx, const llmcad_global_weights *src, void 
     return LLMCAD_OK;
 }
 
-// path_fill: entries of out->accepted_path behind the path, up to this many in all, become -1
+// path_fill: entries of out->accepted_path behind the path become -1, up to this many in all
 static int verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int32_t prefix_len, const int32_t *tree_tokens,
                        const int32_t *parent_idx, int32_t n, const llmcad_result *out, int path_fill, void *stream)
 {
@@ -822,7 +822,7 @@ int llmcad_verify_tree_host(llmcad_ctx *ctx, const void *packed, void *kv_cache,
     dev.argmax = ctx->argmax_dev();
     dev.accepted_path = ctx->path_dev();
     dev.scalars = ctx->scalars_dev();
-    rc = verify_tree(ctx, packed, kv_cache, prefix_len, ctx->tokens_dev(), ctx->parent_dev(), n, &dev, 0, stream);
+    rc = verify_tree(ctx, packed, kv_cache, prefix_len, ctx->tokens_dev(), ctx->parent_dev(), n, &dev, n, stream);
     if (rc != LLMCAD_OK) return rc;
     // argmax[128], path[128] and scalars[8] are contiguous in the context's integer buffer
     CUDA_TRY(cudaMemcpyAsync(out->argmax, ctx->argmax_dev(), n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));

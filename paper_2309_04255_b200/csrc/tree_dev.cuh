@@ -128,11 +128,11 @@ __device__ __forceinline__ void path_search(PathSearch &s, const int32_t *parent
     if (report && c == 0) s.n_all = max(max(s.below[0], s.below[1]), max(s.below[2], s.below[3]));
 }
 
-// The outputs of a pass: accepted_path (entries past the path are -1) and scalars, by one block.
+// The outputs of a pass: the path, -1 in what its first path_len entries hold behind it, and scalars, by one block.
 template <typename Best>
-__device__ __forceinline__ void report_path(const PathSearch &s, Best best_of, int P, int max_tree, int32_t *path, int32_t *scalars)
+__device__ __forceinline__ void report_path(const PathSearch &s, Best best_of, int P, int path_len, int32_t *path, int32_t *scalars)
 {
-    for (int j = threadIdx.x; j < max_tree; j += blockDim.x) path[j] = j < s.len ? s.path[j] : -1;
+    for (int j = threadIdx.x; j < max(s.len, path_len); j += blockDim.x) path[j] = j < s.len ? s.path[j] : -1;
     if (threadIdx.x == 0) {
         scalars[LLMCAD_S_ACCEPTED_LEN] = s.len;
         scalars[LLMCAD_S_NEXT_TOKEN] = best_of(s.path[s.len - 1]);
@@ -144,9 +144,9 @@ __device__ __forceinline__ void report_path(const PathSearch &s, Best best_of, i
     }
 }
 // The same for a pass that an earlier phase refused: an empty result. The status word is not written.
-__device__ __forceinline__ void report_refused(int P, int max_tree, int32_t *path, int32_t *scalars)
+__device__ __forceinline__ void report_refused(int P, int path_len, int32_t *path, int32_t *scalars)
 {
-    for (int j = threadIdx.x; j < max_tree; j += blockDim.x) path[j] = -1;
+    for (int j = threadIdx.x; j < path_len; j += blockDim.x) path[j] = -1;
     if (threadIdx.x == 0) {
         scalars[LLMCAD_S_ACCEPTED_LEN] = 0;
         scalars[LLMCAD_S_NEXT_TOKEN] = -1;

@@ -1,0 +1,59 @@
+"""What the entry points promise their callers around the pass itself: which outputs are written, how far, and in
+which order with other work of the stream."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2309_04255_b200 import binding as B
+from paper_2309_04255_b200 import inputs as gen
+
+from gpu_util import Twin, check_acceptance_against_oracle
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+SMALL = {"f32": gen.ModelConfig("f32", 2, 256, 4, 64, 688, 1024, "f32"),
+         "bf16": gen.ModelConfig("bf16", 2, 512, 4, 128, 1408, 2048, "bf16")}
+
+
+def planted(twin, P, parent, tokens, seed, rounds=4):
+    """Tokens of which the target accepts several levels: each round plants its choices one level deeper."""
+    for _ in range(rounds):
+        tokens = gen.plant_tokens(parent, tokens, twin.gpu_pass(P, tokens, parent)["argmax"], seed, prob=1.0)
+    return tokens
+
+
+def host_buffers(n, vocab):
+    return {"logits": torch.empty((n, vocab), dtype=torch.float32).pin_memory(), "argmax": torch.empty(n, dtype=torch.int32).pin_memory(),
+            "accepted_path": torch.full((n + 3,), 77, dtype=torch.int32).pin_memory(), "scalars": torch.zeros(8, dtype=torch.int32).pin_memory()}
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_host_entry_returns_the_verified_path(dtype):
+    """llmcad_verify_tree_host on trees of which several levels are accepted, two different ones in a row on one context:
+    all n entries of the path, -1 behind it, and nothing past them; everything else as the device entry gives it. A
+    refused tree gives an empty path."""
+    cfg, P = SMALL[dtype], 40
+    twin = Twin(cfg, P + 40, scale=3.0)
+    twin.fill_prefix_synthetic(P)
+    lengths = set()
+    for seed, n in ((3, 24), (5, 31), (3, 24)):
+        parent = gen.tree_random(n, 8, "uniform4", seed)
+        tokens = planted(twin, P, parent, gen.gen_tokens(cfg, n, seed), seed)
+        dev = twin.gpu_pass(P, tokens, parent)
+        acc = check_acceptance_against_oracle(dev, tokens, parent)
+        assert acc.accepted_len >= 3 and acc.path.tolist() != list(range(acc.accepted_len))
+        lengths.add(tuple(acc.path.tolist()))
+        host = host_buffers(n, cfg.vocab)
+        twin.v.verify_tree_host(P, torch.as_tensor(tokens).pin_memory(), torch.as_tensor(parent).pin_memory(), host)
+        for k in ("logits", "argmax", "scalars"):
+            assert np.array_equal(host[k].numpy(), dev[k]), k
+        assert host["accepted_path"].tolist() == acc.path.tolist() + [-1] * (n - acc.accepted_len) + [77] * 3
+    assert len(lengths) == 2
+    bad = parent.copy()
+    bad[2] = 2
+    host = host_buffers(n, cfg.vocab)
+    twin.v.verify_tree_host(P, torch.as_tensor(tokens).pin_memory(), torch.as_tensor(bad).pin_memory(), host)
+    assert host["scalars"].tolist() == [0, -1, P, 0, 0, 0, B.ERR_BAD_TREE, 0]
+    assert host["accepted_path"].tolist() == [-1] * n + [77] * 3
