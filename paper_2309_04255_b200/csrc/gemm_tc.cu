@@ -783,8 +783,11 @@ gemm_stream_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant_
 // accumulator buffer back on the first CTA's barrier. Weights travel as tensor-map boxes of 512-byte rows over
 // the packed tiles: a plain bulk copy can only complete on a barrier of its own CTA.
 //
-// kWide (128 < nodes <= 256, prefill): hi and lo activation planes are multiplied one after the other into the
-// same 256 columns; the MMA is at full rate at N = 256 either way and twice the nodes fit tensor memory.
+// kWide (128 < nodes <= 256, prefill): hi and lo activation planes are multiplied one after the other, each into 256
+// columns of its own, which is all of tensor memory: one accumulator buffer, so the next tile's MMAs wait for the dump.
+// Both planes in the same columns left room for two buffers (512 tokens at 7B: 15.3 instead of 15.8 ms), but the tensor
+// cores cut a sum off to its accumulator's bits at every MMA, always towards zero (5.8e-8 of the sum per k-block), and so
+// did it twice as often (2 layers of the 7B shape without attention, logits against 64 bits: 1.01e-5 instead of 7.8e-6).
 __device__ __forceinline__ uint32_t map_to_cta0(uint32_t addr)
 {
     uint32_t r;
@@ -959,8 +962,9 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
             for (int i = begin; i < end && !timed_out; ++seg) {
                 const int pt = i / ppt, seg_end = min(end, (pt + 1) * ppt);
                 int kb = (i - pt * ppt) * PK;
-                const int buf = seg & 1;
-                if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
+                const int buf = kWide ? 0 : seg & 1;
+                const uint32_t use = kWide ? seg : seg >> 1;
+                if (!mbar_wait_all(smem_u32(&ctl.tmem_empty[buf]), (use & 1u) ^ 1u, abort_flag, wait_limit)) { timed_out = true; break; }
                 const uint32_t d0 = tmem + buf * nb;
                 uint32_t acc = 0;
                 for (; i < seg_end; ++i, kb += PK) {
@@ -977,8 +981,8 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
                             for (int pl = 0; pl < (kWide ? 2 : 1); ++pl)
 #pragma unroll
                                 for (int k4 = 0; k4 < kBlockK / 16; ++k4)
-                                    tc_mma_pair(d0, a_desc + k * (kATileBytes >> 4) + 2 * k4, b_desc + ((k * b_tile_bytes + pl * b_half) >> 4) + 2 * k4, idesc,
-                                                k > 0 || pl > 0 || k4 > 0 ? 1u : acc);
+                                    tc_mma_pair(d0 + pl * nb, a_desc + k * (kATileBytes >> 4) + 2 * k4, b_desc + ((k * b_tile_bytes + pl * b_half) >> 4) + 2 * k4, idesc,
+                                                k > 0 || k4 > 0 ? 1u : acc);
                         }
                         tc_commit_pair(empty);
                         if (i + 1 == seg_end) tc_commit_pair(smem_u32(&ctl.tmem_full[buf]));
@@ -999,9 +1003,9 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
         const size_t slot_stride = slot_floats(p.n_pad);
         uint32_t seg = 0;
         for (int i = begin; i < end && !timed_out; ++seg) {
-            const int pt = i / ppt, v = 2 * pt + rank, buf = seg & 1;
+            const int pt = i / ppt, v = 2 * pt + rank, buf = kWide ? 0 : seg & 1;
             i = min(end, (pt + 1) * ppt);
-            if (!mbar_wait_warp(smem_u32(&ctl.tmem_full[buf]), (seg >> 1) & 1u, abort_flag, lane, wait_limit)) { timed_out = true; break; }
+            if (!mbar_wait_warp(smem_u32(&ctl.tmem_full[buf]), (kWide ? seg : seg >> 1) & 1u, abort_flag, lane, wait_limit)) { timed_out = true; break; }
             tc_fence_after();
             if (threadIdx.x == 64 && seg == 0) LLMCAD_TRACE(4);
             const uint32_t t_lane = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + buf * nb;
@@ -1011,7 +1015,7 @@ gemm_pair_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ 
                 int c0 = 0;
                 for (; c0 + 32 <= p.n_pad; c0 += 32) {
                     float t[32];
-                    if (p.comp && !kWide) tc_ld32_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
+                    if (p.comp) tc_ld32_sum2(t_lane + c0, t_lane + p.n_pad + c0, t);
                     else tc_ld32(t_lane + c0, t);
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) dump4(dst + (size_t)(c0 + j) * 32, t + j);
@@ -1769,7 +1773,7 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     const size_t act_bytes = (size_t)nb * kBlockK * 2 / (p.pairs && !d.w4 && !wide_in ? 2 : 1);
     const size_t stage_bytes = (size_t)pair_k * ((size_t)kATileBytes + act_bytes);
     // One CTA per SM with the whole shared memory as the ring.
-    // two accumulator buffers of MMA N columns each
+    // two accumulators of MMA N columns each: two buffers or, wide, the sums of the hi and of the lo plane
     int cols = 2 * nb, pow2 = 32;
     while (pow2 < cols) pow2 <<= 1;
     p.tmem_cols = pow2;

@@ -131,6 +131,36 @@ def test_prompt_chunks_of_up_to_256_tokens(cuts):
             assert np.abs(got - want).max() <= (2.0 ** -8 + BF16_TOL) * np.abs(want).max()
 
 
+def test_wide_prompt_chunks_are_as_exact_as_narrow_ones():
+    """The last token's logits of a model without attention (wo = 0: no rounded cache entry reaches them) against 64 bits,
+    256 tokens in one chunk and the same token at the end of a chunk of 128. Both carry 16-bit activations (2^-17 each) and
+    lose up to 5.8e-8 per k-block of 64 products to the accumulators, over at most 64 (gate, up) or 86 (down) of them:
+    below 2e-5 of the norm, where a lost lo plane costs 2e-3; and they agree to 10 % (the cuts of the k ranges differ),
+    where accumulating both planes in one sum costs 30 %."""
+    cfg = gen.ModelConfig("ffn", 2, 4096, 32, 128, 11008, 2048, "bf16")
+    errs = {128: [], 256: []}
+    for seed in range(3):
+        v = B.Verifier(cfg, 264)
+        glob = {k: gen.gen_tensor_device(cfg, k, -1, DEV, seed) for k in ("tok_embed", "final_norm", "lm_head")}
+        v.pack_globals(glob)
+        tokens = dev_i32(gen.gen_prefix_tokens(cfg, 256, seed))
+        norm = lambda x, g: x * torch.rsqrt((x * x).mean() + cfg.rms_eps) * g.double()
+        x = glob["tok_embed"][int(tokens[-1])].double()
+        for l in range(cfg.n_layers):
+            w = {k: gen.gen_tensor_device(cfg, k, l, DEV, seed) for k in gen.LAYER_TENSORS}
+            w["wo"].zero_()
+            v.pack_layer(l, w)
+            h = norm(x, w["ffn_norm"])
+            x = x + w["w_down"].double() @ (torch.nn.functional.silu(w["w_gate"].double() @ h) * (w["w_up"].double() @ h))
+        ref = glob["lm_head"].double() @ norm(x, glob["final_norm"])
+        for n in errs:
+            got = v.prefill(0, tokens[256 - n:], want_logits=True).double()
+            assert v.last_status() == 0
+            errs[n].append(((got - ref).norm() / ref.norm()).item())
+    assert max(errs[128] + errs[256]) <= 2e-5
+    assert sum(errs[256]) <= 1.1 * sum(errs[128])
+
+
 def test_prompt_with_a_bad_token_in_a_wide_chunk():
     twin = Twin(PROMPT_CFG, 300)
     tokens = gen.gen_prefix_tokens(PROMPT_CFG, 250, seed=1)
