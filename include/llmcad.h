@@ -121,7 +121,7 @@ typedef struct {
 typedef struct {
     float *logits;          /* [N][vocab] fp32, or NULL when not wanted */
     int32_t *argmax;        /* [N]: lowest index of each node's maximum logit */
-    int32_t *accepted_path; /* [max_tree]: node indices of the verified path, root first */
+    int32_t *accepted_path; /* [max_tree]: node indices of the verified path, root first, then -1 */
     int32_t *scalars;       /* [8], see LLMCAD_S_* */
 } llmcad_result;
 
@@ -129,7 +129,7 @@ typedef struct {
 typedef struct {
     float *logits;          /* [N][vocab] or NULL */
     int32_t *argmax;        /* [N] */
-    int32_t *accepted_path; /* [max_tree] */
+    int32_t *accepted_path; /* [N]: the path, then -1 */
     int32_t *scalars;       /* [8] */
 } llmcad_host_result;
 
@@ -200,12 +200,16 @@ int llmcad_tree_prep(const int32_t *parent_idx, int32_t n, int32_t prefix_len, i
                      uint32_t *anc /*[n][4]*/, int32_t *status, void *stream);
 
 /* Depth-first verified-sequence search and rollback of Sec. 3.2 on a given argmax
- * array: writes accepted_path and scalars, and moves the verified nodes' K/V rows
- * of every layer from slot prefix_len+path[j] to slot prefix_len+j.
- * kv_cache may be NULL (search only). All DEVICE. */
+ * array: writes accepted_path ([n]: the path, then -1) and scalars, and moves the
+ * verified nodes' K/V rows of every layer from slot prefix_len+path[j] to slot prefix_len+j.
+ * kv_cache may be NULL (search only). All DEVICE.
+ * llmcad_accept_compact_fill: the same with an accepted_path of path_len >= n entries. */
 int llmcad_accept_compact(llmcad_ctx *ctx, void *kv_cache, int32_t prefix_len, const int32_t *tree_tokens,
                           const int32_t *parent_idx, const int32_t *argmax, int32_t n,
                           int32_t *accepted_path, int32_t *scalars, void *stream);
+int llmcad_accept_compact_fill(llmcad_ctx *ctx, void *kv_cache, int32_t prefix_len, const int32_t *tree_tokens,
+                               const int32_t *parent_idx, const int32_t *argmax, int32_t n,
+                               int32_t *accepted_path, int32_t path_len, int32_t *scalars, void *stream);
 
 /* Tree-masked attention alone (one layer), the masked self-attention of Sec. 3.2 "Tree
  * decoder": node i attends to every prefix slot and to the tree nodes whose bit is set in

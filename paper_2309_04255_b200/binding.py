@@ -29,7 +29,7 @@ EXPORTS = [
     "llmcad_version", "llmcad_strerror", "llmcad_last_cuda_error", "llmcad_create", "llmcad_destroy",
     "llmcad_kv_cache_bytes", "llmcad_packed_weight_bytes", "llmcad_pack_layer", "llmcad_pack_globals",
     "llmcad_verify_tree", "llmcad_verify_tree_host", "llmcad_prefill", "llmcad_tree_prep",
-    "llmcad_accept_compact", "llmcad_tree_attention", "llmcad_skinny_gemm", "llmcad_launch_count",
+    "llmcad_accept_compact", "llmcad_accept_compact_fill", "llmcad_tree_attention", "llmcad_skinny_gemm", "llmcad_launch_count",
     "llmcad_last_status", "llmcad_set_kernel_timing", "llmcad_get_kernel_timing", "llmcad_set_gemm_trace", "llmcad_tiled_weight_bytes", "llmcad_tile_weight", "llmcad_skinny_gemm_tiled", "llmcad_tree_attention_noalloc", "llmcad_noalloc_last_error",
     "llmcad_tree_confidence", "llmcad_update_threshold", "llmcad_extend_tree", "llmcad_tree_branches", "llmcad_branch_pacer",
     "llmcad_set_wait_limit_ns", "llmcad_selftest_wait_timeout",
@@ -96,6 +96,7 @@ def lib():
         L.llmcad_prefill.argtypes = [vp, vp, vp, i32, vp, i32, vp, vp]
         L.llmcad_tree_prep.argtypes = [vp, i32, i32, vp, vp, vp, vp, vp]
         L.llmcad_accept_compact.argtypes = [vp, vp, i32, vp, vp, vp, i32, vp, vp, vp]
+        L.llmcad_accept_compact_fill.argtypes = [vp, vp, i32, vp, vp, vp, i32, vp, i32, vp, vp]
         L.llmcad_tree_attention.argtypes = [vp, vp, vp, vp, i32, i32, vp, i32, vp, vp]
         L.llmcad_skinny_gemm.argtypes = [vp, vp, vp, vp, i32, i32, i32, vp]
         L.llmcad_launch_count.argtypes = [vp]
@@ -212,9 +213,16 @@ class Verifier:
     def verify_tree(self, prefix_len: int, tokens: torch.Tensor, parent: torch.Tensor, out=None, want_logits=True):
         n = tokens.numel()
         out = out or self.new_outputs(n, want_logits)
-        r = Result(_ptr(out["logits"]), _ptr(out["argmax"]), _ptr(out["accepted_path"]), _ptr(out["scalars"]))
+        path = out["accepted_path"]
+        r = Result(_ptr(out["logits"]), _ptr(out["argmax"]), _ptr(path), _ptr(out["scalars"]))
+        short = path.numel() < self.max_tree
+        if short:       # the pass writes max_tree entries: a caller's shorter buffer gets its part of them afterwards
+            whole = self._i32.new_empty(self.max_tree)
+            r.accepted_path = whole.data_ptr()
         _check(lib().llmcad_verify_tree(self.ctx, self.packed.data_ptr(), self.kv.data_ptr(), prefix_len, _ptr(tokens),
                                         _ptr(parent), n, C.byref(r), _stream()), "llmcad_verify_tree")
+        if short:
+            path.copy_(whole[:path.numel()])
         return out
 
     def extend_tree(self, prefix_len: int, tokens: torch.Tensor, parent: torch.Tensor, n_old: int, top_k: int = 4,
@@ -256,8 +264,8 @@ class Verifier:
         n = tokens.numel()
         path = self._i32.new_empty(self.max_tree)
         scalars = self._i32.new_empty(8)
-        _check(lib().llmcad_accept_compact(self.ctx, self.kv.data_ptr() if compact else None, prefix_len, _ptr(tokens),
-                                           _ptr(parent), _ptr(argmax), n, _ptr(path), _ptr(scalars), _stream()),
+        _check(lib().llmcad_accept_compact_fill(self.ctx, self.kv.data_ptr() if compact else None, prefix_len, _ptr(tokens),
+                                                _ptr(parent), _ptr(argmax), n, _ptr(path), self.max_tree, _ptr(scalars), _stream()),
                "llmcad_accept_compact")
         return path, scalars
 

@@ -903,14 +903,21 @@ int llmcad_accept_compact(llmcad_ctx *ctx, void *kv_cache, int32_t prefix_len, c
                           const int32_t *parent_idx, const int32_t *argmax, int32_t n, int32_t *accepted_path,
                           int32_t *scalars, void *stream)
 {
+    return llmcad_accept_compact_fill(ctx, kv_cache, prefix_len, tree_tokens, parent_idx, argmax, n, accepted_path, n, scalars, stream);
+}
+
+int llmcad_accept_compact_fill(llmcad_ctx *ctx, void *kv_cache, int32_t prefix_len, const int32_t *tree_tokens,
+                               const int32_t *parent_idx, const int32_t *argmax, int32_t n, int32_t *accepted_path,
+                               int32_t path_len, int32_t *scalars, void *stream)
+{
     if (!ctx || !tree_tokens || !parent_idx || !argmax || !accepted_path || !scalars) return LLMCAD_ERR_INVALID_ARG;
-    if (n < 1 || prefix_len < 0) return LLMCAD_ERR_INVALID_ARG;
+    if (n < 1 || prefix_len < 0 || path_len < n) return LLMCAD_ERR_INVALID_ARG;
     if (n > ctx->cfg.max_tree) return LLMCAD_ERR_UNSUPPORTED;
     if ((long long)prefix_len + n > ctx->cfg.max_seq) return LLMCAD_ERR_CAPACITY;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const llmcad_config &c = ctx->cfg;
     // the search trusts the tree: the kernel validates it first (a malformed tree lands in scalars[status])
-    CUDA_TRY(launch_search_rollback(parent_idx, tree_tokens, argmax, n, prefix_len, c.vocab, 1, accepted_path, c.max_tree, scalars,
+    CUDA_TRY(launch_search_rollback(parent_idx, tree_tokens, argmax, n, prefix_len, c.vocab, 1, accepted_path, path_len, scalars,
                                     kv_cache, c.dtype, c.n_layers, c.n_heads, c.max_seq, c.head_dim, st));
     ctx->launches++;
     return LLMCAD_OK;

@@ -57,3 +57,31 @@ def test_host_entry_returns_the_verified_path(dtype):
     twin.v.verify_tree_host(P, torch.as_tensor(tokens).pin_memory(), torch.as_tensor(bad).pin_memory(), host)
     assert host["scalars"].tolist() == [0, -1, P, 0, 0, 0, B.ERR_BAD_TREE, 0]
     assert host["accepted_path"].tolist() == [-1] * n + [77] * 3
+
+
+def test_paths_stay_inside_the_callers_buffers():
+    """llmcad_accept_compact on a path buffer of n entries, and verify_tree on outputs of the caller whose path has n: the
+    path, -1 up to n, and nothing behind (the buffers are the front of larger ones, so that a longer write would show). A
+    path length below n is refused."""
+    cfg, P, n = SMALL["f32"], 9, 20
+    twin = Twin(cfg, P + n + 1, scale=3.0)
+    twin.fill_prefix_synthetic(P)
+    v = twin.v
+    parent = gen.tree_random(n, 8, "uniform4", 4)
+    tokens = planted(twin, P, parent, gen.gen_tokens(cfg, n, 4), 4)
+    ref = twin.gpu_pass(P, tokens, parent)
+    acc = check_acceptance_against_oracle(ref, tokens, parent)
+    want = acc.path.tolist() + [-1] * (n - acc.accepted_len) + [77] * (256 - n)
+    t, p, amax = (torch.as_tensor(np.asarray(a, np.int32), device=DEV) for a in (tokens, parent, ref["argmax"]))
+    for q, expect in ((p, want), (torch.full_like(p, 5), [-1] * n + [77] * (256 - n))):     # the second tree is refused
+        room = torch.full((256,), 77, dtype=torch.int32, device=DEV)
+        sc = torch.zeros(8, dtype=torch.int32, device=DEV)
+        args = (v.ctx, None, P, t.data_ptr(), q.data_ptr(), amax.data_ptr(), n, room.data_ptr())
+        assert B.lib().llmcad_accept_compact(*args, sc.data_ptr(), B._stream()) == B.OK
+        assert room.tolist() == expect
+    assert B.lib().llmcad_accept_compact_fill(*args, n - 1, sc.data_ptr(), B._stream()) == B.ERR_INVALID_ARG
+    out = v.new_outputs(n)
+    room = torch.full((256,), 77, dtype=torch.int32, device=DEV)
+    out["accepted_path"] = room[:n]
+    assert v.verify_tree(P, t, p, out=out)["accepted_path"] is out["accepted_path"]
+    assert room.tolist() == want and out["scalars"].tolist() == ref["scalars"].tolist()
