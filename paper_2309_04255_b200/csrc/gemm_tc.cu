@@ -1532,7 +1532,7 @@ gemm_finish_kernel(const __grid_constant__ GemmParams p)
         for (int n0 = 0; n0 < p.n_pad; n0 += LLMCAD_MAX_TREE) {
             const int node = n0 + col128;
             float acc = 0.f;
-            if (node < p.n_pad) {
+            if (node < ep.n) {             // (the sums of a call on the last row alone start there: none lie behind them)
                 const float *col = ep.ssq_in + node;
                 int t = slice;
                 for (; t + 7 * kSlices < ep.ssq_in_parts; t += 8 * kSlices) {
