@@ -15,6 +15,9 @@ namespace llmcad {
 // at position prefix_len + depth, their row of the residual stream and, with gain != null (the tensor-core
 // path folds the first RMSNorm into the QKV GEMM), gain * x as a GEMM input (hi and, if comp, lo plane)
 // and the row's sum of squares.
+//
+// This kernel lets its dependents go only after its own dependency has resolved: the first GEMM requests
+// weights before its own, and those may have been written right before the call, on this stream.
 template <typename T>
 __global__ void __launch_bounds__(256)
 prep_embed_kernel(const int32_t *__restrict__ parent, const int32_t *__restrict__ tokens, int n_tree, int n_old, int P, int vocab,
@@ -24,8 +27,8 @@ prep_embed_kernel(const int32_t *__restrict__ parent, const int32_t *__restrict_
     __shared__ MaskTable t;
     __shared__ float red[8];
     const int i = blockIdx.x;
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     const int err = mask_table(t, parent, tokens, n_tree, vocab);
     if (i == 0 && threadIdx.x == 0) {
         if (!keep) *status = err;
@@ -97,8 +100,8 @@ chain_embed_kernel(const int32_t *__restrict__ tokens, int n, int P, int vocab, 
 {
     __shared__ float red[8];
     const int i = blockIdx.x;
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     int bad = 0;
     for (int c = threadIdx.x; c < n; c += 256) { const int tk = __ldg(tokens + c); bad |= tk < 0 || tk >= vocab; }
     const int err = __syncthreads_or(bad) ? LLMCAD_ERR_BAD_TOKEN : 0;

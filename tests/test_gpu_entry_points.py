@@ -85,3 +85,45 @@ def test_paths_stay_inside_the_callers_buffers():
     out["accepted_path"] = room[:n]
     assert v.verify_tree(P, t, p, out=out)["accepted_path"] is out["accepted_path"]
     assert room.tolist() == want and out["scalars"].tolist() == ref["scalars"].tolist()
+
+
+@pytest.mark.parametrize("op", ["verify", "prefill"])
+def test_weights_packed_right_before_a_pass_are_the_ones_it_uses(op):
+    """Two sets of weights packed in turn, each followed by a pass on the same stream with nothing in between: every pass
+    gives bit for bit what it gives after a synchronisation. (The first GEMM requests weights ahead of its dependency; that
+    it does so after the packing is an order of launches which no single run proves.)"""
+    cfg, P, n = SMALL["bf16"], 30, 16
+    m = 150 if op == "prefill" else n             # a wide chunk starts with a kernel of its own
+    v = B.Verifier(cfg, P + m + 1)
+    v.kv_view().normal_(generator=torch.Generator(device=DEV).manual_seed(1))
+    tokens = torch.as_tensor(gen.gen_tokens(cfg, m, 2), device=DEV)
+    parent = torch.as_tensor(gen.tree_random(n, 6, "uniform4", 2), device=DEV)
+    sets = []
+    for seed in (0, 1):
+        glob = {k: w.to(DEV) for k, w in gen.gen_globals(cfg, seed).items()}
+        layers = [{k: w.to(DEV) for k, w in gen.gen_layer(cfg, l, seed).items()} for l in range(cfg.n_layers)]
+        sets.append((glob, layers))
+
+    def pack(s):                                   # as the binding does, without its synchronisation
+        glob, layers = sets[s]
+        g = B.GlobalWeights(**{k: w.data_ptr() for k, w in glob.items()})
+        B._check(B.lib().llmcad_pack_globals(v.ctx, g, v.packed.data_ptr(), B._stream()), "pack")
+        for l, w in reversed(list(enumerate(layers))):      # the layer that the pass reads first comes last
+            lw = B.LayerWeights(**{k: t.data_ptr() for k, t in w.items()})
+            B._check(B.lib().llmcad_pack_layer(v.ctx, l, lw, v.packed.data_ptr(), B._stream()), "pack")
+
+    def run():
+        return v.verify_tree(P, tokens, parent)["logits"] if op == "verify" else v.prefill(P, tokens, want_logits=True)
+
+    refs = []
+    for s in (0, 1):
+        pack(s)
+        torch.cuda.synchronize()
+        refs.append(run().clone())
+    assert not torch.equal(refs[0], refs[1])
+    outs = []
+    for i in range(40):
+        pack(i & 1)
+        outs.append(run().clone())
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, refs[i & 1]) for i, o in enumerate(outs))
