@@ -429,6 +429,7 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
                 // the lm_head on the last row alone
                 if ((rc = ensure_act_maps(ctx, 16)) != LLMCAD_OK) return rc;
                 gemms[i].set(ctx, -1, 0, 0, d, specs[i].ep, 16);
+                gemms[i].p.pairs = 0;          // the map below has both planes in a box, which CTA pairs split
                 if (!make_act_map_bf16(&gemms[i].maps.x, static_cast<char *>(ctx->xn) + (size_t)(n - 1) * d * ctx->elem, 1, d, 16, ctx->comp ? 2 : 1, kLoRows,
                                        ctx->comp ? 2 : 1)) {
                     snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for an activation row");

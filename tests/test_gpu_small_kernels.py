@@ -131,6 +131,18 @@ def test_prompt_chunks_of_up_to_256_tokens(cuts):
             assert np.abs(got - want).max() <= (2.0 ** -8 + BF16_TOL) * np.abs(want).max()
 
 
+def test_prompts_with_cta_pairs_at_every_size():
+    """The threshold of the CTA pairs is a tuning aid (read once per process, hence the child): from 16 nodes on, where the
+    last row's lm_head, which has 16 padded nodes whatever the prompt, would take them too."""
+    import os, subprocess, sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    script = ("import sys; sys.path[:0] = [sys.argv[1], sys.argv[1] + '/..']; import test_gpu_small_kernels as T\n"
+              "for cuts in ([5], [64, 191], [300, 140]): T.test_prompt_chunks_of_up_to_256_tokens(cuts)\nprint('ok')")
+    r = subprocess.run([sys.executable, "-c", script, here], env=dict(os.environ, LLMCAD_CTA_PAIR_MIN="16"), capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout[-2000:] + r.stderr[-4000:]
+
+
 def test_wide_prompt_chunks_are_as_exact_as_narrow_ones():
     """The last token's logits of a model without attention (wo = 0: no rounded cache entry reaches them) against 64 bits,
     256 tokens in one chunk and the same token at the end of a chunk of 128. Both carry 16-bit activations (2^-17 each) and
