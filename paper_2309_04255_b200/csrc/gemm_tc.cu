@@ -1739,7 +1739,7 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
     const int nb = p.n_pad * (p.comp && !wide ? 2 : 1);       // MMA N
     if (nb > 256 || p.n_pad < 16 || p.n_pad % 16 || (wide && (!p.pairs || !p.comp || p.n_pad != 256))) return cudaErrorInvalidValue;
     int pair_k = nb > 128 ? 1 : kMaxPairK;
-    if (tune.pair_k) pair_k = tune.pair_k;
+    if (tune.pair_k && !wide) pair_k = tune.pair_k;
     GemmDesc &d = p.g;
     d.pair_k = pair_k;
     // the items are split evenly over one CTA (CTA pair) per SM (two SMs), fewer when there are fewer items
@@ -1812,12 +1812,12 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
     if (attr_set.needed()) {
         cudaError_t e = cudaSuccess;
         typedef void (*SKernel)(GemmMaps, GemmParams);
-        const SKernel all[8] = {gemm_stream_kernel<1>, gemm_stream_kernel<2>, gemm_w4_kernel<1>, gemm_w4_kernel<2>,
-                                gemm_pair_kernel<1, false>, gemm_pair_kernel<2, false>, gemm_pair_kernel<1, true>, gemm_pair_kernel<2, true>};
+        const SKernel all[7] = {gemm_stream_kernel<1>, gemm_stream_kernel<2>, gemm_w4_kernel<1>, gemm_w4_kernel<2>,
+                                gemm_pair_kernel<1, false>, gemm_pair_kernel<2, false>, gemm_pair_kernel<1, true>};
         // An SM splits its on-chip memory between shared memory and L1 when it is empty, to fit the kernel that
         // arrives; a streaming CTA of 195 KB would get a 196 KB split, and the finishing CTA of the same GEMM
         // could not settle beside it. Every kernel of the GEMM asks for the largest shared-memory split.
-        for (int i = 0; i < 8 && e == cudaSuccess; ++i) {
+        for (int i = 0; i < 7 && e == cudaSuccess; ++i) {
             e = cudaFuncSetAttribute(all[i], cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(all[i], cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         }
@@ -1831,7 +1831,7 @@ cudaError_t launch_gemm_tc(const GemmMaps &maps, GemmParams &p, int n_sms, size_
 #define LLMCAD_BY_K(KERNEL1, KERNEL2) \
     (pair_k == 1 ? cudaLaunchKernelEx(&lc.cfg, KERNEL1, maps, p) : cudaLaunchKernelEx(&lc.cfg, KERNEL2, maps, p))
         if (d.w4) e = LLMCAD_BY_K(gemm_w4_kernel<1>, gemm_w4_kernel<2>);
-        else if (p.pairs && wide_in) e = LLMCAD_BY_K((gemm_pair_kernel<1, true>), (gemm_pair_kernel<2, true>));
+        else if (p.pairs && wide_in) e = cudaLaunchKernelEx(&lc.cfg, gemm_pair_kernel<1, true>, maps, p);
         else if (p.pairs) e = LLMCAD_BY_K((gemm_pair_kernel<1, false>), (gemm_pair_kernel<2, false>));
         else e = LLMCAD_BY_K(gemm_stream_kernel<1>, gemm_stream_kernel<2>);
 #undef LLMCAD_BY_K
