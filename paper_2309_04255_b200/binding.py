@@ -166,7 +166,6 @@ class Verifier:
         self.tdtype = torch.float32 if cfg.dtype == "f32" else torch.bfloat16
         self._i32 = torch.empty(1, dtype=torch.int32, device=self.device)      # new_empty of these is the cheapest allocation
         self._f32 = torch.empty(1, dtype=torch.float32, device=self.device)
-        self._kv_view = None
 
     def close(self):
         if getattr(self, "ctx", None):
@@ -194,12 +193,22 @@ class Verifier:
         torch.cuda.current_stream().synchronize()
 
     # ---- cache views
+    @property
+    def kv(self) -> torch.Tensor:
+        """The cache's bytes; may be replaced by another tensor of the same size."""
+        return self._kv
+
+    @kv.setter
+    def kv(self, t):
+        self._kv, self._kv_view = t, None       # the view would keep the old cache's memory
+
     def kv_view(self) -> torch.Tensor:
         """[L][2][H][max_seq][hd] view of the cache in the model dtype."""
-        if self._kv_view is None or self._kv_view[0] is not self.kv:
+        view = self._kv_view
+        if view is None or view.data_ptr() != self._kv.data_ptr():
             c = self.cfg
-            self._kv_view = (self.kv, self.kv.view(self.tdtype).view(c.n_layers, 2, c.n_heads, self.max_seq, c.head_dim))
-        return self._kv_view[1]
+            self._kv_view = view = self._kv.view(self.tdtype).view(c.n_layers, 2, c.n_heads, self.max_seq, c.head_dim)
+        return view
 
     # ---- the pass
     def new_outputs(self, n: int, want_logits: bool = True):
@@ -219,7 +228,7 @@ class Verifier:
         if short:       # the pass writes max_tree entries: a caller's shorter buffer gets its part of them afterwards
             whole = self._i32.new_empty(self.max_tree)
             r.accepted_path = whole.data_ptr()
-        _check(lib().llmcad_verify_tree(self.ctx, self.packed.data_ptr(), self.kv.data_ptr(), prefix_len, _ptr(tokens),
+        _check(lib().llmcad_verify_tree(self.ctx, self.packed.data_ptr(), self._kv.data_ptr(), prefix_len, _ptr(tokens),
                                         _ptr(parent), n, C.byref(r), _stream()), "llmcad_verify_tree")
         if short:
             path.copy_(whole[:path.numel()])
@@ -237,7 +246,7 @@ class Verifier:
             "topk_probs": self._f32.new_empty((n_new, max(top_k, 1))),
             "status": self._i32.new_empty(1),
         }
-        _check(lib().llmcad_extend_tree(self.ctx, _ptr(self.packed), _ptr(self.kv), prefix_len, _ptr(tokens), _ptr(parent),
+        _check(lib().llmcad_extend_tree(self.ctx, _ptr(self.packed), _ptr(self._kv), prefix_len, _ptr(tokens), _ptr(parent),
                                         n_old, n_tree, top_k, _ptr(out["logits"]), _ptr(out["topk_ids"]),
                                         _ptr(out["topk_probs"]), _ptr(out["status"]), _stream()), "llmcad_extend_tree")
         return out
@@ -248,14 +257,14 @@ class Verifier:
         lg = out.get("logits")
         r = Result(lg.data_ptr() if lg is not None else None, out["argmax"].data_ptr(),
                    out["accepted_path"].data_ptr(), out["scalars"].data_ptr())
-        _check(lib().llmcad_verify_tree_host(self.ctx, self.packed.data_ptr(), self.kv.data_ptr(), prefix_len,
+        _check(lib().llmcad_verify_tree_host(self.ctx, self.packed.data_ptr(), self._kv.data_ptr(), prefix_len,
                                              tokens.data_ptr(), parent.data_ptr(), n, C.byref(r), _stream()),
                "llmcad_verify_tree_host")
         return out
 
     def prefill(self, prefix_len: int, tokens: torch.Tensor, want_logits: bool = False):
         lg = torch.empty(self.cfg.vocab, dtype=torch.float32, device=self.device) if want_logits else None
-        _check(lib().llmcad_prefill(self.ctx, self.packed.data_ptr(), self.kv.data_ptr(), prefix_len, _ptr(tokens),
+        _check(lib().llmcad_prefill(self.ctx, self.packed.data_ptr(), self._kv.data_ptr(), prefix_len, _ptr(tokens),
                                     tokens.numel(), _ptr(lg), _stream()), "llmcad_prefill")
         return lg
 
@@ -264,8 +273,8 @@ class Verifier:
         n = tokens.numel()
         path = self._i32.new_empty(self.max_tree)
         scalars = self._i32.new_empty(8)
-        _check(lib().llmcad_accept_compact_fill(self.ctx, self.kv.data_ptr() if compact else None, prefix_len, _ptr(tokens),
-                                                _ptr(parent), _ptr(argmax), n, _ptr(path), self.max_tree, _ptr(scalars), _stream()),
+        _check(lib().llmcad_accept_compact_fill(self.ctx, self._kv.data_ptr() if compact else None, prefix_len, _ptr(tokens),
+                                                _ptr(parent), _ptr(argmax), n, path.data_ptr(), self.max_tree, scalars.data_ptr(), _stream()),
                "llmcad_accept_compact")
         return path, scalars
 

@@ -127,3 +127,20 @@ def test_weights_packed_right_before_a_pass_are_the_ones_it_uses(op):
         outs.append(run().clone())
     torch.cuda.synchronize()
     assert all(torch.equal(o, refs[i & 1]) for i, o in enumerate(outs))
+
+
+def test_a_replaced_cache_is_the_one_in_use_and_the_old_one_is_freed():
+    """The binding keeps its view of the cache between calls; neither another tensor in `kv` nor another storage under the
+    same tensor leaves it on old memory, and a dropped cache is freed at once."""
+    cfg = gen.ModelConfig("cache", 2, 512, 4, 128, 1408, 2048, "bf16")
+    v = B.Verifier(cfg, 4096)
+    nbytes = v.kv.numel()
+    v.kv_view().fill_(1)
+    held = torch.cuda.memory_allocated()
+    v.kv = None
+    assert torch.cuda.memory_allocated() <= held - nbytes
+    v.kv = torch.zeros(nbytes, dtype=torch.uint8, device=DEV)
+    assert v.kv_view().data_ptr() == v.kv.data_ptr() and not v.kv_view().any()
+    v.kv.data = torch.full((nbytes,), 0, dtype=torch.uint8, device=DEV)
+    v.kv_view().fill_(2)
+    assert v.kv_view().data_ptr() == v.kv.data_ptr() and v.kv.any()
