@@ -103,14 +103,16 @@ struct llmcad_ctx {
     // Tensor-core path: activations travel as bf16 hi + lo planes (common.cuh); a tuning aid
     // (LLMCAD_COMP=0) turns the lo planes off.
     bool comp = false;
-    // activations of up to 128 nodes; xn, q, att and h hold two planes of 128 rows (hi, lo)
+    // activations of `rows` nodes (128, or 256 for the chunks of a prompt); xn, q, att and h hold a hi plane and, with
+    // comp, kLoRows rows behind its start a lo plane
+    int rows = LLMCAD_MAX_TREE;
     void *arena = nullptr;    // the one allocation that holds every workspace below
-    float *x = nullptr;       // residual stream [128][d] fp32
-    void *xn = nullptr;       // normalised GEMM input [2][128][d]
-    void *q = nullptr;        // rotated queries [2][128][d]
-    void *att = nullptr;      // attention output [2][128][d]
-    void *h = nullptr;        // SwiGLU output [2][128][f]
-    void *kv_lo = nullptr;    // bf16 remainders of the current layer's tree keys and values [2][H][128][hd]
+    float *x = nullptr;       // residual stream [rows][d] fp32
+    void *xn = nullptr;       // normalised GEMM input, planes of [rows][d]
+    void *q = nullptr;        // rotated queries, the same
+    void *att = nullptr;      // attention output, the same
+    void *h = nullptr;        // SwiGLU output, planes of [rows][f]
+    void *kv_lo = nullptr;    // comp: bf16 remainders of the current layer's tree keys and values [2][H][kLoRows][hd]
     float *logits = nullptr;  // [128][V], used when the caller does not want logits
     TreeBuffers tb{};
     // the one-kernel fp32 pass (pass_small.cu): allowed, and its own workspaces
@@ -232,12 +234,12 @@ int ensure_act_maps(llmcad_ctx *ctx, int n_pad)
     const void *bufs[3] = {ctx->xn, ctx->att, ctx->h};
     for (int i = 0; i < 3; ++i) {
         const int cols = i == 2 ? c.d_ffn : c.d_model;
-        if (n_pad <= LLMCAD_MAX_TREE) ok &= make_act_map_bf16(&ctx->act_maps[slot][i], bufs[i], kLoRows, cols, n_pad, planes, kLoRows, planes);
+        if (n_pad <= LLMCAD_MAX_TREE) ok &= make_act_map_bf16(&ctx->act_maps[slot][i], bufs[i], ctx->rows, cols, n_pad, planes, kLoRows, planes);
         // a CTA pair: one plane, or half of the rows of the only plane
         if (gemm_takes_pairs(n_pad, ctx->comp))
             ok &= n_pad > LLMCAD_MAX_TREE
-                      ? make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], kLoRows, cols, n_pad / 2, planes, kLoRows, planes)    // half of the rows, both planes
-                      : make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], kLoRows, cols, ctx->comp ? n_pad : n_pad / 2, planes, kLoRows, 1);
+                      ? make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], ctx->rows, cols, n_pad / 2, planes, kLoRows, planes)    // half of the rows, both planes
+                      : make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], ctx->rows, cols, ctx->comp ? n_pad : n_pad / 2, planes, kLoRows, 1);
     }
     if (!ok) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed for an activation buffer");
@@ -631,17 +633,24 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
         wants.push_back({p, arena_bytes});
         arena_bytes = align_up(arena_bytes + bytes, 1024);
     };
-    want((void **)&ctx->x, kLoRows * d * 4);
-    want(&ctx->xn, 2 * kLoRows * d * ctx->elem);
-    want(&ctx->q, 2 * kLoRows * d * ctx->elem);
-    want(&ctx->att, 2 * kLoRows * d * ctx->elem);
-    want(&ctx->h, 2 * kLoRows * f * ctx->elem);
-    want(&ctx->kv_lo, 2 * kLoRows * d * ctx->elem);
+    // Prompts go in chunks of kLoRows tokens where the GEMMs on CTA pairs and the tcgen05 attention kernel serve the
+    // layers: the weights are then read half as often, and at 256 columns the MMAs of hi and lo planes set the pace.
+    // (INT4 weights: the kernel that expands them works on 128 nodes at most.)
+    ctx->wide_chunks = ctx->tc_gemm && ctx->comp && !ctx->w4 && ctx->tc_attn && !(cfg->flags & LLMCAD_FLAG_MMA_ATTN) &&
+                       attention_prefers_t5(LLMCAD_MAX_TREE) && cfg->max_tree == LLMCAD_MAX_TREE;
+    ctx->rows = ctx->wide_chunks ? kLoRows : LLMCAD_MAX_TREE;
+    const size_t rows = ctx->rows, planes_rows = ctx->comp ? kLoRows + rows : rows;
+    want((void **)&ctx->x, rows * d * 4);
+    want(&ctx->xn, planes_rows * d * ctx->elem);
+    want(&ctx->q, planes_rows * d * ctx->elem);
+    want(&ctx->att, planes_rows * d * ctx->elem);
+    want(&ctx->h, planes_rows * f * ctx->elem);
+    want(&ctx->kv_lo, ctx->comp ? 2 * kLoRows * d * ctx->elem : 0);
     want((void **)&ctx->logits, (size_t)128 * cfg->vocab * 4);
     want((void **)&ctx->tb.depth, 128 * 4);
     want((void **)&ctx->tb.pos, 128 * 4);
     want((void **)&ctx->tb.anc, 128 * 16);
-    want((void **)&ctx->tb.rope_cs, kLoRows * (hd / 2) * sizeof(float2));
+    want((void **)&ctx->tb.rope_cs, rows * (hd / 2) * sizeof(float2));
     want((void **)&ctx->inv_freq, (hd / 2) * sizeof(double));
     want((void **)&ctx->ibuf, (520 + 128) * 4);
     {
@@ -651,10 +660,6 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
             if ((int)((rows + 127) / 128) > max_tiles) max_tiles = (int)((rows + 127) / 128);
         const int max_pad = (cfg->max_tree + 15) / 16 * 16;
         ctx->partial_floats = ctx->tc_gemm ? gemm_tc_partial_floats(ctx->n_sms, max_tiles, max_pad) : 64;
-        // Prompts go in chunks of kLoRows tokens where the GEMMs on CTA pairs and the tcgen05 attention kernel serve the
-        // layers: the weights are then read half as often, and at 256 columns the MMAs of hi and lo planes set the pace.
-        ctx->wide_chunks = ctx->tc_gemm && ctx->comp && !ctx->w4 && ctx->tc_attn && !(cfg->flags & LLMCAD_FLAG_MMA_ATTN) &&
-                           attention_prefers_t5(LLMCAD_MAX_TREE) && cfg->max_tree == LLMCAD_MAX_TREE;
         if (ctx->wide_chunks) {
             const size_t wide = gemm_tc_wide_partial_floats(ctx->n_sms, (int)(d > f ? d : f), (int)d);
             if (wide > ctx->partial_floats) ctx->partial_floats = wide;

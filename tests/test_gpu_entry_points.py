@@ -144,3 +144,20 @@ def test_a_replaced_cache_is_the_one_in_use_and_the_old_one_is_freed():
     v.kv.data = torch.full((nbytes,), 0, dtype=torch.uint8, device=DEV)
     v.kv_view().fill_(2)
     assert v.kv_view().data_ptr() == v.kv.data_ptr() and v.kv.any()
+
+
+@pytest.mark.parametrize("dtype,flags,mb", [("f32", 0, 24), ("bf16", B.FLAG_INT4_WEIGHTS, 82), ("bf16", B.FLAG_SIMT_GEMM, 24)])
+def test_a_context_holds_no_room_for_chunks_it_never_runs(dtype, flags, mb):
+    """Only bf16 contexts on the tensor cores run prompts in chunks of 256; the others hold activations of 128 nodes. d 4096,
+    f 11008: 128 rows of x, xn, q, att (d) and h (f) are 14 MB in fp32, 8 in bf16; with INT4, where hi and lo plane lie 256
+    rows apart, they and the remainders of K and V are 24, the segments of the GEMMs 53."""
+    import ctypes
+    cfg = gen.ModelConfig("room", 1, 4096, 32, 128, 11008, 512, dtype)
+    c = B.make_config(cfg, 64, flags=flags)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    h = ctypes.c_void_p()
+    assert B.lib().llmcad_create(ctypes.byref(c), ctypes.byref(h)) == B.OK
+    used = free - torch.cuda.mem_get_info()[0]
+    B.lib().llmcad_destroy(h)
+    assert 4e6 < used <= mb * 1e6
