@@ -25,8 +25,8 @@
 //
 // Warp roles of the streaming kernel (224 threads): warp 0 = weight producer, warp 1 = TMEM
 // allocator + MMA issuer, warps 2..5 = accumulator dump (tcgen05.ld of their 32 lanes each),
-// warp 6 = activation loader (TMA). Accumulators are double-buffered in TMEM when two buffers fit,
-// so that the dump of one segment overlaps the MMAs of the next.
+// warp 6 = activation loader (TMA). Accumulators are double-buffered in TMEM, so that the dump of one
+// segment overlaps the MMAs of the next.
 //
 // Programmatic stream serialization: the ring is filled with weight tiles while the previous
 // kernels of the pass are still running; activations and the workspace wait for the grid
@@ -54,7 +54,7 @@ namespace {
 constexpr int kTileM = 128;     // weight rows per tile
 constexpr int kBlockK = 64;     // bf16 elements per k-block = one 128-byte swizzle row
 constexpr int kThreads = 224;   // producer, MMA issuer, 4 epilogue warps, activation loader
-constexpr int kFinThreads = 384;  // finishing kernel: 12 warps, up to 112 registers each beside a resident streaming CTA
+constexpr int kFinThreads = 384;  // finishing kernel: 12 warps, three per scheduler
 // An SM's registers come in four banks of 16K, one per warp scheduler: beside the streaming CTA's two warps per
 // scheduler (96 registers a thread) three finishing warps fit with up to 106 each.
 constexpr int kFinMaxRegs = 96;
@@ -1719,9 +1719,10 @@ const Tuning &tuning()
 }
 }  // namespace
 
-// Pairs from 80 nodes on (measured in whole passes, one kernel per CTA against pairs: 48 nodes 2 % slower, 64 nodes
-// level, 128 nodes 4-5 % faster; 16 and 32 nodes 3-6 % slower, the two cluster barriers at either end of the kernel
-// sit in every hand-over). The MMA's N has to be a multiple of 32.
+// Pairs from 80 nodes on. Measured in passes of 16 layers of the 7B shape and 10 of the 13B shape against one kernel per
+// CTA: 16 and 32 nodes 3-6 % slower (the two cluster barriers at either end of the kernel sit in every hand-over), 45
+// nodes 1 % slower at 7B and 1 % faster at 13B, 64 nodes 1-3 % faster, 80 nodes 1.5-2.4 %, 128 nodes 7 %. The MMA's N has
+// to be a multiple of 32.
 bool gemm_takes_pairs(int n_pad, bool comp)
 {
     if (n_pad > 128) return true;
@@ -1733,8 +1734,9 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
 {
     const Tuning &tune = tuning();
     // Ring items of two k-blocks (one 32 KB weight copy each) unless the activation tiles are so wide
-    // (hi | lo planes of more than 64 nodes) that only two stages would fit; measured on B200:
-    // single k-blocks cost 10-17 % up to 64 nodes and gain 6 % at 128.
+    // (hi | lo planes of more than 64 nodes) that only two stages would fit. Measured on B200 in passes of 16 layers
+    // of the 7B shape: single k-blocks cost 1.4 % at 1 and 16 nodes and 0.5 % at 32, are level at 45 and 64 (there 13B
+    // widths gain up to 2 %), and gain 2.3 % at 80 and 128.
     const bool wide = p.n_pad > 128;
     const int nb = p.n_pad * (p.comp && !wide ? 2 : 1);       // MMA N
     if (nb > 256 || p.n_pad < 16 || p.n_pad % 16 || (wide && (!p.pairs || !p.comp || p.n_pad != 256))) return cudaErrorInvalidValue;

@@ -22,7 +22,7 @@ struct GemmDesc {
                              // or nullptr: row-major weights through the tensor map
     int up_tile_offset;      // first tile of the up projection in the tiled sequence
     int w4;                  // 1: w_tiled holds INT4 tiles (pack.cu, 4224 bytes per tile and k-block) that the kernel
-                             // turns into bf16 tiles in shared memory on their way to the MMA
+                             // expands to bf16 in tensor memory, where the MMA reads them
     EpiParams ep;
 };
 

@@ -2,11 +2,12 @@
 //
 // The fp32 configuration is a small model: a pass is a chain of 5 L + 3 steps of a microsecond or two each. As
 // one kernel per step it was bound by the hand-over between kernels and by steps that kept few loads in flight
-// (2 layers, d 256: 33 kernels, 194 us at 15 nodes; 2.1 ms at 128 nodes and 2000 prefix keys). Here one CTA per
+// (2 layers, d 256: 33 kernels, 203 us at 15 nodes; 2.4 ms at 128 nodes and 2000 prefix keys). Here one CTA per
 // SM stays for the whole pass, steps are separated by grid barriers (1.1-1.3 us each on 148 SMs, the slowest
 // CTA's lead included), and what a step can fetch without the previous one, its first weights, it requests
-// before the barrier: 54 us and 0.36 ms. What bounds it now is latency: a GEMM step is a barrier, one round trip
-// to L2 for its input rows, ~1 us of arithmetic, and the stores.
+// before the barrier: 59 us and 0.35 ms (4 layers of d 512 to 2048, 1 to 128 nodes: 1.3 to 23 times as fast;
+// level at d 4096 with one node and a short prefix). What bounds it now is latency: a GEMM step is a barrier, one
+// round trip to L2 for its input rows, ~1 us of arithmetic, and the stores.
 //
 //   GEMM steps    input rows are staged in shared memory (RMSNorm gain applied and sums of squares taken on the
 //                 way in; the norm factor multiplies the finished sums). A warp owns two output rows (a rotary
