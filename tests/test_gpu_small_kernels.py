@@ -82,7 +82,25 @@ def test_one_kernel_fp32_pass(P, n, H, hd, f, V):
     assert tw.v.launch_count() - l0 == 2
 
 
-@pytest.mark.parametrize("n_out,n_in,n", [(128, 64, 64), (300, 520, 64), (640, 128, 96), (257, 72, 128), (4096, 1000, 120), (9600, 4096, 128)])
+def ctas_of_next_gemm(v, run):
+    """CTAs of the streaming kernel in the one GEMM that run() launches, by their time stamps."""
+    trace = torch.zeros(1, 256, 16, dtype=torch.int64, device=DEV)
+    v.set_gemm_trace(trace)
+    y = run()
+    torch.cuda.synchronize()
+    v.set_gemm_trace(None)
+    assert v.last_status() == 0
+    return y, int((trace[0, :, 0] != 0).sum())
+
+
+def pair_plan(n_out, n_in):
+    """CTAs when pairs of them share items of (two weight tiles, two k-blocks)."""
+    items = -(-n_out // 256) * -(-n_in // 128)
+    groups = min(torch.cuda.get_device_properties(0).multi_processor_count // 2, items)
+    return 2 * -(-items // -(-items // groups))
+
+
+@pytest.mark.parametrize("n_out,n_in,n", [(128, 64, 96), (100, 136, 128), (300, 520, 128), (640, 128, 96), (257, 72, 128), (4096, 1000, 120), (9600, 4096, 128)])
 def test_gemm_on_cta_pairs(n_out, n_in, n):
     """Weight tiles paired over two CTAs: one tile only (its pair is empty), an odd number of them, a ragged last
     k-block, an odd number of k-blocks, half of the activation rows per CTA. bf16 inputs, fp32 sums: the error of
@@ -93,9 +111,29 @@ def test_gemm_on_cta_pairs(n_out, n_in, n):
     g = torch.Generator(device=DEV).manual_seed(n_out + n_in + n)
     w = torch.randn(n_out, n_in, generator=g, device=DEV).to(torch.bfloat16)
     x = torch.randn(n, n_in, generator=g, device=DEV).to(torch.bfloat16)
-    y = v.skinny_gemm_tiled(v.tile_weight(w), n_out, x)
-    assert v.last_status() == 0
+    tiled = v.tile_weight(w)
+    y, ctas = ctas_of_next_gemm(v, lambda: v.skinny_gemm_tiled(tiled, n_out, x))
+    assert ctas == pair_plan(n_out, n_in)
     ref = x.double() @ w.double().t()
+    assert (y.double() - ref).abs().max() <= 2e-6 * n_in ** 0.5 * ref.abs().max()
+
+
+@pytest.mark.parametrize("n_out,n_in,n", [(128, 64, 96), (100, 192, 128), (300, 576, 128), (640, 128, 96), (4096, 1088, 120)])
+def test_int4_gemm_cut_for_cta_pairs(n_out, n_in, n):
+    """The INT4 GEMM deals its tiles out as the bf16 GEMM does on CTA pairs, at the same edges: bit for bit the bf16 GEMM
+    over the dequantised weights, and that within the bound above."""
+    cfg = gen.ModelConfig("g", 0, 256, 2, 128, 256, 512, "bf16")
+    v = B.Verifier(cfg, 16)
+    g = torch.Generator(device=DEV).manual_seed(n_out + n_in + n)
+    w = torch.randn(n_out, n_in, generator=g, device=DEV).to(torch.bfloat16)
+    x = torch.randn(n, n_in, generator=g, device=DEV).to(torch.bfloat16)
+    q, e = B.quantize_int4(w)
+    wq = (q.view(n_out, -1, 64).double() * torch.exp2(e.double())[:, :, None]).view(n_out, n_in).to(torch.bfloat16)
+    packed, tiled = v.tile_weight_int4(w), v.tile_weight(wq)
+    y, ctas = ctas_of_next_gemm(v, lambda: v.skinny_gemm_tiled_int4(packed, n_out, x))
+    assert ctas == pair_plan(n_out, n_in)
+    assert torch.equal(y, v.skinny_gemm_tiled(tiled, n_out, x))
+    ref = x.double() @ wq.double().t()
     assert (y.double() - ref).abs().max() <= 2e-6 * n_in ** 0.5 * ref.abs().max()
 
 
