@@ -129,7 +129,7 @@ typedef struct {
 typedef struct {
     float *logits;          /* [N][vocab] or NULL */
     int32_t *argmax;        /* [N] */
-    int32_t *accepted_path; /* [N]: the path, then -1 */
+    int32_t *accepted_path; /* [N]: the path, then 0 */
     int32_t *scalars;       /* [8] */
 } llmcad_host_result;
 

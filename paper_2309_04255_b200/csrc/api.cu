@@ -828,7 +828,7 @@ int llmcad_verify_tree_host(llmcad_ctx *ctx, const void *packed, void *kv_cache,
     dev.argmax = ctx->argmax_dev();
     dev.accepted_path = ctx->path_dev();
     dev.scalars = ctx->scalars_dev();
-    rc = verify_tree(ctx, packed, kv_cache, prefix_len, ctx->tokens_dev(), ctx->parent_dev(), n, &dev, n, stream);
+    rc = verify_tree(ctx, packed, kv_cache, prefix_len, ctx->tokens_dev(), ctx->parent_dev(), n, &dev, 0, stream);
     if (rc != LLMCAD_OK) return rc;
     // argmax[128], path[128] and scalars[8] are contiguous in the context's integer buffer
     CUDA_TRY(cudaMemcpyAsync(out->argmax, ctx->argmax_dev(), n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -837,6 +837,8 @@ int llmcad_verify_tree_host(llmcad_ctx *ctx, const void *packed, void *kv_cache,
     if (out->logits != nullptr)
         CUDA_TRY(cudaMemcpyAsync(out->logits, ctx->logits, (size_t)n * ctx->cfg.vocab * sizeof(float), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
+    const int32_t len = out->scalars[LLMCAD_S_ACCEPTED_LEN];
+    for (int32_t k = len < 0 ? 0 : len; k < n; ++k) out->accepted_path[k] = 0;     // not an earlier call's path
     return LLMCAD_OK;
 }
 

@@ -32,7 +32,7 @@ def host_buffers(n, vocab):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_host_entry_returns_the_verified_path(dtype):
     """llmcad_verify_tree_host on trees of which several levels are accepted, two different ones in a row on one context:
-    all n entries of the path, -1 behind it, and nothing past them; everything else as the device entry gives it. A
+    all n entries of the path, 0 behind it, and nothing past them; everything else as the device entry gives it. A
     refused tree gives an empty path."""
     cfg, P = SMALL[dtype], 40
     twin = Twin(cfg, P + 40, scale=3.0)
@@ -49,14 +49,14 @@ def test_host_entry_returns_the_verified_path(dtype):
         twin.v.verify_tree_host(P, torch.as_tensor(tokens).pin_memory(), torch.as_tensor(parent).pin_memory(), host)
         for k in ("logits", "argmax", "scalars"):
             assert np.array_equal(host[k].numpy(), dev[k]), k
-        assert host["accepted_path"].tolist() == acc.path.tolist() + [-1] * (n - acc.accepted_len) + [77] * 3
+        assert host["accepted_path"].tolist() == acc.path.tolist() + [0] * (n - acc.accepted_len) + [77] * 3
     assert len(lengths) == 2
     bad = parent.copy()
     bad[2] = 2
     host = host_buffers(n, cfg.vocab)
     twin.v.verify_tree_host(P, torch.as_tensor(tokens).pin_memory(), torch.as_tensor(bad).pin_memory(), host)
     assert host["scalars"].tolist() == [0, -1, P, 0, 0, 0, B.ERR_BAD_TREE, 0]
-    assert host["accepted_path"].tolist() == [-1] * n + [77] * 3
+    assert host["accepted_path"].tolist() == [0] * n + [77] * 3
 
 
 def test_paths_stay_inside_the_callers_buffers():
