@@ -76,7 +76,7 @@ __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile i
     if (mbar_try(bar, parity)) return true;
     uint64_t t0 = 0;
     for (uint32_t it = 1;; ++it) {
-        __nanosleep(20);
+        __nanosleep(20);      // (the producer only: 35.8 us with and without at 8192 keys and 128 nodes)
         if (mbar_try(bar, parity)) return true;
         if ((it & 255u) == 0) {
             if (*abort_flag) return false;

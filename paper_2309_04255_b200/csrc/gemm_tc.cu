@@ -1303,7 +1303,7 @@ gemm_w4_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                     t_idle = 0;
                     continue;
                 }
-                __nanosleep(32);
+                __nanosleep(32);      // (a pass of the 7B shape takes 2319 us with and 2318 without it: the expansion paces it, not this thread)
                 if (t_idle == 0) t_idle = global_timer_ns();
                 else if (*abort_flag || global_timer_ns() - t_idle > wait_limit) { timed_out = true; break; }
             }
