@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "gemm_tc.cuh"
 #include "pass_small.cuh"
+#include "pass_stream.cuh"
 
 using namespace llmcad;
 
@@ -117,6 +118,10 @@ struct llmcad_ctx {
     TreeBuffers tb{};
     // the one-kernel fp32 pass (pass_small.cu): allowed, and its own workspaces
     bool small_pass = false;
+    // the one-kernel bf16 pass over few nodes (pass_stream.cu): allowed, and its own workspaces
+    bool stream_pass = false;
+    float *st_qkv = nullptr, *st_part = nullptr, *st_ssq = nullptr;
+    uint32_t *st_bar = nullptr;
     bool wide_chunks = false;      // prefill: chunks of kLoRows tokens
     float *sp_att = nullptr;
     float2 *sp_ml = nullptr;
@@ -342,6 +347,9 @@ bool use_small_pass(const llmcad_ctx *ctx, int n_keys);
 SmallPass small_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent,
                             int n_tree, int n_old, float *logits, int32_t *status, bool keep_status);
 int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st);
+bool use_stream_pass(const llmcad_ctx *ctx, int n);
+bool stream_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent, int n_tree,
+                        int n_old, float *logits, int32_t *status, bool keep_status, bool last_row, StreamPass &p);
 
 // Decoder forward over the nodes n_old .. n_tree-1 of a tree of n_tree nodes (all of them when
 // n_old = 0): tree prep of the whole tree, embedding, all layers; K/V of node i go to cache slot
@@ -362,6 +370,12 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
     int rc;
     if (use_small_pass(ctx, P + n_tree))
         return run_small_pass(ctx, small_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status), st);
+    StreamPass sp;
+    if (use_stream_pass(ctx, n) && stream_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status, last_row, sp)) {
+        ctx->launches++;
+        CUDA_TRY(launch_stream_pass(sp, ctx->n_sms, st));
+        return LLMCAD_OK;
+    }
     if ((rc = ensure_weight_maps(ctx, packed, n_pad)) != LLMCAD_OK) return rc;
     if ((rc = ensure_act_maps(ctx, n_pad)) != LLMCAD_OK) return rc;
 
@@ -544,6 +558,36 @@ int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st)
     return LLMCAD_OK;
 }
 
+// Whether n new nodes go through the one kernel of pass_stream.cu (measuring launches one by one needs the others).
+bool use_stream_pass(const llmcad_ctx *ctx, int n)
+{
+    return ctx->stream_pass && !ctx->use_counters && !ctx->timing && ctx->trace == nullptr && stream_pass_prefers(n);
+}
+
+bool stream_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent, int n_tree,
+                        int n_old, float *logits, int32_t *status, bool keep_status, bool last_row, StreamPass &p)
+{
+    const llmcad_config &c = ctx->cfg;
+    const PackedLayout &y = ctx->lay;
+    p = StreamPass{};
+    p.L = c.n_layers; p.d = c.d_model; p.H = c.n_heads; p.f = c.d_ffn; p.V = c.vocab; p.S = c.max_seq;
+    p.eps = c.rms_eps;
+    p.base = static_cast<const char *>(packed);
+    p.w_off[SG_QKV] = y.wqkv; p.w_off[SG_O] = y.wo; p.w_off[SG_GU] = y.wgu; p.w_off[SG_DOWN] = y.wdown; p.w_off[SG_HEAD] = y.lm_head;
+    p.g[SG_GU].upper = tiled_weight_bytes(c.d_ffn, c.d_model);
+    p.attn_norm = y.attn_norm; p.ffn_norm = y.ffn_norm; p.layer_bytes = y.layer_bytes; p.tok_embed = y.tok_embed; p.final_norm = y.final_norm;
+    p.kv = static_cast<char *>(kv_cache);
+    p.inv_freq = ctx->inv_freq;
+    p.tokens = tokens; p.parent = parent; p.P = P; p.n_tree = n_tree; p.n_old = n_old;
+    p.xn = ctx->xn; p.att = ctx->att; p.h = ctx->h;
+    p.qkv = ctx->st_qkv; p.part = ctx->st_part; p.ssq = ctx->st_ssq; p.bar = ctx->st_bar;
+    p.logits = logits;
+    p.head_first = logits != nullptr && last_row ? n_tree - n_old - 1 : 0;
+    p.status = status; p.keep_status = keep_status ? 1 : 0;
+    p.wait_limit_ns = ctx->wait_limit_ns;
+    return plan_stream_pass(p, ctx->n_sms);
+}
+
 int check_pass_args(const llmcad_ctx *ctx, const void *packed, const void *kv, int P, const void *tok, const void *par, int n)
 {
     if (ctx == nullptr || packed == nullptr || kv == nullptr || tok == nullptr || par == nullptr) return LLMCAD_ERR_INVALID_ARG;
@@ -677,6 +721,14 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
             want((void **)&ctx->sp_best, 128 * 8);
             want((void **)&ctx->sp_bar, 2 * 4);
         }
+    }
+    ctx->stream_pass = ctx->tc_gemm && ctx->comp && ctx->tc_attn && cfg->flags == 0 && cfg->n_layers > 0 &&
+                       stream_pass_serves(cfg->d_model, cfg->d_ffn, cfg->head_dim, cfg->n_heads, cfg->vocab, ctx->n_sms);
+    if (ctx->stream_pass) {
+        want((void **)&ctx->st_qkv, stream_pass_floats_qkv(cfg->d_model) * 4);
+        want((void **)&ctx->st_part, stream_pass_floats_part(ctx->n_sms) * 4);
+        want((void **)&ctx->st_ssq, (size_t)2 * kStreamMaxNodes * ctx->n_sms * 4);
+        want((void **)&ctx->st_bar, (size_t)(2 + cfg->n_heads) * 4);
     }
     const size_t ssq_floats = (size_t)4 * ((d + 127) / 128) * kLoRows;
     want((void **)&ctx->ssq[0], ssq_floats * 4);

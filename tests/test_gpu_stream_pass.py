@@ -1,0 +1,92 @@
+"""The one-kernel bf16 pass over few nodes (pass_stream.cu) against the oracle, at the edges of how it cuts its work: models
+with fewer pairs of rows than CTAs, K that ends inside a k-block, an odd vocabulary, rows of a CTA on both sides of a weight
+tile, prefixes around a tile of 32 keys, trees whose first nodes are in the cache already, prompts of a few tokens."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2309_04255_b200 import binding as B
+from paper_2309_04255_b200 import inputs as gen
+
+from gpu_util import BF16_TOL, Twin, argmax_agrees_where_decided, check_acceptance_against_oracle, logits_close
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+MODELS = {"one-head": gen.ModelConfig("one-head", 1, 128, 1, 128, 352, 512, "bf16"),
+          "odd": gen.ModelConfig("odd", 3, 640, 5, 128, 1376, 2051, "bf16"),
+          "small": gen.ModelConfig("small", 2, 512, 4, 128, 1408, 2048, "bf16"),
+          "7b": gen.shrink(gen.MODELS["7b"], 1), "30b": gen.shrink(gen.MODELS["30b"], 1)}
+# hi + lo activations keep 16 bits and the logits some 1e-5; K and V of a pass's own nodes are rounded to bf16 only in the
+# cache, where earlier nodes of a tree are read back (2^-9 each)
+TOL = 1e-3
+
+
+def tree(n, seed):
+    return gen.tree_random(n, 4, "uniform4", seed) if n > 1 else np.array([-1], np.int32)
+
+
+@pytest.mark.parametrize("model,P,n", [("one-head", 0, 1), ("one-head", 31, 4), ("odd", 33, 3), ("odd", 1, 2), ("odd", 300, 4), ("small", 0, 4),
+                                       ("small", 32, 1), ("small", 100, 3), ("7b", 33, 1), ("7b", 128, 4), ("30b", 40, 2)])
+def test_pass_over_few_nodes(model, P, n):
+    cfg = MODELS[model]
+    tw = Twin(cfg, P + n + 40, scale=3.0 if cfg.d_model < 1024 else 1.0, seed=n)
+    tw.fill_prefix_synthetic(P)
+    parent, tokens = tree(n, P), gen.gen_tokens(cfg, n, P)
+    ref = tw.oracle_pass(P, tokens, parent)
+    before, launches = tw.v.kv_view().clone(), tw.v.launch_count()
+    out = tw.gpu_pass(P, tokens, parent)
+    assert tw.v.launch_count() - launches == 3        # the pass, argmax, search: this kernel, not the one per step
+    logits_close(out["logits"], ref.logits, TOL)
+    argmax_agrees_where_decided(out["argmax"], ref.logits, BF16_TOL)
+    acc = check_acceptance_against_oracle(out, tokens, parent)
+    after = tw.v.kv_view()
+    assert torch.equal(after[:, :, :, :P], before[:, :, :, :P]) and torch.equal(after[:, :, :, P + n:], before[:, :, :, P + n:])
+    for layer in range(cfg.n_layers):
+        for which, rows in ((0, ref.tree_k[layer]), (1, ref.tree_v[layer])):
+            want = rows[acc.path].reshape(acc.accepted_len, cfg.n_heads, cfg.head_dim).transpose(1, 0, 2)
+            have = after[layer, which, :, P:P + acc.accepted_len].double().cpu().numpy()
+            assert np.abs(have - want).max() <= 2 ** -8 * np.abs(want).max()
+    again = tw.gpu_pass(P, tokens, parent)
+    assert np.array_equal(again["logits"], out["logits"]) and np.array_equal(again["scalars"], out["scalars"])
+
+
+@pytest.mark.parametrize("model,P,cuts", [("odd", 30, [3, 4, 8, 9]), ("small", 300, [30, 33, 70, 74]), ("7b", 40, [1, 5, 8])])
+def test_extension_by_few_nodes(model, P, cuts):
+    """A tree grown by one to four nodes per call behind calls of any size: earlier nodes are keys with a mask."""
+    cfg = MODELS[model]
+    n = cuts[-1]
+    tw = Twin(cfg, P + n + 8, scale=3.0 if cfg.d_model < 1024 else 1.0)
+    tw.fill_prefix_synthetic(P)
+    parent, tokens = gen.tree_random(n, 12, "uniform4", n), gen.gen_tokens(cfg, n)
+    ref = tw.oracle_pass(P, tokens, parent)
+    old = 0
+    for m in cuts:
+        out = tw.v.extend_tree(P, torch.as_tensor(tokens[:m], device=DEV), torch.as_tensor(parent[:m], device=DEV), old, top_k=2)
+        assert out["status"].item() == 0
+        logits_close(out["logits"].cpu().numpy(), ref.logits[old:m], BF16_TOL)
+        old = m
+
+
+@pytest.mark.parametrize("P,n", [(0, 1), (0, 4), (257, 2), (30, 131)])
+def test_prompts_that_are_or_end_in_few_tokens(P, n):
+    """The last row's logits and the cache of a prompt of a few tokens, or whose last chunk is (131 = 128 + 3 where chunks
+    are of 128 tokens), as one pass over the same chain gives them."""
+    cfg = MODELS["small"]
+    tw = Twin(cfg, P + n + 8, scale=3.0, keep_host=False)
+    tw.fill_prefix_synthetic(P)
+    tokens = torch.as_tensor(gen.gen_tokens(cfg, n), device=DEV)
+    last = tw.v.prefill(P, tokens, want_logits=True)
+    assert tw.v.last_status() == 0
+    cache = tw.v.kv_view()[:, :, :, :P + n].clone()
+    # the same prompt in two calls, cut elsewhere
+    if n > 1:
+        tw.v.prefill(P, tokens[:n - 1])
+        again = tw.v.prefill(P + n - 1, tokens[n - 1:], want_logits=True)
+        logits_close(again.cpu().numpy()[None], last.double().cpu().numpy()[None], BF16_TOL)
+        d = (tw.v.kv_view()[:, :, :, :P + n].double() - cache.double()).abs().max().item()
+        assert d <= BF16_TOL * cache.double().abs().max().item()
+    bad = tokens.clone()
+    bad[-1] = cfg.vocab
+    tw.v.prefill(P, bad)
+    assert tw.v.last_status() == B.ERR_BAD_TOKEN
