@@ -1702,7 +1702,7 @@ GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool
 namespace {
 // tuning aids from the environment, read once per process
 struct Tuning {
-    int pair_k = 0, stages_cap = 0, w4_xstages = kMaxXStages, w4_pstages = kMaxPStages, cta_pair_min = 80;
+    int pair_k = 0, stages_cap = 0, w4_xstages = kMaxXStages, w4_pstages = kMaxPStages, cta_pair_min = 64;
     Tuning()
     {
         if (const char *e = getenv("LLMCAD_GEMM_PAIR_K")) { const int v = atoi(e); if (v == 1 || v == 2) pair_k = v; }
@@ -1719,10 +1719,10 @@ const Tuning &tuning()
 }
 }  // namespace
 
-// Pairs from 80 nodes on. Measured in passes of 16 layers of the 7B shape and 10 of the 13B shape against one kernel per
+// Pairs from 64 nodes on. Measured in passes of 16 layers of the 7B shape and 10 of the 13B shape against one kernel per
 // CTA: 16 and 32 nodes 3-6 % slower (the two cluster barriers at either end of the kernel sit in every hand-over), 45
-// nodes 1 % slower at 7B and 1 % faster at 13B, 64 nodes 1-3 % faster, 80 nodes 1.5-2.4 %, 128 nodes 7 %. The MMA's N has
-// to be a multiple of 32.
+// nodes 1-2 % slower at 7B and 1-2 % faster at 13B, 64 nodes level at 7B (1745 / 1750 us), 3-4 % faster at 13B (1650 /
+// 1590) and 30B widths (12 layers: 2890 / 2815), 80 nodes 1.5-2.4 %, 128 nodes 7 %. The MMA's N has to be a multiple of 32.
 bool gemm_takes_pairs(int n_pad, bool comp)
 {
     if (n_pad > 128) return true;
