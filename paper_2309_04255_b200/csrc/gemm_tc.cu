@@ -1735,14 +1735,21 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
     const Tuning &tune = tuning();
     // Ring items of two k-blocks (one 32 KB weight copy each) unless the activation tiles are so wide
     // (hi | lo planes of more than 64 nodes) that only two stages would fit. Measured on B200 in passes of 16 layers
-    // of the 7B shape: single k-blocks cost 1.4 % at 1 and 16 nodes and 0.5 % at 32, are level at 45 and 64 (there 13B
-    // widths gain up to 2 %), and gain 2.3 % at 80 and 128.
+    // of the 7B shape: single k-blocks cost 1.4 % at 1 and 16 nodes and 0.5 % at 32, and gain 2.3 % at 80 and 128. At 33
+    // to 48 nodes three stages of two k-blocks leave 28 KB of shared memory unused, seven of one k-block fill it: 1673 ->
+    // 1652 us (16 layers of the 7B shape, 45 nodes), 1482 -> 1458 (10 of 13B). The work is cut by two k-blocks there all
+    // the same, so that the sums stay those of the INT4 kernel.
     const bool wide = p.n_pad > 128;
     const int nb = p.n_pad * (p.comp && !wide ? 2 : 1);       // MMA N
     if (nb > 256 || p.n_pad < 16 || p.n_pad % 16 || (wide && (!p.pairs || !p.comp || p.n_pad != 256))) return cudaErrorInvalidValue;
     int pair_k = nb > 128 ? 1 : kMaxPairK;
     if (tune.pair_k && !wide) pair_k = tune.pair_k;
     GemmDesc &d = p.g;
+    int cut = 1;              // items by which the work is cut
+    if (pair_k == 2 && nb >= 96 && !p.pairs && !d.w4 && d.kb_per_tile % 2 == 0) {
+        pair_k = 1;
+        cut = 2;
+    }
     d.pair_k = pair_k;
     // the items are split evenly over one CTA (CTA pair) per SM (two SMs), fewer when there are fewer items
     d.group = p.pairs ? 2 : 1;
@@ -1750,8 +1757,8 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
     const long long total = (long long)(p.pairs ? (vtiles + 1) / 2 : vtiles) * pairs_per_tile(d);
     if (total < 1) return cudaErrorInvalidValue;
     long long groups = n_sms / d.group;
-    if (groups > total) groups = total;
-    const long long ipc = (total + groups - 1) / groups;
+    if (groups > total / cut) groups = total / cut;
+    const long long ipc = (total / cut + groups - 1) / groups * cut;
     d.items_per_cta = (int)ipc;
     d.grid = (int)((total + ipc - 1) / ipc) * d.group;
     return cudaSuccess;
