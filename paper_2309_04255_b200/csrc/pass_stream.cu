@@ -570,21 +570,40 @@ __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, 
     else meet(e, c);           // the scratch may be written again
 }
 
-// Merges partial attention rows: out = sum_s O_s 2^(m_s - M), l likewise, for four dims of one row.
+// Merges partial attention rows: out = sum_s O_s 2^(m_s - M), l likewise, for four dims of one row; four rows' loads at a
+// time are under way together.
 template <typename Row>
 __device__ __forceinline__ float4 merge_rows(int count, Row row, int dim, float &M, float &L)
 {
     M = -INFINITY;
     L = 0.f;
-    for (int s = 0; s < count; ++s) M = fmaxf(M, row(s, kHdim).x);
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < count; ++s) {
-        const float4 ml = row(s, kHdim);
-        if (ml.x == -INFINITY) continue;
-        const float w = exp2f(ml.x - M);
-        const float4 v = row(s, dim);
-        L += ml.y * w;
-        a.x += v.x * w; a.y += v.y * w; a.z += v.z * w; a.w += v.w * w;
+    for (int s0 = 0; s0 < count; s0 += 4) {
+        float4 v[4], ml[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int s = min(s0 + u, count - 1);
+            ml[u] = row(s, kHdim);
+            v[u] = row(s, dim);
+        }
+        float mx = M;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (s0 + u >= count) ml[u].x = -INFINITY;
+            mx = fmaxf(mx, ml[u].x);
+        }
+        if (mx == -INFINITY) continue;                       // no key that these rows see
+        const float old = exp2f(M - mx);
+        M = mx;
+        L *= old;
+        a.x *= old; a.y *= old; a.z *= old; a.w *= old;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (ml[u].x == -INFINITY) continue;              // (its outputs were never written)
+            const float w = exp2f(ml[u].x - M);
+            L += ml[u].y * w;
+            a.x += v[u].x * w; a.y += v[u].y * w; a.z += v[u].z * w; a.w += v[u].w * w;
+        }
     }
     return a;
 }
@@ -831,23 +850,19 @@ __device__ __forceinline__ bool load_inputs(const StreamPass &p, Ctl &ctl, uint3
         const int k32_bytes = 2 * (p.n_tree - p.n_old - (head ? p.head_first : 0)) * 64, x_kb = p.x_stage_bytes / (2 * k32_bytes);
         const char *src = static_cast<const char *>(kind == SG_O ? p.att : kind == SG_DOWN ? p.h : p.xn);
         if (++step == 5) step = 0;
-        // Polls only once this CTA has arrived itself, and with relaxed loads: an acquire at every poll slows the
-        // shared-memory loads of the whole SM down, threefold while the main loop of a phase runs.
+        // Polls only once this CTA has arrived itself: every poll takes L1 along.
         const bool first = ph <= 5 * p.L;                     // the parts of the lm_head have the same input
         if (first && !thread_wait(smem_u32(&ctl.gone), ph & 1u, ctl, p.wait_limit_ns)) return false;
         target += first ? gridDim.x : 0;
         uint64_t t0 = 0;
-        uint32_t seen;
-        for (uint32_t it = 1; first; ++it) {
-            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(p.bar) : "memory");
-            if (seen >= target) break;
+        for (uint32_t it = 1; first && ld_acquire_gpu_u32(p.bar) < target; ++it) {
             if ((it & 63u) == 0) {
                 const uint64_t now = global_timer_ns();
                 if (t0 == 0) t0 = now;
                 else if (ctl.abort_flag || now - t0 > p.wait_limit_ns) return false;
             }
         }
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        if (first) mbar_arrive(smem_u32(&ctl.ready));
         asm volatile("fence.proxy.async;" ::: "memory");      // the input was written by ordinary stores
         for (int kb = 0; kb < n_kb; kb += x_kb, ++xs) {
             const int st = xs % kXStages;
@@ -857,9 +872,7 @@ __device__ __forceinline__ bool load_inputs(const StreamPass &p, Ctl &ctl, uint3
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"(x_ring + st * p.x_stage_bytes), "l"(src + (size_t)(2 * kb) * k32_bytes), "r"(bytes), "r"(full)
                          : "memory");
-            if (kb == 0 && first) mbar_arrive(smem_u32(&ctl.ready));
         }
-        if (n_kb == 0 && first) mbar_arrive(smem_u32(&ctl.ready));
     }
     return true;
 }
