@@ -209,7 +209,7 @@ struct TimedLaunch {
 int ensure_weight_maps(llmcad_ctx *ctx, const void *packed, int n_pad)
 {
     ctx->maps_for = packed;
-    if (!ctx->tc_gemm || ctx->weight_maps_for == packed || !gemm_takes_pairs(n_pad, ctx->comp)) return LLMCAD_OK;
+    if (!ctx->tc_gemm || ctx->weight_maps_for == packed || !gemm_takes_pairs(n_pad, ctx->comp, ctx->cfg.d_model)) return LLMCAD_OK;
     const llmcad_config &c = ctx->cfg;
     const int d = c.d_model, f = c.d_ffn;
     const char *base = static_cast<const char *>(packed);
@@ -241,7 +241,7 @@ int ensure_act_maps(llmcad_ctx *ctx, int n_pad)
         const int cols = i == 2 ? c.d_ffn : c.d_model;
         if (n_pad <= LLMCAD_MAX_TREE) ok &= make_act_map_bf16(&ctx->act_maps[slot][i], bufs[i], ctx->rows, cols, n_pad, planes, kLoRows, planes);
         // a CTA pair: one plane, or half of the rows of the only plane
-        if (gemm_takes_pairs(n_pad, ctx->comp))
+        if (gemm_takes_pairs(n_pad, ctx->comp, ctx->cfg.d_model))
             ok &= n_pad > LLMCAD_MAX_TREE
                       ? make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], ctx->rows, cols, n_pad / 2, planes, kLoRows, planes)    // half of the rows, both planes
                       : make_act_map_bf16(&ctx->pair_maps[slot][i], bufs[i], ctx->rows, cols, ctx->comp ? n_pad : n_pad / 2, planes, kLoRows, 1);
@@ -271,7 +271,7 @@ struct TcGemm {
     void set(llmcad_ctx *ctx, int l, int which, int act, int n_in, const EpiParams &ep, int n_pad)
     {
         const bool w4 = ctx->w4 && l >= 0;
-        p.pairs = gemm_takes_pairs(n_pad, ctx->comp);
+        p.pairs = gemm_takes_pairs(n_pad, ctx->comp, ctx->cfg.d_model);
         maps.x = p.pairs && !w4 ? ctx->pair_maps[n_pad / 16][act] : ctx->act_maps[n_pad / 16][act];
         if (p.pairs && !w4) maps.w = l < 0 ? ctx->weight_maps.back() : ctx->weight_maps[4 * (size_t)l + which];
         p.g = make_gemm_desc(n_in, ep, weight_ptr(ctx, l, which), w4);
@@ -1059,7 +1059,7 @@ int llmcad_skinny_gemm_tiled(llmcad_ctx *ctx, const void *w_tiled, const void *x
     ep.mode = EPI_PLAIN; ep.n = n; ep.n_out = n_out; ep.y = y; ep.ldy = n_out;
     const int n_pad = (n + 15) / 16 * 16;
     TcGemm g;
-    g.p.pairs = gemm_takes_pairs(n_pad, false);
+    g.p.pairs = gemm_takes_pairs(n_pad, false, 0);
     if (!make_act_map_bf16(&g.maps.x, x, n, n_in, g.p.pairs ? n_pad / 2 : n_pad, 1, n, 1) ||
         (g.p.pairs && !make_packed_map(&g.maps.w, w_tiled, tiled_weight_bytes(n_out, n_in)))) {
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
@@ -1111,7 +1111,7 @@ int llmcad_skinny_gemm_tiled_int4(llmcad_ctx *ctx, const void *w_tiled, const vo
         snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
         return LLMCAD_ERR_CUDA;
     }
-    g.p.pairs = gemm_takes_pairs(n_pad, false);
+    g.p.pairs = gemm_takes_pairs(n_pad, false, 0);
     g.p.g = make_gemm_desc(n_in, ep, w_tiled, true);
     g.p.n_pad = n_pad;
     return g.launch(ctx, status, st);

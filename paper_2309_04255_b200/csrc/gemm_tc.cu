@@ -1702,7 +1702,7 @@ GemmDesc make_gemm_desc(int n_in, const EpiParams &ep, const void *w_tiled, bool
 namespace {
 // tuning aids from the environment, read once per process
 struct Tuning {
-    int pair_k = 0, stages_cap = 0, w4_xstages = kMaxXStages, w4_pstages = kMaxPStages, cta_pair_min = 64;
+    int pair_k = 0, stages_cap = 0, w4_xstages = kMaxXStages, w4_pstages = kMaxPStages, cta_pair_min = -1;
     Tuning()
     {
         if (const char *e = getenv("LLMCAD_GEMM_PAIR_K")) { const int v = atoi(e); if (v == 1 || v == 2) pair_k = v; }
@@ -1719,15 +1719,18 @@ const Tuning &tuning()
 }
 }  // namespace
 
-// Pairs from 64 nodes on. Measured in passes of 16 layers of the 7B shape and 10 of the 13B shape against one kernel per
-// CTA: 16 and 32 nodes 3-6 % slower (the two cluster barriers at either end of the kernel sit in every hand-over), 45
-// nodes 1-2 % slower at 7B and 1-2 % faster at 13B, 64 nodes level at 7B (1745 / 1750 us), 3-4 % faster at 13B (1650 /
-// 1590) and 30B widths (12 layers: 2890 / 2815), 80 nodes 1.5-2.4 %, 128 nodes 7 %. The MMA's N has to be a multiple of 32.
-bool gemm_takes_pairs(int n_pad, bool comp)
+// Pairs from 65 nodes on (80 padded), and from 49 on (64 padded) in passes of models at least 4096 wide. Against one
+// kernel per CTA, whole passes: 16 and 32 nodes 3-6 % slower (the two cluster barriers at either end of the kernel sit in
+// every hand-over), 45 nodes 1-2 % slower at 7B and 1-2 % faster at 13B, 80 nodes 1.5-2.4 % faster, 128 nodes 7 %. At 49 and
+// 64 nodes it is the width that decides (us, pairs / not, 3 or 4 layers): d 512 182.6 / 170.2 and 180.3 / 168.4, d 2048 282.8 /
+// 270.5 and 282.8 / 271.6, d 3072 361.1 / 353.2 and 361.8 / 354.5, 7B 502.8 / 499.2 and 500.1 / 508.1, 13B 526.3 / 538.0 and 517.1 /
+// 542.8, 30B 761.7 / 770.0 and 763.5 / 779.5. A GEMM on its own (d_model 0) takes them from 65 on: with 64 nodes 4096 x 4096 would
+// take 18.0 us instead of 16.5, 1536 x 512 12.4 instead of 10.3. The MMA's N has to be a multiple of 32.
+bool gemm_takes_pairs(int n_pad, bool comp, int d_model)
 {
     if (n_pad > 128) return true;
-    const int nb = n_pad * (comp ? 2 : 1);
-    return tuning().cta_pair_min > 0 && n_pad >= tuning().cta_pair_min && nb % 32 == 0;
+    const int nb = n_pad * (comp ? 2 : 1), tuned = tuning().cta_pair_min, least = tuned >= 0 ? tuned : d_model >= 4096 ? 64 : 80;
+    return least > 0 && n_pad >= least && nb % 32 == 0;
 }
 
 cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)

@@ -70,8 +70,9 @@ bool make_act_map_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64
 // Tensor map over a packed weight matrix of `bytes` bytes (a sequence of 16 KB tiles): one box = one tile.
 bool make_packed_map(CUtensorMap *map, const void *tiled, uint64_t bytes);
 
-// Whether a GEMM with bf16 weights on this many (padded) nodes runs on CTA pairs. comp: hi and lo planes.
-bool gemm_takes_pairs(int n_pad, bool comp);
+// Whether a GEMM with bf16 weights on this many (padded) nodes runs on CTA pairs (with INT4 weights: is cut as if it did).
+// comp: hi and lo planes; d_model: the width of the model whose pass it belongs to, 0 for a GEMM on its own.
+bool gemm_takes_pairs(int n_pad, bool comp, int d_model);
 // Any three-dimensional bf16 tensor with 128-byte swizzle and zero fill outside its bounds: dims and box
 // innermost first, strides (bytes) of dimensions 1 and 2.
 bool make_tensor_map_bf16_3d(CUtensorMap *map, const void *base, const uint64_t dims[3], const uint64_t strides_bytes[2],

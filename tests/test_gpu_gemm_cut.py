@@ -1,14 +1,16 @@
 """How the GEMMs of a pass over 33 to 64 nodes cut their work: ring items of one k-block up to 48 nodes, cut by two where K
-has an even number of them, and CTA pairs from 49 on. Whole passes against the oracle, and bit for bit against an INT4
-context, whose kernel is cut the same way and shares no ring with them."""
+has an even number of them, and CTA pairs from 49 on in wide models. Whole passes against the oracle, and bit for bit
+against an INT4 context, whose kernel is cut the same way and shares no ring with them."""
 import numpy as np
 import pytest
 import torch
 
+from paper_2309_04255_b200 import binding as B
 from paper_2309_04255_b200 import inputs as gen
 
 from gpu_util import argmax_agrees_where_decided, check_acceptance_against_oracle, logits_close
 from test_gpu_int4 import Int4Twin
+from test_gpu_small_kernels import ctas_of_next_gemm, pair_plan
 
 pytestmark = pytest.mark.gpu
 
@@ -29,3 +31,39 @@ def test_passes_of_33_to_64_nodes(d, heads, f, n):
     o16 = twin.v16.verify_tree(50, t, p)
     assert np.array_equal(o16["logits"].cpu().numpy(), out["logits"])
     assert np.array_equal(o16["scalars"].cpu().numpy(), out["scalars"])
+
+
+def single_plan(n_out, n_in):
+    """CTAs when each has items of (one weight tile, two k-blocks) of its own."""
+    items = -(-n_out // 128) * -(-n_in // 128)
+    groups = min(torch.cuda.get_device_properties(0).multi_processor_count, items)
+    return -(-items // -(-items // groups))
+
+
+# widths at which the two plans differ in their number of CTAs (148 SMs)
+@pytest.mark.parametrize("d,f,n,pairs", [(640, 1408, 49, False), (640, 1408, 64, False), (1152, 3072, 64, False), (4096, 11008, 49, True), (4096, 11008, 64, True),
+                                         (4096, 11008, 48, False)])
+def test_which_passes_of_up_to_64_nodes_take_cta_pairs(d, f, n, pairs):
+    """Narrow models lose by pairs at 49 to 64 nodes, wide ones gain; by the CTAs of the first QKV GEMM of a pass."""
+    cfg = gen.ModelConfig("width", 1, d, d // 128, 128, f, 1000, "bf16")
+    v = B.Verifier(cfg, n + 16)
+    v.pack_globals({k: gen.gen_tensor_device(cfg, k, -1, v.device) for k in ("tok_embed", "final_norm", "lm_head")})
+    v.pack_layer(0, {k: gen.gen_tensor_device(cfg, k, 0, v.device) for k in gen.LAYER_TENSORS})
+    t, p = (torch.as_tensor(np.asarray(a, np.int32), device=v.device) for a in (gen.gen_tokens(cfg, n, n), gen.tree_random(n, 10, "uniform4", n)))
+    assert single_plan(3 * d, d) != pair_plan(3 * d, d)
+    out, ctas = ctas_of_next_gemm(v, lambda: v.verify_tree(0, t, p))
+    assert out["scalars"][B.S_STATUS].item() == 0
+    assert ctas == (pair_plan if pairs else single_plan)(3 * d, d)
+
+
+@pytest.mark.parametrize("n", [49, 64])
+def test_gemm_on_its_own_takes_no_cta_pairs_up_to_64_nodes(n):
+    n_out, n_in = 640, 640
+    v = B.Verifier(gen.ModelConfig("g", 0, 256, 2, 128, 256, 512, "bf16"), 16)
+    g = torch.Generator(device=v.device).manual_seed(n)
+    w, x = (torch.randn(s, generator=g, device=v.device).to(torch.bfloat16) for s in ((n_out, n_in), (n, n_in)))
+    tiled = v.tile_weight(w)
+    y, ctas = ctas_of_next_gemm(v, lambda: v.skinny_gemm_tiled(tiled, n_out, x))
+    assert ctas == single_plan(n_out, n_in) != pair_plan(n_out, n_in)
+    ref = x.double() @ w.double().t()
+    assert (y.double() - ref).abs().max() <= 2e-6 * n_in ** 0.5 * ref.abs().max()
