@@ -272,6 +272,7 @@ struct TcGemm {
     {
         const bool w4 = ctx->w4 && l >= 0;
         p.pairs = gemm_takes_pairs(n_pad, ctx->comp, ctx->cfg.d_model);
+        p.wide_model = ctx->cfg.d_model >= 3072;
         maps.x = p.pairs && !w4 ? ctx->pair_maps[n_pad / 16][act] : ctx->act_maps[n_pad / 16][act];
         if (p.pairs && !w4) maps.w = l < 0 ? ctx->weight_maps.back() : ctx->weight_maps[4 * (size_t)l + which];
         p.g = make_gemm_desc(n_in, ep, weight_ptr(ctx, l, which), w4);

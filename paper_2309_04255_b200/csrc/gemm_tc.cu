@@ -1740,8 +1740,11 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
     // (hi | lo planes of more than 64 nodes) that only two stages would fit. Measured on B200 in passes of 16 layers
     // of the 7B shape: single k-blocks cost 1.4 % at 1 and 16 nodes and 0.5 % at 32, and gain 2.3 % at 80 and 128. At 33
     // to 48 nodes three stages of two k-blocks leave 28 KB of shared memory unused, seven of one k-block fill it: 1673 ->
-    // 1652 us (16 layers of the 7B shape, 45 nodes), 1482 -> 1458 (10 of 13B). The work is cut by two k-blocks there all
-    // the same, so that the sums stay those of the INT4 kernel.
+    // 1652 us (16 layers of the 7B shape, 45 nodes), 1482 -> 1458 (10 of 13B), d 3072 (4 layers) 339.1 -> 337.4. Narrower models
+    // have too few k-blocks per CTA to gain (d 2560 level, d 2048 261.8 -> 263.4, d 1024 190.2 -> 192.1), and a GEMM on its own
+    // with as many MMA columns loses (1536 x 512, 112 nodes: 10.7 -> 12.0), so both keep two. All GEMMs of a pass take the
+    // same: with the large ones alone on single k-blocks d 3072 takes 341.7. The work is cut by two k-blocks either way, so
+    // that the sums stay those of the INT4 kernel.
     const bool wide = p.n_pad > 128;
     const int nb = p.n_pad * (p.comp && !wide ? 2 : 1);       // MMA N
     if (nb > 256 || p.n_pad < 16 || p.n_pad % 16 || (wide && (!p.pairs || !p.comp || p.n_pad != 256))) return cudaErrorInvalidValue;
@@ -1749,7 +1752,7 @@ cudaError_t plan_gemm_tc(GemmParams &p, int n_sms)
     if (tune.pair_k && !wide) pair_k = tune.pair_k;
     GemmDesc &d = p.g;
     int cut = 1;              // items by which the work is cut
-    if (pair_k == 2 && nb >= 96 && !p.pairs && !d.w4 && d.kb_per_tile % 2 == 0) {
+    if (p.wide_model && p.comp && p.n_pad == 48 && !tune.pair_k && !p.pairs && !d.w4 && d.kb_per_tile % 2 == 0) {
         pair_k = 1;
         cut = 2;
     }

@@ -36,6 +36,7 @@ struct GemmParams {
     int comp;           // 1: activations come as hi + lo planes; the MMA N is 2 * n_pad and the two columns of a node are added
     int pairs;          // 1: items are dealt out to CTA pairs; with bf16 weights (gemm_pair_kernel) maps.w is the packed matrix (make_packed_map), maps.x has boxes of half
                         // of the MMA's rows (gemm_takes_pairs)
+    int wide_model;     // 1: part of a pass of a model at least 3072 wide (plan_gemm_tc)
     int stages;         // depth of the shared-memory ring (INT4 weights: of the ring of expanded items in tensor memory)
     int pstages;        // INT4 weights: depth of the ring of packed items that feeds it
     int astages;        // INT4 weights: depth of the ring of activation items (with bf16 weights they share the weights' stages)

@@ -103,3 +103,30 @@ def check_acceptance_against_oracle(out, tokens, parent):
 def cache_rows(v: B.Verifier, upto: int) -> np.ndarray:
     """[L][2][H][upto][hd] as float64."""
     return v.kv_view()[:, :, :, :upto].double().cpu().numpy()
+
+
+def kernels_of(call):
+    """Names (as the linker sees them) of the kernels that `call` launches, in order: captured into a graph, not run. What
+    `call` sets up on its first run has to be there already."""
+    from cuda.bindings import driver as drv, runtime as rt
+
+    def ok(r):
+        assert int(r[0]) == 0, r[0]
+        return r[1] if len(r) == 2 else r[1:]
+
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(st):
+        ok(rt.cudaStreamBeginCapture(st.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed) + (None,))
+        call()
+        graph = ok(rt.cudaStreamEndCapture(st.cuda_stream))
+    _, count = ok(rt.cudaGraphGetNodes(graph))
+    nodes, _ = ok(rt.cudaGraphGetNodes(graph, count))
+    names = []
+    for node in nodes:
+        if int(ok(rt.cudaGraphNodeGetType(node))) == int(rt.cudaGraphNodeType.cudaGraphNodeTypeKernel):
+            params = ok(drv.cuGraphKernelNodeGetParams(drv.CUgraphNode(int(node))))
+            name = ok(drv.cuFuncGetName(params.func)) if int(params.func) else ok(drv.cuKernelGetName(params.kern))
+            names.append(name.decode())
+    rt.cudaGraphDestroy(graph)
+    return names

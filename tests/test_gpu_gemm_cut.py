@@ -1,5 +1,5 @@
-"""How the GEMMs of a pass over 33 to 64 nodes cut their work: ring items of one k-block up to 48 nodes, cut by two where K
-has an even number of them, and CTA pairs from 49 on in wide models. Whole passes against the oracle, and bit for bit
+"""How the GEMMs of a pass over 33 to 64 nodes cut their work: ring items of one k-block up to 48 nodes in wide models, cut by
+two where K has an even number of them, and CTA pairs from 49 on in wider ones. Whole passes against the oracle, and bit for bit
 against an INT4 context, whose kernel is cut the same way and shares no ring with them."""
 import numpy as np
 import pytest
@@ -8,7 +8,7 @@ import torch
 from paper_2309_04255_b200 import binding as B
 from paper_2309_04255_b200 import inputs as gen
 
-from gpu_util import argmax_agrees_where_decided, check_acceptance_against_oracle, logits_close
+from gpu_util import argmax_agrees_where_decided, check_acceptance_against_oracle, kernels_of, logits_close
 from test_gpu_int4 import Int4Twin
 from test_gpu_small_kernels import ctas_of_next_gemm, pair_plan
 
@@ -33,6 +33,45 @@ def test_passes_of_33_to_64_nodes(d, heads, f, n):
     assert np.array_equal(o16["scalars"].cpu().numpy(), out["scalars"])
 
 
+def small_model(d, f, max_seq):
+    cfg = gen.ModelConfig("width", 1, d, d // 128, 128, f, 1000, "bf16")
+    v = B.Verifier(cfg, max_seq)
+    v.pack_globals({k: gen.gen_tensor_device(cfg, k, -1, v.device) for k in ("tok_embed", "final_norm", "lm_head")})
+    v.pack_layer(0, {k: gen.gen_tensor_device(cfg, k, 0, v.device) for k in gen.LAYER_TENSORS})
+    return cfg, v
+
+
+def tree(v, cfg, n):
+    return (torch.as_tensor(np.asarray(a, np.int32), device=v.device) for a in (gen.gen_tokens(cfg, n, n), gen.tree_random(n, 10, "uniform4", n)))
+
+
+def stream_variants(names):
+    """k-blocks per ring item of the streaming GEMM kernels among `names`."""
+    return sorted({int(n.split("gemm_stream_kernelILi")[1][0]) for n in names if "gemm_stream_kernelILi" in n})
+
+
+@pytest.mark.parametrize("d,f,n,k_blocks", [(512, 1408, 33, 2), (512, 1408, 48, 2), (2048, 5632, 48, 2), (3072, 8192, 33, 1), (3072, 8192, 48, 1), (3072, 8192, 32, 2)])
+def test_which_passes_take_ring_items_of_one_k_block(d, f, n, k_blocks):
+    """Narrow models lose by them at 33 to 48 nodes (the sums are the same either way)."""
+    cfg, v = small_model(d, f, n + 16)
+    t, p = tree(v, cfg, n)
+    out = v.verify_tree(0, t, p)
+    assert out["scalars"][B.S_STATUS].item() == 0
+    assert stream_variants(kernels_of(lambda: v.verify_tree(0, t, p, out=out))) == [k_blocks]
+
+
+@pytest.mark.parametrize("n,tiled", [(48, True), (96, False), (128, False), (112, True)])
+def test_gemm_on_its_own_keeps_ring_items_of_two_k_blocks(n, tiled):
+    """As many columns of the MMA as a pass of 48 nodes and more, and a twentieth to a sixth slower with one."""
+    n_out, n_in = 1536, 512
+    v = B.Verifier(gen.ModelConfig("g", 0, 256, 2, 128, 256, 512, "bf16"), 16)
+    w, x = (torch.randn(s, device=v.device).to(torch.bfloat16) for s in ((n_out, n_in), (n, n_in)))
+    wt = v.tile_weight(w)
+    call = (lambda: v.skinny_gemm_tiled(wt, n_out, x)) if tiled else (lambda: v.skinny_gemm(w, x))
+    call()
+    assert stream_variants(kernels_of(call)) == [2]
+
+
 def single_plan(n_out, n_in):
     """CTAs when each has items of (one weight tile, two k-blocks) of its own."""
     items = -(-n_out // 128) * -(-n_in // 128)
@@ -45,11 +84,8 @@ def single_plan(n_out, n_in):
                                          (4096, 11008, 48, False)])
 def test_which_passes_of_up_to_64_nodes_take_cta_pairs(d, f, n, pairs):
     """Narrow models lose by pairs at 49 to 64 nodes, wide ones gain; by the CTAs of the first QKV GEMM of a pass."""
-    cfg = gen.ModelConfig("width", 1, d, d // 128, 128, f, 1000, "bf16")
-    v = B.Verifier(cfg, n + 16)
-    v.pack_globals({k: gen.gen_tensor_device(cfg, k, -1, v.device) for k in ("tok_embed", "final_norm", "lm_head")})
-    v.pack_layer(0, {k: gen.gen_tensor_device(cfg, k, 0, v.device) for k in gen.LAYER_TENSORS})
-    t, p = (torch.as_tensor(np.asarray(a, np.int32), device=v.device) for a in (gen.gen_tokens(cfg, n, n), gen.tree_random(n, 10, "uniform4", n)))
+    cfg, v = small_model(d, f, n + 16)
+    t, p = tree(v, cfg, n)
     assert single_plan(3 * d, d) != pair_plan(3 * d, d)
     out, ctas = ctas_of_next_gemm(v, lambda: v.verify_tree(0, t, p))
     assert out["scalars"][B.S_STATUS].item() == 0
