@@ -993,8 +993,13 @@ bool plan_stream_pass(StreamPass &p, int n_sms)
 {
     const int n = p.n_tree - p.n_old;
     const int tiles = (p.P + p.n_old + kKeys - 1) / kKeys;
-    p.splits = n_sms / p.H;
-    if (p.splits > tiles) p.splits = tiles > 0 ? tiles : 1;
+    // Key ranges of a head: as many as there are CTAs for, but no fewer than four tiles each, which a CTA's four pairs of warps
+    // take side by side. The last CTA of a head merges its ranges one after the other: with a tile each (us a pass of 4
+    // layers and 4 nodes, a tile / four tiles at least / one kernel per step) 1 head and 4096 keys take 214 / 135 / 155, 2 heads
+    // and 2048 161 / 125 / 144, 4 heads and 512 127 / 123 / 148, 32 heads and 64 367 / 361 / 392. With eight at least, 512 keys
+    // are 3 % slower.
+    const int ranges = tiles > 4 ? (tiles + 3) / 4 : 1;
+    p.splits = n_sms / p.H < ranges ? n_sms / p.H : ranges;
     const int units[SG_KINDS] = {3 * p.d / 2, p.d / 2, p.f, p.d / 2, (p.V + 1) / 2};
     const int K[SG_KINDS] = {p.d, p.d, p.d, p.f, p.d};
     size_t red = 0;
