@@ -14,7 +14,7 @@
 //   warp 12       polls the grid barrier, then copies the phase's input into a ring of its own. Inputs are stored by
 //                 whoever produces them as the B fragments of the MMA: [32 columns of K][node, plane][32], so that a
 //                 lane's 16 bytes serve two MMAs.
-//   warps 0-7     mma.sync m16n8k16: weights on the M side, (node, hi/lo plane) on the N side. Groups of warps take the
+//   warps 0-7     mma.sync m16n8k16: weights on the M side, (node, hi/lo plane) as the eight columns of the N side. Groups of warps take the
 //                 k-blocks in turn; the sums are added in shared memory in a fixed order, and the epilogue (norm factor,
 //                 rotary, K/V write, SwiGLU, residual) runs where they lie. The residual stream stays in shared memory.
 //   attention     (head, key range) per CTA: prefix tiles of 32 keys come through the weight ring, scores and outputs
@@ -338,40 +338,32 @@ struct ATile {
 // A k-block's operands of a warp: M tiles of 16 rows, two times 32 columns (the second is left out where K ends in the
 // middle). Lane (g, t) holds columns 8t .. 8t+7 of 32 on both sides, the first four for one MMA and the others for the
 // next. What lanes of columns and rows that do not exist read (other data of the rings) ends in sums that nobody takes.
-template <int NT, int M>
+template <int M>
 struct Block {
-    uint4 b[2][NT], lo[2][M], up[2][M];
+    uint4 b[2], lo[2][M], up[2][M];
     __device__ __forceinline__ void load(const ATile &at, uint32_t w, uint32_t x, int x_step, bool whole)
     {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-#pragma unroll
-            for (int j = 0; j < NT; ++j) b[q][j] = lds128(x + q * x_step + j * 512);
+            b[q] = lds128(x + q * x_step);
 #pragma unroll
             for (int i = 0; i < M; ++i) {
                 lo[q][i] = lds128(w + at.lo[q] + i * at.mt_stride);
                 up[q][i] = lds128(w + at.up[q] + i * at.mt_stride);
             }
         }
-        if (!whole) {
-#pragma unroll
-            for (int j = 0; j < NT; ++j) b[1][j] = make_uint4(0, 0, 0, 0);     // the weights there are zero
-        }
+        if (!whole) b[1] = make_uint4(0, 0, 0, 0);     // the weights there are zero
     }
-    __device__ __forceinline__ void mma(float (&acc)[kMt][NT][4]) const
+    __device__ __forceinline__ void mma(float (&acc)[kMt][4]) const
     {
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll
-            for (int i = 0; i < M; ++i)
-#pragma unroll
-                for (int j = 0; j < NT; ++j) mma_bf16(acc[i][j], lo[q][i].x, up[q][i].x, lo[q][i].y, up[q][i].y, b[q][j].x, b[q][j].y);
+            for (int i = 0; i < M; ++i) mma_bf16(acc[i], lo[q][i].x, up[q][i].x, lo[q][i].y, up[q][i].y, b[q].x, b[q].y);
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll
-            for (int i = 0; i < M; ++i)
-#pragma unroll
-                for (int j = 0; j < NT; ++j) mma_bf16(acc[i][j], lo[q][i].z, up[q][i].z, lo[q][i].w, up[q][i].w, b[q][j].z, b[q][j].w);
+            for (int i = 0; i < M; ++i) mma_bf16(acc[i], lo[q][i].z, up[q][i].z, lo[q][i].w, up[q][i].w, b[q].z, b[q].w);
     }
 };
 
@@ -380,8 +372,8 @@ struct Walk {
     uint32_t full, empty, ring, x_ring, xfull, xempty;                // shared-memory addresses
     int slots, slot_bytes, x_stage_bytes, kg, kb_item, kb_all, n_items, n_k32, x_kb, x_bytes_kb;
 };
-template <int NT, int M>
-__device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][NT][4], const ATile at, const Walk k, int kq, Place pl, uint32_t &xs, const Ctl &ctl, uint64_t limit, int lane)
+template <int M>
+__device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][4], const ATile at, const Walk k, int kq, Place pl, uint32_t &xs, const Ctl &ctl, uint64_t limit, int lane)
 {
     int kb = kq, item = 0, in_item = kq, x_st = 0, in_x = kq;         // kb = item * kb_item + in_item = x_st * x_kb + in_x
     bool landed = false;                                              // the item has been seen to land
@@ -410,7 +402,7 @@ __device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][NT][4], const ATile 
         ++x_st;
     };
     if (!x_wait()) return false;
-    Block<NT, M> blk;
+    Block<M> blk;
     while (kb < k.kb_all) {
         for (; in_item >= k.kb_item; in_item -= k.kb_item)
             if (!give_back()) return false;
@@ -436,7 +428,6 @@ __device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][NT][4], const ATile 
 }
 
 // One GEMM phase.
-template <int NT>
 __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, int layer, int part)
 {
     const StreamPass &p = e.p;
@@ -476,18 +467,16 @@ __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, 
 #pragma unroll
             for (int j = 0; j < kMaxSms / 32; ++j) sq[j] = e.lane + 32 * j < (int)gridDim.x ? __ldcg(ssq + e.lane + 32 * j) : 0.f;
         }
-        float acc[kMt][NT][4];
+        float acc[kMt][4];
 #pragma unroll
-        for (int i = 0; i < kMt; ++i)
-#pragma unroll
-            for (int j = 0; j < NT; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
+        for (int i = 0; i < kMt; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
 
         const Walk walk{smem_u32(&e.ctl.full[0]), smem_u32(&e.ctl.empty[0]), e.ring, e.ring + p.x_off + e.lane * 16, smem_u32(&e.ctl.xfull[0]),
                         smem_u32(&e.ctl.xempty[0]), p.slots, p.slot_bytes, p.x_stage_bytes, g.kg, g.kb_item, g.kb_all, g.n_items,
                         g.K / 32, g.x_kb, C * 128};
-        if (mtn == 2) c.ok = gemm_walk<NT, 2>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
-        else if (mtn == 3) c.ok = gemm_walk<NT, 3>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
-        else c.ok = gemm_walk<NT, 1>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);      // (no tile at all: a tile of other data)
+        if (mtn == 2) c.ok = gemm_walk<2>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+        else if (mtn == 3) c.ok = gemm_walk<3>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+        else c.ok = gemm_walk<1>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);      // (no tile at all: a tile of other data)
         if (!c.ok) return;
         c.at.add(g.n_items, p.slots);
 
@@ -497,9 +486,7 @@ __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, 
         for (int i = 0; i < kMt; ++i) {
             if (i < mtn) {
                 const int unit = (mq + i * g.mg) * 8 + pu;
-#pragma unroll
-                for (int j = 0; j < NT; ++j)
-                    if (j * 4 + t < n) red[(kq * n + j * 4 + t) * units_pad + unit] = make_float2(acc[i][j][0] + acc[i][j][1], acc[i][j][2] + acc[i][j][3]);
+                if (t < n) red[(kq * n + t) * units_pad + unit] = make_float2(acc[i][0] + acc[i][1], acc[i][2] + acc[i][3]);
             }
         }
         if (norm && e.warp < n) {
@@ -632,12 +619,12 @@ __device__ __forceinline__ void attention_phase(const Env &e, Consumer &c, int l
             const float *k0 = q0 + (size_t)kStreamMaxNodes * d, *v0 = k0 + (size_t)kStreamMaxNodes * d;
             const int nd = kWarps - 1 - e.warp;
             if (nd < n) {
-                float4 q[8], v[8], acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 q[8], v[kStreamMaxNodes], acc = make_float4(0.f, 0.f, 0.f, 0.f);
                 const int key = e.lane >> 2, qd = (e.lane & 3) * 4, tn = p.n_old + key;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) q[i] = __ldcg(reinterpret_cast<const float4 *>(q0 + (size_t)nd * d + 16 * i + qd));
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = j <= nd ? __ldcg(reinterpret_cast<const float4 *>(v0 + (size_t)j * d + 4 * e.lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int j = 0; j < kStreamMaxNodes; ++j) v[j] = j <= nd ? __ldcg(reinterpret_cast<const float4 *>(v0 + (size_t)j * d + 4 * e.lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 float dot = 0.f;
                 if (key <= nd) {
 #pragma unroll
@@ -656,7 +643,7 @@ __device__ __forceinline__ void attention_phase(const Env &e, Consumer &c, int l
                 float sum = pr;
                 for (int o = 16; o > 2; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = 0; j < kStreamMaxNodes; ++j) {
                     const float wj = __shfl_sync(0xffffffffu, pr, j * 4);
                     if (wj == 0.f) continue;               // a row that is not seen has no say, whatever it holds
                     acc.x = fmaf(wj, v[j].x, acc.x); acc.y = fmaf(wj, v[j].y, acc.y); acc.z = fmaf(wj, v[j].z, acc.z); acc.w = fmaf(wj, v[j].w, acc.w);
@@ -801,7 +788,6 @@ __device__ __forceinline__ void attention_phase(const Env &e, Consumer &c, int l
     arrive_grid(e, c);
 }
 
-template <int NT>
 __device__ __forceinline__ void consume(const Env &e, Consumer &c)
 {
     const StreamPass &p = e.p;
@@ -833,7 +819,7 @@ __device__ __forceinline__ void consume(const Env &e, Consumer &c)
         const int steps = l < p.L ? 5 : p.logits != nullptr ? p.head_parts : 0;
         for (int st = 0; st < steps && c.ok; ++st) {
             if (l < p.L && st == 1) attention_phase(e, c, l);
-            else gemm_phase<NT>(e, c, l < p.L ? gemm_kind(st) : SG_HEAD, l, l < p.L ? 0 : st);
+            else gemm_phase(e, c, l < p.L ? gemm_kind(st) : SG_HEAD, l, l < p.L ? 0 : st);
         }
     }
 }
@@ -878,8 +864,6 @@ __device__ __forceinline__ bool load_inputs(const StreamPass &p, Ctl &ctl, uint3
     return true;
 }
 
-// NT: tiles of eight columns on the N side (two columns per node)
-template <int NT>
 __global__ void __launch_bounds__(kThreads, 1)
 stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__ CUtensorMap kv_map)
 {
@@ -931,7 +915,7 @@ stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__
     } else if (warp < kWarps) {
         Env e{p, ctl, base, reinterpret_cast<float *>(smp + p.red_off), reinterpret_cast<float2 *>(smp + p.cs_off), p.n_tree - p.n_old, warp, lane};
         Consumer c;
-        consume<NT>(e, c);
+        consume(e, c);
         ok = c.ok;
     } else if (producer) {
         while (!prod.done()) {
@@ -966,19 +950,21 @@ stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__
 
 bool stream_pass_serves(int d, int f, int hd, int H, int V, int n_sms)
 {
-    // a CTA's rows of the residual stream are one unit per lane, K whole MMA steps, and 16-row tiles eight a warp at most
+    // a CTA's rows of the residual stream are one unit per lane, K is whole halves of a k-block, and a phase has 16 tiles of 16
+    // rows at most: kMt of them per warp once the warps share the rows
     auto per_cta = [&](long long units) { return (units + n_sms - 1) / n_sms; };
     return hd == kHdim && n_sms <= kMaxSms && H <= n_sms && d % 128 == 0 && f % 32 == 0 && per_cta(d / 2) <= kMaxResidUnits &&
            per_cta(3 * d / 2) <= 128 && per_cta(f) <= 128 && per_cta(((long long)V + 1) / 2) <= 128;
 }
 
-// Up to four nodes, (node, plane) is one tile of eight columns and a warp's loads of weights feed one MMA each. Whole
-// passes, us, this kernel against one kernel per step: 7B shape (32 layers, prefix 512) 2560 / 2818 with one node,
-// 2620 / 2827 with four, 3241 / 2844 with eight; 13B widths (20 layers, prefix 1024) 2400 / 2516, 2423 / 2524, 2842 / 2535.
+// Up to four nodes, (node, plane) is one tile of eight columns and a warp's loads of weights feed one MMA each; a variant with
+// two tiles, for eight nodes, lost. Whole passes, us, this kernel against one kernel per step: 7B shape (32 layers, prefix
+// 512) 2511 / 2811 with one node, 2620 / 2827 with four, 3241 / 2844 with eight; 13B widths (20 layers, prefix 1024) 2400 / 2516,
+// 2423 / 2524, 2842 / 2535.
 bool stream_pass_prefers(int n)
 {
     static const int max_n = [] { const char *e = getenv("LLMCAD_STREAM_PASS_MAX_N"); return e ? atoi(e) : 4; }();   // tuning aid; 0: never
-    return n <= max_n && n <= kStreamMaxNodes;
+    return n <= kStreamMaxNodes && n <= max_n;
 }
 
 size_t stream_pass_floats_qkv(int d) { return (size_t)3 * kStreamMaxNodes * d; }
@@ -1003,7 +989,7 @@ bool plan_stream_pass(StreamPass &p, int n_sms)
     const int units[SG_KINDS] = {3 * p.d / 2, p.d / 2, p.f, p.d / 2, (p.V + 1) / 2};
     const int K[SG_KINDS] = {p.d, p.d, p.d, p.f, p.d};
     size_t red = 0;
-    // two stages of inputs, 32 k-blocks of one node each, or 16 of four
+    // two stages of inputs, 32 k-blocks of one node each, or 16 of four nodes
     p.x_stage_bytes = n == 1 ? 8192 : 16384;
     int U[SG_KINDS], kbs[SG_KINDS];
     for (int i = 0; i < SG_KINDS; ++i) {
@@ -1083,13 +1069,10 @@ cudaError_t launch_stream_pass(const StreamPass &p, int n_sms, cudaStream_t st)
     // rows behind the prefix read as zero
     if (!make_tensor_map_bf16_3d(&map, p.kv, dims, strides, box)) return cudaErrorInvalidValue;
 
-    auto kernel = p.n_tree - p.n_old <= 4 ? stream_pass_kernel<1> : stream_pass_kernel<2>;
     static PerDeviceOnce attr_set;
     if (attr_set.needed()) {
-        for (auto k : {stream_pass_kernel<1>, stream_pass_kernel<2>}) {
-            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem + 1024);
-            if (e != cudaSuccess) return e;
-        }
+        const cudaError_t e = cudaFuncSetAttribute(stream_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem + 1024);
+        if (e != cudaSuccess) return e;
         attr_set.mark();
     }
     cudaLaunchConfig_t cfg = {};
@@ -1102,7 +1085,7 @@ cudaError_t launch_stream_pass(const StreamPass &p, int n_sms, cudaStream_t st)
     attr.val.cooperative = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p, map);
+    return cudaLaunchKernelEx(&cfg, stream_pass_kernel, p, map);
 }
 
 }  // namespace llmcad

@@ -7,7 +7,7 @@
 
 namespace llmcad {
 
-constexpr int kStreamMaxNodes = 8;      // computed nodes of a pass
+constexpr int kStreamMaxNodes = 4;      // computed nodes of a pass
 
 // One of the five GEMM shapes of a pass. Its units (a rotary pair of rows, gate and up row of a feature, or two
 // adjacent rows) are dealt out to the CTAs; a CTA's eight warps are kg groups, which take the k-blocks in turn, of
