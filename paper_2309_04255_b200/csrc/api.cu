@@ -344,11 +344,13 @@ int run_attention(llmcad_ctx *ctx, const void *q, const void *k, const void *v, 
     return LLMCAD_OK;
 }
 
-bool use_small_pass(const llmcad_ctx *ctx, int n_keys);
+constexpr int kNoRoom = -1000;       // a cooperative launch was refused: the kernels per step serve the call
+int cooperative_result(llmcad_ctx *ctx, cudaError_t e, const char *what);
+bool use_small_pass(const llmcad_ctx *ctx, int n_keys, cudaStream_t st);
 SmallPass small_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent,
                             int n_tree, int n_old, float *logits, int32_t *status, bool keep_status);
 int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st);
-bool use_stream_pass(const llmcad_ctx *ctx, int n);
+bool use_stream_pass(const llmcad_ctx *ctx, int n, cudaStream_t st);
 bool stream_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent, int n_tree,
                         int n_old, float *logits, int32_t *status, bool keep_status, bool last_row, StreamPass &p);
 
@@ -369,13 +371,13 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
     const int n_pad = wide ? kLoRows : (n + 15) / 16 * 16;
     const char *base = static_cast<const char *>(packed);
     int rc;
-    if (use_small_pass(ctx, P + n_tree))
-        return run_small_pass(ctx, small_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status), st);
+    if (use_small_pass(ctx, P + n_tree, st)) {
+        rc = run_small_pass(ctx, small_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status), st);
+        if (rc != kNoRoom) return rc;
+    }
     StreamPass sp;
-    if (use_stream_pass(ctx, n) && stream_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status, last_row, sp)) {
-        ctx->launches++;
-        CUDA_TRY(launch_stream_pass(sp, ctx->n_sms, st));
-        return LLMCAD_OK;
+    if (use_stream_pass(ctx, n, st) && stream_pass_params(ctx, packed, kv_cache, P, tokens, parent, n_tree, n_old, logits, status, keep_status, last_row, sp)) {
+        if ((rc = cooperative_result(ctx, launch_stream_pass(sp, ctx->n_sms, st), "launch_stream_pass")) != kNoRoom) return rc;
     }
     if ((rc = ensure_weight_maps(ctx, packed, n_pad)) != LLMCAD_OK) return rc;
     if ((rc = ensure_act_maps(ctx, n_pad)) != LLMCAD_OK) return rc;
@@ -522,11 +524,64 @@ int run_forward(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, cons
     return LLMCAD_OK;
 }
 
+// A process that shares the device may have fewer SMs than it was created with: that is refused at the launch.
+int cooperative_result(llmcad_ctx *ctx, cudaError_t e, const char *what)
+{
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return kNoRoom;
+    }
+    ctx->launches++;
+    return cuda_ok(e, what) ? LLMCAD_OK : LLMCAD_ERR_CUDA;
+}
+
+// Driver calls that tell what a stream may use.
+struct SmQuery {
+    decltype(&cuStreamGetGreenCtx) stream_ctx = nullptr;
+    decltype(&cuGreenCtxGetDevResource) green_resource = nullptr;
+    decltype(&cuCtxGetCurrent) current = nullptr;
+    decltype(&cuCtxGetDevResource) resource = nullptr;
+    bool ok;
+    SmQuery()
+    {
+        ok = find("cuStreamGetGreenCtx", stream_ctx) && find("cuGreenCtxGetDevResource", green_resource) && find("cuCtxGetCurrent", current) &&
+             find("cuCtxGetDevResource", resource);
+    }
+    template <typename F>
+    static bool find(const char *name, F &f)
+    {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint(name, &ptr, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) return false;
+        f = reinterpret_cast<F>(ptr);
+        return true;
+    }
+};
+
+// Whether a launch on `st` has every SM of the device. The one-kernel passes are a CTA per SM that all have to run at once;
+// on a stream of a green context, or under one, there are fewer, and a cooperative launch of too many CTAs is not
+// refused there: it never starts. Asked per call (0.3 us): handles of streams and contexts are used again.
+bool has_every_sm(const llmcad_ctx *ctx, cudaStream_t st)
+{
+    static const SmQuery d;
+    if (!d.ok) return false;
+    CUdevResource r;
+    CUgreenCtx green = nullptr;
+    if (d.stream_ctx(st, &green) != CUDA_SUCCESS) return false;
+    if (green != nullptr) {
+        if (d.green_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return false;
+    } else {
+        CUcontext c = nullptr;
+        if (d.current(&c) != CUDA_SUCCESS || c == nullptr || d.resource(c, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return false;
+    }
+    return (int)r.sm.smCount >= ctx->n_sms;
+}
+
 // Whether this pass goes through the one kernel of pass_small.cu (n_keys keys, prefix and tree).
-bool use_small_pass(const llmcad_ctx *ctx, int n_keys)
+bool use_small_pass(const llmcad_ctx *ctx, int n_keys, cudaStream_t st)
 {
     const llmcad_config &c = ctx->cfg;
-    return ctx->small_pass && !ctx->timing && small_pass_serves(c.d_model, c.d_ffn, c.head_dim, c.n_heads, n_keys);
+    return ctx->small_pass && !ctx->timing && small_pass_serves(c.d_model, c.d_ffn, c.head_dim, c.n_heads, n_keys) && has_every_sm(ctx, st);
 }
 
 // What every pass through that kernel has in common; the caller adds what follows the logits.
@@ -554,15 +609,13 @@ SmallPass small_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache,
 
 int run_small_pass(llmcad_ctx *ctx, const SmallPass &p, cudaStream_t st)
 {
-    ctx->launches++;
-    CUDA_TRY(launch_small_pass(p, ctx->n_sms, st));
-    return LLMCAD_OK;
+    return cooperative_result(ctx, launch_small_pass(p, ctx->n_sms, st), "launch_small_pass");
 }
 
 // Whether n new nodes go through the one kernel of pass_stream.cu (measuring launches one by one needs the others).
-bool use_stream_pass(const llmcad_ctx *ctx, int n)
+bool use_stream_pass(const llmcad_ctx *ctx, int n, cudaStream_t st)
 {
-    return ctx->stream_pass && !ctx->use_counters && !ctx->timing && ctx->trace == nullptr && stream_pass_prefers(n);
+    return ctx->stream_pass && !ctx->use_counters && !ctx->timing && ctx->trace == nullptr && stream_pass_prefers(n) && has_every_sm(ctx, st);
 }
 
 bool stream_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int P, const int32_t *tokens, const int32_t *parent, int n_tree,
@@ -844,11 +897,11 @@ static int verify_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int3
     const llmcad_config &c = ctx->cfg;
     int32_t *status = out->scalars + LLMCAD_S_STATUS;
     float *logits = out->logits != nullptr ? out->logits : ctx->logits;
-    if (use_small_pass(ctx, prefix_len + n)) {
+    if (use_small_pass(ctx, prefix_len + n, st)) {
         SmallPass sp = small_pass_params(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n, 0, logits, status, false);
         sp.verify = 1;
         sp.argmax = out->argmax; sp.path = out->accepted_path; sp.scalars = out->scalars; sp.path_fill = path_fill;
-        return run_small_pass(ctx, sp, st);
+        if ((rc = run_small_pass(ctx, sp, st)) != kNoRoom) return rc;
     }
     if ((rc = run_forward(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n, logits, status, st)) != LLMCAD_OK)
         return rc;
@@ -933,11 +986,11 @@ int llmcad_extend_tree(llmcad_ctx *ctx, const void *packed, void *kv_cache, int3
     if (top_k > ctx->cfg.vocab) return LLMCAD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float *lg = logits != nullptr ? logits : ctx->logits;
-    if (use_small_pass(ctx, prefix_len + n_tree)) {
+    if (use_small_pass(ctx, prefix_len + n_tree, st)) {
         SmallPass sp = small_pass_params(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n_tree, n_old, lg, status, false);
         sp.top_k = top_k;
         sp.topk_ids = topk_ids; sp.topk_probs = topk_probs;
-        return run_small_pass(ctx, sp, st);
+        if ((rc = run_small_pass(ctx, sp, st)) != kNoRoom) return rc;
     }
     if ((rc = run_forward(ctx, packed, kv_cache, prefix_len, tree_tokens, parent_idx, n_tree, lg, status, st, n_old)) != LLMCAD_OK)
         return rc;

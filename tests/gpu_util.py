@@ -105,17 +105,17 @@ def cache_rows(v: B.Verifier, upto: int) -> np.ndarray:
     return v.kv_view()[:, :, :, :upto].double().cpu().numpy()
 
 
-def kernels_of(call):
-    """Names (as the linker sees them) of the kernels that `call` launches, in order: captured into a graph, not run. What
-    `call` sets up on its first run has to be there already."""
+def kernels_of(call, st=None):
+    """Names (as the linker sees them) of the kernels that `call` launches (on `st`, or a stream of its own), in order: captured
+    into a graph, not run. What `call` sets up on its first run has to be there already."""
     from cuda.bindings import driver as drv, runtime as rt
 
     def ok(r):
         assert int(r[0]) == 0, r[0]
         return r[1] if len(r) == 2 else r[1:]
 
-    st = torch.cuda.Stream()
-    st.wait_stream(torch.cuda.current_stream())
+    st = st or torch.cuda.Stream()
+    torch.cuda.synchronize()
     with torch.cuda.stream(st):
         ok(rt.cudaStreamBeginCapture(st.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed) + (None,))
         call()
