@@ -40,7 +40,7 @@ int llmcad_set_gemm_trace(llmcad_ctx *ctx, uint64_t *trace, int32_t capacity);
 int64_t llmcad_launch_count(const llmcad_ctx *ctx);
 
 /* Every device-side wait of this context's kernels (the shared-memory barriers between the roles of
- * a CTA; no kernel waits for another CTA) gives up after `ns` nanoseconds; the kernel
+ * a CTA; in the one-kernel passes, which are launched cooperatively, the grid barrier too) gives up after `ns` nanoseconds; the kernel
  * then sets LLMCAD_ERR_TIMEOUT in the status word, lets all its roles fall out of their loops,
  * frees its tensor memory and returns. Default 2 s; 0 restores the default. */
 int llmcad_set_wait_limit_ns(llmcad_ctx *ctx, uint64_t ns);
@@ -52,6 +52,12 @@ int llmcad_set_wait_limit_ns(llmcad_ctx *ctx, uint64_t ns);
  * Synchronises `stream` and returns the device status word, LLMCAD_ERR_TIMEOUT when the path
  * works, or a negative host-detected error. The context is usable afterwards. */
 int llmcad_selftest_wait_timeout(llmcad_ctx *ctx, void *stream);
+
+/* The same self-test of the one-kernel pass over up to four nodes, whose CTAs also wait for one another at a grid barrier
+ * (contexts and streams that take that kernel, LLMCAD_ERR_UNSUPPORTED otherwise): a pass of one node over an empty prefix whose
+ * inputs are withheld behind the first barrier, so that the waits of every role of every CTA run out. packed and
+ * kv_cache as for llmcad_verify_tree; the cache is not written. Limit, return value and what is left as above. */
+int llmcad_selftest_pass_timeout(llmcad_ctx *ctx, const void *packed, void *kv_cache, void *stream);
 
 /* Micro-benchmarks of the machine, context-free, on the current device (no tensor of the library is involved).
  *

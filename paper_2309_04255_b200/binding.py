@@ -32,7 +32,7 @@ EXPORTS = [
     "llmcad_accept_compact", "llmcad_accept_compact_fill", "llmcad_tree_attention", "llmcad_skinny_gemm", "llmcad_launch_count",
     "llmcad_last_status", "llmcad_set_kernel_timing", "llmcad_get_kernel_timing", "llmcad_set_gemm_trace", "llmcad_tiled_weight_bytes", "llmcad_tile_weight", "llmcad_skinny_gemm_tiled", "llmcad_tree_attention_noalloc", "llmcad_noalloc_last_error",
     "llmcad_tree_confidence", "llmcad_update_threshold", "llmcad_extend_tree", "llmcad_tree_branches", "llmcad_branch_pacer",
-    "llmcad_set_wait_limit_ns", "llmcad_selftest_wait_timeout",
+    "llmcad_set_wait_limit_ns", "llmcad_selftest_wait_timeout", "llmcad_selftest_pass_timeout",
     "llmcad_quantize_int4", "llmcad_tiled_weight_int4_bytes", "llmcad_tile_weight_int4", "llmcad_skinny_gemm_tiled_int4",
     "llmcad_probe_bulk_copy", "llmcad_probe_mma_sync",
 ]
@@ -119,6 +119,7 @@ def lib():
         L.llmcad_skinny_gemm_tiled_int4.argtypes = [vp, vp, vp, vp, i32, i32, i32, vp]
         L.llmcad_set_wait_limit_ns.argtypes = [vp, C.c_uint64]
         L.llmcad_selftest_wait_timeout.argtypes = [vp, vp]
+        L.llmcad_selftest_pass_timeout.argtypes = [vp, vp, vp, vp]
         L.llmcad_probe_bulk_copy.argtypes = [vp, sz, i32, i32, vp, C.POINTER(C.c_double), C.POINTER(C.c_double)]
         L.llmcad_probe_mma_sync.argtypes = [i32, i32, vp, C.POINTER(C.c_double), C.POINTER(C.c_double)]
         _lib = L
@@ -345,10 +346,17 @@ class Verifier:
         _check(lib().llmcad_set_wait_limit_ns(self.ctx, int(ns)), "llmcad_set_wait_limit_ns")
 
     def selftest_wait_timeout(self) -> int:
-        """Runs a small GEMM chain whose grid barrier cannot complete; returns the device status word."""
+        """Runs a small GEMM whose activation copies are withheld; returns the device status word."""
         code = lib().llmcad_selftest_wait_timeout(self.ctx, _stream())
         if code < 0:
             raise LlmcadError(code, "llmcad_selftest_wait_timeout")
+        return code
+
+    def selftest_pass_timeout(self) -> int:
+        """Runs a one-kernel pass whose inputs are withheld; returns the device status word."""
+        code = lib().llmcad_selftest_pass_timeout(self.ctx, self.packed.data_ptr(), self.kv.data_ptr(), _stream())
+        if code < 0:
+            raise LlmcadError(code, "llmcad_selftest_pass_timeout")
         return code
 
 

@@ -1334,4 +1334,24 @@ int llmcad_selftest_wait_timeout(llmcad_ctx *ctx, void *stream)
     return v;
 }
 
+int llmcad_selftest_pass_timeout(llmcad_ctx *ctx, const void *packed, void *kv_cache, void *stream)
+{
+    if (ctx == nullptr) return LLMCAD_ERR_INVALID_ARG;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // a root alone: token 0, and the -1 that begins the parents of a chain
+    int rc = check_pass_args(ctx, packed, kv_cache, 0, ctx->tokens_dev(), ctx->chain_dev(), 1);
+    if (rc != LLMCAD_OK) return rc;
+    if (ctx->wait_limit_ns > 100000000ull) return LLMCAD_ERR_INVALID_ARG;
+    int32_t *status = ctx->scalars_dev() + LLMCAD_S_STATUS;
+    StreamPass sp;
+    if (!use_stream_pass(ctx, 1, st) ||
+        !stream_pass_params(ctx, packed, kv_cache, 0, ctx->tokens_dev(), ctx->chain_dev(), 1, 0, ctx->logits, status, false, false, sp))
+        return LLMCAD_ERR_UNSUPPORTED;
+    CUDA_TRY(cudaMemsetAsync(ctx->tokens_dev(), 0, sizeof(int32_t), st));
+    sp.withhold_input = 1;
+    rc = cooperative_result(ctx, launch_stream_pass(sp, ctx->n_sms, st), "launch_stream_pass");
+    if (rc != LLMCAD_OK) return rc == kNoRoom ? LLMCAD_ERR_UNSUPPORTED : rc;
+    return llmcad_last_status(ctx, stream);
+}
+
 }  // extern "C"

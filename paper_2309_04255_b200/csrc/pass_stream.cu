@@ -854,6 +854,7 @@ __device__ __forceinline__ bool load_inputs(const StreamPass &p, Ctl &ctl, uint3
         for (int kb = 0; kb < n_kb; kb += x_kb, ++xs) {
             const int st = xs % kXStages;
             if (!thread_wait(smem_u32(&ctl.xempty[st]), ((xs / kXStages) & 1u) ^ 1u, ctl, p.wait_limit_ns)) return false;
+            if (p.withhold_input) continue;
             const uint32_t full = smem_u32(&ctl.xfull[st]), bytes = (min(2 * (kb + x_kb), n_k32) - 2 * kb) * k32_bytes;
             mbar_expect_tx(full, bytes);
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"

@@ -48,6 +48,7 @@ struct StreamPass {
     int32_t *status;
     int keep_status;                    // the status word of an earlier chunk of the same call stands
     uint64_t wait_limit_ns;
+    int withhold_input;                 // self-test of the wait limit: the copies of the phases' inputs are never issued
     int slots, slot_bytes, x_stage_bytes, x_off, red_off, q_off, cs_off;    // shared memory layout
 };
 constexpr int kStreamHeadParts = 4;

@@ -1,6 +1,8 @@
 """The one-kernel bf16 pass over few nodes (pass_stream.cu) against the oracle, at the edges of how it cuts its work: models
 with fewer pairs of rows than CTAs, K that ends inside a k-block, an odd vocabulary, rows of a CTA on both sides of a weight
 tile, prefixes around a tile of 32 keys, trees whose first nodes are in the cache already, prompts of a few tokens."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -119,3 +121,42 @@ def test_prompts_that_are_or_end_in_few_tokens(P, n):
     bad[-1] = cfg.vocab
     tw.v.prefill(P, bad)
     assert tw.v.last_status() == B.ERR_BAD_TOKEN
+
+
+@pytest.mark.parametrize("model,P", [("small", 40), ("odd", 700), ("7b", 200)])
+def test_bounded_waits_run_out_and_the_context_survives(model, P):
+    """With the limit at 1 ms and the inputs withheld behind the first grid barrier, the waits of consumers, producers and the
+    loader of every CTA run out: TIMEOUT, promptly, with nothing written, and again. The barrier words are back at zero
+    afterwards: passes of one and four nodes (P = 700: several key ranges per head and their counters) are bit for bit what
+    they were."""
+    cfg = MODELS[model]
+    tw = Twin(cfg, P + 16, scale=3.0 if cfg.d_model < 1024 else 1.0, keep_host=False)
+    tw.fill_prefix_synthetic(P)
+    passes = [(tree(n, P), gen.gen_tokens(cfg, n, P)) for n in (1, 4)]
+    before = [tw.gpu_pass(P, tokens, parent) for parent, tokens in passes]
+    cache = tw.v.kv_view().clone()
+    with pytest.raises(B.LlmcadError) as e:          # refuses to run with the default limit of 2 s
+        tw.v.selftest_pass_timeout()
+    assert e.value.code == B.ERR_INVALID_ARG
+    tw.v.set_wait_limit_ns(1_000_000)
+    for _ in range(2):
+        t0 = time.perf_counter()
+        assert tw.v.selftest_pass_timeout() == B.ERR_TIMEOUT
+        assert time.perf_counter() - t0 < 1.0
+    assert torch.equal(tw.v.kv_view(), cache)
+    tw.v.set_wait_limit_ns(0)
+    for (parent, tokens), was in zip(passes, before):
+        now = tw.gpu_pass(P, tokens, parent)
+        assert now["scalars"][B.S_STATUS] == 0
+        for key in ("logits", "argmax", "scalars", "accepted_path"):
+            assert np.array_equal(now[key], was[key]), key
+
+
+def test_timeout_self_test_is_refused_where_the_kernel_is_not_taken():
+    cfg = MODELS["small"]
+    for flags in (B.FLAG_MMA_ATTN, B.FLAG_SIMT_GEMM):
+        tw = Twin(cfg, 64, flags=flags, keep_host=False)
+        tw.v.set_wait_limit_ns(1_000_000)
+        with pytest.raises(B.LlmcadError) as e:
+            tw.v.selftest_pass_timeout()
+        assert e.value.code == B.ERR_UNSUPPORTED
