@@ -628,7 +628,8 @@ bool stream_pass_params(llmcad_ctx *ctx, const void *packed, void *kv_cache, int
     p.eps = c.rms_eps;
     p.base = static_cast<const char *>(packed);
     p.w_off[SG_QKV] = y.wqkv; p.w_off[SG_O] = y.wo; p.w_off[SG_GU] = y.wgu; p.w_off[SG_DOWN] = y.wdown; p.w_off[SG_HEAD] = y.lm_head;
-    p.g[SG_GU].upper = tiled_weight_bytes(c.d_ffn, c.d_model);
+    p.w4 = ctx->w4 ? 1 : 0;
+    p.g[SG_GU].upper = ctx->w4 ? tiled_weight_int4_bytes(c.d_ffn, c.d_model) : tiled_weight_bytes(c.d_ffn, c.d_model);
     p.attn_norm = y.attn_norm; p.ffn_norm = y.ffn_norm; p.layer_bytes = y.layer_bytes; p.tok_embed = y.tok_embed; p.final_norm = y.final_norm;
     p.kv = static_cast<char *>(kv_cache);
     p.inv_freq = ctx->inv_freq;
@@ -776,7 +777,7 @@ int llmcad_create(const llmcad_config *cfg, llmcad_ctx **out)
             want((void **)&ctx->sp_bar, 2 * 4);
         }
     }
-    ctx->stream_pass = ctx->tc_gemm && ctx->comp && ctx->tc_attn && cfg->flags == 0 && cfg->n_layers > 0 &&
+    ctx->stream_pass = ctx->tc_gemm && ctx->comp && ctx->tc_attn && (cfg->flags & ~LLMCAD_FLAG_INT4_WEIGHTS) == 0 && cfg->n_layers > 0 &&
                        stream_pass_serves(cfg->d_model, cfg->d_ffn, cfg->head_dim, cfg->n_heads, cfg->vocab, ctx->n_sms);
     if (ctx->stream_pass) {
         want((void **)&ctx->st_qkv, stream_pass_floats_qkv(cfg->d_model) * 4);

@@ -17,6 +17,10 @@
 //   warps 0-7     mma.sync m16n8k16: weights on the M side, (node, hi/lo plane) as the eight columns of the N side. Groups of warps take the
 //                 k-blocks in turn; the sums are added in shared memory in a fixed order, and the epilogue (norm factor,
 //                 rotary, K/V write, SwiGLU, residual) runs where they lie. The residual stream stays in shared memory.
+//   INT4 weights  take the same plan, operands and order of sums (the passes are equal bit for bit): codes and exponents go through
+//                 the ring as they are packed, by ordinary asynchronous copies, and are expanded on the way into the MMA. 7B widths,
+//                 4 layers, prefix 512, one / four nodes: 305 / 329 us, with one kernel per step 312 / 314; 13B (3 layers) 322 / 344,
+//                 313 / 316; d 512 112 / 119, 151 / 152. The latency of a k-block per warp bounds it, not the HBM.
 //   attention     (head, key range) per CTA: prefix tiles of 32 keys come through the weight ring, scores and outputs
 //                 by mma.sync with hi and lo planes as the two halves of the 16 rows, the new nodes' keys and values in
 //                 fp32; the CTA that finishes a head last merges its key ranges.
@@ -37,10 +41,12 @@ namespace {
 constexpr int kWarps = 8;                       // consumers
 // A copy costs its warp ~90 cycles to issue and an item ~500 more, all of it latency: one producer got 13 of the 26 bytes
 // a cycle that an SM's share of the HBM is.
-constexpr int kProducers = 4;
-constexpr int kThreads = 32 * (kWarps + kProducers + 1);
+// INT4 items are many copies of 16 bytes per lane; there every slot of the ring up to seven has a producer of its own.
+template <bool W4> constexpr int kProducers = W4 ? 7 : 4;
+template <bool W4> constexpr int kThreads = 32 * (kWarps + kProducers<W4> + 1);
 constexpr int kMaxSlots = 16;                   // items the ring can hold
 constexpr int kMaxItemKb = 6;                   // k-blocks of an item at most
+constexpr int kMaxItemKbW4 = 32;                // the same, of INT4 weights (16: 3 % slower, 8: 6 %)
 constexpr int kXStages = 2;                     // of the ring of inputs
 constexpr int kMt = 3;                          // 16-row tiles of a warp at most
 constexpr int kHdim = 128, kKeys = 32;          // head size, keys of a prefix tile
@@ -105,12 +111,39 @@ struct Ctl {
     MaskTable table;
 };
 
+// ---- INT4 weights (layer matrices only, see pack.cu): a k-block of a CTA's rows in the ring is, per run of rows, the codes of
+// its columns 0 .. 31 and then 32 .. 63, 16 bytes a row; behind the runs their exponents, a byte a row, from a multiple of
+// 16 rows on (copies move 16 bytes).
+__device__ __host__ __forceinline__ int exp_chunks(int row0, int rows_run) { return ((row0 & 15) + rows_run + 15) >> 4; }
+__device__ __host__ __forceinline__ int w4_kb_bytes(int row0, int rows_run, int runs) { return runs * (rows_run * 32 + exp_chunks(row0, rows_run) * 16); }
+// Two codes of a word as a bf16 pair: OR 0x4300 into each half: 128 + u (u = q + 8); (128 + u) * 2^e - 136 * 2^e = q * 2^e, exact.
+// The bf16 bits of 2^e are (e + 127) << 7, those of -136 * 2^e are that + 0x8388.
+__device__ __forceinline__ uint32_t expand2(uint32_t word, uint32_t scale)
+{
+    uint32_t t, r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xea;" : "=r"(t) : "r"(word), "r"(0x000f000fu), "r"(0x43004300u));
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(t), "r"(scale), "r"(scale + 0x83888388u));
+    return r;
+}
+
 // (volatile: they stay behind the barrier wait in front of them)
 __device__ __forceinline__ uint4 lds128(uint32_t a)
 {
     uint4 r;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(a));
     return r;
+}
+__device__ __forceinline__ uint32_t lds32v(uint32_t a)
+{
+    uint32_t r;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(r) : "r"(a));
+    return r;
+}
+__device__ __forceinline__ uint32_t exp_scale(uint32_t a)
+{
+    int e;
+    asm volatile("ld.shared.s8 %0, [%1];" : "=r"(e) : "r"(a));
+    return (uint32_t)(e + 127) * 0x00800080u;
 }
 __device__ __forceinline__ uint32_t lds32(uint32_t a)
 {
@@ -158,9 +191,15 @@ __device__ __forceinline__ bool thread_wait(uint32_t bar, uint32_t parity, const
     }
     return true;
 }
-__device__ __forceinline__ bool wait_all(uint32_t bar, uint32_t parity, const Ctl &ctl, uint64_t limit)
+// (The loop that watches the clock is called, not inlined: a walk has four waits, a phase three walks, and what straight-line
+// code costs here is its fetch.)
+__device__ __noinline__ bool wait_watched(uint32_t bar, uint32_t parity, const Ctl &ctl, uint64_t limit)
 {
     return mbar_wait_all(bar, parity, const_cast<volatile int *>(&ctl.abort_flag), limit);
+}
+__device__ __forceinline__ bool wait_all(uint32_t bar, uint32_t parity, const Ctl &ctl, uint64_t limit)
+{
+    return __all_sync(0xffffffffu, mbar_try(bar, parity)) || wait_watched(bar, parity, ctl, limit);
 }
 
 // ---- a place in the ring: slot and the parity of its turn
@@ -176,6 +215,7 @@ struct Place {
 
 // ---- weight producer: a warp that fetches the items of its slots, every kProducers-th of the ring. (A slot belongs to
 // one producer, which so sees each of its turns: a barrier tells two of them apart and no more.)
+template <bool W4>
 struct Producer {
     const StreamPass &p;
     const CUtensorMap *map;
@@ -185,19 +225,27 @@ struct Producer {
     Place at;
     int issued = 0;
     int ph = -1, pos = 0;                      // the next item: phase and k-block or tile in it
-    bool attention = false;
+    bool attention = false, codes = false;     // codes: an INT4 matrix
     int layer = 0, kb_all = 0, kb_item = 1, kb_bytes = 0;    // kb_all: k-blocks or tiles in all
     // what this lane copies of an item: one run of rows of one k-block, cut where a tile of 128 rows ends
     const char *src = nullptr;
     int my_k = 1 << 30, my_dst = 0, my_bytes = 0;
-    const int lane = threadIdx.x & 31, rank = (int)(threadIdx.x >> 5) - kWarps, phases;
+    // INT4: the CTA's rows, bytes from a weight tile to the next one below it and from run to run, and this lane's 16 exponents
+    int row0 = 0, rows_run = 0, rows = 0, exp_dst = -1;
+    uint32_t tile_bytes = 0, exp_src = 0;
+    size_t upper = 0;
+    const int lane = threadIdx.x & 31, rank = (int)(threadIdx.x >> 5) - kWarps, step, phases;
     __device__ Producer(const StreamPass &p_, const CUtensorMap *m, Ctl &c, uint32_t r)
-        : p(p_), map(m), ctl(c), ring(r), phases(5 * p_.L + (p_.logits != nullptr ? p_.head_parts : 0))
+        : p(p_), map(m), ctl(c), ring(r), step(W4 ? min(kProducers<W4>, p_.slots) : kProducers<W4>), phases(5 * p_.L + (p_.logits != nullptr ? p_.head_parts : 0))
     {
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     }
     __device__ void start()
     {
+        if (rank >= step) {            // (a ring of fewer slots)
+            ph = phases;
+            return;
+        }
         next_phase();
         skip(rank);
     }
@@ -221,6 +269,20 @@ struct Producer {
             kb_all = s.U > 0 ? g.kb_all : 0;
             if (kb_all == 0) continue;
             kb_item = g.kb_item;
+            codes = W4 && !head;
+            if (W4 && codes) {
+                const int runs = g.upper ? 2 : 1, chunks = exp_chunks(s.row0, s.rows_run), run = lane >= chunks ? 1 : 0;
+                row0 = s.row0; rows_run = s.rows_run; rows = s.rows;
+                upper = g.upper;
+                tile_bytes = kb_all * kW4TileBytes;
+                kb_bytes = w4_kb_bytes(row0, rows_run, runs);
+                const int r = (row0 & ~15) + 16 * (lane - run * chunks);
+                exp_dst = lane < runs * chunks ? rows * 32 + lane * 16 : -1;
+                exp_src = (r >> 7) * tile_bytes + 4096 + (r & 127);
+                src = p.base + p.w_off[kind] + p.layer_bytes * (size_t)layer;
+                if (run) exp_src += (uint32_t)upper;
+                continue;
+            }
             kb_bytes = s.rows * 128;
             const int pieces = ((s.row0 & 127) + s.rows_run + 127) >> 7, per_k = (g.upper ? 2 : 1) * pieces;
             my_k = lane / per_k;
@@ -247,7 +309,16 @@ struct Producer {
     {
         const uint32_t full = smem_u32(&ctl.full[at.slot]), dst = ring + at.slot * p.slot_bytes;
         const int nkb = min(kb_item, kb_all - pos);
+        if (W4 && codes && !attention) {
+            fetch_codes(full, dst, nkb);
+            ++issued;
+            skip(at.slot + step < p.slots ? step : p.slots - at.slot + rank);
+            return;
+        }
+        // (INT4: the slot's last content may have come by ordinary copies)
+        if (W4) asm volatile("fence.proxy.async;" ::: "memory");
         if (lane == 0) mbar_expect_tx(full, attention ? kKvItem : nkb * kb_bytes);
+        else if (W4) mbar_arrive(full);
         __syncwarp();
         if (attention) {
             if (lane < 4)
@@ -261,7 +332,31 @@ struct Producer {
                          : "memory");
         }
         ++issued;
-        skip(at.slot + kProducers < p.slots ? kProducers : p.slots - at.slot + rank);
+        skip(at.slot + step < p.slots ? step : p.slots - at.slot + rank);
+    }
+    // An item of an INT4 matrix: 16 bytes per lane and copy. (Bulk copies would be three per run, piece and k-block, of 48 to
+    // 1300 bytes each.) Every lane arrives when its copies have landed.
+    __device__ void fetch_codes(uint32_t full, const uint32_t dst0, int nkb)
+    {
+        auto copy = [&](uint32_t to, const char *from) {
+            asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "l"(policy) : "memory");
+        };
+        const char *first = src + (size_t)pos * kW4TileBytes;
+        for (int x = lane; x < rows; x += 32) {
+            const int run = x >= rows_run ? 1 : 0, in_run = x - run * rows_run, r = row0 + in_run;
+            const char *from = first + (run ? upper : 0) + (size_t)((r >> 7) * tile_bytes + (r & 127) * 16);
+            uint32_t to = dst0 + run * rows_run * 32 + in_run * 16;
+            for (int k = 0; k < nkb; ++k, from += kW4TileBytes, to += kb_bytes) {
+                copy(to, from);
+                copy(to + rows_run * 16, from + 2048);
+            }
+        }
+        if (exp_dst >= 0) {
+            const char *from = first + exp_src;
+            uint32_t to = dst0 + exp_dst;
+            for (int k = 0; k < nkb; ++k, from += kW4TileBytes, to += kb_bytes) copy(to, from);
+        }
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full) : "memory");
     }
 };
 
@@ -334,6 +429,7 @@ __device__ __forceinline__ void emit_resid(const Env &e, int node, bool has, int
 struct ATile {
     int lo[2], up[2];          // first and second row of its unit, for the even and odd 32 columns of a k-block
     int kb_bytes, mt_stride;
+    int exp_lo, exp_up, exp_stride;      // INT4: their exponents
 };
 // A k-block's operands of a warp: M tiles of 16 rows, two times 32 columns (the second is left out where K ends in the
 // middle). Lane (g, t) holds columns 8t .. 8t+7 of 32 on both sides, the first four for one MMA and the others for the
@@ -367,12 +463,53 @@ struct Block {
     }
 };
 
+// The same of INT4 weights: eight codes per row and lane in place of 16 bytes. The MMAs are those above, in their order, on the
+// same bf16 values: a pass with INT4 weights is the pass with the dequantised ones bit for bit.
+template <int M>
+struct CodeBlock {
+    uint4 b[2];
+    uint32_t code[2][2][M], scale[2][M];        // [half][first, second row]
+    __device__ __forceinline__ void load(const ATile &at, uint32_t a, uint32_t x, int x_step, bool)
+    {
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            scale[0][i] = exp_scale(a + at.exp_lo + i * at.exp_stride);
+            scale[1][i] = exp_scale(a + at.exp_up + i * at.exp_stride);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            b[q] = lds128(x + q * x_step);
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                code[q][0][i] = lds32v(a + at.lo[q] + i * at.mt_stride);
+                code[q][1][i] = lds32v(a + at.up[q] + i * at.mt_stride);
+            }
+        }
+    }
+    template <int ROUND>
+    __device__ __forceinline__ void round(float (&acc)[kMt][4]) const
+    {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const uint32_t c0 = code[q][0][i] >> (8 * ROUND), c1 = code[q][1][i] >> (8 * ROUND), s0 = scale[0][i], s1 = scale[1][i];
+                mma_bf16(acc[i], expand2(c0, s0), expand2(c1, s1), expand2(c0 >> 4, s0), expand2(c1 >> 4, s1), ROUND ? b[q].z : b[q].x, ROUND ? b[q].w : b[q].y);
+            }
+    }
+    __device__ __forceinline__ void mma(float (&acc)[kMt][4]) const
+    {
+        round<0>(acc);
+        round<1>(acc);
+    }
+};
+
 // The main loop of a GEMM phase for a warp: k-blocks kq, kq + kg, ... of `kb_all`. False when a wait ran out.
 struct Walk {
     uint32_t full, empty, ring, x_ring, xfull, xempty;                // shared-memory addresses
     int slots, slot_bytes, x_stage_bytes, kg, kb_item, kb_all, n_items, n_k32, x_kb, x_bytes_kb;
 };
-template <int M>
+template <int M, typename Operands>
 __device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][4], const ATile at, const Walk k, int kq, Place pl, uint32_t &xs, const Ctl &ctl, uint64_t limit, int lane)
 {
     int kb = kq, item = 0, in_item = kq, x_st = 0, in_x = kq;         // kb = item * kb_item + in_item = x_st * x_kb + in_x
@@ -402,7 +539,7 @@ __device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][4], const ATile at, 
         ++x_st;
     };
     if (!x_wait()) return false;
-    Block<M> blk;
+    Operands blk;
     while (kb < k.kb_all) {
         for (; in_item >= k.kb_item; in_item -= k.kb_item)
             if (!give_back()) return false;
@@ -428,6 +565,7 @@ __device__ __forceinline__ bool gemm_walk(float (&acc)[kMt][4], const ATile at, 
 }
 
 // One GEMM phase.
+template <bool W4>
 __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, int layer, int part)
 {
     const StreamPass &p = e.p;
@@ -458,6 +596,20 @@ __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, 
         at.lo[h] = row_l * 128 + mq * mt_bytes + (((h * 4 + t) << 4) ^ sw);
         at.up[h] = row_l * 128 + mq * mt_bytes + (g.upper ? s.rows_run * 128 : 128) + (((h * 4 + t) << 4) ^ sw_up);
     }
+    const bool codes = W4 && !head;
+    if (W4 && codes) {
+        const int mt_rows = g.upper ? 8 : 16, row = row_l + mq * mt_rows;
+        at.kb_bytes = w4_kb_bytes(s.row0, s.rows_run, g.upper ? 2 : 1);
+        at.mt_stride = g.mg * mt_rows * 16;
+        at.exp_stride = g.mg * mt_rows;
+        at.exp_lo = s.rows * 32 + (s.row0 & 15) + row;
+        at.exp_up = at.exp_lo + (g.upper ? exp_chunks(s.row0, s.rows_run) * 16 : 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            at.lo[h] = (h * s.rows_run + row) * 16 + t * 4;
+            at.up[h] = at.lo[h] + (g.upper ? s.rows_run * 32 : 16);
+        }
+    }
     if (part == 0 && !wait_ready(e, c)) return;
     if (s.U > 0) {
         // requested now, used behind the main loop: the sums of squares of a node per warp
@@ -474,9 +626,13 @@ __device__ __forceinline__ void gemm_phase(const Env &e, Consumer &c, int kind, 
         const Walk walk{smem_u32(&e.ctl.full[0]), smem_u32(&e.ctl.empty[0]), e.ring, e.ring + p.x_off + e.lane * 16, smem_u32(&e.ctl.xfull[0]),
                         smem_u32(&e.ctl.xempty[0]), p.slots, p.slot_bytes, p.x_stage_bytes, g.kg, g.kb_item, g.kb_all, g.n_items,
                         g.K / 32, g.x_kb, C * 128};
-        if (mtn == 2) c.ok = gemm_walk<2>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
-        else if (mtn == 3) c.ok = gemm_walk<3>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
-        else c.ok = gemm_walk<1>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);      // (no tile at all: a tile of other data)
+        if (W4 && codes) {
+            if (mtn == 2) c.ok = gemm_walk<2, CodeBlock<2>>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+            else if (mtn == 3) c.ok = gemm_walk<3, CodeBlock<3>>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+            else c.ok = gemm_walk<1, CodeBlock<1>>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+        } else if (mtn == 2) c.ok = gemm_walk<2, Block<2>>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+        else if (mtn == 3) c.ok = gemm_walk<3, Block<3>>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);
+        else c.ok = gemm_walk<1, Block<1>>(acc, at, walk, kq, c.at, c.xs, e.ctl, p.wait_limit_ns, e.lane);      // (no tile at all: a tile of other data)
         if (!c.ok) return;
         c.at.add(g.n_items, p.slots);
 
@@ -788,6 +944,7 @@ __device__ __forceinline__ void attention_phase(const Env &e, Consumer &c, int l
     arrive_grid(e, c);
 }
 
+template <bool W4>
 __device__ __forceinline__ void consume(const Env &e, Consumer &c)
 {
     const StreamPass &p = e.p;
@@ -819,7 +976,7 @@ __device__ __forceinline__ void consume(const Env &e, Consumer &c)
         const int steps = l < p.L ? 5 : p.logits != nullptr ? p.head_parts : 0;
         for (int st = 0; st < steps && c.ok; ++st) {
             if (l < p.L && st == 1) attention_phase(e, c, l);
-            else gemm_phase(e, c, l < p.L ? gemm_kind(st) : SG_HEAD, l, l < p.L ? 0 : st);
+            else gemm_phase<W4>(e, c, l < p.L ? gemm_kind(st) : SG_HEAD, l, l < p.L ? 0 : st);
         }
     }
 }
@@ -865,7 +1022,8 @@ __device__ __forceinline__ bool load_inputs(const StreamPass &p, Ctl &ctl, uint3
     return true;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool W4>
+__global__ void __launch_bounds__(kThreads<W4>, 1)
 stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__ CUtensorMap kv_map)
 {
     extern __shared__ uint8_t sm_raw[];
@@ -873,13 +1031,13 @@ stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__
     const uint32_t raw = smem_u32(sm_raw), base = (raw + 1023u) & ~1023u;     // swizzled tiles want 1024-byte alignment
     uint8_t *smp = sm_raw + (base - raw);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    Producer prod(p, &kv_map, ctl, base);
+    Producer<W4> prod(p, &kv_map, ctl, base);
     if (warp == kWarps) {
         if (lane < SG_HEAD + p.head_parts) ctl.share[lane] = lane < SG_HEAD ? share_of(p.g[lane]) : part_of(share_of(p.g[SG_HEAD]), lane - SG_HEAD, p.head_parts);
         if (lane == 31) ctl.attn = attn_share(p);
         if (lane == 0) {
             for (int s = 0; s < kMaxSlots; ++s) {
-                mbar_init(smem_u32(&ctl.full[s]), 1);
+                mbar_init(smem_u32(&ctl.full[s]), W4 ? 32 : 1);
                 mbar_init(smem_u32(&ctl.empty[s]), kWarps);
             }
             for (int s = 0; s < kXStages; ++s) {
@@ -895,7 +1053,7 @@ stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__
         }
     }
     __syncthreads();
-    const bool producer = warp >= kWarps && warp < kWarps + kProducers;
+    const bool producer = warp >= kWarps && warp < kWarps + kProducers<W4>;
     if (producer) {
         prod.start();
         while (!prod.done() && prod.free_now()) prod.fetch();
@@ -912,11 +1070,11 @@ stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__
     if (err || stands) {
         // nothing to do but to let the weights land: the first turn of this producer's slots
         if (producer)
-            for (int i = 0; i < prod.issued && ok; ++i) ok = wait_all(smem_u32(&ctl.full[warp - kWarps + i * kProducers]), 0, ctl, p.wait_limit_ns);
+            for (int i = 0; i < prod.issued && ok; ++i) ok = wait_all(smem_u32(&ctl.full[warp - kWarps + i * prod.step]), 0, ctl, p.wait_limit_ns);
     } else if (warp < kWarps) {
         Env e{p, ctl, base, reinterpret_cast<float *>(smp + p.red_off), reinterpret_cast<float2 *>(smp + p.cs_off), p.n_tree - p.n_old, warp, lane};
         Consumer c;
-        consume(e, c);
+        consume<W4>(e, c);
         ok = c.ok;
     } else if (producer) {
         while (!prod.done()) {
@@ -928,6 +1086,7 @@ stream_pass_kernel(const __grid_constant__ StreamPass p, const __grid_constant__
         ok = load_inputs(p, ctl, base + (uint32_t)p.x_off);
     }
     __syncwarp();
+    if (W4) asm volatile("cp.async.wait_all;" ::: "memory");
     if (!ok) {
         ctl.abort_flag = 1;
         atomicCAS(p.status, 0, LLMCAD_ERR_TIMEOUT);
@@ -1024,11 +1183,11 @@ bool plan_stream_pass(StreamPass &p, int n_sms)
     // The ring: slots of one size, the one that leaves most weights in flight on average over a layer's GEMMs. An item has
     // as many k-blocks as fit (and as there are lanes for, a copy each).
     const int ring = (int)((kStreamSmem - red - cs) / 1024 * 1024) - kXStages * p.x_stage_bytes;
-    auto item_kb = [&](int i, int slot) {
+    auto item_kb = [&](int i, int slot, bool codes) {
         const bool two = p.g[i].upper != 0;
-        const int runs = (two ? 2 : 1) * ((((two ? 1 : 2) * U[i] + 126) >> 7) + 1);
-        int kb = slot / (U[i] * 256);
-        for (int most_kb : {32 / runs, kMaxItemKb, kbs[i]}) kb = kb < most_kb ? kb : most_kb;
+        const int rows_run = (two ? 1 : 2) * U[i], runs = (two ? 2 : 1) * (((rows_run + 126) >> 7) + 1);
+        int kb = slot / (codes ? w4_kb_bytes(15, rows_run, two ? 2 : 1) : U[i] * 256);
+        for (int most_kb : {codes ? kMaxItemKbW4 : 32 / runs, codes ? kMaxItemKbW4 : kMaxItemKb, kbs[i]}) kb = kb < most_kb ? kb : most_kb;
         return kb;
     };
     double best = 0;
@@ -1037,21 +1196,22 @@ bool plan_stream_pass(StreamPass &p, int n_sms)
         if (slots > kMaxSlots) slots = kMaxSlots;
         double time = 0, bytes = 0;
         for (int i = 0; i < SG_HEAD; ++i) {
-            const int kb = item_kb(i, slot);
+            // (also with INT4 weights a slot has room for a k-block in bf16: both take the same models)
+            const int kb = item_kb(i, slot, false) == 0 ? 0 : item_kb(i, slot, p.w4 != 0);
             if (kb == 0) { time = 1e30; break; }
             const double all = (double)units[i] * kbs[i];
             bytes += all;
             time += all / ((double)slots * kb * U[i]);
         }
-        if (item_kb(SG_HEAD, slot) == 0 || bytes / time <= best) continue;
+        if (item_kb(SG_HEAD, slot, false) == 0 || bytes / time <= best) continue;
         best = bytes / time;
         p.slot_bytes = slot;
         p.slots = slots;
     }
-    if (best == 0 || p.slots < kProducers) return false;
+    if (best == 0 || p.slots < kProducers<false>) return false;
     for (int i = 0; i < SG_KINDS; ++i) {
         StreamGemm &g = p.g[i];
-        g.kb_item = item_kb(i, p.slot_bytes);
+        g.kb_item = item_kb(i, p.slot_bytes, p.w4 && i != SG_HEAD);
         g.n_items = (g.kb_all + g.kb_item - 1) / g.kb_item;
     }
     p.x_off = ring;
@@ -1072,13 +1232,15 @@ cudaError_t launch_stream_pass(const StreamPass &p, int n_sms, cudaStream_t st)
 
     static PerDeviceOnce attr_set;
     if (attr_set.needed()) {
-        const cudaError_t e = cudaFuncSetAttribute(stream_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem + 1024);
-        if (e != cudaSuccess) return e;
+        for (auto k : {stream_pass_kernel<false>, stream_pass_kernel<true>}) {
+            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem + 1024);
+            if (e != cudaSuccess) return e;
+        }
         attr_set.mark();
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_sms);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(p.w4 ? kThreads<true> : kThreads<false>);
     cfg.dynamicSmemBytes = kStreamSmem + 1024;
     cfg.stream = st;
     cudaLaunchAttribute attr;
@@ -1086,7 +1248,7 @@ cudaError_t launch_stream_pass(const StreamPass &p, int n_sms, cudaStream_t st)
     attr.val.cooperative = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, stream_pass_kernel, p, map);
+    return cudaLaunchKernelEx(&cfg, p.w4 ? stream_pass_kernel<true> : stream_pass_kernel<false>, p, map);
 }
 
 }  // namespace llmcad

@@ -30,6 +30,7 @@ struct StreamPass {
     size_t w_off[SG_KINDS];             // inside a layer; SG_HEAD: from the base
     size_t attn_norm, ffn_norm, layer_bytes, tok_embed, final_norm;
     StreamGemm g[SG_KINDS];
+    int w4;                             // the layer matrices are INT4 tiles
     char *kv;
     const double *inv_freq;
     // the tree: the nodes n_old .. n_tree-1 are computed

@@ -106,6 +106,44 @@ def test_int4_pass_against_oracle_and_against_bf16_over_dequantised_weights(case
     assert layer_bytes(c4) < 0.27 * layer_bytes(c16)
 
 
+FEW = {"small": gen.ModelConfig("small-bf16", 2, 512, 4, 128, 1408, 2048, "bf16"), "one-head": gen.ModelConfig("one-head", 1, 128, 1, 128, 320, 512, "bf16"),
+       "odd": gen.ModelConfig("odd", 3, 640, 5, 128, 1344, 2051, "bf16"), "7b": gen.shrink(gen.MODELS["7b"], 1), "30b": gen.shrink(gen.MODELS["30b"], 1)}
+
+
+@pytest.mark.parametrize("model,P,ns", [("one-head", 33, (1, 4)), ("odd", 0, (2, 3)), ("odd", 700, (1, 2, 3, 4, 5)), ("small", 300, (1, 4, 5)), ("7b", 129, (1, 4)), ("30b", 40, (3,))])
+def test_int4_passes_over_few_nodes(model, P, ns):
+    """Up to four nodes go through the one-kernel pass in both contexts: the same bits, as from five on; and the oracle's logits.
+    The same of the nodes that extend a tree and of prompts that are or end in a few tokens."""
+    cfg = FEW[model]
+    twin = Int4Twin(cfg, P + 24, scale=3.0 if cfg.d_model < 1024 else 1.0, seed=P)
+    twin.fill_prefix_synthetic(P)
+    both = (twin.v, twin.v16)
+    twin.v16.kv_view()[:, :, :, :P] = twin.v.kv_view()[:, :, :, :P]
+    dev = lambda a: torch.as_tensor(np.asarray(a, np.int32), device=DEV)
+    for n in ns:
+        parent = gen.tree_random(n, 4, "uniform4", n) if n > 1 else np.array([-1], np.int32)
+        tokens = gen.gen_tokens(cfg, n, seed=n)
+        ref = twin.oracle_pass(P, tokens, parent)
+        out = [v.verify_tree(P, dev(tokens), dev(parent)) for v in both]
+        for key in ("logits", "argmax", "scalars", "accepted_path"):
+            assert torch.equal(out[0][key], out[1][key]), (n, key)
+        host = {k: t.cpu().numpy() for k, t in out[0].items()}
+        logits_close(host["logits"], ref.logits, 1e-3)
+        check_acceptance_against_oracle(host, tokens, parent)
+        length = int(host["scalars"][B.S_ACCEPTED_LEN])
+        assert torch.equal(twin.v.kv_view()[:, :, :, :P + length], twin.v16.kv_view()[:, :, :, :P + length]), n
+    n = 12
+    parent, tokens = dev(gen.tree_random(n, 6, "uniform4", n)), dev(gen.gen_tokens(cfg, n, seed=n))
+    for old, new in ((0, 3), (3, 9), (9, 10), (10, 12)):
+        a, b = (v.extend_tree(P, tokens[:new], parent[:new], old, top_k=3) for v in both)
+        assert all(torch.equal(a[key], b[key]) for key in a), (old, new)
+    for start, count in ((P, 3), (P + 3, 1), (P + 4, 16)):
+        a, b = (v.prefill(start, tokens.repeat(2)[:count], want_logits=True) for v in both)
+        assert torch.equal(a, b), count
+    assert torch.equal(twin.v.kv_view()[:, :, :, :P + 20], twin.v16.kv_view()[:, :, :, :P + 20])
+    assert twin.v.last_status() == 0 and twin.v16.last_status() == 0
+
+
 def test_int4_contexts_are_refused_where_they_cannot_work():
     import ctypes
     h = ctypes.c_void_p()
