@@ -16,6 +16,11 @@
  *   - `stream` arguments are a cudaStream_t passed as void*. Calls enqueue work on
  *     that stream and return without synchronising unless stated otherwise.
  *   - A context is not thread-safe and serves one stream at a time.
+ *   - Passes over up to four new nodes (bf16 and INT4 weights), and fp32 passes of small models, run as one kernel that takes
+ *     every SM at once: alone they are faster, but work on other streams waits meanwhile instead of filling gaps. A
+ *     bf16 context that is to run beside others, a draft model's next to the target's, can be created with
+ *     LLMCAD_FLAG_MMA_ATTN, which keeps one kernel per step. Streams that have only some of the device's SMs (green contexts)
+ *     take the kernels per step by themselves.
  *   - Return value: LLMCAD_OK or a negative host-detected error. Errors found on
  *     the device (malformed tree, token id out of range, a wait that ran out) are
  *     written to scalars[LLMCAD_S_STATUS]; all later phases of that pass then do

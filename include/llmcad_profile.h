@@ -16,13 +16,16 @@ extern "C" {
 /* Per-launch timing of kernels in isolation. While enabled, every skinny-GEMM launch (kind 0) and
  * every tree-attention launch (kind 1) of this context is bracketed by CUDA events on the
  * launching stream (which keeps consecutive kernels from overlapping under programmatic dependent
- * launch: the figures are those of a kernel running alone). llmcad_get_kernel_timing waits for the
+ * launch: the figures are those of a kernel running alone). Passes that are one kernel otherwise (fp32 passes of small
+ * models, bf16 and INT4 passes over up to four new nodes) go through the kernels per step while this is on, so that there is
+ * something to time; their results then differ in the last bits. llmcad_get_kernel_timing waits for the
  * recorded launches of `kind`, returns their summed duration and count since the last query, and
  * forgets them. */
 int llmcad_set_kernel_timing(llmcad_ctx *ctx, int32_t enable);
 int llmcad_get_kernel_timing(llmcad_ctx *ctx, int32_t kind, double *total_ms /*HOST*/, int64_t *n_launches /*HOST*/);
 
-/* Timeline of the kernels inside an undisturbed pass. While `trace` (DEVICE, [capacity][256][16]
+/* Timeline of the kernels inside an undisturbed pass (of five new nodes or more; with fewer a traced bf16 or INT4 pass goes through
+ * the kernels per step, as above). While `trace` (DEVICE, [capacity][256][16]
  * uint64, or NULL to stop) is set, the next `capacity` tensor-core GEMMs and attention launches of
  * this context each fill one [256][16] slice: per CTA, nanosecond timestamps (%globaltimer). A GEMM
  * (streaming kernel + finishing kernel) shares one slice: streaming CTA entry (0), set-up done (1),
